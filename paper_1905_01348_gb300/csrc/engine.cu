@@ -269,25 +269,45 @@ static pt_status exchange_x_t(pt_system* sys, const double2* X, int ncols, doubl
   return to_basis<T>(sys, fv, sys->w_r, ncols, out, 1, nullptr, nullptr);
 }
 
-template <typename Tc>
 static pt_status gemm(pt_system* sys, int opA, int opB, int M, int N, int K, double2 alpha, const double2* A, long lda,
                       const double2* B, long ldb, double2 beta, double2* C, long ldc,
                       int structure = pt::GEMM_GENERAL) {
-  PT_CK(pt::gemm<Tc>(opA, opB, M, N, K, alpha, A, lda, 0, B, ldb, 0, beta, C, ldc, 0, 1, sys->gemm_ws,
-                     sys->gemm_ws_elems, sys->s, structure));
+  PT_CK(pt::gemm64(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sys->gemm_ws, sys->gemm_ws_elems, sys->s,
+                   structure));
   return PT_OK;
 }
 
 static const double2 kOne = {1.0, 0.0}, kZero = {0.0, 0.0}, kMinusOne = {-1.0, 0.0};
 
-// Product of complex64 copies on the tensor cores (mixed precision, 3xTF32 with FP32
-// accumulation); C stays complex128. A bounded wait that expires inside the kernel sets
-// status[4], which tc_status() reports.
-static pt_status gemm32(pt_system* sys, int opA, int opB, int M, int N, int K, double2 alpha, const float2* A, long lda,
-                        const float2* B, long ldb, double2 beta, double2* C, long ldc,
-                        int structure = pt::GEMM_GENERAL) {
-  PT_CK(pt::gemm_tc(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, sys->gemm_ws, sys->gemm_ws_elems,
-                    sys->status + 4, sys->s, structure));
+static pt_status to32(pt_system* sys, const double2* src, float2* dst, long n) {
+  PT_CK(pt::convert_c128_to_c64(src, dst, n, sys->s));
+  return PT_OK;
+}
+
+// A complex128 operand of a mixed-precision product (`count` values) and the place of its
+// complex64 copy; `ready` when the copy is there already.
+struct Operand32 {
+  const double2* p;
+  float2* copy;
+  long ld, count;
+  bool ready;
+};
+
+// Mixed-precision product, C complex128: on the tensor cores from complex64 copies of the
+// operands (3xTF32 with FP32 accumulation), made here where they are not ready; outputs too
+// small for those tiles go to the FP32 CUDA-core kernel, which rounds as it reads. A bounded
+// wait that expires inside the kernel sets status[4], which tc_status() reports.
+static pt_status gemm32(pt_system* sys, int opA, int opB, int M, int N, int K, double2 alpha, const Operand32& A,
+                        const Operand32& B, double2 beta, double2* C, long ldc, int structure = pt::GEMM_GENERAL) {
+  if (pt::tc_too_small(M, N)) {
+    PT_CK(pt::gemm32_small(opA, opB, M, N, K, alpha, A.p, A.ld, B.p, B.ld, beta, C, ldc, sys->gemm_ws,
+                           sys->gemm_ws_elems, sys->s, structure));
+    return PT_OK;
+  }
+  if (!A.ready) PT_TRY(to32(sys, A.p, A.copy, A.count));
+  if (!B.ready) PT_TRY(to32(sys, B.p, B.copy, B.count));
+  PT_CK(pt::gemm_tc(opA, opB, M, N, K, alpha, A.copy, A.ld, B.copy, B.ld, beta, C, ldc, sys->gemm_ws,
+                    sys->gemm_ws_elems, sys->status + 4, sys->s, structure));
   return PT_OK;
 }
 
@@ -334,11 +354,6 @@ pt_status tc_status(pt_system* sys) {
   return PT_OK;
 }
 
-static pt_status to32(pt_system* sys, const double2* src, float2* dst, long n) {
-  PT_CK(pt::convert_c128_to_c64(src, dst, n, sys->s));
-  return PT_OK;
-}
-
 // SCF-iteration forms. In mixed precision the real-space orbitals, the
 // density they give and the local-potential product run in FP32; in FP64
 // mode these are the FP64 routines above.
@@ -376,19 +391,20 @@ pt_status apply_local_scf(pt_system* sys, const double2* c, double2* out) {
   return PT_OK;
 }
 
-// S = A^H B and C -= A S (the PT projection, Alg. 3): on the tensor cores in mixed
-// precision unless fp64 is asked for (refinement iterations)
-pt_status projection(pt_system* sys, const double2* A, double2* HB, bool fp64) {
+// S = A^H HB and HB -= A S (the PT projection, Alg. 3): in mixed precision unless fp64 is
+// asked for (refinement iterations). a_ready: ga32 holds the complex64 copy of A.
+pt_status projection(pt_system* sys, const double2* A, double2* HB, bool fp64, bool a_ready) {
   const int ne = sys->ne, npw = sys->npw;
+  const long n = (long)npw * ne;
   if (sys->mixed && !fp64) {
-    PT_TRY(to32(sys, A, sys->ga32, (long)npw * ne));
-    PT_TRY(to32(sys, HB, sys->gb32, (long)npw * ne));
-    PT_TRY(gemm32(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, sys->ga32, npw, sys->gb32, npw, kZero, sys->S, ne));
-    PT_TRY(to32(sys, sys->S, sys->gs32, (long)ne * ne));
-    PT_TRY(gemm32(sys, pt::OP_N, pt::OP_N, npw, ne, ne, kMinusOne, sys->ga32, npw, sys->gs32, ne, kOne, HB, npw));
+    Operand32 a{A, sys->ga32, npw, n, a_ready};
+    const Operand32 b{HB, sys->gb32, npw, n, false}, t{sys->S, sys->gs32, ne, (long)ne * ne, false};
+    PT_TRY(gemm32(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, a, b, kZero, sys->S, ne));
+    a.ready = a_ready || !pt::tc_too_small(ne, ne);
+    PT_TRY(gemm32(sys, pt::OP_N, pt::OP_N, npw, ne, ne, kMinusOne, a, t, kOne, HB, npw));
   } else {
-    PT_TRY(gemm<double>(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, A, npw, HB, npw, kZero, sys->S, ne));
-    PT_TRY(gemm<double>(sys, pt::OP_N, pt::OP_N, npw, ne, ne, kMinusOne, A, npw, sys->S, ne, kOne, HB, npw));
+    PT_TRY(gemm(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, A, npw, HB, npw, kZero, sys->S, ne));
+    PT_TRY(gemm(sys, pt::OP_N, pt::OP_N, npw, ne, ne, kMinusOne, A, npw, sys->S, ne, kOne, HB, npw));
   }
   return PT_OK;
 }
@@ -399,14 +415,13 @@ pt_status read_status(pt_system* sys, int* h) { return read_small(sys, h, sys->s
 pt_status orthonormalize(pt_system* sys, const double2* src, double2* dst) {
   Phase phase_("orthonormalize");
   const int ne = sys->ne, npw = sys->npw;
-  PT_TRY(gemm<double>(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, src, npw, src, npw, kZero, sys->S, ne,
+  PT_TRY(gemm(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, src, npw, src, npw, kZero, sys->S, ne,
                       pt::GEMM_HERM));
-  PT_CK(pt::cholesky(sys->S, ne, sys->status, sys->s));
+  PT_CK(pt::cholesky_inverse(sys->S, sys->Linv, ne, sys->status, sys->s));
   int h = 0;
   PT_TRY(read_status(sys, &h));
   if (h != 0) { sys->err = "orthonormalisation: overlap matrix is not positive definite"; return PT_ERR_NOT_PD; }
-  PT_CK(pt::tri_inverse(sys->S, sys->Linv, ne, sys->s));
-  PT_TRY(gemm<double>(sys, pt::OP_N, pt::OP_H, npw, ne, ne, kOne, src, npw, sys->Linv, ne, kZero, dst, npw,
+  PT_TRY(gemm(sys, pt::OP_N, pt::OP_H, npw, ne, ne, kOne, src, npw, sys->Linv, ne, kZero, dst, npw,
                       pt::GEMM_TRI_B));
   return PT_OK;
 }
@@ -419,29 +434,28 @@ pt_status ace_from_w(pt_system* sys, const double2* psi_src) {
   const int ne = sys->ne, npw = sys->npw;
   const bool ace = sys->p.fock_mode == PT_FOCK_ACE && sys->p.alpha != 0.0;
   const double2* psi = psi_src ? psi_src : sys->psi;
-  if (sys->mixed && ace) {
-    PT_TRY(to32(sys, psi, sys->ga32, (long)npw * ne));
-    PT_TRY(to32(sys, sys->wg, sys->gb32, (long)npw * ne));
-    PT_TRY(gemm32(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kMinusOne, sys->ga32, npw, sys->gb32, npw, kZero, sys->Mneg, ne));
-  } else
-    PT_TRY(gemm<double>(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kMinusOne, psi, npw, sys->wg, npw, kZero, sys->Mneg, ne));
+  const long n = (long)npw * ne;
+  if (sys->mixed && ace)
+    PT_TRY(gemm32(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kMinusOne, Operand32{psi, sys->ga32, npw, n, false},
+                  Operand32{sys->wg, sys->gb32, npw, n, false}, kZero, sys->Mneg, ne));
+  else
+    PT_TRY(gemm(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kMinusOne, psi, npw, sys->wg, npw, kZero, sys->Mneg, ne));
   sys->have_ace = false;
   if (!ace) return PT_OK;
   PT_CK(cudaMemcpyAsync(sys->S, sys->Mneg, sizeof(double2) * ne * ne, cudaMemcpyDeviceToDevice, sys->s));
-  PT_CK(pt::cholesky(sys->S, ne, sys->status, sys->s));
+  PT_CK(pt::cholesky_inverse(sys->S, sys->Linv, ne, sys->status, sys->s));
   int h = 0;
   PT_TRY(read_status(sys, &h));
   if (h != 0) { sys->err = "ACE: -M is not positive definite"; return PT_ERR_NOT_PD; }
-  PT_CK(pt::tri_inverse(sys->S, sys->Linv, ne, sys->s));
   if (sys->mixed) {
-    // W is still in gb32; xi and its complex64 copy for the FP32 ACE products
-    PT_TRY(to32(sys, sys->Linv, sys->gs32, (long)ne * ne));
-    PT_TRY(gemm32(sys, pt::OP_N, pt::OP_H, npw, ne, ne, kOne, sys->gb32, npw, sys->gs32, ne, kZero, sys->xi, npw,
-                  pt::GEMM_TRI_B));
-    PT_TRY(to32(sys, sys->xi, sys->xi32, (long)npw * ne));
+    // xi and its complex64 copy for the tensor-core products; W may still be in gb32
+    PT_TRY(gemm32(sys, pt::OP_N, pt::OP_H, npw, ne, ne, kOne,
+                  Operand32{sys->wg, sys->gb32, npw, n, !pt::tc_too_small(ne, ne)},
+                  Operand32{sys->Linv, sys->gs32, ne, (long)ne * ne, false}, kZero, sys->xi, npw, pt::GEMM_TRI_B));
+    PT_TRY(to32(sys, sys->xi, sys->xi32, n));
   } else
-    PT_TRY(gemm<double>(sys, pt::OP_N, pt::OP_H, npw, ne, ne, kOne, sys->wg, npw, sys->Linv, ne, kZero, sys->xi, npw,
-                        pt::GEMM_TRI_B));
+    PT_TRY(gemm(sys, pt::OP_N, pt::OP_H, npw, ne, ne, kOne, sys->wg, npw, sys->Linv, ne, kZero, sys->xi, npw,
+                pt::GEMM_TRI_B));
   sys->have_ace = true;
   return PT_OK;
 }
@@ -458,13 +472,14 @@ pt_status exchange_data(pt_system* sys) {
 pt_status ace_apply(pt_system* sys, const double2* X, int ncols, double2* out, bool fp64) {
   const int ne = sys->ne, npw = sys->npw;
   if (sys->mixed && !fp64) {
-    PT_TRY(to32(sys, X, sys->ga32, (long)npw * ncols));
-    PT_TRY(gemm32(sys, pt::OP_H, pt::OP_N, ne, ncols, npw, kOne, sys->xi32, npw, sys->ga32, npw, kZero, sys->Z, ne));
-    PT_TRY(to32(sys, sys->Z, sys->gs32, (long)ne * ncols));
-    PT_TRY(gemm32(sys, pt::OP_N, pt::OP_N, npw, ncols, ne, kMinusOne, sys->xi32, npw, sys->gs32, ne, kOne, out, npw));
+    const Operand32 xi{sys->xi, sys->xi32, npw, (long)npw * ne, true};
+    PT_TRY(gemm32(sys, pt::OP_H, pt::OP_N, ne, ncols, npw, kOne, xi,
+                  Operand32{X, sys->ga32, npw, (long)npw * ncols, false}, kZero, sys->Z, ne));
+    PT_TRY(gemm32(sys, pt::OP_N, pt::OP_N, npw, ncols, ne, kMinusOne, xi,
+                  Operand32{sys->Z, sys->gs32, ne, (long)ne * ncols, false}, kOne, out, npw));
   } else {
-    PT_TRY(gemm<double>(sys, pt::OP_H, pt::OP_N, ne, ncols, npw, kOne, sys->xi, npw, X, npw, kZero, sys->Z, ne));
-    PT_TRY(gemm<double>(sys, pt::OP_N, pt::OP_N, npw, ncols, ne, kMinusOne, sys->xi, npw, sys->Z, ne, kOne, out, npw));
+    PT_TRY(gemm(sys, pt::OP_H, pt::OP_N, ne, ncols, npw, kOne, sys->xi, npw, X, npw, kZero, sys->Z, ne));
+    PT_TRY(gemm(sys, pt::OP_N, pt::OP_N, npw, ncols, ne, kMinusOne, sys->xi, npw, sys->Z, ne, kOne, out, npw));
   }
   return PT_OK;
 }
@@ -503,8 +518,8 @@ pt_status relax(pt_system* sys) {
     PT_TRY(kerker_mix(sys));
     PT_TRY(local_potential(sys, sys->rho_mix));
     PT_TRY(apply_local_from_real(sys, sys->psi, sys->hpsi));
-    PT_TRY(gemm<double>(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, sys->psi, npw, sys->hpsi, npw, kZero, sys->S, ne));
-    PT_TRY(gemm<double>(sys, pt::OP_N, pt::OP_N, npw, ne, ne, kMinusOne, sys->psi, npw, sys->S, ne, kOne, sys->hpsi, npw));
+    PT_TRY(gemm(sys, pt::OP_H, pt::OP_N, ne, ne, npw, kOne, sys->psi, npw, sys->hpsi, npw, kZero, sys->S, ne));
+    PT_TRY(gemm(sys, pt::OP_N, pt::OP_N, npw, ne, ne, kMinusOne, sys->psi, npw, sys->S, ne, kOne, sys->hpsi, npw));
     PT_CK(pt::precond_step(sys->psi, sys->hpsi, sys->kin, npw, n, sys->p.relax_tau, sys->s));
     PT_TRY(orthonormalize(sys, sys->psi, sys->psi_f));
     std::swap(sys->psi, sys->psi_f);
@@ -615,7 +630,10 @@ pt_status cn_iterate(pt_system* sys, StepCtx* c) {
   }
   {
     Phase p_("PT residual");
-    PT_TRY(projection(sys, sys->psi_f, sys->hpsi, hi));
+    // the ACE product has left the complex64 copy of psi_f in ga32
+    const bool copied = sys->mixed && !hi && sys->p.alpha != 0.0 && sys->p.fock_mode == PT_FOCK_ACE &&
+                        !pt::tc_too_small(ne, ne);
+    PT_TRY(projection(sys, sys->psi_f, sys->hpsi, hi, copied));
     PT_CK(pt::pt_residual(sys->psi_f, sys->hpsi, sys->psi_half, hdt, sys->rbuf, n, sys->part, sys->red + 0, sys->s));
   }
   // Anderson (per band)

@@ -187,7 +187,7 @@ pt_status read_small(pt_system* sys, void* dst, const void* d_src, size_t bytes)
 // kept until exit: freeing page-locked memory can synchronise the device)
 void* pinned_block_get();
 void pinned_block_put(void* block);
-pt_status projection(pt_system* sys, const double2* A, double2* HB, bool fp64 = false);
+pt_status projection(pt_system* sys, const double2* A, double2* HB, bool fp64 = false, bool a_ready = false);
 pt_status orthonormalize(pt_system* sys, const double2* src, double2* dst);
 pt_status ace_from_w(pt_system* sys, const double2* psi_src = nullptr);
 pt_status exchange_data(pt_system* sys);

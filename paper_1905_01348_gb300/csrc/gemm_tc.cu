@@ -387,6 +387,12 @@ static cudaError_t launch_tc(int M, int N, int K, int kchunk, int ksplit, int tr
   return cudaGetLastError();
 }
 
+// An output that would leave most of its 128 x 128 tiles empty.
+bool tc_too_small(long M, long N) {
+  const long tiles = ((M + TC_M - 1) / TC_M) * ((N + TC_NC - 1) / TC_NC);
+  return tiles * TC_M * TC_NC > 3 * ((M + 15) / 16 * 16) * ((N + 15) / 16 * 16);
+}
+
 cudaError_t gemm_tc(int opA, int opB, int M, int N, int K, double2 alpha, const float2* A, long lda, const float2* B,
                     long ldb, double2 beta, double2* C, long ldc, double2* ws, size_t ws_elems, int* d_err,
                     cudaStream_t s, int structure) {
@@ -394,20 +400,14 @@ cudaError_t gemm_tc(int opA, int opB, int M, int N, int K, double2 alpha, const 
   if (structure == GEMM_HERM || d_err == nullptr) return cudaErrorInvalidValue;
   const int tri_b = structure == GEMM_TRI_B ? 1 : 0;
   const long tiles = (long)((M + TC_M - 1) / TC_M) * ((N + TC_NC - 1) / TC_NC);
-  // split the reduction over the basis so that the tiles fill the SMs (one CTA each) about once
-  static std::atomic<int> sm_count[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-  int sms = sm_count[dev & 63].load(std::memory_order_relaxed);
-  if (sms == 0) {
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    sms = std::max(1, sms);
-    sm_count[dev & 63].store(sms, std::memory_order_relaxed);
-  }
-  const long slots = sms;
+  if (tc_too_small(M, N))
+    return gemm32_small(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_elems, s, structure);
+  // split the reduction over the basis so that the tiles fill the SMs (one CTA each) about
+  // once, down to one accumulation window of 64 complex k per chunk
+  const long slots = sm_count();
   int ksplit = 1;
   if (K > 1024 && tiles < slots && ws != nullptr) {
-    ksplit = (int)std::max<long>(1, std::min<long>(slots / tiles, (K + 511) / 512));
+    ksplit = (int)std::max<long>(1, std::min<long>(slots / tiles, (K + 63) / 64));
     while (ksplit > 1 && (size_t)ksplit * M * N > ws_elems) --ksplit;
   }
   int kchunk = (K + ksplit - 1) / ksplit;

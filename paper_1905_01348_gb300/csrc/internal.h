@@ -140,18 +140,27 @@ int fock_build_tiles(int n_occ, int n_x, int tile, int sym, int tiles_per_launch
                      int** launch_first, int** launch_count, int* n_launch);
 
 // ---- dense linear algebra (linalg.cu) -------------------------------------
-// C(M x N) = alpha * op(A) op(B) + beta * C, complex, column-major, batched by strides.
+// C(M x N) = alpha * op(A) op(B) + beta * C, complex128, column-major, on the CUDA cores.
 // A element (i, k) of op(A) == N: A[i + k * lda]; == H: conj(A[k + i * lda]).
-// Inputs stored as complex128; Tc is the compute / accumulate precision.
 // structure: GEMM_HERM for C = A^H A (only the lower half is computed, the upper
 // half is its conjugate mirror); GEMM_TRI_B when op(B) is upper triangular.
 enum { OP_N = 0, OP_H = 1 };
 enum { GEMM_GENERAL = 0, GEMM_HERM = 1, GEMM_TRI_B = 2 };
-template <typename Tc>
-cudaError_t gemm(int opA, int opB, int M, int N, int K, double2 alpha, const double2* A, long lda, long strideA,
-                 const double2* B, long ldb, long strideB, double2 beta, double2* C, long ldc, long strideC,
-                 int batch, double2* splitk_ws, size_t splitk_ws_elems, cudaStream_t s,
-                 int structure = GEMM_GENERAL);
+cudaError_t gemm64(int opA, int opB, int M, int N, int K, double2 alpha, const double2* A, long lda, const double2* B,
+                   long ldb, double2 beta, double2* C, long ldc, double2* splitk_ws, size_t splitk_ws_elems,
+                   cudaStream_t s, int structure = GEMM_GENERAL);
+// The same with FP32 multiply-adds (FP64 sums over the split), for outputs too small for
+// the tensor-core tiles (tc_too_small): from complex64 operands, or from complex128 ones
+// rounded to complex64 as they are read.
+bool tc_too_small(long M, long N);
+cudaError_t gemm32_small(int opA, int opB, int M, int N, int K, double2 alpha, const float2* A, long lda,
+                         const float2* B, long ldb, double2 beta, double2* C, long ldc, double2* splitk_ws,
+                         size_t splitk_ws_elems, cudaStream_t s, int structure = GEMM_GENERAL);
+cudaError_t gemm32_small(int opA, int opB, int M, int N, int K, double2 alpha, const double2* A, long lda,
+                         const double2* B, long ldb, double2 beta, double2* C, long ldc, double2* splitk_ws,
+                         size_t splitk_ws_elems, cudaStream_t s, int structure = GEMM_GENERAL);
+// Multiprocessors of the current device.
+int sm_count();
 // The same product from complex64 copies of A and B on the tensor cores (gemm_tc.cu):
 // 3xTF32 with FP32 accumulation, C complex128; GEMM_GENERAL or GEMM_TRI_B. `d_err`
 // (device int) gets bit 0 set when a bounded wait inside the kernel expires.
@@ -161,12 +170,10 @@ cudaError_t gemm_tc(int opA, int opB, int M, int N, int K, double2 alpha, const 
 // C = alpha sum_kz part[kz] + beta C over ksplit partials part[(kz N + j) M + i], fixed order.
 cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const double2* part, double2 beta, double2* C,
                           long ldc, cudaStream_t s);
-// In-place lower Cholesky of an n x n Hermitian matrix (column-major, lower
-// triangle used and overwritten, upper set to 0). *d_status = 1 on a
-// non-positive pivot.
-cudaError_t cholesky(double2* A, int n, int* d_status, cudaStream_t s);
-// Linv = L^{-1} for lower-triangular L (n x n, column-major).
-cudaError_t tri_inverse(const double2* L, double2* Linv, int n, cudaStream_t s);
+// In-place lower Cholesky of an n x n Hermitian matrix (column-major, lower triangle
+// used and overwritten, upper set to 0) and Linv = L^{-1}. *d_status = 1 on a
+// non-positive pivot (A and Linv are then unfinished).
+cudaError_t cholesky_inverse(double2* A, double2* Linv, int n, int* d_status, cudaStream_t s);
 
 std::string cuda_msg(cudaError_t e);
 

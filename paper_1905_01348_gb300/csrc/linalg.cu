@@ -2,13 +2,12 @@
 //   overlap / projection products S = Psi^H (H Psi), Psi S (Alg. 3),
 //   M = Psi^H W, xi^H X, xi Y (ACE), Psi^H Psi and Psi L^{-H} (Sec. 3.4),
 //   Cholesky factorisations (orthonormalisation, -M of ACE) and L^{-1}.
-// GEMM: 64 x 64 output tiles, 256 threads with 4 x 4 complex micro-tiles,
-// operands staged in shared memory in the compute precision (double-buffered,
-// next slice prefetched into registers); the long reduction over the basis is
-// split over blocks (split-K) into a workspace and summed in a fixed order, so
-// results are deterministic. Hermitian products (Psi^H Psi) compute half the
-// tiles; products with a triangular factor stop the reduction at the diagonal.
+// GEMM: 16 x 16 output tiles on the CUDA cores; a long reduction is split over blocks
+// (split-K) into a workspace and summed in a fixed order, so results are deterministic.
+// Hermitian products (Psi^H Psi) compute half the tiles; products with a triangular
+// factor stop the reduction at the diagonal.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "common.cuh"
@@ -16,99 +15,72 @@
 
 namespace pt {
 
-constexpr int GBM = 64, GBN = 64;
-template <typename C> __device__ __forceinline__ C to_compute(double2 v) { return cvt<C>(v); }
-template <typename C> __device__ __forceinline__ C to_compute(float2 v);
-template <> __device__ __forceinline__ float2 to_compute<float2>(float2 v) { return v; }
-template <typename Tc> struct GemmK { static constexpr int V = 16; };
-template <> struct GemmK<double> { static constexpr int V = 8; };
-
 // Output structure the caller promises (skipped work is exactly zero or implied):
 //   GEMM_HERM   C = A^H A is Hermitian: only tiles on or below the diagonal are
 //               computed; the upper triangle is written as the conjugate mirror.
 //   GEMM_TRI_B  op(B) is upper triangular (op(B)[k][j] = 0 for k > j): the
-//               reduction for output columns [n0, n0 + 64) stops at n0 + 64.
-// One block computes a 64 x 64 tile over its K chunk with 256 threads (4 x 4
-// complex register tiles). The next K slice is fetched into registers while the
-// current one is multiplied from the other of two shared-memory buffers, so
-// there is one barrier per K slice. TI is the storage type of A and B
-// (complex128, or complex64 mirrors for FP32 products: converting FP64 inputs
-// inside the product loop would run every re-read element through the FP64
-// pipe, which on this GPU is as costly as the products themselves).
-template <typename Tc, typename TI>
-__global__ void __launch_bounds__(256) k_gemm(int opA, int opB, int M, int N, int K, int kchunk, int ksplit, int structure,
-                                              double2 alpha, const TI* __restrict__ A, long lda, long sA,
-                                              const TI* __restrict__ B, long ldb, long sB, double2 beta,
-                                              double2* __restrict__ Cm, long ldc, long sC,
-                                              double2* __restrict__ part) {
-  using C = cplx<Tc>;
-  constexpr int GK = GemmK<Tc>::V;
-  constexpr int PA = GBM * GK / 256;   // A elements per thread per slice
-  constexpr int PB = GBN * GK / 256;
-  __shared__ C As[2][GK][GBM + 1];
-  __shared__ C Bs[2][GK][GBN + 1];
+//               reduction for the output columns [n0, n0 + 16) stops at n0 + 16.
+//
+// One block of 64 threads computes a 16 x 16 tile over its K chunk, 2 x 2 complex values
+// per thread; the next K slice is fetched into registers while the current one is
+// multiplied from the other of two shared-memory buffers. In FP64 nothing but the
+// multiply-adds counts (an SM does two a clock, one warp instruction in 16 clocks), so
+// the small tile costs no time and saves the work of padding and of the skipped
+// triangle. FP32 (the small products of mixed precision) takes the same kernel: C is the
+// complex type of the arithmetic, TI that of A and B in memory.
+constexpr int GT = 16, GK = 16;
+
+template <typename C> __device__ __forceinline__ C mk_as(double2 v) { return cvt<C>(v); }
+template <typename C> __device__ __forceinline__ C mk_as(float2 v) { return v; }
+__device__ __forceinline__ double2 ld_op(const double2* p) { return *p; }
+__device__ __forceinline__ float2 ld_op(const float2* p) { return __ldg(p); }
+
+template <typename C, typename TI>
+__global__ void __launch_bounds__(64) k_gemm(int opA, int opB, int M, int N, int K, int kchunk, int ksplit, int structure,
+                                             double2 alpha, const TI* __restrict__ A, long lda,
+                                             const TI* __restrict__ B, long ldb, double2 beta,
+                                             double2* __restrict__ Cm, long ldc, double2* __restrict__ part) {
+  constexpr int P = GT * GK / 64;   // operand elements per thread per slice
+  __shared__ C As[2][GK][GT + 1];
+  __shared__ C Bs[2][GK][GT + 1];
   const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.x * GBM, n0 = blockIdx.y * GBN;
-  if (structure == GEMM_HERM && m0 + GBM <= n0) return;   // strictly above the diagonal
-  const int bz = blockIdx.z / ksplit, kz = blockIdx.z % ksplit;
-  const TI* Ab = A + (long)bz * sA;
-  const TI* Bb = B + (long)bz * sB;
+  const int tx = tid & 7, ty = tid >> 3;
+  const int m0 = blockIdx.x * GT, n0 = blockIdx.y * GT, kz = blockIdx.z;
+  if (structure == GEMM_HERM && m0 < n0) return;   // above the diagonal
   const int kbeg = kz * kchunk;
   int kend = min(K, kbeg + kchunk);
-  if (structure == GEMM_TRI_B) kend = min(kend, n0 + GBN);
-  C acc[4][4];
+  if (structure == GEMM_TRI_B) kend = min(kend, n0 + GT);
+  C acc[2][2];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = mk((Tc)0, (Tc)0);
-  C ra[PA], rb[PB];   // next slice, already in the compute precision
+    for (int b = 0; b < 2; ++b) acc[a][b] = C{};
+  C ra[P], rb[P];   // next slice
   auto fetch = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < PA; ++q) {
-      const int idx = tid + q * 256;
-      int i, k;
-      if (opA == OP_N) { i = idx % GBM; k = idx / GBM; }
-      else { k = idx % GK; i = idx / GK; }
-      const int gi = m0 + i, gk = k0 + k;
-      TI v{};
-      if (gi < M && gk < kend) {
-        if (opA == OP_N) v = Ab[gi + (long)gk * lda];
-        else { v = Ab[gk + (long)gi * lda]; v.y = -v.y; }
+    for (int q = 0; q < P; ++q) {
+      const int u = tid & 15, w = (tid >> 4) + 4 * q;   // u runs along the contiguous direction
+      const int ia = opA == OP_N ? u : w, ka = opA == OP_N ? w : u;
+      const int jb = opB == OP_N ? w : u, kb = opB == OP_N ? u : w;
+      TI va{}, vb{};
+      if (m0 + ia < M && k0 + ka < kend) {
+        if (opA == OP_N) va = ld_op(A + (m0 + ia) + (long)(k0 + ka) * lda);
+        else { va = ld_op(A + (k0 + ka) + (long)(m0 + ia) * lda); va.y = -va.y; }
       }
-      ra[q] = to_compute<C>(v);
-    }
-#pragma unroll
-    for (int q = 0; q < PB; ++q) {
-      const int idx = tid + q * 256;
-      int j, k;
-      if (opB == OP_N) { k = idx % GK; j = idx / GK; }
-      else { j = idx % GBN; k = idx / GBN; }
-      const int gj = n0 + j, gk = k0 + k;
-      TI v{};
-      if (gj < N && gk < kend) {
-        if (opB == OP_N) v = Bb[gk + (long)gj * ldb];
-        else { v = Bb[gj + (long)gk * ldb]; v.y = -v.y; }
+      if (n0 + jb < N && k0 + kb < kend) {
+        if (opB == OP_N) vb = ld_op(B + (k0 + kb) + (long)(n0 + jb) * ldb);
+        else { vb = ld_op(B + (n0 + jb) + (long)(k0 + kb) * ldb); vb.y = -vb.y; }
       }
-      rb[q] = to_compute<C>(v);
+      ra[q] = mk_as<C>(va);
+      rb[q] = mk_as<C>(vb);
     }
   };
   auto stash = [&](int buf) {
 #pragma unroll
-    for (int q = 0; q < PA; ++q) {
-      const int idx = tid + q * 256;
-      int i, k;
-      if (opA == OP_N) { i = idx % GBM; k = idx / GBM; }
-      else { k = idx % GK; i = idx / GK; }
-      As[buf][k][i] = ra[q];
-    }
-#pragma unroll
-    for (int q = 0; q < PB; ++q) {
-      const int idx = tid + q * 256;
-      int j, k;
-      if (opB == OP_N) { k = idx % GK; j = idx / GK; }
-      else { j = idx % GBN; k = idx / GBN; }
-      Bs[buf][k][j] = rb[q];
+    for (int q = 0; q < P; ++q) {
+      const int u = tid & 15, w = (tid >> 4) + 4 * q;
+      if (opA == OP_N) As[buf][w][u] = ra[q]; else As[buf][u][w] = ra[q];
+      if (opB == OP_N) Bs[buf][u][w] = rb[q]; else Bs[buf][w][u] = rb[q];
     }
   };
   int buf = 0;
@@ -120,82 +92,94 @@ __global__ void __launch_bounds__(256) k_gemm(int opA, int opB, int M, int N, in
   for (int k0 = kbeg; k0 < kend; k0 += GK) {
     const bool more = k0 + GK < kend;
     if (more) fetch(k0 + GK);   // in flight during the products below
+    auto one = [&](int k) {
+      C av[2], bv[2];
 #pragma unroll
-    for (int k = 0; k < GK; ++k) {
-      C av[4], bv[4];
+      for (int a = 0; a < 2; ++a) av[a] = As[buf][k][tx + 8 * a];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[buf][k][tx + 16 * a];
+      for (int b = 0; b < 2; ++b) bv[b] = Bs[buf][k][ty + 8 * b];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[buf][k][ty + 16 * b];
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
+        for (int b = 0; b < 2; ++b) {
           acc[a][b].x = fma(av[a].x, bv[b].x, acc[a][b].x);
           acc[a][b].x = fma(-av[a].y, bv[b].y, acc[a][b].x);
           acc[a][b].y = fma(av[a].x, bv[b].y, acc[a][b].y);
           acc[a][b].y = fma(av[a].y, bv[b].x, acc[a][b].y);
         }
+    };
+    if (kend - k0 >= GK) {
+#pragma unroll
+      for (int k = 0; k < GK; ++k) one(k);
+    } else {
+      for (int k = 0; k < kend - k0; ++k) one(k);
     }
     if (more) stash(buf ^ 1);
     __syncthreads();
     buf ^= 1;
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = m0 + tx + 16 * a, j = n0 + ty + 16 * b;
-      if (i < M && j < N) {
-        if (structure == GEMM_HERM && i < j) continue;   // mirrored from (j, i)
-        const double2 v = to_d(acc[a][b]);
-        if (ksplit > 1) {
-          part[(((long)kz * gridDim.z / ksplit + bz) * N + j) * (long)M + i] = v;
-        } else {
-          double2 r = make_double2(alpha.x * v.x - alpha.y * v.y, alpha.x * v.y + alpha.y * v.x);
-          double2* c = Cm + (long)bz * sC + i + (long)j * ldc;
-          if (beta.x != 0.0 || beta.y != 0.0) {
-            const double2 o = *c;
-            r.x += beta.x * o.x - beta.y * o.y;
-            r.y += beta.x * o.y + beta.y * o.x;
-          }
-          *c = r;
-          if (structure == GEMM_HERM && i != j) {
-            double2* cm = Cm + (long)bz * sC + j + (long)i * ldc;
-            double2 rm = make_double2(alpha.x * v.x + alpha.y * v.y, alpha.y * v.x - alpha.x * v.y);  // alpha conj(v)
-            if (beta.x != 0.0 || beta.y != 0.0) {
-              const double2 o = *cm;
-              rm.x += beta.x * o.x - beta.y * o.y;
-              rm.y += beta.x * o.y + beta.y * o.x;
-            }
-            *cm = rm;
-          }
-        }
+    for (int b = 0; b < 2; ++b) {
+      const int i = m0 + tx + 8 * a, j = n0 + ty + 8 * b;
+      if (i >= M || j >= N || (structure == GEMM_HERM && i < j)) continue;   // i < j: mirrored from (j, i)
+      const double2 v = to_d(acc[a][b]);
+      if (ksplit > 1) {
+        part[((long)kz * N + j) * (long)M + i] = v;
+        continue;
       }
+      auto put = [&](double2* c, double2 r) {
+        if (beta.x != 0.0 || beta.y != 0.0) {
+          const double2 o = *c;
+          r.x += beta.x * o.x - beta.y * o.y;
+          r.y += beta.x * o.y + beta.y * o.x;
+        }
+        *c = r;
+      };
+      put(Cm + i + (long)j * ldc, make_double2(alpha.x * v.x - alpha.y * v.y, alpha.x * v.y + alpha.y * v.x));
+      if (structure == GEMM_HERM && i != j)   // alpha conj(v)
+        put(Cm + j + (long)i * ldc, make_double2(alpha.x * v.x + alpha.y * v.y, alpha.y * v.x - alpha.x * v.y));
     }
 }
 
-// Sums the split-K partials in a fixed order. For GEMM_HERM the partials exist
+// Sums the split-K partials in a fixed order: G threads per entry (lanes 32 / G apart) sum
+// consecutive runs of partials, then add up pairwise. For GEMM_HERM the partials exist
 // on and below the diagonal; an entry above it is the conjugate of its mirror.
-__global__ void k_splitk_reduce(int M, int N, int batch, int ksplit, int structure, double2 alpha,
-                                const double2* __restrict__ part, double2 beta, double2* __restrict__ Cm, long ldc,
-                                long sC) {
-  const long total = (long)batch * M * N;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-    const int i = (int)(t % M);
-    const long rest = t / M;
-    const int j = (int)(rest % N);
-    const int bz = (int)(rest / N);
-    const bool mirror = structure == GEMM_HERM && i < j;
-    const int pi = mirror ? j : i, pj = mirror ? i : j;
+template <int G>
+__global__ void k_splitk_reduce(int M, int N, int ksplit, int structure, double2 alpha, const double2* __restrict__ part,
+                                double2 beta, double2* __restrict__ Cm, long ldc) {
+  constexpr int E = 32 / G;   // entries per warp
+  const long total = (long)M * N;
+  const int lane = threadIdx.x & 31, g = lane / E;
+  const int run = (ksplit + G - 1) / G;
+  const int z0 = g * run, z1 = min(ksplit, z0 + run);
+  const long warps = (long)gridDim.x * (blockDim.x >> 5);
+  for (long w = blockIdx.x * (long)(blockDim.x >> 5) + (threadIdx.x >> 5); w * E < total; w += warps) {
+    const long t = w * E + lane % E;
     double2 s = make_double2(0.0, 0.0);
-    for (int kz = 0; kz < ksplit; ++kz) {
-      const double2 v = part[(((long)kz * batch + bz) * N + pj) * (long)M + pi];
-      s.x += v.x;
-      s.y += v.y;
+    int i = 0, j = 0;
+    bool mirror = false;
+    if (t < total) {
+      i = (int)(t % M);
+      j = (int)(t / M);
+      mirror = structure == GEMM_HERM && i < j;
+      const double2* p = part + (mirror ? (long)i * M + j : (long)j * M + i);
+#pragma unroll 4
+      for (int kz = z0; kz < z1; ++kz) {
+        const double2 v = p[(long)kz * total];
+        s.x += v.x;
+        s.y += v.y;
+      }
     }
+#pragma unroll
+    for (int o = E; o < 32; o <<= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    }
+    if (t >= total || g != 0) continue;
     if (mirror) s.y = -s.y;
-    double2* c = Cm + (long)bz * sC + i + (long)j * ldc;
+    double2* c = Cm + i + (long)j * ldc;
     double2 r = make_double2(alpha.x * s.x - alpha.y * s.y, alpha.x * s.y + alpha.y * s.x);
     if (beta.x != 0.0 || beta.y != 0.0) {
       const double2 o = *c;
@@ -206,118 +190,233 @@ __global__ void k_splitk_reduce(int M, int N, int batch, int ksplit, int structu
   }
 }
 
-template <typename Tc, typename TI>
-static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alpha, const TI* A, long lda, long strideA,
-                             const TI* B, long ldb, long strideB, double2 beta, double2* C, long ldc, long strideC,
-                             int batch, double2* ws, size_t ws_elems, cudaStream_t s, int structure) {
-  constexpr int GK = GemmK<Tc>::V;
-  if (M <= 0 || N <= 0 || batch <= 0) return cudaSuccess;
-  if (structure == GEMM_HERM && M != N) return cudaErrorInvalidValue;
-  const int tm = (M + GBM - 1) / GBM, tn = (N + GBN - 1) / GBN;
-  const long tiles = structure == GEMM_HERM ? (long)tm * (tm + 1) / 2 * batch : (long)tm * tn * batch;
-  // split the reduction so that tiles x ksplit fills the resident block slots once
-  // (a second, mostly empty wave would cost as much as the first)
-  static std::atomic<int> slot_count[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-  int slots = slot_count[dev & 63].load(std::memory_order_relaxed);
-  if (slots == 0) {
-    int sms = 0, per_sm = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemm<Tc, TI>, 256, 0);
-    slots = std::max(1, sms * std::max(1, per_sm));
-    slot_count[dev & 63].store(slots, std::memory_order_relaxed);
-  }
-  int ksplit = 1;
-  if (K > 1024 && tiles < slots) {
-    ksplit = (int)std::max<long>(1, std::min<long>(slots / tiles, (K + 511) / 512));
-    while (ksplit > 1 && (size_t)ksplit * batch * M * N > ws_elems) --ksplit;
-  }
-  int kchunk = (K + ksplit - 1) / ksplit;
-  kchunk = ((kchunk + GK - 1) / GK) * GK;
-  ksplit = std::max(1, (K + kchunk - 1) / kchunk);
-  if (K == 0) { ksplit = 1; kchunk = GK; }
-  dim3 grid(tm, tn, (unsigned)(batch * ksplit));
-  k_gemm<Tc, TI><<<grid, 256, 0, s>>>(opA, opB, M, N, K, kchunk, ksplit, structure, alpha, A, lda, strideA, B, ldb,
-                                  strideB, beta, C, ldc, strideC, ws); launched();
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || ksplit == 1) return e;
-  const long total = (long)batch * M * N;
-  const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);
-  k_splitk_reduce<<<blocks, 256, 0, s>>>(M, N, batch, ksplit, structure, alpha, ws, beta, C, ldc, strideC); launched();
+static cudaError_t reduce_partials(int M, int N, int ksplit, int structure, double2 alpha, const double2* part,
+                                   double2 beta, double2* C, long ldc, cudaStream_t s) {
+  const long total = (long)M * N;
+  // eight threads per entry while one per entry would leave the chip mostly idle
+  const int G = ksplit >= 8 && total < 65536 ? 8 : 1;
+  const int blocks = (int)std::min<long>((total * G + 255) / 256, 152L * 16);
+  if (G == 8) k_splitk_reduce<8><<<blocks, 256, 0, s>>>(M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  else k_splitk_reduce<1><<<blocks, 256, 0, s>>>(M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  launched();
   return cudaGetLastError();
 }
 
-template <typename Tc>
-cudaError_t gemm(int opA, int opB, int M, int N, int K, double2 alpha, const double2* A, long lda, long strideA,
-                 const double2* B, long ldb, long strideB, double2 beta, double2* C, long ldc, long strideC, int batch,
-                 double2* ws, size_t ws_elems, cudaStream_t s, int structure) {
-  return gemm_impl<Tc, double2>(opA, opB, M, N, K, alpha, A, lda, strideA, B, ldb, strideB, beta, C, ldc, strideC,
-                                batch, ws, ws_elems, s, structure);
+int sm_count() {
+  static std::atomic<int> count[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+  int sms = count[dev & 63].load(std::memory_order_relaxed);
+  if (sms == 0) {
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(1, sms);
+    count[dev & 63].store(sms, std::memory_order_relaxed);
+  }
+  return sms;
 }
 
-template cudaError_t gemm<double>(int, int, int, int, int, double2, const double2*, long, long, const double2*, long,
-                                  long, double2, double2*, long, long, int, double2*, size_t, cudaStream_t, int);
+// Chunks of the reduction: the blocks of an SM share its multiply pipe, so the time goes as
+// the blocks of the fullest SM times the chunk length. Take the fewest chunks within 3%
+// of the least such time that the workspace allows, none shorter than `least_chunk`.
+static int choose_split(long tiles, int K, int least_chunk, long out_elems, size_t ws_elems) {
+  const long sms = sm_count();
+  const long most = std::max<long>(1, std::min<long>({(long)(K / least_chunk), (long)(ws_elems / out_elems), 4 * sms}));
+  auto cost = [&](long ks) { return (double)((tiles * ks + sms - 1) / sms) * (double)((K + ks - 1) / ks); };
+  double least = cost(1);
+  for (long ks = 2; ks <= most; ++ks) least = std::min(least, cost(ks));
+  for (long ks = 1; ks <= most; ++ks)
+    if (cost(ks) <= 1.03 * least) return (int)ks;
+  return 1;
+}
+
+template <typename C, typename TI>
+static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alpha, const TI* A, long lda, const TI* B,
+                             long ldb, double2 beta, double2* Cm, long ldc, double2* ws, size_t ws_elems,
+                             cudaStream_t s, int structure) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  if (structure == GEMM_HERM && M != N) return cudaErrorInvalidValue;
+  const int tm = (M + GT - 1) / GT, tn = (N + GT - 1) / GT;
+  if (tn > 65535) return cudaErrorInvalidValue;
+  const long tiles = structure == GEMM_HERM ? (long)tm * (tm + 1) / 2 : (long)tm * tn;
+  // FP64 chunks down to one slice pay (its multiply-adds are the time); FP32 ones cost a
+  // partial to sum, so they keep four slices
+  const int least = sizeof(C) == sizeof(double2) ? 8 : 64;
+  const int ksplit = K > 0 && ws != nullptr ? choose_split(tiles, K, least, (long)M * N, ws_elems) : 1;
+  const int kchunk = std::max(1, (K + ksplit - 1) / ksplit);
+  k_gemm<C, TI><<<dim3(tm, tn, (unsigned)ksplit), 64, 0, s>>>(opA, opB, M, N, K, kchunk, ksplit, structure, alpha, A,
+                                                              lda, B, ldb, beta, Cm, ldc, ws);
+  launched();
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || ksplit == 1) return e;
+  return reduce_partials(M, N, ksplit, structure, alpha, ws, beta, Cm, ldc, s);
+}
+
+cudaError_t gemm64(int opA, int opB, int M, int N, int K, double2 alpha, const double2* A, long lda, const double2* B,
+                   long ldb, double2 beta, double2* C, long ldc, double2* ws, size_t ws_elems, cudaStream_t s,
+                   int structure) {
+  return gemm_impl<double2>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_elems, s, structure);
+}
+
+cudaError_t gemm32_small(int opA, int opB, int M, int N, int K, double2 alpha, const float2* A, long lda,
+                         const float2* B, long ldb, double2 beta, double2* C, long ldc, double2* ws, size_t ws_elems,
+                         cudaStream_t s, int structure) {
+  return gemm_impl<float2>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_elems, s, structure);
+}
+
+cudaError_t gemm32_small(int opA, int opB, int M, int N, int K, double2 alpha, const double2* A, long lda,
+                         const double2* B, long ldb, double2 beta, double2* C, long ldc, double2* ws, size_t ws_elems,
+                         cudaStream_t s, int structure) {
+  return gemm_impl<float2>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_elems, s, structure);
+}
 
 cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const double2* part, double2 beta, double2* C,
                           long ldc, cudaStream_t s) {
-  const long total = (long)M * N;
-  const int blocks = (int)std::min<long>((total + 255) / 256, 152L * 16);
-  k_splitk_reduce<<<blocks, 256, 0, s>>>(M, N, 1, ksplit, GEMM_GENERAL, alpha, part, beta, C, ldc, 0); launched();
-  return cudaGetLastError();
+  return reduce_partials(M, N, ksplit, GEMM_GENERAL, alpha, part, beta, C, ldc, s);
 }
 
 // ---------------------------------------------------------------------------
-// Cholesky, right-looking, one column per pair of launches (pivot, update).
-__global__ void k_chol_pivot(double2* A, int n, int j, int* status) {
-  __shared__ double djj;
+// Cholesky, right-looking by panels of CB columns: one block factors the diagonal block
+// and inverts its factor, the rows below are multiplied by that inverse, and the trailing
+// matrix takes the rank-CB update: 3 launches per CB columns. Bound by FP64 (two
+// multiply-adds a clock and SM) in the single diagonal block, so only one thread takes
+// each pivot's reciprocal square root.
+constexpr int CB = 32;
+
+// Factor of the nb x nb block at (j0, j0), zeros above its diagonal, and the factor's
+// inverse into the same block of Linv.
+__global__ void __launch_bounds__(256) k_chol_diag(double2* __restrict__ A, double2* __restrict__ Linv, int n, int j0,
+                                                   int* __restrict__ status) {
+  __shared__ double2 a[CB][CB + 1], x[CB][CB + 1];
+  __shared__ double rinv[CB];
+  __shared__ int bad;
   if (*status != 0) return;
-  if (threadIdx.x == 0) {
-    const double d = A[j + (long)j * n].x;
-    if (!(d > 0.0)) { *status = 1; djj = 0.0; }
-    else { djj = sqrt(d); A[j + (long)j * n] = make_double2(djj, 0.0); }
+  const int tid = threadIdx.x, nb = min(CB, n - j0);
+  double2* Ab = A + j0 + (long)j0 * n;
+  double2* Xb = Linv + j0 + (long)j0 * n;
+  if (tid == 0) bad = 0;
+  for (int t = tid; t < nb * nb; t += 256) {
+    const int i = t % nb, k = t / nb;
+    a[i][k] = i >= k ? Ab[i + (long)k * n] : make_double2(0.0, 0.0);
+    x[i][k] = make_double2(i == k ? 1.0 : 0.0, 0.0);
   }
   __syncthreads();
-  if (djj == 0.0) return;
-  const double inv = 1.0 / djj;
-  for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-    double2 v = A[i + (long)j * n];
-    A[i + (long)j * n] = make_double2(v.x * inv, v.y * inv);
+  for (int j = 0; j < nb; ++j) {
+    if (tid == 0) {
+      const double d = a[j][j].x;
+      if (!(d > 0.0)) {
+        bad = 1;
+      } else {
+        const double r = rsqrt(d);
+        a[j][j] = make_double2(d * r, 0.0);
+        rinv[j] = r;
+      }
+    }
+    __syncthreads();
+    if (bad) {
+      if (tid == 0) *status = 1;
+      return;
+    }
+    if (tid > j && tid < nb) {
+      const double r = rinv[j];
+      a[tid][j] = make_double2(a[tid][j].x * r, a[tid][j].y * r);
+    }
+    __syncthreads();
+    const int m = nb - 1 - j;
+    for (int t = tid; t < m * m; t += 256) {
+      const int i = j + 1 + t % m, k = j + 1 + t / m;
+      if (i < k) continue;
+      const double2 u = a[i][j], w = a[k][j];
+      a[i][k].x -= u.x * w.x + u.y * w.y;
+      a[i][k].y -= u.y * w.x - u.x * w.y;
+    }
+    __syncthreads();
+  }
+  for (int i = 0; i < nb; ++i) {   // rows of the inverse
+    if (tid <= i) {
+      const double r = rinv[i];
+      x[i][tid] = make_double2(x[i][tid].x * r, x[i][tid].y * r);
+    }
+    __syncthreads();
+    const int m = nb - 1 - i;
+    for (int t = tid; t < m * (i + 1); t += 256) {
+      const int k = i + 1 + t % m, c = t / m;
+      const double2 l = a[k][i], v = x[i][c];
+      x[k][c].x -= l.x * v.x - l.y * v.y;
+      x[k][c].y -= l.x * v.y + l.y * v.x;
+    }
+    __syncthreads();
+  }
+  for (int t = tid; t < nb * nb; t += 256) {
+    const int i = t % nb, k = t / nb;
+    Ab[i + (long)k * n] = a[i][k];
+    Xb[i + (long)k * n] = x[i][k];
   }
 }
 
-// A[i][k] -= A[i][j] conj(A[k][j]) for j < k <= i
-__global__ void k_chol_update(double2* A, int n, int j, const int* status) {
+// Rows below the diagonal block: A21 <- A21 L11^{-H}, eight rows per block; the block's part
+// of the columns j0.. above the diagonal (rows of A12) is zeroed.
+__global__ void __launch_bounds__(256) k_chol_panel(double2* __restrict__ A, const double2* __restrict__ Linv, int n,
+                                                    int j0, const int* __restrict__ status) {
+  __shared__ double2 a[8][CB + 1], x[CB][CB + 1];
   if (*status != 0) return;
-  const int k = j + 1 + blockIdx.x;
-  if (k >= n) return;
-  const double2 akj = A[k + (long)j * n];
-  for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-    const double2 aij = A[i + (long)j * n];
-    double2* t = A + i + (long)k * n;
-    double2 v = *t;
-    v.x -= aij.x * akj.x + aij.y * akj.y;
-    v.y -= aij.y * akj.x - aij.x * akj.y;
-    *t = v;
+  const int tid = threadIdx.x, i0 = j0 + CB + 8 * blockIdx.x;
+  const int r = tid & 7, k = tid >> 3;
+  for (int t = tid; t < CB * CB; t += 256) x[t % CB][t / CB] = Linv[j0 + t % CB + (long)(j0 + t / CB) * n];
+  const bool in = i0 + r < n;
+  double2* p = A + i0 + r + (long)(j0 + k) * n;
+  a[r][k] = in ? *p : make_double2(0.0, 0.0);
+  __syncthreads();
+  double2 s = make_double2(0.0, 0.0);
+  for (int m = 0; m <= k; ++m) {
+    const double2 u = a[r][m], w = x[k][m];
+    s.x += u.x * w.x + u.y * w.y;
+    s.y += u.y * w.x - u.x * w.y;
   }
+  if (!in) return;
+  *p = s;
+  A[j0 + k + (long)(i0 + r) * n] = make_double2(0.0, 0.0);
 }
 
-__global__ void k_zero_upper(double2* A, int n) {
-  const long total = (long)n * n;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total; t += (long)gridDim.x * blockDim.x) {
-    const int i = (int)(t % n), k = (int)(t / n);
-    if (i < k) A[t] = make_double2(0.0, 0.0);
+// A22 -= L21 L21^H on and below the diagonal, one 16 x 16 tile per block
+__global__ void __launch_bounds__(256) k_chol_trail(double2* __restrict__ A, int n, int j0,
+                                                    const int* __restrict__ status) {
+  __shared__ double2 u[CB][17], w[CB][17];
+  if (blockIdx.x < blockIdx.y || *status != 0) return;
+  const int tid = threadIdx.x, base = j0 + CB;
+  const int i0 = base + 16 * blockIdx.x, k0 = base + 16 * blockIdx.y;
+  for (int t = tid; t < 16 * CB; t += 256) {
+    const int i = t & 15, m = t >> 4;
+    const double2 z = make_double2(0.0, 0.0);
+    u[m][i] = i0 + i < n ? A[i0 + i + (long)(j0 + m) * n] : z;
+    w[m][i] = k0 + i < n ? A[k0 + i + (long)(j0 + m) * n] : z;
   }
+  __syncthreads();
+  const int i = i0 + (tid & 15), k = k0 + (tid >> 4);
+  if (i >= n || k > i) return;
+  double2 s = A[i + (long)k * n];
+#pragma unroll 8
+  for (int m = 0; m < CB; ++m) {
+    const double2 a = u[m][tid & 15], b = w[m][tid >> 4];
+    s.x -= a.x * b.x + a.y * b.y;
+    s.y -= a.y * b.x - a.x * b.y;
+  }
+  A[i + (long)k * n] = s;
 }
 
-cudaError_t cholesky(double2* A, int n, int* d_status, cudaStream_t s) {
+__global__ void k_tri_inverse(const double2* __restrict__ L, double2* __restrict__ Li, int n);
+
+cudaError_t cholesky_inverse(double2* A, double2* Linv, int n, int* d_status, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(d_status, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
-  for (int j = 0; j < n; ++j) {
-    k_chol_pivot<<<1, 256, 0, s>>>(A, n, j, d_status); launched();
-    if (j + 1 < n) { k_chol_update<<<n - j - 1, 128, 0, s>>>(A, n, j, d_status); launched(); }
+  for (int j0 = 0; j0 < n; j0 += CB) {
+    k_chol_diag<<<1, 256, 0, s>>>(A, Linv, n, j0, d_status); launched();
+    const int rest = n - j0 - CB;
+    if (rest <= 0) continue;
+    k_chol_panel<<<(rest + 7) / 8, 256, 0, s>>>(A, Linv, n, j0, d_status); launched();
+    const unsigned t = (unsigned)((rest + 15) / 16);
+    k_chol_trail<<<dim3(t, t), 256, 0, s>>>(A, n, j0, d_status); launched();
   }
-  k_zero_upper<<<std::max(1, std::min(1024, (n * n + 255) / 256)), 256, 0, s>>>(A, n); launched();
+  if (n > CB) { k_tri_inverse<<<n, 128, sizeof(double2) * n, s>>>(A, Linv, n); launched(); }
   return cudaGetLastError();
 }
 
@@ -345,11 +444,6 @@ __global__ void k_tri_inverse(const double2* __restrict__ L, double2* __restrict
     __syncthreads();
   }
   for (int i = threadIdx.x; i < n; i += blockDim.x) Li[i + (long)c * n] = i < c ? make_double2(0.0, 0.0) : b[i];
-}
-
-cudaError_t tri_inverse(const double2* L, double2* Linv, int n, cudaStream_t s) {
-  k_tri_inverse<<<n, 128, sizeof(double2) * n, s>>>(L, Linv, n); launched();
-  return cudaGetLastError();
 }
 
 }  // namespace pt

@@ -266,7 +266,9 @@ size_t carve(pt_system* sys, const pt_params* p, uintptr_t base) {
   t->Mneg = c.take<double2>(ne * ne);
   t->Linv = c.take<double2>(ne * ne);
   t->Z = c.take<double2>(ne * ne);
-  t->gemm_ws_elems = (size_t)16 * ne * ne + 4096;
+  // split-K partials: enough chunks that 128 x 128 tiles (and 16 x 16 ones) fill 152 SMs
+  const size_t tiles_tc = (size_t)((ne + 127) / 128) * ((ne + 127) / 128);
+  t->gemm_ws_elems = std::max<size_t>(16, 152 / tiles_tc) * ne * ne + 65536;
   t->gemm_ws = c.take<double2>(t->gemm_ws_elems);
   t->gram = c.take<double2>((size_t)ne * std::max(1, m) * std::max(1, m));
   t->rhs = c.take<double2>((size_t)ne * std::max(1, m));
