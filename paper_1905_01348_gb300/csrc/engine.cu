@@ -565,6 +565,9 @@ pt_status set_kinetic(pt_system* sys, int64_t n) { return set_kinetic_t(sys, (do
 // ACE and the observables. cn_step runs them in order; a batch interleaves the phases of
 // several systems, each on its own stream, with identical arithmetic.
 
+// the residual's block partials inside sys->part, clear of the other reductions' partials
+static constexpr long kResidPart = 7168;
+
 pt_status cn_begin(pt_system* sys, StepCtx* c) {
   const int ne = sys->ne, npw = sys->npw;
   const long n = (long)npw * ne;
@@ -634,9 +637,9 @@ pt_status cn_iterate(pt_system* sys, StepCtx* c) {
     const bool copied = sys->mixed && !hi && sys->p.alpha != 0.0 && sys->p.fock_mode == PT_FOCK_ACE &&
                         !pt::tc_too_small(ne, ne);
     PT_TRY(projection(sys, sys->psi_f, sys->hpsi, hi, copied));
-    PT_CK(pt::pt_residual(sys->psi_f, sys->hpsi, sys->psi_half, hdt, sys->rbuf, n, sys->part, sys->red + 0, sys->s));
   }
-  // Anderson (per band)
+  // Anderson (per band); the residual goes into rprev, the next iterate into xprev, which
+  // then changes places with psi_f
   {
     Phase and_("Anderson");
     int newslot = -1;
@@ -650,22 +653,21 @@ pt_status cn_iterate(pt_system* sys, StepCtx* c) {
       }
       sys->and_order.push_back(newslot);
     }
+    const int f32 = sys->mixed ? 1 : 0;
     const size_t hs = sys->mixed ? sizeof(float2) : sizeof(double2);
-    PT_CK(pt::anderson_push(sys->psi_f, sys->rbuf, sys->xprev, sys->rprev,
-                            sys->dX + (newslot >= 0 ? newslot : 0) * stride * hs,
-                            sys->dR + (newslot >= 0 ? newslot : 0) * stride * hs, n, newslot >= 0 ? 1 : 0,
-                            sys->mixed ? 1 : 0, sys->s));
+    const size_t at = (newslot >= 0 ? newslot : 0) * stride * hs;
+    PT_CK(pt::residual_push(sys->psi_f, sys->hpsi, sys->psi_half, hdt, sys->xprev, sys->rprev, sys->dX + at,
+                            sys->dR + at, n, newslot >= 0 ? 1 : 0, f32, sys->part + kResidPart, sys->s));
     c->have_prev = true;
     pt::SlotList sl{};
     sl.k = (int)sys->and_order.size();
     for (int q = 0; q < sl.k; ++q) sl.s[q] = sys->and_order[q];
-    if (sl.k > 0) {
-      PT_CK(pt::anderson_dots(sys->dR, stride, sl, newslot, sys->rbuf, npw, ne, m, sys->gram, sys->rhs,
-                              sys->mixed ? 1 : 0, sys->s));
-      PT_CK(pt::anderson_solve(sys->gram, sys->rhs, sl, m, ne, sys->gamma, sys->s));
-    }
-    PT_CK(pt::anderson_update(sys->psi_f, sys->rbuf, sys->dX, sys->dR, stride, sl, sys->gamma, std::max(m, 1), npw, n,
-                              sys->p.anderson_beta, sys->mixed ? 1 : 0, sys->s));
+    if (sl.k > 0)
+      PT_CK(pt::anderson_gamma(sys->dR, stride, sl, newslot, sys->rprev, npw, ne, m, sys->gram, sys->gamma,
+                               sys->gemm_ws, f32, sys->s));
+    PT_CK(pt::anderson_update(sys->psi_f, sys->rprev, sys->dX, sys->dR, stride, sl, sys->gamma, std::max(m, 1), npw, n,
+                              sys->p.anderson_beta, f32, sys->xprev, sys->s));
+    std::swap(sys->psi_f, sys->xprev);
   }
   // new density and its change (FP64 real-space orbitals and density once refining)
   Phase rho_("density");
@@ -716,6 +718,7 @@ pt_status cn_outer(pt_system* sys, StepCtx* c, bool* again) {
 }
 
 pt_status cn_orthonormalize(pt_system* sys, StepCtx* c) {
+  PT_CK(pt::residual_norm2(sys->part + kResidPart, (long)sys->npw * sys->ne, sys->red, sys->s));
   PT_TRY(read_small(sys, c->hres, sys->red, sizeof(c->hres)));
   // orthonormalise; the real-space orbitals of Psi_{n+1} for its exchange and density
   PT_TRY(orthonormalize(sys, sys->psi_f, sys->psi));

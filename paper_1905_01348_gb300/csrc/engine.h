@@ -70,7 +70,7 @@ struct pt_system {
   double *hfac = nullptr, *kfac = nullptr, *rho_mix = nullptr, *vion = nullptr, *vloc = nullptr, *vh = nullptr, *rho = nullptr, *rho2 = nullptr;
   double* d_atoms = nullptr;
   float* vloc32 = nullptr;
-  double2 *psi = nullptr, *psi_half = nullptr, *psi_f = nullptr, *hpsi = nullptr, *tmp = nullptr, *rbuf = nullptr;
+  double2 *psi = nullptr, *psi_half = nullptr, *psi_f = nullptr, *hpsi = nullptr, *tmp = nullptr;
   double2 *wg = nullptr, *xi = nullptr, *xprev = nullptr, *rprev = nullptr;
   // Anderson history: complex128, or complex64 in mixed precision
   unsigned char *dX = nullptr, *dR = nullptr;
@@ -98,7 +98,7 @@ struct pt_system {
   unsigned char *sphf_rowlive = nullptr, *sphf_planelive = nullptr;
   double2 *S = nullptr, *Mneg = nullptr, *Linv = nullptr, *Z = nullptr, *gemm_ws = nullptr;
   size_t gemm_ws_elems = 0;
-  double2 *gram = nullptr, *rhs = nullptr, *gamma = nullptr;
+  double2 *gram = nullptr, *gamma = nullptr;
   double *part = nullptr, *red = nullptr;
   int* status = nullptr;
   pt::PairTile *d_tiles_sym = nullptr, *d_tiles_x = nullptr;

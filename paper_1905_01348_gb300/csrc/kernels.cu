@@ -36,12 +36,20 @@ __device__ __forceinline__ void block_sums(double (&v)[NS], double* part) {
   }
 }
 
+// out[q] = sum of part[b ns + q] over the nblocks partials, in an order that depends on
+// nblocks alone: one warp per sum, lane l adding partials l, l + 32, ... first.
 __global__ void k_finalize(const double* __restrict__ part, int nblocks, int ns, double* __restrict__ out) {
-  const int s = threadIdx.x;
-  if (s >= ns) return;
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q >= ns) return;
   double t = 0.0;
-  for (int b = 0; b < nblocks; ++b) t += part[b * ns + s];
-  out[s] = t;
+#pragma unroll 4
+  for (int b = lane; b < nblocks; b += 32) t += part[b * ns + q];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if (lane == 0) out[q] = t;
+}
+
+static void finalize(const double* part, int nblocks, int ns, double* out, cudaStream_t s) {
+  k_finalize<<<1, 32 * ns, 0, s>>>(part, nblocks, ns, out); launched();
 }
 
 // ---- density ------------------------------------------------------------------
@@ -183,28 +191,6 @@ cudaError_t half_step(const double2* psi, const double2* R, double hdt, double2*
   return cudaGetLastError();
 }
 
-// r = -(psi_f + i dt/2 T - psi_half); block partials of |r|^2
-__global__ void k_resid(const double2* __restrict__ psi_f, const double2* __restrict__ T, const double2* __restrict__ ph,
-                        double hdt, double2* __restrict__ r, long n, double* __restrict__ part) {
-  double acc[1] = {0.0};
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
-    const double2 p = psi_f[t], q = T[t], h = ph[t];
-    // i hdt (qx + i qy) = -hdt qy + i hdt qx
-    const double2 R = make_double2(p.x - hdt * q.y - h.x, p.y + hdt * q.x - h.y);
-    r[t] = make_double2(-R.x, -R.y);
-    acc[0] += R.x * R.x + R.y * R.y;
-  }
-  block_sums<1>(acc, part);
-}
-
-cudaError_t pt_residual(const double2* psi_f, const double2* T, const double2* ph, double hdt, double2* r, long n,
-                        double* part, double* out_norm2, cudaStream_t s) {
-  const unsigned b = nblk(n, 256, 1024);
-  k_resid<<<b, 256, 0, s>>>(psi_f, T, ph, hdt, r, n, part); launched();
-  k_finalize<<<1, 32, 0, s>>>(part, b, 1, out_norm2); launched();
-  return cudaGetLastError();
-}
-
 // y = x - tau * P * R, P = 1 / (1 + kin) per basis vector (start-state relaxation)
 __global__ void k_precond_step(double2* __restrict__ x, const double2* __restrict__ R, const double* __restrict__ kin,
                                int npw, long n, double tau) {
@@ -224,185 +210,205 @@ cudaError_t precond_step(double2* x, const double2* R, const double* kin, int np
 }
 
 // ---- Anderson mixing (Sec. 3.4), per band -------------------------------------------
-// push: dX[slot] = x - x_prev, dR[slot] = r - r_prev (when have_prev), then x_prev = x, r_prev = r
+// r = -(x + i dt/2 T - psi_half) (the fixed-point residual, Alg. 1 and 3) with block partials
+// of |r|^2, and the history entries dX[slot] = x - x_prev, dR[slot] = r - r_prev when there
+// is a previous iterate. r overwrites r_prev: one pass over the orbitals instead of three.
 // History entries are stored as H: complex128, or complex64 in mixed precision
 // (the differences of successive iterates and residuals, whose rounding to FP32
 // only perturbs the least-squares extrapolation, not the fixed point).
 template <typename H>
-__global__ void k_anderson_push(const double2* __restrict__ x, const double2* __restrict__ r, double2* __restrict__ xp,
-                                double2* __restrict__ rp, H* __restrict__ dx, H* __restrict__ dr, long n,
-                                int have_prev) {
+__global__ void __launch_bounds__(256) k_resid_push(const double2* __restrict__ x, const double2* __restrict__ T,
+                                                    const double2* __restrict__ ph, double hdt,
+                                                    const double2* __restrict__ xp, double2* __restrict__ r,
+                                                    H* __restrict__ dx, H* __restrict__ dr, long n, int have_prev,
+                                                    double* __restrict__ part) {
+  using A = decltype(H::x);
+  double acc[1] = {0.0};
+#pragma unroll 2
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
-    const double2 a = x[t], b = r[t];
+    const double2 p = x[t], q = T[t], h = ph[t];
+    // i hdt (qx + i qy) = -hdt qy + i hdt qx
+    const double2 v = make_double2(-(p.x - hdt * q.y - h.x), -(p.y + hdt * q.x - h.y));
     if (have_prev) {
-      const double2 c = xp[t], d = rp[t];
-      dx[t] = {(decltype(H::x))(a.x - c.x), (decltype(H::x))(a.y - c.y)};
-      dr[t] = {(decltype(H::x))(b.x - d.x), (decltype(H::x))(b.y - d.y)};
+      const double2 c = xp[t], d = r[t];
+      dx[t] = {(A)(p.x - c.x), (A)(p.y - c.y)};
+      dr[t] = {(A)(v.x - d.x), (A)(v.y - d.y)};
     }
-    xp[t] = a;
-    rp[t] = b;
+    r[t] = v;
+    acc[0] += v.x * v.x + v.y * v.y;
   }
+  block_sums<1>(acc, part);
 }
 
-cudaError_t anderson_push(const double2* x, const double2* r, double2* xp, double2* rp, void* dx, void* dr, long n,
-                          int have_prev, int f32, cudaStream_t s) {
+static unsigned resid_blocks(long n) { return nblk(n, 256, 1024); }
+
+cudaError_t residual_push(const double2* x, const double2* T, const double2* ph, double hdt, const double2* xp,
+                          double2* r, void* dx, void* dr, long n, int have_prev, int f32, double* part,
+                          cudaStream_t s) {
+  const unsigned b = resid_blocks(n);
   if (f32)
-    k_anderson_push<float2><<<nblk(n, 256), 256, 0, s>>>(x, r, xp, rp, (float2*)dx, (float2*)dr, n, have_prev);
+    k_resid_push<float2><<<b, 256, 0, s>>>(x, T, ph, hdt, xp, r, (float2*)dx, (float2*)dr, n, have_prev, part);
   else
-    k_anderson_push<double2><<<nblk(n, 256), 256, 0, s>>>(x, r, xp, rp, (double2*)dx, (double2*)dr, n, have_prev);
+    k_resid_push<double2><<<b, 256, 0, s>>>(x, T, ph, hdt, xp, r, (double2*)dx, (double2*)dr, n, have_prev, part);
   launched();
   return cudaGetLastError();
 }
 
-// For each band b: gram[b][slot_q][new] = <dR_{slot_q}, dR_new>_b (and its
-// conjugate at [new][slot_q]) and rhs[b][q] = <dR_{slot_q}, r>_b for the
-// history slots in order (oldest first). One block per band; the slots are
-// processed four at a time to bound registers.
+cudaError_t residual_norm2(const double* part, long n, double* out, cudaStream_t s) {
+  finalize(part, (int)resid_blocks(n), 1, out, s);
+  return cudaGetLastError();
+}
+
+// Partial sums over one of kDotChunks chunks of the basis of <dR_q, dR_new> and <dR_q, r>
+// for band blockIdx.y, one warp per history slot q: the warps of a block walk the same
+// stretch together, so dR_new and r come from DRAM once per block and from L1 for the
+// other slots, and every lane carries four sums whatever the history depth.
 // Complex64 history (mixed precision): the products are formed in FP32 and
-// summed in FP32 over each thread's share of the basis (about npw / 256 terms);
-// the per-thread sums are reduced in FP64. FP64 otherwise. The Gram matrix and
+// summed in FP32 over each lane's share of the chunk (about npw / 256 terms);
+// the lanes' sums are reduced in FP64. FP64 otherwise. The Gram matrix and
 // right-hand side feed the FP64 solve either way.
+constexpr int kDotChunks = 8;
+
 template <typename H>
 __global__ void k_anderson_dots(const H* __restrict__ dR, long slot_stride, SlotList sl, int newslot,
-                                const double2* __restrict__ r, int npw, int mdim, double2* __restrict__ gram,
-                                double2* __restrict__ rhs) {
+                                const double2* __restrict__ r, int npw, double4_16a* __restrict__ part) {
   using A = decltype(H::x);
-  const int b = blockIdx.x;
-  const int k = sl.k;
+  const int b = blockIdx.y, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int len = (npw + kDotChunks - 1) / kDotChunks;
+  const int g0 = blockIdx.x * len, g1 = min(npw, g0 + len);
   const long boff = (long)b * npw;
   const H* dn = dR + (long)newslot * slot_stride + boff;
+  const H* du = dR + (long)sl.s[q] * slot_stride + boff;
   const double2* rb = r + boff;
-  __shared__ double sh[16][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int q0 = 0; q0 < k; q0 += 4) {
-    A acc[16];
-#pragma unroll
-    for (int c = 0; c < 16; ++c) acc[c] = (A)0;
-    for (int g = threadIdx.x; g < npw; g += blockDim.x) {
-      const H vnd = dn[g];
-      const double2 vrd = rb[g];
-      const A vnx = vnd.x, vny = vnd.y, vrx = (A)vrd.x, vry = (A)vrd.y;
-#pragma unroll
-      for (int qq = 0; qq < 4; ++qq) {
-        if (q0 + qq < k) {
-          const H ud = dR[(long)sl.s[q0 + qq] * slot_stride + boff + g];
-          const A ux = ud.x, uy = ud.y;
-          acc[4 * qq + 0] += ux * vnx + uy * vny;
-          acc[4 * qq + 1] += ux * vny - uy * vnx;
-          acc[4 * qq + 2] += ux * vrx + uy * vry;
-          acc[4 * qq + 3] += ux * vry - uy * vrx;
-        }
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      double x = (double)acc[c];
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      if (lane == 0) sh[c][warp] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < 4 && q0 + (int)threadIdx.x < k) {
-      const int qq = threadIdx.x, q = q0 + qq;
-      double v[4];
-      for (int c = 0; c < 4; ++c) {
-        double t = 0.0;
-        for (int w = 0; w < nw; ++w) t += sh[4 * qq + c][w];
-        v[c] = t;
-      }
-      const long gb = (long)b * mdim * mdim;
-      const int sq = sl.s[q];
-      if (sq == newslot) {
-        gram[gb + (long)sq * mdim + sq] = make_double2(v[0], 0.0);
-      } else {
-        gram[gb + (long)sq * mdim + newslot] = make_double2(v[0], v[1]);
-        gram[gb + (long)newslot * mdim + sq] = make_double2(v[0], -v[1]);
-      }
-      rhs[(long)b * mdim + q] = make_double2(v[2], v[3]);
-    }
-    __syncthreads();
+  A a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+#pragma unroll 4
+  for (int g = g0 + lane; g < g1; g += 32) {
+    const H v = dn[g], u = du[g];
+    const double2 w = rb[g];
+    const A wx = (A)w.x, wy = (A)w.y;
+    a0 += u.x * v.x + u.y * v.y;
+    a1 += u.x * v.y - u.y * v.x;
+    a2 += u.x * wx + u.y * wy;
+    a3 += u.x * wy - u.y * wx;
   }
+  double d[4] = {(double)a0, (double)a1, (double)a2, (double)a3};
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    for (int o = 16; o > 0; o >>= 1) d[c] += __shfl_down_sync(0xffffffffu, d[c], o);
+  if (lane == 0) part[((long)b * sl.k + q) * kDotChunks + blockIdx.x] = make_double4_16a(d[0], d[1], d[2], d[3]);
 }
 
-cudaError_t anderson_dots(const void* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r,
-                          int npw, int ne, int mdim, double2* gram, double2* rhs, int f32, cudaStream_t s) {
-  if (sl.k > kSlotMax) return cudaErrorInvalidValue;
-  if (f32)
-    k_anderson_dots<float2><<<ne, 256, 0, s>>>((const float2*)dR, slot_stride, sl, newslot, r, npw, mdim, gram, rhs);
-  else
-    k_anderson_dots<double2><<<ne, 256, 0, s>>>((const double2*)dR, slot_stride, sl, newslot, r, npw, mdim, gram, rhs);
-  launched();
-  return cudaGetLastError();
-}
-
-// Solve (G + 1e-14 tr(G) I) gamma = rhs per band by Cholesky; gamma = 0 when
-// the trace is zero or a pivot is not positive. One thread per band.
-__global__ void k_anderson_solve(const double2* __restrict__ gram, const double2* __restrict__ rhs, SlotList sl,
-                                 int mdim, int ne, double2* __restrict__ gamma) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= ne) return;
-  const int k = sl.k;
-  double2 L[kSlotMax][kSlotMax];
-  double2 y[kSlotMax];
-  const long gb = (long)b * mdim * mdim;
+// Gathers the sums into gram[b][slot_q][new] (and its conjugate at [new][slot_q]) and the
+// right-hand side <dR_q, r> (slots in order, oldest first), then solves
+// (G + 1e-14 tr(G) I) gamma = rhs per band by Cholesky; gamma = 0 when the trace is zero
+// or a pivot is not positive. One warp per band, the matrix in shared memory: the k^3 / 6
+// multiply-adds of a column's update are spread over the lanes.
+__global__ void __launch_bounds__(32) k_anderson_solve(const double4_16a* __restrict__ part, SlotList sl, int newslot,
+                                                       int mdim, double2* __restrict__ gram,
+                                                       double2* __restrict__ gamma) {
+  __shared__ double2 L[kSlotMax][kSlotMax + 1];
+  const int b = blockIdx.x, lane = threadIdx.x, k = sl.k;
+  double2* G = gram + (long)b * mdim * mdim;
+  double2 y = make_double2(0.0, 0.0);   // right-hand side, then the solution, of row `lane`
+  const int mine = lane < k ? sl.s[lane] : 0;
+  if (lane < k) {
+    const double4_16a* p = part + ((long)b * k + lane) * kDotChunks;
+    double4_16a t = p[0];
+#pragma unroll
+    for (int c = 1; c < kDotChunks; ++c) {
+      t.x += p[c].x;
+      t.y += p[c].y;
+      t.z += p[c].z;
+      t.w += p[c].w;
+    }
+    if (mine == newslot) {
+      G[(long)mine * mdim + mine] = make_double2(t.x, 0.0);
+    } else {
+      G[(long)mine * mdim + newslot] = make_double2(t.x, t.y);
+      G[(long)newslot * mdim + mine] = make_double2(t.x, -t.y);
+    }
+    y = make_double2(t.z, t.w);
+  }
+  __syncwarp();
+  // L L^H = A with A[i][j] = G[s_i][s_j]  (G[s][t] = <dR_s, dR_t>)
+  for (int t = lane; t < k * k; t += 32) {
+    const int i = t / k, j = t % k;
+    if (j <= i) L[i][j] = G[(long)sl.s[i] * mdim + sl.s[j]];
+  }
+  __syncwarp();
   double tr = 0.0;
-  for (int q = 0; q < k; ++q) tr += gram[gb + (long)sl.s[q] * mdim + sl.s[q]].x;
+  for (int q = 0; q < k; ++q) tr += L[q][q].x;
   bool ok = tr > 0.0;
   const double shift = 1e-14 * tr;
-  // L L^H = A with A[i][j] = G[s_i][s_j]  (G[s][t] = <dR_s, dR_t>)
+  double inv = 0.0;   // 1 / L[lane][lane]
   for (int j = 0; j < k && ok; ++j) {
-    double d = gram[gb + (long)sl.s[j] * mdim + sl.s[j]].x + shift;
-    for (int p = 0; p < j; ++p) d -= L[j][p].x * L[j][p].x + L[j][p].y * L[j][p].y;
+    const double d = L[j][j].x + shift;
     if (!(d > 0.0)) { ok = false; break; }
-    const double ljj = sqrt(d);
-    L[j][j] = make_double2(ljj, 0.0);
-    for (int i = j + 1; i < k; ++i) {
-      double2 a = gram[gb + (long)sl.s[i] * mdim + sl.s[j]];
-      for (int p = 0; p < j; ++p) {
-        // a -= L[i][p] * conj(L[j][p])
-        a.x -= L[i][p].x * L[j][p].x + L[i][p].y * L[j][p].y;
-        a.y -= L[i][p].y * L[j][p].x - L[i][p].x * L[j][p].y;
-      }
-      L[i][j] = make_double2(a.x / ljj, a.y / ljj);
+    const double r = rsqrt(d);
+    if (lane == j) inv = r;
+    if (lane > j && lane < k) L[lane][j] = make_double2(L[lane][j].x * r, L[lane][j].y * r);
+    __syncwarp();
+    const int m = k - 1 - j;
+    for (int t = lane; t < m * m; t += 32) {
+      const int i = j + 1 + t % m, p = j + 1 + t / m;
+      if (p > i) continue;
+      const double2 u = L[i][j], w = L[p][j];
+      L[i][p].x -= u.x * w.x + u.y * w.y;
+      L[i][p].y -= u.y * w.x - u.x * w.y;
     }
+    __syncwarp();
   }
   if (!ok) {
-    for (int q = 0; q < k; ++q) gamma[(long)b * mdim + q] = make_double2(0.0, 0.0);
+    if (lane < k) gamma[(long)b * mdim + lane] = make_double2(0.0, 0.0);
     return;
   }
   for (int i = 0; i < k; ++i) {   // L y = rhs
-    double2 a = rhs[(long)b * mdim + i];
-    for (int p = 0; p < i; ++p) {
-      a.x -= L[i][p].x * y[p].x - L[i][p].y * y[p].y;
-      a.y -= L[i][p].x * y[p].y + L[i][p].y * y[p].x;
+    if (lane == i) { y.x *= inv; y.y *= inv; }
+    const double yx = __shfl_sync(0xffffffffu, y.x, i), yy = __shfl_sync(0xffffffffu, y.y, i);
+    if (lane > i && lane < k) {
+      const double2 l = L[lane][i];
+      y.x -= l.x * yx - l.y * yy;
+      y.y -= l.x * yy + l.y * yx;
     }
-    y[i] = make_double2(a.x / L[i][i].x, a.y / L[i][i].x);
   }
   for (int i = k - 1; i >= 0; --i) {   // L^H g = y
-    double2 a = y[i];
-    for (int p = i + 1; p < k; ++p) {
-      const double2 gp = y[p];
-      a.x -= L[p][i].x * gp.x + L[p][i].y * gp.y;
-      a.y -= L[p][i].x * gp.y - L[p][i].y * gp.x;
+    if (lane == i) { y.x *= inv; y.y *= inv; }
+    const double yx = __shfl_sync(0xffffffffu, y.x, i), yy = __shfl_sync(0xffffffffu, y.y, i);
+    if (lane < i) {
+      const double2 l = L[i][lane];
+      y.x -= l.x * yx + l.y * yy;
+      y.y -= l.x * yy - l.y * yx;
     }
-    y[i] = make_double2(a.x / L[i][i].x, a.y / L[i][i].x);
   }
-  for (int q = 0; q < k; ++q) gamma[(long)b * mdim + q] = y[q];
+  if (lane < k) gamma[(long)b * mdim + lane] = y;
 }
 
-cudaError_t anderson_solve(const double2* gram, const double2* rhs, const SlotList& sl, int mdim, int ne,
-                           double2* gamma, cudaStream_t s) {
-  k_anderson_solve<<<(ne + 63) / 64, 64, 0, s>>>(gram, rhs, sl, mdim, ne, gamma); launched();
+cudaError_t anderson_gamma(const void* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r,
+                           int npw, int ne, int mdim, double2* gram, double2* gamma, void* part, int f32,
+                           cudaStream_t s) {
+  if (sl.k < 1 || sl.k > kSlotMax) return cudaErrorInvalidValue;
+  if (ne > 65535) return cudaErrorInvalidValue;
+  const dim3 grid(kDotChunks, (unsigned)ne);
+  if (f32)
+    k_anderson_dots<float2><<<grid, 32 * sl.k, 0, s>>>((const float2*)dR, slot_stride, sl, newslot, r, npw,
+                                                       (double4_16a*)part);
+  else
+    k_anderson_dots<double2><<<grid, 32 * sl.k, 0, s>>>((const double2*)dR, slot_stride, sl, newslot, r, npw,
+                                                        (double4_16a*)part);
+  k_anderson_solve<<<ne, 32, 0, s>>>((const double4_16a*)part, sl, newslot, mdim, gram, gamma);
+  launched(2);
   return cudaGetLastError();
 }
 
-// x <- x + beta r - sum_q (dX_q + beta dR_q) gamma_q  (per band)
-// x += beta r - sum_q gamma_q (dX_q + beta dR_q). One block row per band (no
+// out = x + beta r - sum_q gamma_q (dX_q + beta dR_q). One block row per band (no
 // division per element). With complex64 history the correction sum is formed
 // in FP32 and added to the FP64 iterate once.
 template <typename H>
-__global__ void k_anderson_update(double2* __restrict__ x, const double2* __restrict__ r, const H* __restrict__ dX,
-                                  const H* __restrict__ dR, long slot_stride, SlotList sl,
-                                  const double2* __restrict__ gamma, int mdim, int npw, double beta) {
+__global__ void __launch_bounds__(256) k_anderson_update(const double2* __restrict__ x, const double2* __restrict__ r,
+                                                         const H* __restrict__ dX, const H* __restrict__ dR,
+                                                         long slot_stride, SlotList sl,
+                                                         const double2* __restrict__ gamma, int mdim, int npw,
+                                                         double beta, double2* __restrict__ out) {
   using A = decltype(H::x);
   const int k = sl.k;
   const int b = blockIdx.y;
@@ -418,6 +424,7 @@ __global__ void k_anderson_update(double2* __restrict__ x, const double2* __rest
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < npw; i += gridDim.x * blockDim.x) {
     const long t = boff + i;
     A cx = 0, cy = 0;
+#pragma unroll 4
     for (int q = 0; q < k; ++q) {
       const long sq = (long)sl.s[q] * slot_stride + t;
       const H a = dX[sq], c = dR[sq];
@@ -426,27 +433,24 @@ __global__ void k_anderson_update(double2* __restrict__ x, const double2* __rest
       cx += ux * gx - uy * gy;
       cy += ux * gy + uy * gx;
     }
-    double2 v = x[t];
-    const double2 rr = r[t];
-    v.x += beta * rr.x - (double)cx;
-    v.y += beta * rr.y - (double)cy;
-    x[t] = v;
+    const double2 v = x[t], rr = r[t];
+    out[t] = make_double2(v.x + (beta * rr.x - (double)cx), v.y + (beta * rr.y - (double)cy));
   }
 }
 
-cudaError_t anderson_update(double2* x, const double2* r, const void* dX, const void* dR, long slot_stride,
+cudaError_t anderson_update(const double2* x, const double2* r, const void* dX, const void* dR, long slot_stride,
                             const SlotList& sl, const double2* gamma, int mdim, int npw, long n, double beta, int f32,
-                            cudaStream_t s) {
+                            double2* out, cudaStream_t s) {
   if (sl.k > kSlotMax) return cudaErrorInvalidValue;
   const int ne = npw > 0 ? (int)(n / npw) : 0;
   if (ne == 0) return cudaSuccess;
   const dim3 grid((unsigned)std::min(32, (npw + 255) / 256), (unsigned)ne);
   if (f32)
     k_anderson_update<float2><<<grid, 256, 0, s>>>(x, r, (const float2*)dX, (const float2*)dR, slot_stride, sl, gamma,
-                                                   mdim, npw, beta);
+                                                   mdim, npw, beta, out);
   else
     k_anderson_update<double2><<<grid, 256, 0, s>>>(x, r, (const double2*)dX, (const double2*)dR, slot_stride, sl,
-                                                    gamma, mdim, npw, beta);
+                                                    gamma, mdim, npw, beta, out);
   launched();
   return cudaGetLastError();
 }
@@ -476,7 +480,7 @@ __global__ void k_drho(const double* __restrict__ a, const double* __restrict__ 
 cudaError_t rho_change(const double* a, const double* b, long N, double* part, double* out, cudaStream_t s) {
   const unsigned nb = nblk(N, 256, 1024);
   k_drho<<<nb, 256, 0, s>>>(a, b, N, part); launched();
-  k_finalize<<<1, 32, 0, s>>>(part, nb, 1, out); launched();
+  finalize(part, nb, 1, out, s);
   return cudaGetLastError();
 }
 
@@ -525,11 +529,11 @@ cudaError_t energy_sums(const double* rho, const double* vion, const double* vh,
                         double* out8, cudaStream_t s) {
   const unsigned nb = nblk(g.N(), 256, 1024);
   k_grid_sums<<<nb, 256, 0, s>>>(rho, vion, vh, use_h, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2], part); launched();
-  k_finalize<<<1, 32, 0, s>>>(part, nb, 6, out8); launched();
+  finalize(part, nb, 6, out8, s);
   const long n = (long)npw * ne;
   const unsigned nb2 = nblk(n, 256, 1024);
   k_kin_sum<<<nb2, 256, 0, s>>>(c, kin, npw, n, part + 6 * 1024); launched();
-  k_finalize<<<1, 32, 0, s>>>(part + 6 * 1024, nb2, 1, out8 + 6); launched();
+  finalize(part + 6 * 1024, nb2, 1, out8 + 6, s);
   if (negM != nullptr) { k_trace_real<<<1, 32, 0, s>>>(negM, ne, out8 + 7); launched(); }
   return cudaGetLastError();
 }

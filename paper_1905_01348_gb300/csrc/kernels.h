@@ -22,18 +22,21 @@ cudaError_t ion_potential(double* v, Grid3 g, const double* cell, const double* 
                           double sigma, cudaStream_t s);
 cudaError_t hartree_factor(double* f, Grid3 g, const double* cell, cudaStream_t s);
 cudaError_t half_step(const double2* psi, const double2* R, double hdt, double2* out, long n, cudaStream_t s);
-cudaError_t pt_residual(const double2* psi_f, const double2* T, const double2* ph, double hdt, double2* r, long n,
-                        double* part, double* out_norm2, cudaStream_t s);
 cudaError_t precond_step(double2* x, const double2* R, const double* kin, int npw, long n, double tau, cudaStream_t s);
-cudaError_t anderson_push(const double2* x, const double2* r, double2* xp, double2* rp, void* dx, void* dr, long n,
-                          int have_prev, int f32, cudaStream_t s);
-cudaError_t anderson_dots(const void* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r,
-                          int npw, int ne, int mdim, double2* gram, double2* rhs, int f32, cudaStream_t s);
-cudaError_t anderson_solve(const double2* gram, const double2* rhs, const SlotList& sl, int mdim, int ne,
-                           double2* gamma, cudaStream_t s);
-cudaError_t anderson_update(double2* x, const double2* r, const void* dX, const void* dR, long slot_stride,
+// r (holding r_prev) <- -(x + i hdt T - ph); dx = x - xp and dr = r - r_prev when have_prev;
+// part (1024 doubles) takes the block partials of |r|^2 that residual_norm2 sums up
+cudaError_t residual_push(const double2* x, const double2* T, const double2* ph, double hdt, const double2* xp,
+                          double2* r, void* dx, void* dr, long n, int have_prev, int f32, double* part,
+                          cudaStream_t s);
+cudaError_t residual_norm2(const double* part, long n, double* out, cudaStream_t s);
+// gram entries of the new slot and gamma per band; part: at least 8 * 4 * sl.k * ne doubles
+cudaError_t anderson_gamma(const void* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r,
+                           int npw, int ne, int mdim, double2* gram, double2* gamma, void* part, int f32,
+                           cudaStream_t s);
+// out = x + beta r - sum_q gamma_q (dX_q + beta dR_q)
+cudaError_t anderson_update(const double2* x, const double2* r, const void* dX, const void* dR, long slot_stride,
                             const SlotList& sl, const double2* gamma, int mdim, int npw, long n, double beta, int f32,
-                            cudaStream_t s);
+                            double2* out, cudaStream_t s);
 cudaError_t kinetic_shifted(const double* gk3, int npw, double ax, double ay, double az, double* kin, cudaStream_t s);
 cudaError_t rho_change(const double* a, const double* b, long N, double* part, double* out, cudaStream_t s);
 // out8: [0] sum vion rho, [1] sum vh rho, [2] sum rho^{4/3}, [3..5] sum r rho,

@@ -221,7 +221,6 @@ size_t carve(pt_system* sys, const pt_params* p, uintptr_t base) {
   t->psi_f = c.take<double2>(pe);
   t->hpsi = c.take<double2>(pe);
   t->tmp = c.take<double2>(pe);
-  t->rbuf = c.take<double2>(pe);
   t->wg = c.take<double2>(pe);
   t->xi = c.take<double2>(pe);
   t->xprev = c.take<double2>(pe);
@@ -271,7 +270,6 @@ size_t carve(pt_system* sys, const pt_params* p, uintptr_t base) {
   t->gemm_ws_elems = std::max<size_t>(16, 152 / tiles_tc) * ne * ne + 65536;
   t->gemm_ws = c.take<double2>(t->gemm_ws_elems);
   t->gram = c.take<double2>((size_t)ne * std::max(1, m) * std::max(1, m));
-  t->rhs = c.take<double2>((size_t)ne * std::max(1, m));
   t->gamma = c.take<double2>((size_t)ne * std::max(1, m));
   t->part = c.take<double>(8192);
   t->red = c.take<double>(64);
