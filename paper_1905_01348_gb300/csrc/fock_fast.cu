@@ -1,476 +1,594 @@
 // FP32 pair pipeline for cubic grids of 32, 48, 64 or 96 points per edge (the
-// Si8 / Si64 / Si216 workloads, and 48 for the Si216 wavefunction grid): the same three passes as fock.cu (Eq. 3,
-// pair loop of Alg. 2) with compile-time line lengths and two-stage radix
-// plans, padded and transposed shared-memory rows (no bank conflicts), the
-// screened-kernel multiply fused between the last forward and the first
-// inverse stage of axis 0, accumulation through per-output contribution
-// lists, asynchronous global->shared copies for the pair intermediate, and
-// no work on the axis-2 frequency slabs that pair products cannot reach.
+// Si8 / Si64 / Si216 workloads, and 48 for the Si216 wavefunction grid): the same three
+// passes as fock.cu (Eq. 3, pair loop of Alg. 2) on packed pairs of lines (fft_pk.cuh):
+// every value in registers and shared memory is a pk2, the same element of two
+// neighbouring grid rows, so that one packed FP32 instruction, one 16-byte shared access
+// and one address serve two lines.
+//
+// Pair intermediate X: [pair slot][i2][i0][i1 / 2] of pk2, a pk2 holding i1 and i1 + 1
+// (the byte count and position of two complex64 values); only the axis-2 slabs that
+// pair products can reach are written or read.
+// Kernel table (fast_khat_index): [i2][i1 / 4][(i1 / 2) % 2][i0] pairs of K(i1), K(i1 + 1),
+// i1 even: the two frequencies one pk2 of F2's inner step holds, in the order its threads read.
 #include <algorithm>
 
 #include "common.cuh"
-#include "fft_ct.cuh"
+#include "fft_pk.cuh"
 #include "internal.h"
 
 namespace pt {
 
 namespace {
 
-constexpr int TT = kTileMax;   // orbitals per tile edge
-constexpr int RR = 4;          // grid rows per block in F1 / F3
+constexpr int TT = kTileMax;      // orbitals per tile edge
 constexpr int NPAIR = TT * TT;
+constexpr int RP = 4;             // row pairs per block in F1 / F3
+constexpr int RR = 2 * RP;        // grid rows per block
+constexpr int QB = 4;             // pairs of a tile worked on together in F1 / F3
 
-template <int L> struct Cfg { static constexpr int NT13 = 256; };
-
-template <int L> constexpr int WS = L + 1;   // work-buffer row stride (complex values)
-
-template <int L> constexpr size_t smem13() { return sizeof(float2) * (size_t)(L + NPAIR * RR * WS<L>); }
-
-// Row layout of the F1 / F3 work buffer: row l (pair p, grid row r) at stride
-// L + 1, and inside each aligned group of 16 elements the 4 x 4 block is
-// transposed (element 4a + b sits at 4b + a). FFT stages access one element of
-// 16 consecutive rows per half-warp (distinct banks through the odd stride);
-// the X loads and stores access 4 rows x 4 consecutive elements per half-warp,
-// which the transpose also spreads over 16 distinct bank pairs.
-template <int L> struct RowsT {
-  __device__ __forceinline__ static int at(int l, int e) {
-    return l * WS<L> + ((e & ~15) | ((e & 3) << 2) | ((e >> 2) & 3));
-  }
+template <int L> struct Sizes {
+  static constexpr int M = L / 8;                       // second radix of the axis-2 lines
+  static constexpr int MP = M + 1;                      // odd: spreads (row pair, k2) over the banks
+  static constexpr int QS = 8 * RP * MP + 2;            // one pair's part of the exchange buffer; 2 mod 8
+  static constexpr int NT = 16 * (M > 8 ? M : 8);       // threads of F1 / F3
+  static constexpr int RS = L == 48 ? L + 2 : L + (M == 12 ? 6 : M == 8 ? 4 : 2);   // orbital row stride
+  static constexpr size_t tw_bytes = sizeof(pk2) * L;
+  static constexpr size_t orb_bytes = sizeof(float2) * 2 * TT * RR * RS;
+  static constexpr size_t smem13 = tw_bytes + orb_bytes + sizeof(pk2) * QB * QS;
+  static constexpr int CP = L / 2;                      // pk2 values of a row of X
+  // F2: L = 4 Q, Q / 2 column pairs of 16 Q values each
+  static constexpr int Q = L / 4;
+  static constexpr int CPQ = Q / 2;
+  static constexpr int SC = 16 * Q + 1;
+  static constexpr int ROT = Q == 16 ? 0 : Q == 12 ? 6 : 4;   // rotation of k2 at odd u: spreads (c', p) over the banks
+  static constexpr size_t smem2 = sizeof(pk2) * (4 * Q + 4 * CPQ + CPQ * SC);
+  // 96: two blocks of 192 threads (one round of steps A and C) beat three of 96 or 128 by 4 to
+  // 5%, and by 12% three of 192, whose 96 registers spill
+  static constexpr int NT2 = L == 96 ? 192 : L == 64 ? 128 : L == 48 ? 96 : 64;
+  static constexpr int MINB2 = L == 96 ? 2 : L == 64 ? 4 : 6;
+  static constexpr int RG = L * (L / RR);               // row groups of a tile
+  static constexpr int RES1 = L == 96 ? 2 : 4;          // resident F1 and F3 blocks per SM
+  static constexpr int RES3 = L == 96 ? 2 : 3;
 };
 
-__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc) {
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// waits until at most N of the thread's newest groups are in flight
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // Axis-2 slab i2 is dead when its frequency lies beyond the pair reach R:
 // the pair products have no component there (the slab stays unwritten in X).
 template <int L> __device__ __forceinline__ bool dead_slab(int i2, int reach) { return i2 > reach && i2 < L - reach; }
 
+// bit k1: slab k2 + 8 k1 is live
+template <int L> __device__ __forceinline__ unsigned live_mask(int k2, int reach) {
+  unsigned m = 0;
+  for (int k1 = 0; k1 < L / 8; ++k1) m |= dead_slab<L>(k2 + 8 * k1, reach) ? 0u : 1u << k1;
+  return m;
+}
+
 // An off-diagonal tile of two full orbital blocks: orbitals 0..3 and 4..7,
 // pair 4a + b = (a, 4 + b).
 __device__ __forceinline__ bool full_tile(const PairTile& tl) { return tl.n_orb == 2 * TT && tl.n_pairs == NPAIR; }
 
-__device__ __forceinline__ const float2* orb_ptr(const PairTile& tl, int o) {
-  return static_cast<const float2*>(tl.in[o]);
+// the tile record into shared memory, asynchronously
+__device__ __forceinline__ void copy_tile(PairTile* dst, const PairTile* src, int tid) {
+  static_assert(sizeof(PairTile) % 16 == 0, "copied by 16 bytes");
+  if (tid < (int)(sizeof(PairTile) / 16))
+    cp_async16(reinterpret_cast<unsigned char*>(dst) + 16 * tid, reinterpret_cast<const unsigned char*>(src) + 16 * tid);
 }
-__device__ __forceinline__ float2* acc_ptr(const PairTile& tl, int o) { return static_cast<float2*>(tl.out[o]); }
+
+// twiddles W_L^(n1 k2) = c - i s as (c, c, s, s) at [k2][n1]
+template <int L> __device__ __forceinline__ void load_twiddles(pk2* tw, const float2* __restrict__ tw_g, int tid, int nt) {
+  constexpr int M = Sizes<L>::M;
+  for (int t = tid; t < L; t += nt) {
+    const float2 w = tw_g[(t / M) * (t % M)];
+    tw[t] = {f2(w.x), f2(-w.y)};
+  }
+}
+
+// RR rows (from element roff) of the tile's orbitals o0 .. o1 - 1 into shared memory by
+// 16-byte asynchronous copies
+template <int L>
+__device__ __forceinline__ void load_orbitals(float2* orb, const PairTile& tl, int o0, int o1, long roff, int tid) {
+  using S = Sizes<L>;
+  constexpr int CH = RR * L / 2, PER = (CH + S::NT - 1) / S::NT;   // 16-byte chunks per orbital and per thread
+  const int end = min(tl.n_orb, o1);
+  for (int o = o0; o < end; ++o) {
+    const float2* src = static_cast<const float2*>(tl.in[o]) + roff;
+    float2* dst = orb + o * (RR * S::RS);
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int e = tid + q * S::NT;
+      if (CH % S::NT == 0 || e < CH) cp_async16(dst + (e / (L / 2)) * S::RS + 2 * (e % (L / 2)), src + 2 * e);
+    }
+  }
+}
+
+// element n of rows 2 rp and 2 rp + 1 of orbital o
+template <int L> __device__ __forceinline__ pk2 orb_at(const float2* orb, int o, int rp, int n) {
+  const float2* p = orb + (o * RR + 2 * rp) * Sizes<L>::RS + n;
+  const float2 u = p[0], v = p[Sizes<L>::RS];
+  return {make_float2(u.x, v.x), make_float2(u.y, v.y)};
+}
+
+// a load that stays where it is written: the compiler would move it down to its use,
+// past the barrier, and its latency with it
+__device__ __forceinline__ pk2 load_now(const pk2* p) {
+  pk2 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+               : "=f"(v.re.x), "=f"(v.re.y), "=f"(v.im.x), "=f"(v.im.y)
+               : "l"(p)
+               : "memory");
+  return v;
+}
+
+// adds v to a row pair in global memory without waiting for the old values; every element
+// has one writer per launch, so the sums keep their order
+__device__ __forceinline__ void red_add(float2* p, float x, float y) {
+  asm volatile("red.global.add.v2.f32 [%0], {%1, %2};\n" ::"l"(p), "f"(x), "f"(y) : "memory");
+}
+template <int L> __device__ __forceinline__ void add_rows(float2* p, pk2 v) {
+  red_add(p, v.re.x, v.im.x);
+  red_add(p + L, v.re.y, v.im.y);
+}
+
+__device__ __forceinline__ pk2 pk_select(bool first, pk2 a, pk2 b) {
+  return {make_float2(first ? a.re.x : b.re.x, first ? a.re.y : b.re.y),
+          make_float2(first ? a.im.x : b.im.x, first ? a.im.y : b.im.y)};
+}
+__device__ __forceinline__ pk2 pk_shfl_xor(pk2 a, int m) {
+  return {make_float2(__shfl_xor_sync(0xffffffffu, a.re.x, m), __shfl_xor_sync(0xffffffffu, a.re.y, m)),
+          make_float2(__shfl_xor_sync(0xffffffffu, a.im.x, m), __shfl_xor_sync(0xffffffffu, a.im.y, m))};
+}
 
 }  // namespace
 
-// F1: pair products of RR grid rows for every pair of the tile (orbital rows
-// read through the read-only cache, four products per thread per round with
-// all their loads issued first), forward FFT along axis 2, store the live
-// slabs of X[slot][i2][i0][i1].
+// F1: pair products of RR grid rows for every pair of the tile, forward FFT along axis 2,
+// store of the live slabs. Resident blocks walk the (tile, row group) items; the next item's
+// orbital rows arrive by asynchronous copies, each orbital's as soon as the current item
+// is done with its place, so no item waits for memory. The pairs are worked on four at a
+// time: (row pair, n1, pair) threads form the products and run the 8-point DFTs, the values
+// cross shared memory once, and (row pair, k2, pair) threads run the M-point DFTs and store
+// from registers (64 contiguous bytes per pair and slab). The pair is the fastest thread
+// index of the first step, so one read of a left orbital serves four pairs; a full tile
+// keeps the right orbitals' values in registers for all of its left ones.
 template <int L>
-__global__ void __launch_bounds__(Cfg<L>::NT13, 4) k_fast_f1(const PairTile* __restrict__ tiles, int tile0,
-                                                          float2* __restrict__ X, const float2* __restrict__ tw_g,
+__global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES1) k_fast_f1(const PairTile* __restrict__ tiles, int n_items,
+                                                          pk2* __restrict__ X, const float2* __restrict__ tw_g,
                                                           int reach) {
-  using A = RowsT<L>;
-  constexpr int NT = Cfg<L>::NT13;
-  constexpr int ROW = RR * L;
-  constexpr long N = (long)L * L * L;
+  using S = Sizes<L>;
+  constexpr int M = S::M, MP = S::MP, QS = S::QS, RG = S::RG;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ PairTile tl;
-  float2* tw = reinterpret_cast<float2*>(smem_raw);
-  float2* work = tw + L;
-  const int tid = threadIdx.x;
-  if (tid == 0) tl = tiles[tile0 + blockIdx.y];
-  for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
+  __shared__ __align__(16) PairTile ring[3];   // the tiles of this item, the next and the one after
+  pk2* tw = reinterpret_cast<pk2*>(smem_raw);
+  float2* orb = reinterpret_cast<float2*>(smem_raw + S::tw_bytes);
+  pk2* ex = reinterpret_cast<pk2*>(smem_raw + S::tw_bytes + S::orb_bytes);
+  const int tid = threadIdx.x, stride = gridDim.x;
+  copy_tile(&ring[0], tiles + blockIdx.x / RG, tid);
+  if (blockIdx.x + stride < n_items) copy_tile(&ring[1], tiles + (blockIdx.x + stride) / RG, tid);
+  load_twiddles<L>(tw, tw_g, tid, S::NT);
+  cp_async_wait_all();
   __syncthreads();
-  constexpr int NB1 = L / RR;
-  const int i0 = blockIdx.x / NB1;
-  const int i1s = (blockIdx.x % NB1) * RR;
-  const long roff = ((long)i0 * L + i1s) * L;
-  const int np = tl.n_pairs;
-  if (full_tile(tl)) {
-    // off-diagonal 4 x 4 tile: pair 4a + b is (a, 4 + b); the eight orbital
-    // values of an element are loaded once (eight loads in flight)
-    for (int e = tid; e < ROW; e += NT) {
-      float2 v[2 * TT];
+  load_orbitals<L>(orb, ring[0], 0, 2 * TT, (long)(blockIdx.x % RG) * (RR * L), tid);
+  const int qa = tid % QB, n1 = (tid / QB) % M, rpa = tid / (QB * M);
+  const int rpb = tid % RP, k2b = (tid / RP) % 8, qb = tid / (8 * RP);
+  const bool first = rpa < RP;   // M < 8: the last threads only take part in the second step
+  const unsigned live = live_mask<L>(k2b, reach);
+  int cur = 0;
+  bool was_full = false;
+  for (int item = blockIdx.x; item < n_items; item += stride) {
+    // After a full item four groups are in flight, orbitals (0, right), 1, 2, 3; a full item
+    // waits for each as it comes to it.
+    const bool piped = was_full && full_tile(ring[cur]);
+    if (piped) cp_async_wait<3>(); else cp_async_wait_all();
+    __syncthreads();
+    const int nxt = cur == 2 ? 0 : cur + 1, far = cur == 0 ? 2 : cur - 1;
+    const PairTile& tl = ring[cur];
+    const bool more = item + stride < n_items;
+    const long noff = (long)((item + stride) % RG) * (RR * L);
+    if (item + 2 * stride < n_items) copy_tile(&ring[far], tiles + (item + 2 * stride) / RG, tid);
+    const int np = tl.n_pairs;
+    const bool full = full_tile(tl);
+    pk2* xb = X + (((long)(item / RG) * NPAIR + qb) * L + k2b) * (L * S::CP) + (item % RG) * RP + rpb;
+    pk2 b[8];
+    if (full && first) {
 #pragma unroll
-      for (int o = 0; o < 2 * TT; ++o) v[o] = __ldg(orb_ptr(tl, o) + roff + e);
-      const int row = e / L, col = e % L;
-#pragma unroll
-      for (int a = 0; a < TT; ++a)
-#pragma unroll
-        for (int b = 0; b < TT; ++b) work[A::at((a * TT + b) * RR + row, col)] = cmulc(v[a], v[TT + b]);
+      for (int n2 = 0; n2 < 8; ++n2) b[n2] = orb_at<L>(orb, TT + qa, rpa, n1 + M * n2);
     }
-  } else {
-    // any tile: four products per thread per round, all eight loads issued before the first use
-    constexpr int U = 4;
-    for (int base = tid; base < np * ROW; base += U * NT) {
-      float2 a[U], b[U];
+    for (int p0 = 0; p0 < np; p0 += QB, xb += (long)QB * L * L * S::CP) {
+      if (first && p0 + qa < np) {
+        if (!full) {
+          const int oj = tl.pj[p0 + qa];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int idx = base + u * NT;
-        if (idx < np * ROW) {
-          const int p = idx / ROW, e = idx % ROW;
-          a[u] = __ldg(orb_ptr(tl, tl.pi[p]) + roff + e);
-          b[u] = __ldg(orb_ptr(tl, tl.pj[p]) + roff + e);
+          for (int n2 = 0; n2 < 8; ++n2) b[n2] = orb_at<L>(orb, oj, rpa, n1 + M * n2);
+        }
+        const int oi = tl.pi[p0 + qa];
+        pk2 v[8];
+#pragma unroll
+        for (int n2 = 0; n2 < 8; ++n2) {
+          const pk2 a = orb_at<L>(orb, oi, rpa, n1 + M * n2);
+          v[n2] = {vfma(a.re, b[n2].re, vmul(a.im, b[n2].im)), vdet(a.re, b[n2].im, a.im, b[n2].re)};
+        }
+        pk_dft<8, false>(v);   // of conj(a) b
+        pk2* dst = ex + qa * QS + rpa * MP + n1;
+        dst[0] = v[0];
+#pragma unroll
+        for (int k2 = 1; k2 < 8; ++k2) dst[k2 * RP * MP] = ptwiddle<false>(v[k2], tw[k2 * M + n1]);
+      }
+      __syncthreads();
+      if (more) {   // places of orbitals this item no longer reads
+        if (full) {
+          load_orbitals<L>(orb, ring[nxt], p0 / QB, p0 / QB + 1, noff, tid);
+          if (p0 == 0) load_orbitals<L>(orb, ring[nxt], TT, 2 * TT, noff, tid);
+        } else if (p0 + QB >= np) {
+          load_orbitals<L>(orb, ring[nxt], 0, 2 * TT, noff, tid);
         }
       }
+      cp_async_commit();
+      if (qb < QB && p0 + qb < np) {
+        pk2 v[M];
+        const pk2* src = ex + qb * QS + (k2b * RP + rpb) * MP;
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int idx = base + u * NT;
-        if (idx < np * ROW) {
-          const int p = idx / ROW, e = idx % ROW;
-          work[A::at(p * RR + e / L, e % L)] = cmulc(a[u], b[u]);
-        }
+        for (int m = 0; m < M; ++m) v[m] = src[m];
+        pk_dft<M, false>(v);
+#pragma unroll
+        for (int k1 = 0; k1 < M; ++k1)
+          if (live & (1u << k1)) xb[(long)k1 * 8 * L * S::CP] = v[k1];
       }
+      if (piped) cp_async_wait<3>();
+      __syncthreads();
     }
-  }
-  __syncthreads();
-  ct_forward_lay<float2, L, NPAIR * RR, NT, A>(work, np * RR, tw, tid);
-  // lanes: r fastest, then i2, so each (pair, i2) writes one run of RR values along i1
-  const long slot0 = (long)blockIdx.y * NPAIR;
-  const int r = tid % RR;
-  for (int p = 0; p < np; ++p) {
-    float2* xp = X + (slot0 + p) * N + (long)i0 * L + i1s + r;
-    for (int i2 = tid / RR; i2 < L; i2 += NT / RR)
-      if (!dead_slab<L>(i2, reach)) xp[(long)i2 * L * L] = work[A::at(p * RR + r, i2)];
+    cur = nxt;
+    was_full = full;
   }
 }
 
-// Register-line transforms of 96-point lines (L = 96 = 12 x 8, n = n1 + 12 n2,
-// k = k2 + 8 k1): two threads share a line, thread half h holding n1 in [6h, 6h + 6)
-// (48 values); the partner is the lane XM apart. Used by F2 at 96^3.
-namespace l96 {
-constexpr int L = 96, W = L + 1;
-
-// Twiddle indices n1 k2 stay below 96 (n1 < 12, k2 < 8), so they need no reduction.
-
-// 8-point DFTs over n2 of the owned n1 = 6h + a, then the twiddle W96^(n1 k2) (forward)
-__device__ __forceinline__ void stage_a_fwd(float2 (&v)[6][8], int h, const float2* tw) {
-  const int h6 = 6 * h;
-#pragma unroll
-  for (int a = 0; a < 6; ++a) {
-    dft<8, false>(v[a]);
-#pragma unroll
-    for (int k2 = 1; k2 < 8; ++k2) v[a][k2] = cmul(v[a][k2], tw[a * k2 + h6 * k2]);
-  }
-}
-
-// inverse 8-point DFTs over k2: v[a][n2] = x[6h + a + 12 n2]
-__device__ __forceinline__ void stage_a_inv(float2 (&v)[6][8]) {
-#pragma unroll
-  for (int a = 0; a < 6; ++a) dft<8, true>(v[a]);
-}
-
-// forward exchange for k2 = 4h + b: z[n1], n1 = 0..11, from the owned v[.][b or 4 + b] and the partner's
-template <int XM = 1>
-__device__ __forceinline__ void exch_fwd(const float2 (&v)[6][8], int h, int b, float2 (&z)[12]) {
-#pragma unroll
-  for (int a = 0; a < 6; ++a) {
-    const float2 mine = h ? v[a][4 + b] : v[a][b];   // my k2 = 4h + b
-    const float2 send = h ? v[a][b] : v[a][4 + b];   // the partner's k2 = 4(1 - h) + b
-    float2 got;
-    got.x = __shfl_xor_sync(0xffffffffu, send.x, XM);
-    got.y = __shfl_xor_sync(0xffffffffu, send.y, XM);
-    z[a] = h ? got : mine;        // n1 = a (owned by half 0)
-    z[6 + a] = h ? mine : got;    // n1 = 6 + a (owned by half 1)
-  }
-}
-
-// inverse twiddle of Z[n1][k2], k2 = 4h + b, then the exchange back into v[a][b], v[a][4 + b]
-template <int XM = 1>
-__device__ __forceinline__ void exch_inv(float2 (&z)[12], int h, int b, const float2* tw, float2 (&v)[6][8]) {
-  const int h4 = 4 * h;
-#pragma unroll
-  for (int n1 = 1; n1 < 12; ++n1) {
-    float2 w = tw[n1 * b + n1 * h4];
-    w.y = -w.y;
-    z[n1] = cmul(z[n1], w);
-  }
-#pragma unroll
-  for (int a = 0; a < 6; ++a) {
-    const float2 mine = h ? z[6 + a] : z[a];          // my n1 = 6h + a
-    const float2 send = h ? z[a] : z[6 + a];          // the partner's n1
-    float2 got;
-    got.x = __shfl_xor_sync(0xffffffffu, send.x, XM);
-    got.y = __shfl_xor_sync(0xffffffffu, send.y, XM);  // my n1, the partner's k2 = 4(1 - h) + b
-    v[a][b] = h ? got : mine;
-    v[a][4 + b] = h ? mine : got;
-  }
-}
-}  // namespace l96
-
-// F2: one live (pair, i2) slab per block: asynchronous copies into the padded
-// work buffer, FFT along axis 1 and axis 0, multiply by the screened kernel
-// (fused between the last forward and first inverse stage of axis 0), inverse
-// along axis 0 and axis 1, store. Blocks are small so that two or more are
-// resident per SM and one block's barrier waits overlap another's work (this
-// beat a single persistent block per SM fed by bulk-copy prefetch, and one
-// block of 384 threads without sub-batches).
-template <int L> struct Cfg2;
-template <> struct Cfg2<32> { static constexpr int NT = 128, SUB = 32, MINB = 4; };
-template <> struct Cfg2<48> { static constexpr int NT = 192, SUB = 48, MINB = 4; };
-template <> struct Cfg2<64> { static constexpr int NT = 256, SUB = 32, MINB = 3; };
-// 96: 192 threads balance both radices (48 lines x 12 radix-8 or 8 radix-12
-// butterflies = 3 or 2 per thread) and leave room for 152 registers without spills.
-template <> struct Cfg2<96> { static constexpr int NT = 192, SUB = 48, MINB = 2; };
-template <int L> constexpr size_t smem2() { return sizeof(float2) * (size_t)(L + L * WS<L>); }
-
+// F2: one live (pair, i2) slab per block: FFT along both of its axes, kernel multiply,
+// inverse FFTs, in place. Shared-memory bandwidth bounds it (every value crosses at 16
+// bytes per pair of lines), so the 2D transform takes three steps instead of two per axis:
+// with L = 4 Q,
+//   A  Q-point DFTs along axis 0 over i0 = n1 + 4 n2 (packed over neighbouring columns i1,
+//      as X stores them), straight from global memory;
+//   B  both radix-4 steps at once, 4 x 4 values per thread: axis 0 over n1 (rows k0 = k2 +
+//      Q k1) and axis 1 over i1 = c + Q p (outputs q, twiddle W_L^(c q)), then a 2 x 2
+//      transpose in registers packs over (q, q + 1) instead of (c, c + 1);
+//   C  Q-point DFTs along axis 1 over c (frequency 4 m + q), kernel multiply, and back;
+// then B and A backwards, storing from registers. Values stay at fixed places (a step's
+// outputs overwrite its own inputs): place (c', u, k2) = c' SC + u Q + k2 with c' = c / 2 and
+// u = (n1, p) before and (k1, c & 1, q / 2) after B; at odd u, k2 is rotated by ROT. Threads
+// of neighbouring c' (A) and of neighbouring k2 (B, C) touch distinct banks.
 template <int L>
-__global__ void __launch_bounds__(Cfg2<L>::NT, Cfg2<L>::MINB) k_fast_f2(float2* __restrict__ X,
-                                                                         const PairTile* __restrict__ tiles, int tile0,
-                                                                         const float* __restrict__ khat_t,
-                                                                         const float2* __restrict__ tw_g, int reach) {
-  constexpr int NT = Cfg2<L>::NT;
-  constexpr int SUB = Cfg2<L>::SUB;
-  static_assert(L % SUB == 0, "the sub-batches of SUB lines must tile the L lines of a slab exactly");
-  constexpr int SLAB = L * L;
-  constexpr int R1 = Plan2<L>::R1, R2 = Plan2<L>::R2;
-  constexpr int W = WS<L>;
+__global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
+    k_fast_f2(pk2* __restrict__ X, const PairTile* __restrict__ tiles, const float2* __restrict__ kt2,
+              const float2* __restrict__ tw_g, int reach) {
+  using S = Sizes<L>;
+  constexpr int Q = S::Q, CP = S::CP, CPQ = S::CPQ, SC = S::SC, ROT = S::ROT, NT = S::NT2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int tid = threadIdx.x;
   const int slot = blockIdx.y;
-  if (slot % NPAIR >= tiles[tile0 + slot / NPAIR].n_pairs) return;
+  if (slot % NPAIR >= tiles[slot / NPAIR].n_pairs) return;
   // live slabs only: blockIdx.x in [0, n_live) maps to frequencies 0..R, then -R..-1
   const int i2 = (int)blockIdx.x <= reach ? (int)blockIdx.x : (int)blockIdx.x + (L - (int)gridDim.x);
-  float2* tw = reinterpret_cast<float2*>(smem_raw);
-  float2* buf = tw + L;
-  for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
-  float2* slab = X + ((long)slot * L + i2) * SLAB;
-  for (int e = tid; e < SLAB; e += NT) cp_async8(buf + (e / L) * W + e % L, slab + e);
-  cp_async_wait_all();
+  pk2* twa = reinterpret_cast<pk2*>(smem_raw);   // W_L^(n1 k2) at [n1][k2]
+  pk2* twb = twa + 4 * Q;                        // W_L^(c q), c = 2 c' and 2 c' + 1, at [q][c']
+  pk2* buf = twb + 4 * CPQ;
+  for (int t = tid; t < 4 * Q; t += NT) {
+    const float2 w = tw_g[(t / Q) * (t % Q)];
+    twa[t] = {f2(w.x), f2(-w.y)};
+  }
+  for (int t = tid; t < 4 * CPQ; t += NT) {
+    const int q = t / CPQ, c = 2 * (t % CPQ);
+    const float2 w = tw_g[q * c], z = tw_g[q * (c + 1)];
+    twb[t] = {make_float2(w.x, z.x), make_float2(-w.y, -z.y)};
+  }
+  pk2* slab = X + ((long)slot * L + i2) * (L * CP);
   __syncthreads();
 #pragma unroll 1
-  for (int l0 = 0; l0 < L; l0 += SUB) ct_stage<float2, false, L, R1, 1, SUB, NT, W, 1>(buf, SUB, tw, tid, l0);
-#pragma unroll 1
-  for (int l0 = 0; l0 < L; l0 += SUB) ct_stage<float2, false, L, R2, R1, SUB, NT, W, 1>(buf, SUB, tw, tid, l0);
-#pragma unroll 1
-  for (int l0 = 0; l0 < L; l0 += SUB) ct_stage<float2, false, L, R1, 1, SUB, NT, 1, W>(buf, SUB, tw, tid, l0);
-  const float* kt = khat_t + (long)i2 * SLAB;
-#pragma unroll 1
-  for (int l0 = 0; l0 < L; l0 += SUB)
-    ct_fused<float2, L, SUB, NT, 1, W>(buf, SUB, tw, tid, [kt](int line, int e) { return __ldg(kt + e * L + line); },
-                                      l0);
-#pragma unroll 1
-  for (int l0 = 0; l0 < L; l0 += SUB) ct_stage<float2, true, L, R1, R2, SUB, NT, 1, W>(buf, SUB, tw, tid, l0);
-#pragma unroll 1
-  for (int l0 = 0; l0 < L; l0 += SUB) ct_stage<float2, true, L, R2, 1, SUB, NT, W, 1>(buf, SUB, tw, tid, l0);
-#pragma unroll 1
-  for (int l0 = 0; l0 < L; l0 += SUB) ct_stage<float2, true, L, R1, R2, SUB, NT, W, 1>(buf, SUB, tw, tid, l0);
-  for (int e = tid; e < SLAB; e += NT) slab[e] = buf[(e / L) * W + e % L];
-}
-
-// F2 for 96-point lines with the lines in registers. Two threads share a line of
-// L = 96 = 12 x 8 points, n = n1 + 12 n2, k = k2 + 8 k1: thread half h holds the
-// points of n1 in [6h, 6h + 6) (48 values). Forward: 8-point DFTs over n2 in registers
-// (twiddle W96^(n1 k2)), then the two halves exchange by warp shuffles so that half h
-// holds k2 in [4h, 4h + 4) for all twelve n1, and 12-point DFTs over n1 give the outputs
-// k2 + 8 k1. The inverse runs the same steps backwards. The slab arrives by cp.async
-// into a shared buffer (rows padded to 97) and leaves from it; between the passes the
-// lines cross shared memory once per pass instead of once per radix stage. Column
-// pass: for each owned k2, forward 12-point DFT, kernel multiply, inverse 12-point DFT,
-// all in registers.
-
-template <int L>
-__global__ void __launch_bounds__(192, 2) k_fast_f2r(float2* __restrict__ X, const PairTile* __restrict__ tiles,
-                                                     int tile0, const float* __restrict__ khat_t,
-                                                     const float2* __restrict__ tw_g, int reach) {
-  static_assert(L == l96::L, "register-line F2 is written for 96-point lines");
-  using namespace l96;
-  constexpr int SLAB = L * L;
-  constexpr int XM = 16;                      // the two halves of a line are the lanes 16 apart
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  float2* tw = reinterpret_cast<float2*>(smem_raw);
-  float2* buf = tw + L;                       // [row][W]
-  const int tid = threadIdx.x, lane = tid & 31;
-  // a half-warp holds the same half h of 16 consecutive lines: its shared-memory accesses
-  // (one row of 16 lines, or 16 columns of one row) fall on distinct banks
-  const int line = (tid >> 5) * 16 + (lane & 15), h = lane >> 4;
-  const int slot = blockIdx.y;
-  if (slot % NPAIR >= tiles[tile0 + slot / NPAIR].n_pairs) return;
-  const int i2 = (int)blockIdx.x <= reach ? (int)blockIdx.x : (int)blockIdx.x + (L - (int)gridDim.x);
-  for (int t = tid; t < L; t += 192) tw[t] = tw_g[t];
-  float2* slab = X + ((long)slot * L + i2) * SLAB;
-  for (int e = tid; e < SLAB; e += 192) cp_async8(buf + (e / L) * W + e % L, slab + e);
-  cp_async_wait_all();
-  __syncthreads();
-  float2 v[6][8];
-  // ---- forward along axis 1 (rows): v[a][n2] = x[6h + a + 12 n2] of row `line`; outputs
-  // k = k2 + 8 k1 back into the row
+  for (int t = tid; t < 8 * Q; t += NT) {
+    const int c2 = t % CP, n1 = t / CP;
+    const pk2* src = slab + n1 * CP + c2;
+    pk2 v[Q];
 #pragma unroll
-  for (int n2 = 0; n2 < 8; ++n2)
+    for (int n2 = 0; n2 < Q; ++n2) v[n2] = src[n2 * 4 * CP];
+    pk_dft<Q, false>(v);
+    const int odd = (c2 / CPQ) & 1;
+    pk2* dst = buf + (c2 % CPQ) * SC + (4 * n1 + c2 / CPQ) * Q + odd * ROT;
+    pk2* wrap = dst - odd * Q;   // of the last ROT values
+    dst[0] = v[0];
 #pragma unroll
-    for (int a = 0; a < 6; ++a) v[a][n2] = buf[line * W + 6 * h + a + 12 * n2];
-  __syncthreads();   // every row is in registers before any is overwritten
-  stage_a_fwd(v, h, tw);
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    float2 z[12];
-    exch_fwd<XM>(v, h, b, z);
-    dft12<false>(z);
-#pragma unroll
-    for (int k1 = 0; k1 < 12; ++k1) buf[line * W + 4 * h + b + 8 * k1] = z[k1];
+    for (int k2 = 1; k2 < Q; ++k2) (k2 < Q - ROT ? dst : wrap)[k2] = ptwiddle<false>(v[k2], twa[n1 * Q + k2]);
   }
   __syncthreads();
-  // ---- axis 0 (columns): column c = line; forward, kernel multiply, inverse, in registers
-  {
-    const int c = line;
+#pragma unroll 1
+  for (int t = tid; t < CPQ * Q; t += NT) {
+    const int c1 = t / Q;
+    pk2* p = buf + c1 * SC + t % Q;                    // even u
+    pk2* r = buf + c1 * SC + (t % Q + ROT) % Q;        // odd u
+    pk2 v[4][4];
 #pragma unroll
-    for (int n2 = 0; n2 < 8; ++n2)
+    for (int u = 0; u < 16; ++u) v[u / 4][u % 4] = (u % 2 ? r : p)[u * Q];
 #pragma unroll
-      for (int a = 0; a < 6; ++a) v[a][n2] = buf[(6 * h + a + 12 * n2) * W + c];
-    stage_a_fwd(v, h, tw);
-    const float* kt = khat_t + (long)i2 * SLAB + c;
+    for (int h = 0; h < 4; ++h) pk_dft4(v[0][h], v[1][h], v[2][h], v[3][h]);
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      float2 z[12];
-      exch_fwd<XM>(v, h, b, z);
-      dft12<false>(z);                                   // frequency k0 = 4h + b + 8 k1 along axis 0
+    for (int h = 0; h < 4; ++h) pk_dft4(v[h][0], v[h][1], v[h][2], v[h][3]);
 #pragma unroll
-      for (int k1 = 0; k1 < 12; ++k1) z[k1] = cscale(z[k1], __ldg(kt + (4 * h + b + 8 * k1) * L));
-      dft12<true>(z);                                    // back to n1, this k2
-      exch_inv<XM>(z, h, b, tw, v);
+    for (int q = 1; q < 4; ++q) {
+      const pk2 w = twb[q * CPQ + c1];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) v[h][q] = ptwiddle<false>(v[h][q], w);
     }
-    stage_a_inv(v);
 #pragma unroll
-    for (int n2 = 0; n2 < 8; ++n2)
+    for (int h = 0; h < 4; ++h)
 #pragma unroll
-      for (int a = 0; a < 6; ++a) buf[(6 * h + a + 12 * n2) * W + c] = v[a][n2];
+      for (int g = 0; g < 2; ++g) {
+        const pk2 a = v[h][2 * g], b = v[h][2 * g + 1];
+        (g ? r : p)[(4 * h + g) * Q] = {make_float2(a.re.x, b.re.x), make_float2(a.im.x, b.im.x)};
+        (g ? r : p)[(4 * h + 2 + g) * Q] = {make_float2(a.re.y, b.re.y), make_float2(a.im.y, b.im.y)};
+      }
   }
   __syncthreads();
-  // ---- inverse along axis 1 (rows): inputs k2 + 8 k1 of row `line`, outputs back into it
+  const float2* kt = kt2 + (long)i2 * (L * CP);
+#pragma unroll 1
+  for (int t = tid; t < 8 * Q; t += NT) {
+    const int k2 = t % Q, k1 = (t / Q) % 4, g = t / (4 * Q);
+    pk2* p = buf + (4 * k1 + g) * Q + (k2 + g * ROT) % Q;
+    pk2 v[Q];
 #pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    float2 z[12];
+    for (int c = 0; c < Q; ++c) v[c] = p[(c >> 1) * SC + 2 * Q * (c & 1)];
+    pk_dft<Q, false>(v);
 #pragma unroll
-    for (int k1 = 0; k1 < 12; ++k1) z[k1] = buf[line * W + 4 * h + b + 8 * k1];
-    dft12<true>(z);
-    exch_inv<XM>(z, h, b, tw, v);
+    for (int m = 0; m < Q; ++m) {
+      const float2 kk = __ldg(kt + m * 8 * Q + t);   // [m][g][k1][k2]: t itself
+      v[m] = {vmul(v[m].re, kk), vmul(v[m].im, kk)};
+    }
+    pk_dft<Q, true>(v);
+#pragma unroll
+    for (int c = 0; c < Q; ++c) p[(c >> 1) * SC + 2 * Q * (c & 1)] = v[c];
   }
-  stage_a_inv(v);
-  __syncthreads();   // every row is in registers before any is overwritten
-#pragma unroll
-  for (int n2 = 0; n2 < 8; ++n2)
-#pragma unroll
-    for (int a = 0; a < 6; ++a) buf[line * W + 6 * h + a + 12 * n2] = v[a][n2];
   __syncthreads();
-  for (int e = tid; e < SLAB; e += 192) slab[e] = buf[(e / L) * W + e % L];
+#pragma unroll 1
+  for (int t = tid; t < CPQ * Q; t += NT) {
+    const int c1 = t / Q;
+    pk2* p = buf + c1 * SC + t % Q;                    // even u
+    pk2* r = buf + c1 * SC + (t % Q + ROT) % Q;        // odd u
+    pk2 v[4][4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h)
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        const pk2 a = (g ? r : p)[(4 * h + g) * Q], b = (g ? r : p)[(4 * h + 2 + g) * Q];
+        v[h][2 * g] = {make_float2(a.re.x, b.re.x), make_float2(a.im.x, b.im.x)};
+        v[h][2 * g + 1] = {make_float2(a.re.y, b.re.y), make_float2(a.im.y, b.im.y)};
+      }
+#pragma unroll
+    for (int q = 1; q < 4; ++q) {
+      const pk2 w = twb[q * CPQ + c1];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) v[h][q] = ptwiddle<true>(v[h][q], w);
+    }
+#pragma unroll
+    for (int h = 0; h < 4; ++h) pk_dft<4, true>(v[h]);
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      pk2 z[4] = {v[0][h], v[1][h], v[2][h], v[3][h]};
+      pk_dft<4, true>(z);
+#pragma unroll
+      for (int n1 = 0; n1 < 4; ++n1) (h % 2 ? r : p)[(4 * n1 + h) * Q] = z[n1];
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int t = tid; t < 8 * Q; t += NT) {
+    const int c2 = t % CP, n1 = t / CP;
+    const int odd = (c2 / CPQ) & 1;
+    const pk2* p = buf + (c2 % CPQ) * SC + (4 * n1 + c2 / CPQ) * Q + odd * ROT;
+    const pk2* wrap = p - odd * Q;
+    pk2 v[Q];
+    v[0] = p[0];
+#pragma unroll
+    for (int k2 = 1; k2 < Q; ++k2) v[k2] = ptwiddle<true>((k2 < Q - ROT ? p : wrap)[k2], twa[n1 * Q + k2]);
+    pk_dft<Q, true>(v);
+    pk2* dst = slab + n1 * CP + c2;
+#pragma unroll
+    for (int n2 = 0; n2 < Q; ++n2) dst[n2 * 4 * CP] = v[n2];
+  }
 }
 
-// F3: inverse FFT along axis 2 for all pairs of the tile, then each output
-// orbital adds its listed contributions to its W rows (one writer per row).
-// The live slabs of X arrive by asynchronous copies straight into shared
-// memory (no registers held while the loads are in flight); dead slabs are zero.
-// Three resident blocks per SM (rather than F1's four) leave F3 the registers to keep the
-// orbital and W loads of its accumulation in flight together (9% faster at 96^3).
+// F3: inverse FFT along axis 2 for four pairs of the tile at a time, the steps of F1
+// backwards, then the accumulation into the W rows (one writer per row). In an
+// off-diagonal tile of two full blocks the four pairs share orbital a: each thread
+// adds psi_a v_ab to its registers' sums for W_b (added to W once, after the last a), and the
+// products psi_b conj(v_ab) of an element's four threads, neighbouring lanes, are summed
+// by two exchanges that leave a quarter of the elements to each, which adds them to W_a.
+// Any other tile adds its contributions output by output. Resident blocks walk the items
+// as in F1: X values are loaded into registers one group of pairs (or item) ahead,
+// orbital rows refill their places asynchronously, and the additions to W do not wait.
 template <int L>
-__global__ void __launch_bounds__(Cfg<L>::NT13, 3) k_fast_f3(const PairTile* __restrict__ tiles, int tile0,
-                                                          const float2* __restrict__ X,
+__global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES3) k_fast_f3(const PairTile* __restrict__ tiles, int n_items,
+                                                          const pk2* __restrict__ X,
                                                           const float2* __restrict__ tw_g, int reach) {
-  using A = RowsT<L>;
-  constexpr int NT = Cfg<L>::NT13;
-  constexpr int ROW = RR * L;
-  constexpr long N = (long)L * L * L;
+  using S = Sizes<L>;
+  constexpr int M = S::M, MP = S::MP, QS = S::QS, RG = S::RG;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ PairTile tl;
-  float2* tw = reinterpret_cast<float2*>(smem_raw);
-  float2* work = tw + L;
-  const int tid = threadIdx.x;
-  if (tid == 0) tl = tiles[tile0 + blockIdx.y];
-  for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
-  __syncthreads();
-  constexpr int NB1 = L / RR;
-  const int i0 = blockIdx.x / NB1;
-  const int i1s = (blockIdx.x % NB1) * RR;
-  const long roff = ((long)i0 * L + i1s) * L;
-  const int np = tl.n_pairs;
-  const long slot0 = (long)blockIdx.y * NPAIR;
-  const int r = tid % RR;
-  for (int p = 0; p < np; ++p) {
-    const float2* xp = X + (slot0 + p) * N + (long)i0 * L + i1s + r;
-    for (int i2 = tid / RR; i2 < L; i2 += NT / RR) {
-      float2* dst = work + A::at(p * RR + r, i2);
-      if (dead_slab<L>(i2, reach)) *dst = make_float2(0.f, 0.f);
-      else cp_async8(dst, xp + (long)i2 * L * L);
-    }
-  }
+  __shared__ __align__(16) PairTile ring[3];
+  pk2* tw = reinterpret_cast<pk2*>(smem_raw);
+  float2* orb = reinterpret_cast<float2*>(smem_raw + S::tw_bytes);
+  pk2* ex = reinterpret_cast<pk2*>(smem_raw + S::tw_bytes + S::orb_bytes);
+  const int tid = threadIdx.x, stride = gridDim.x;
+  copy_tile(&ring[0], tiles + blockIdx.x / RG, tid);
+  if (blockIdx.x + stride < n_items) copy_tile(&ring[1], tiles + (blockIdx.x + stride) / RG, tid);
+  load_twiddles<L>(tw, tw_g, tid, S::NT);
   cp_async_wait_all();
   __syncthreads();
-  ct_inverse_lay<float2, L, NPAIR * RR, NT, A>(work, np * RR, tw, tid);
-  if (full_tile(tl)) {
-    // off-diagonal 4 x 4 tile: output a (< 4) takes psi_{4+b} conj(v_ab) over b, output
-    // 4 + b takes psi_a v_ab over a, in the order of the contribution lists; all orbital
-    // and W loads of an element are issued together
-    for (int e = tid; e < ROW; e += NT) {
-      const int row = e / L, col = e % L;
-      float2 v[2 * TT], w[2 * TT];
-      float2* dst[2 * TT];
+  load_orbitals<L>(orb, ring[0], 0, 2 * TT, (long)(blockIdx.x % RG) * (RR * L), tid);
+  const int qa = tid % QB, n1 = (tid / QB) % M, rpa = tid / (QB * M);
+  const int rpb = tid % RP, k2b = (tid / RP) % 8, qb = tid / (8 * RP);
+  const bool second = rpa < RP;   // M < 8: the last threads only take part in the first step
+  const unsigned live = live_mask<L>(k2b, reach);
+  const pk2 zero = {f2(0.f), f2(0.f)};
+  pk2 x[M];
+  // X values of pairs p0.. of an item into registers
+  auto load_x = [&](int item, int p0, int np) {
+    if (qb < QB && p0 + qb < np) {
+      const pk2* src = X + (((long)(item / RG) * NPAIR + p0 + qb) * L + k2b) * (L * S::CP) + (item % RG) * RP + rpb;
 #pragma unroll
-      for (int o = 0; o < 2 * TT; ++o) {
-        v[o] = __ldg(orb_ptr(tl, o) + roff + e);
-        dst[o] = tl.is_out[o] ? acc_ptr(tl, o) + roff + e : nullptr;
-        if (tl.is_out[o]) w[o] = *dst[o];
-      }
+      for (int k1 = 0; k1 < M; ++k1)
+        x[k1] = live & (1u << k1) ? load_now(src + (long)k1 * 8 * L * S::CP) : zero;
+    }
+  };
+  load_x(blockIdx.x, 0, ring[0].n_pairs);
+  int cur = 0;
+  bool was_full = false;
+  for (int item = blockIdx.x; item < n_items; item += stride) {
+    // After a full item five groups are in flight: the right orbitals, 0, 1, 2, 3.
+    const bool piped = was_full && full_tile(ring[cur]);
+    if (piped) cp_async_wait<4>(); else cp_async_wait_all();
+    __syncthreads();
+    const int nxt = cur == 2 ? 0 : cur + 1, far = cur == 0 ? 2 : cur - 1;
+    const PairTile& tl = ring[cur];
+    const bool more = item + stride < n_items;
+    const long noff = (long)((item + stride) % RG) * (RR * L);
+    if (item + 2 * stride < n_items) copy_tile(&ring[far], tiles + (item + 2 * stride) / RG, tid);
+    const int np = tl.n_pairs;
+    const bool full = full_tile(tl);
+    const long roff = (long)(item % RG) * (RR * L), aoff = roff + (long)2 * rpa * L + n1;
+    pk2 b[8], wb[8];
+    if (full && second) {
 #pragma unroll
-      for (int a = 0; a < TT; ++a) {
-        if (!tl.is_out[a]) continue;
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int b = 0; b < TT; ++b) acc = cadd(acc, cmul_conj(v[TT + b], work[A::at((a * TT + b) * RR + row, col)]));
-        *dst[a] = cadd(w[a], acc);
-      }
-#pragma unroll
-      for (int b = 0; b < TT; ++b) {
-        if (!tl.is_out[TT + b]) continue;
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int a = 0; a < TT; ++a) acc = cadd(acc, cmul(v[a], work[A::at((a * TT + b) * RR + row, col)]));
-        *dst[TT + b] = cadd(w[TT + b], acc);
+      for (int n2 = 0; n2 < 8; ++n2) {
+        b[n2] = orb_at<L>(orb, TT + qa, rpa, n1 + M * n2);
+        wb[n2] = zero;
       }
     }
-    return;
-  }
-  for (int o = 0; o < tl.n_orb; ++o) {
-    const int n = tl.out_n[o];
-    if (!tl.is_out[o] || n == 0) continue;
-    float2* dst = acc_ptr(tl, o) + roff;
-    for (int e = tid; e < ROW; e += NT) {
-      const int r = e / L, i2 = e % L;
-      float2 acc = make_float2(0.f, 0.f);
-      for (int c = 0; c < n; ++c) {
-        const float2 v = work[A::at(tl.out_pair[o][c] * RR + r, i2)];
-        const float2 a = __ldg(orb_ptr(tl, tl.out_other[o][c]) + roff + e);
-        acc = cadd(acc, tl.out_conj[o][c] ? cmul_conj(a, v) : cmul(a, v));
+    for (int p0 = 0; p0 < np; p0 += QB) {
+      if (qb < QB && p0 + qb < np) {
+        pk_dft<M, true>(x);
+        pk2* dst = ex + qb * QS + (k2b * RP + rpb) * MP;
+        dst[0] = x[0];
+#pragma unroll
+        for (int m = 1; m < M; ++m) dst[m] = ptwiddle<true>(x[m], tw[k2b * M + m]);
       }
-      dst[e] = cadd(dst[e], acc);
+      if (p0 + QB < np) load_x(item, p0 + QB, np);
+      else if (more) load_x(item + stride, 0, ring[nxt].n_pairs);
+      if (piped) {
+        if (p0 == 0) cp_async_wait<3>(); else cp_async_wait<4>();
+      }
+      __syncthreads();
+      if (p0 == 0) {
+        if (full && more) load_orbitals<L>(orb, ring[nxt], TT, 2 * TT, noff, tid);
+        cp_async_commit();
+      }
+      pk2* mine = ex + qa * QS + rpa * MP + n1;
+      if (full) {
+        if (second) {
+          const int a = p0 / QB;
+          pk2 v[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = mine[q * RP * MP];
+          pk_dft<8, true>(v);
+#pragma unroll
+          for (int n2 = 0; n2 < 8; ++n2) {
+            const pk2 pa = orb_at<L>(orb, a, rpa, n1 + M * n2), y = v[n2];
+            wb[n2].re = vminus(vfma(pa.re, y.re, wb[n2].re), vmul(pa.im, y.im));
+            wb[n2].im = vfma(pa.im, y.re, vfma(pa.re, y.im, wb[n2].im));
+            v[n2] = {vfma(b[n2].re, y.re, vmul(b[n2].im, y.im)), vdet(b[n2].im, y.re, b[n2].re, y.im)};
+          }
+          const bool lo1 = (qa & 1) == 0, lo2 = (qa & 2) == 0;
+          pk2 s[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h)
+            s[h] = padd(pk_select(lo1, v[h], v[4 + h]), pk_shfl_xor(pk_select(lo1, v[4 + h], v[h]), 1));
+          const int n2a = 4 * (qa & 1) + (qa & 2);   // this thread's elements of W_a: n2a and n2a + 1
+          float2* w = static_cast<float2*>(tl.out[a]) + aoff + M * n2a;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const pk2 r = padd(pk_select(lo2, s[h], s[2 + h]), pk_shfl_xor(pk_select(lo2, s[2 + h], s[h]), 2));
+            if (tl.is_out[a]) add_rows<L>(w + M * h, r);
+          }
+        }
+      } else {
+        if (second && p0 + qa < np) {
+          pk2 v[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = mine[q * RP * MP];
+          pk_dft<8, true>(v);
+#pragma unroll
+          for (int n2 = 0; n2 < 8; ++n2) mine[n2 * RP * MP] = v[n2];
+        }
+        __syncthreads();
+        for (int o = 0; o < tl.n_orb; ++o) {
+          if (!tl.is_out[o]) continue;
+          for (int e = tid; e < RP * L; e += S::NT) {
+            const int rp = e / L, n = e % L;
+            pk2 s = zero;
+            bool any = false;
+            for (int c = 0; c < tl.out_n[o]; ++c) {
+              const int p = tl.out_pair[o][c];
+              if (p < p0 || p >= p0 + QB) continue;
+              any = true;
+              const pk2 y = ex[(p - p0) * QS + ((n / M) * RP + rp) * MP + n % M];
+              const pk2 a = orb_at<L>(orb, tl.out_other[o][c], rp, n);
+              if (tl.out_conj[o][c]) {
+                s.re = vfma(a.im, y.im, vfma(a.re, y.re, s.re));
+                s.im = vminus(vfma(a.im, y.re, s.im), vmul(a.re, y.im));
+              } else {
+                s.re = vminus(vfma(a.re, y.re, s.re), vmul(a.im, y.im));
+                s.im = vfma(a.im, y.re, vfma(a.re, y.im, s.im));
+              }
+            }
+            if (any) add_rows<L>(static_cast<float2*>(tl.out[o]) + roff + (long)2 * rp * L + n, s);
+          }
+        }
+      }
+      __syncthreads();
+      if (more) {   // places of orbitals this item no longer reads
+        if (full) load_orbitals<L>(orb, ring[nxt], p0 / QB, p0 / QB + 1, noff, tid);
+        else if (p0 + QB >= np) load_orbitals<L>(orb, ring[nxt], 0, 2 * TT, noff, tid);
+      }
+      cp_async_commit();
     }
+    if (full && second && tl.is_out[TT + qa]) {
+      float2* w = static_cast<float2*>(tl.out[TT + qa]) + aoff;
+#pragma unroll
+      for (int n2 = 0; n2 < 8; ++n2) add_rows<L>(w + M * n2, wb[n2]);
+    }
+    cur = nxt;
+    was_full = full;
   }
 }
 
 template <int L>
 static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* scratch, const float2* tw,
                                cudaStream_t s) {
+  using S = Sizes<L>;
   static std::atomic<unsigned long long> attr_done{0};
   if (const unsigned long long bit = device_bit_todo(attr_done)) {
-    cudaError_t e = cudaFuncSetAttribute(k_fast_f1<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem13<L>());
+    cudaError_t e = cudaFuncSetAttribute(k_fast_f1<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem13);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_fast_f3<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem13<L>());
+    e = cudaFuncSetAttribute(k_fast_f3<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem13);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_fast_f2<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2<L>());
+    e = cudaFuncSetAttribute(k_fast_f2<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem2);
     if (e != cudaSuccess) return e;
-    if constexpr (L == 96) {
-      e = cudaFuncSetAttribute(k_fast_f2r<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2<L>());
-      if (e != cudaSuccess) return e;
-    }
     attr_done.fetch_or(bit, std::memory_order_release);
   }
-  float2* X = (float2*)scratch;
+  pk2* X = (pk2*)scratch;
+  const float2* kt2 = reinterpret_cast<const float2*>(khat_t);
   const int reach = 2 * plan.g2_reach + 1 < L ? plan.g2_reach : L;
   const int n_live = reach >= L ? L : 2 * reach + 1;
+  const int sms = sm_count();   // F1 and F3 run the blocks the chip holds at once
   for (int l = 0; l < plan.n_launch; ++l) {
-    const int t0 = plan.launch_first[l], nt = plan.launch_count[l];
-    dim3 g13((unsigned)(L * (L / RR)), (unsigned)nt);
-    k_fast_f1<L><<<g13, Cfg<L>::NT13, smem13<L>(), s>>>(plan.d_tiles, t0, X, tw, reach);
+    const PairTile* tiles = plan.d_tiles + plan.launch_first[l];
+    const int nt = plan.launch_count[l], items = nt * S::RG;
+    const unsigned g1 = (unsigned)std::min(items, S::RES1 * sms), g3 = (unsigned)std::min(items, S::RES3 * sms);
+    k_fast_f1<L><<<g1, S::NT, S::smem13, s>>>(tiles, items, X, tw, reach);
     dim3 g2((unsigned)n_live, (unsigned)(nt * NPAIR));
-    if constexpr (L == 96) k_fast_f2r<L><<<g2, 192, smem2<L>(), s>>>(X, plan.d_tiles, t0, khat_t, tw, reach);
-    else k_fast_f2<L><<<g2, Cfg2<L>::NT, smem2<L>(), s>>>(X, plan.d_tiles, t0, khat_t, tw, reach);
-    k_fast_f3<L><<<g13, Cfg<L>::NT13, smem13<L>(), s>>>(plan.d_tiles, t0, X, tw, reach);
+    k_fast_f2<L><<<g2, S::NT2, S::smem2, s>>>(X, tiles, kt2, tw, reach);
+    k_fast_f3<L><<<g3, S::NT, S::smem13, s>>>(tiles, items, X, tw, reach);
     launched(3);
   }
   return cudaGetLastError();
@@ -478,6 +596,11 @@ static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* 
 
 bool fock_fast_supported(Grid3 g) {
   return g.n0 == g.n1 && g.n1 == g.n2 && (g.n0 == 32 || g.n0 == 48 || g.n0 == 64 || g.n0 == 96);
+}
+
+size_t fast_khat_index(int L, int i0, int i1, int i2) {
+  const int Q = L / 4, m = i1 / 4, g = (i1 / 2) % 2;
+  return ((((size_t)i2 * Q + m) * 2 + g) * 4 + i0 / Q) * Q * 2 + (size_t)(i0 % Q) * 2 + i1 % 2;
 }
 
 cudaError_t fock_pairs_fast(const FockPlan& plan, Grid3 g, const float* khat_t, void* scratch, const float2* tw_L,

@@ -153,7 +153,14 @@ cudaError_t upload_fft_tables(const pt_params* p, Grid3 g, bool mixed, double2* 
   if (e == cudaSuccess) {
     if (mixed) {
       kf.resize(kt.size());
-      for (size_t k = 0; k < kt.size(); ++k) kf[k] = (float)kt[k];
+      if (pt::fock_fast_supported(g)) {
+        size_t k = 0;
+        for (int i2 = 0; i2 < g.n2; ++i2)
+          for (int i0 = 0; i0 < g.n0; ++i0)
+            for (int i1 = 0; i1 < g.n1; ++i1) kf[pt::fast_khat_index(g.n0, i0, i1, i2)] = (float)kt[k++];
+      } else {
+        for (size_t k = 0; k < kt.size(); ++k) kf[k] = (float)kt[k];
+      }
       e = cudaMemcpyAsync(khat32, kf.data(), sizeof(float) * kf.size(), cudaMemcpyHostToDevice, s);
     } else {
       e = cudaMemcpyAsync(khat64, kt.data(), sizeof(double) * kt.size(), cudaMemcpyHostToDevice, s);
