@@ -78,8 +78,15 @@ pt_status real_orbitals(pt_system* sys, const double2* c) {
   return PT_OK;
 }
 
+// vloc (with its FP32 copy in mixed precision) and vh of the density rho
 pt_status local_potential(pt_system* sys, const double* rho) {
-  const int use_h = sys->p.use_hartree ? 1 : 0;
+  const bool use_h = sys->p.use_hartree != 0;
+  const pt::ConvSink sink{nullptr, sys->vion, rho, sys->p.use_lda ? (1.0 - sys->p.alpha) : 0.0,
+                          use_h ? sys->vh : nullptr, sys->vloc, sys->mixed ? sys->vloc32 : nullptr};
+  if (use_h && pt::convolve_supported(sys->g)) {
+    PT_CK(pt::convolve(rho, nullptr, sys->hfac, sys->hbuf, sink, sys->g, sys->tw, sys->s));
+    return PT_OK;
+  }
   if (use_h) {
     PT_CK(pt::rho_to_complex(rho, sys->hbuf, sys->N, sys->s));
     PT_CK(pt::fft_rows<double>(sys->hbuf, sys->hbuf, 1, sys->g, 0, 1.0, nullptr, sys->tw, sys->s));
@@ -88,8 +95,7 @@ pt_status local_potential(pt_system* sys, const double* rho) {
     PT_CK(pt::fft_cols<double>(sys->hbuf, 1, sys->g, 1, 1, 0, 1.0, nullptr, sys->tw, sys->s));
     PT_CK(pt::fft_rows<double>(sys->hbuf, sys->hbuf, 1, sys->g, 1, 1.0, nullptr, sys->tw, sys->s));
   }
-  const double w_lda = sys->p.use_lda ? (1.0 - sys->p.alpha) : 0.0;
-  PT_CK(pt::assemble_vloc(sys->vion, sys->hbuf, rho, sys->N, use_h, w_lda, sys->vh, sys->vloc, sys->s));
+  PT_CK(pt::assemble_vloc(use_h ? sys->hbuf : nullptr, sink, sys->N, sys->s));
   return PT_OK;
 }
 
@@ -97,6 +103,12 @@ pt_status local_potential(pt_system* sys) { return local_potential(sys, sys->rho
 
 // rho_mix += F^-1[ b |G|^2/(|G|^2 + q0^2) F[rho - rho_mix] ]
 static pt_status kerker_mix(pt_system* sys) {
+  if (pt::convolve_supported(sys->g)) {
+    pt::ConvSink sink{};
+    sink.acc = sys->rho_mix;
+    PT_CK(pt::convolve(sys->rho, sys->rho_mix, sys->kfac, sys->hbuf, sink, sys->g, sys->tw, sys->s));
+    return PT_OK;
+  }
   PT_CK(pt::diff_to_complex(sys->rho, sys->rho_mix, sys->hbuf, sys->N, sys->s));
   PT_CK(pt::fft_rows<double>(sys->hbuf, sys->hbuf, 1, sys->g, 0, 1.0, nullptr, sys->tw, sys->s));
   PT_CK(pt::fft_cols<double>(sys->hbuf, 1, sys->g, 1, 0, 0, 1.0, nullptr, sys->tw, sys->s));
@@ -370,7 +382,6 @@ pt_status density_scf(pt_system* sys, double* rho) {
 
 pt_status apply_local_scf(pt_system* sys, const double2* c, double2* out) {
   if (!sys->mixed) return apply_local_from_real(sys, c, out);
-  PT_CK(pt::to_float(sys->vloc, sys->vloc32, sys->N, sys->s));
   float2* hb = reinterpret_cast<float2*>(sys->hbuf);
   for (int c0 = 0; c0 < sys->ne; c0 += sys->hb) {
     const int cnt = std::min(sys->hb, sys->ne - c0);

@@ -13,6 +13,7 @@
 
 #include "common.cuh"
 #include "fft.cuh"
+#include "fft_ct.cuh"
 #include "internal.h"
 
 namespace pt {
@@ -170,6 +171,135 @@ cudaError_t fft_cols(void* data, long nvol, Grid3 g, int axis, int inverse, int 
 #undef PT_COLS
   launched();
   return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Convolution of a real field with a reciprocal-space factor (the Hartree solve, the Kerker
+// mixing) on cubic grids of 32, 48 or 64 points: a block transforms a whole plane (axes 1 and
+// 2) in shared memory, so the solve takes three launches instead of seven, with the field's
+// load, the factor and the potential's assembly inside them. One volume is too little work
+// to fill the chip: launches and latency bound it (32^3: 100 us in seven launches).
+namespace {
+
+template <int L> struct ConvCfg {
+  static constexpr int NT = L == 32 ? 128 : L == 48 ? 192 : 256;   // plane kernels
+  static constexpr int NC = 8;                                     // columns of an axis-0 block
+  static constexpr int NT0 = L == 48 ? 96 : 64;
+  static constexpr size_t smem_plane = sizeof(double2) * (L + L * (L + 1));
+  static constexpr size_t smem_axis0 = sizeof(double2) * (L + L * (NC + 1));
+};
+
+// plane i0 of a (minus b, when given), transformed along axes 2 and 1
+template <int L>
+__global__ void __launch_bounds__(ConvCfg<L>::NT) k_conv_plane_fwd(const double* __restrict__ a,
+                                                                   const double* __restrict__ b,
+                                                                   double2* __restrict__ out,
+                                                                   const double2* __restrict__ tw_g) {
+  constexpr int NT = ConvCfg<L>::NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* tw = reinterpret_cast<double2*>(smem_raw);
+  double2* buf = tw + L;
+  const int tid = threadIdx.x;
+  const long off = (long)blockIdx.x * L * L;
+  for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
+#pragma unroll 4
+  for (int e = tid; e < L * L; e += NT) {
+    double v = a[off + e];
+    if (b != nullptr) v -= b[off + e];
+    buf[(e / L) * (L + 1) + e % L] = make_double2(v, 0.0);
+  }
+  __syncthreads();
+  ct_forward<double2, L, L, NT, L + 1, 1>(buf, L, tw, tid);
+  ct_forward<double2, L, L, NT, 1, L + 1>(buf, L, tw, tid);
+#pragma unroll 4
+  for (int e = tid; e < L * L; e += NT) out[off + e] = buf[(e / L) * (L + 1) + e % L];
+}
+
+// axis 0 of NC columns: forward, times f, inverse, in place
+template <int L>
+__global__ void __launch_bounds__(ConvCfg<L>::NT0) k_conv_axis0(double2* __restrict__ data,
+                                                                const double* __restrict__ f,
+                                                                const double2* __restrict__ tw_g) {
+  constexpr int NT = ConvCfg<L>::NT0, NC = ConvCfg<L>::NC;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* tw = reinterpret_cast<double2*>(smem_raw);
+  double2* buf = tw + L;
+  const int tid = threadIdx.x;
+  const long off = (long)blockIdx.x * NC;
+  for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
+#pragma unroll 4
+  for (int e = tid; e < L * NC; e += NT) buf[(e / NC) * (NC + 1) + e % NC] = data[(long)(e / NC) * L * L + off + e % NC];
+  __syncthreads();
+  ct_forward<double2, L, NC, NT, 1, NC + 1>(buf, NC, tw, tid);
+  for (int e = tid; e < L * NC; e += NT) {
+    double2& v = buf[(e / NC) * (NC + 1) + e % NC];
+    v = cscale(v, f[(long)(e / NC) * L * L + off + e % NC]);
+  }
+  __syncthreads();
+  ct_inverse<double2, L, NC, NT, 1, NC + 1>(buf, NC, tw, tid);
+#pragma unroll 4
+  for (int e = tid; e < L * NC; e += NT) data[(long)(e / NC) * L * L + off + e % NC] = buf[(e / NC) * (NC + 1) + e % NC];
+}
+
+// plane i0 back along axes 1 and 2; the real part goes to the sink
+template <int L>
+__global__ void __launch_bounds__(ConvCfg<L>::NT) k_conv_plane_inv(const double2* __restrict__ in, ConvSink sink,
+                                                                   const double2* __restrict__ tw_g) {
+  constexpr int NT = ConvCfg<L>::NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* tw = reinterpret_cast<double2*>(smem_raw);
+  double2* buf = tw + L;
+  const int tid = threadIdx.x;
+  const long off = (long)blockIdx.x * L * L;
+  for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
+#pragma unroll 4
+  for (int e = tid; e < L * L; e += NT) buf[(e / L) * (L + 1) + e % L] = in[off + e];
+  __syncthreads();
+  ct_inverse<double2, L, L, NT, 1, L + 1>(buf, L, tw, tid);
+  ct_inverse<double2, L, L, NT, L + 1, 1>(buf, L, tw, tid);
+#pragma unroll 2
+  for (int e = tid; e < L * L; e += NT) {
+    const double h = buf[(e / L) * (L + 1) + e % L].x;
+    if (sink.acc != nullptr) sink.acc[off + e] += h;
+    else sink_potential(sink, off + e, h);
+  }
+}
+
+template <int L>
+cudaError_t convolve_t(const double* a, const double* b, const double* f, double2* work, const ConvSink& sink,
+                       const double2* tw, cudaStream_t s) {
+  using G = ConvCfg<L>;
+  static std::atomic<unsigned long long> attr_done{0};
+  if (const unsigned long long bit = device_bit_todo(attr_done)) {
+    cudaError_t e = cudaFuncSetAttribute(k_conv_plane_fwd<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)G::smem_plane);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_conv_plane_inv<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem_plane);
+    if (e != cudaSuccess) return e;
+    attr_done.fetch_or(bit, std::memory_order_release);
+  }
+  k_conv_plane_fwd<L><<<L, G::NT, G::smem_plane, s>>>(a, b, work, tw);
+  k_conv_axis0<L><<<L * L / G::NC, G::NT0, G::smem_axis0, s>>>(work, f, tw);
+  k_conv_plane_inv<L><<<L, G::NT, G::smem_plane, s>>>(work, sink, tw);
+  launched(3);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+bool convolve_supported(Grid3 g) {
+  return g.n0 == g.n1 && g.n1 == g.n2 && (g.n0 == 32 || g.n0 == 48 || g.n0 == 64);
+}
+
+cudaError_t convolve(const double* a, const double* b, const double* f, double2* work, const ConvSink& sink, Grid3 g,
+                     const DevTwiddles& tw, cudaStream_t s) {
+  const double2* t = tw_for<double>(tw, g.n0);
+  switch (g.n0) {
+    case 32: return convolve_t<32>(a, b, f, work, sink, t, s);
+    case 48: return convolve_t<48>(a, b, f, work, sink, t, s);
+    case 64: return convolve_t<64>(a, b, f, work, sink, t, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // ---------------------------------------------------------------------------

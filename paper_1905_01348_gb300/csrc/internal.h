@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <cmath>
 #include <cstdint>
 #include <cstddef>
 #include <string>
@@ -49,6 +50,47 @@ template <typename T>
 cudaError_t gather_basis(const void* in, double2* out, long out_ld, long nvol, Grid3 g, const int* basis,
                          int npw, double scale, const double* kin, const double2* x, long x_ld, int accumulate,
                          cudaStream_t s);
+// Where a convolution's result h goes: acc += h when acc is given, otherwise the local
+// potential: vh = h, vloc = vion + h + w_lda * Slater(rho) and its FP32 copy (when given).
+struct ConvSink {
+  double* acc;
+  const double* vion;
+  const double* rho;
+  double w_lda;
+  double* vh;
+  double* vloc;
+  float* vloc32;
+};
+#ifdef __CUDACC__
+// Cube root of x >= 0 to FP64 rounding from an FP32 one by two Newton steps on y^3 = x (8 FP64
+// operations; the slope 1 / (3 y^2) to FP32 is enough, each step leaves its error times the
+// last step's). FP64 is 1 / 64 of the FP32 rate here, and the density's cube roots were most
+// of the potential's time on small grids.
+__device__ __forceinline__ double cbrt_pos(double x) {
+  if (!(x > 1e-30 && x < 1e30)) return cbrt(x);
+  const float f = cbrtf((float)x);
+  const double c = (double)(1.0f / (3.0f * f * f));
+  double y = (double)f;
+  y = fma(fma(-y * y, y, x), c, y);
+  return fma(fma(-y * y, y, x), c, y);
+}
+// vh, vloc (and vloc32) of grid point r with Hartree potential h (vh null: no Hartree)
+__device__ __forceinline__ void sink_potential(const ConvSink& k, long r, double h) {
+  double v = k.vion[r];
+  if (k.vh != nullptr) {
+    k.vh[r] = h;
+    v += h;
+  }
+  if (k.w_lda != 0.0) v += k.w_lda * -cbrt_pos(3.0 / M_PI * k.rho[r]);
+  k.vloc[r] = v;
+  if (k.vloc32 != nullptr) k.vloc32[r] = (float)v;
+}
+#endif
+// h = F^-1[f F[a - b]] (b may be null; f carries the 1 / N) on the supported cubic grids;
+// work: one complex128 volume.
+bool convolve_supported(Grid3 g);
+cudaError_t convolve(const double* a, const double* b, const double* f, double2* work, const ConvSink& sink, Grid3 g,
+                     const DevTwiddles& tw, cudaStream_t s);
 cudaError_t convert_c128_to_c64(const double2* in, float2* out, long n, cudaStream_t s);
 
 // ---- sphere-pruned FP32 transforms for cubic 32/64/96 grids (fft_sphere.cu) --

@@ -94,33 +94,15 @@ cudaError_t density32(const float2* psi_r, long N, int ne, double* rho, cudaStre
   return cudaGetLastError();
 }
 
-__global__ void k_to_float(const double* __restrict__ a, float* __restrict__ b, long n) {
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) b[t] = (float)a[t];
-}
-
-cudaError_t to_float(const double* a, float* b, long n, cudaStream_t s) {
-  k_to_float<<<nblk(n, 256), 256, 0, s>>>(a, b, n); launched();
-  return cudaGetLastError();
-}
-
 // ---- local potential -----------------------------------------------------------
 __global__ void k_rho_to_complex(const double* __restrict__ rho, double2* __restrict__ buf, long N) {
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x)
     buf[r] = make_double2(rho[r], 0.0);
 }
 
-__global__ void k_vloc(const double* __restrict__ vion, const double2* __restrict__ vh_c, const double* __restrict__ rho,
-                       long N, int use_h, double w_lda, double* __restrict__ vh, double* __restrict__ vloc) {
-  for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x) {
-    double v = vion[r];
-    if (use_h) {
-      const double h = vh_c[r].x;
-      vh[r] = h;
-      v += h;
-    }
-    if (w_lda != 0.0) v += w_lda * (-cbrt(3.0 * rho[r] / M_PI));
-    vloc[r] = v;
-  }
+__global__ void k_vloc(const double2* __restrict__ vh_c, ConvSink sink, long N) {
+  for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x)
+    sink_potential(sink, r, vh_c != nullptr ? vh_c[r].x : 0.0);
 }
 
 cudaError_t rho_to_complex(const double* rho, double2* buf, long N, cudaStream_t s) {
@@ -128,9 +110,8 @@ cudaError_t rho_to_complex(const double* rho, double2* buf, long N, cudaStream_t
   return cudaGetLastError();
 }
 
-cudaError_t assemble_vloc(const double* vion, const double2* vh_c, const double* rho, long N, int use_h, double w_lda,
-                          double* vh, double* vloc, cudaStream_t s) {
-  k_vloc<<<nblk(N, 256), 256, 0, s>>>(vion, vh_c, rho, N, use_h, w_lda, vh, vloc); launched();
+cudaError_t assemble_vloc(const double2* vh_c, const ConvSink& sink, long N, cudaStream_t s) {
+  k_vloc<<<nblk(N, 256), 256, 0, s>>>(vh_c, sink, N); launched();
   return cudaGetLastError();
 }
 
@@ -497,7 +478,7 @@ __global__ void k_grid_sums(const double* __restrict__ rho, const double* __rest
     const double p = rho[t];
     acc[0] += vion[t] * p;
     if (use_h) acc[1] += vh[t] * p;
-    acc[2] += cbrt(p) * p;
+    acc[2] += cbrt_pos(p) * p;
     acc[3] += (a0 * i0 / n0) * p;
     acc[4] += (a1 * i1 / n1) * p;
     acc[5] += (a2 * i2 / n2) * p;

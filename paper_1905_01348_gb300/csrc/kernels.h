@@ -14,10 +14,9 @@ struct SlotList {
 
 cudaError_t density(const double2* psi_r, long N, int ne, double* rho, cudaStream_t s);
 cudaError_t density32(const float2* psi_r, long N, int ne, double* rho, cudaStream_t s);
-cudaError_t to_float(const double* a, float* b, long n, cudaStream_t s);
 cudaError_t rho_to_complex(const double* rho, double2* buf, long N, cudaStream_t s);
-cudaError_t assemble_vloc(const double* vion, const double2* vh_c, const double* rho, long N, int use_h, double w_lda,
-                          double* vh, double* vloc, cudaStream_t s);
+// the local potential from the Hartree potential vh_c (real parts; null without Hartree)
+cudaError_t assemble_vloc(const double2* vh_c, const ConvSink& sink, long N, cudaStream_t s);
 cudaError_t ion_potential(double* v, Grid3 g, const double* cell, const double* d_atoms, int na, double depth,
                           double sigma, cudaStream_t s);
 cudaError_t hartree_factor(double* f, Grid3 g, const double* cell, cudaStream_t s);
