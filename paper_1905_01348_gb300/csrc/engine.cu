@@ -145,6 +145,16 @@ pt_status apply_local_from_real(pt_system* sys, const double2* c, double2* out) 
 pt_status apply_local(pt_system* sys, const double2* X, double2* out, int ncols) {
   for (int c0 = 0; c0 < ncols; c0 += sys->hb) {
     const int cnt = std::min(sys->hb, ncols - c0);
+    if (sys->use_sphere) {
+      // only the rows and planes the basis sphere reaches: 54% of the full transforms' FP64
+      // work at the workloads' cutoff (FP64-bound)
+      const double2* x = X + (long)c0 * sys->npw;
+      PT_TRY(to_real<double>(sys, x, cnt, sys->hbuf));
+      PT_CK(pt::sphere_from_real(sys->hbuf, sys->vloc, sys->hbuf, cnt, sys->g, sys->sph, sys->basis,
+                                 std::sqrt(sys->vol) / sys->N, sys->kin, x, sys->npw, out + (long)c0 * sys->npw,
+                                 sys->npw, 0, tw_for(sys, sys->g.n0, (double*)nullptr), sys->s));
+      continue;
+    }
     PT_CK(pt::scatter_basis<double>(X + (long)c0 * sys->npw, sys->npw, sys->hbuf, cnt, sys->g, sys->basis, sys->npw,
                                     1.0 / std::sqrt(sys->vol), sys->s));
     PT_CK(pt::fft_rows<double>(sys->hbuf, sys->hbuf, cnt, sys->g, 1, 1.0, nullptr, sys->tw, sys->s));
