@@ -21,6 +21,7 @@
 // skipped inputs are zero and the skipped outputs are not needed.
 #include "common.cuh"
 #include "fft_ct.cuh"
+#include "fft_pk.cuh"
 #include "internal.h"
 
 namespace pt {
@@ -178,7 +179,257 @@ __global__ void __launch_bounds__(SNT) k_sph_rows_fwd(const C* __restrict__ vol,
   }
 }
 
-template <typename C, int L>
+// ---- FP32: packed pairs of lines (fft_pk.cuh) --------------------------------------
+// The FP32 passes are bound by memory traffic once their transforms are cheap: a pk2 holds
+// two neighbouring lines (i2, i2 + 1 in the column passes, two live rows in the row
+// passes), loads and stores go straight between global memory and registers, and a value
+// crosses shared memory once per pass, between the 8-point and the M-point DFTs (L = 8 M).
+constexpr int CPB = 8;    // column pairs per block (16 columns)
+constexpr int RPB = 8;    // row pairs per block
+
+template <int L> struct Pk {
+  static constexpr int M = L / 8;
+  static constexpr int NT = 8 * (M > 8 ? M : 8);
+  static constexpr int LS = L + 1;   // odd: neighbouring pairs on distinct banks
+};
+
+// twiddles W_L^(n1 k2) = c - i s as (c, c, s, s) at [k2][n1]
+template <int L> __device__ __forceinline__ void load_tw(pk2* tw, const float2* __restrict__ tw_g, int tid) {
+  for (int t = tid; t < L; t += Pk<L>::NT) {
+    const float2 w = tw_g[(t / Pk<L>::M) * (t % Pk<L>::M)];
+    tw[t] = {f2(w.x), f2(-w.y)};
+  }
+}
+
+__device__ __forceinline__ pk2 pk_load(const float2* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  return {make_float2(v.x, v.z), make_float2(v.y, v.w)};
+}
+__device__ __forceinline__ void pk_store(float2* p, pk2 v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v.re.x, v.im.x, v.re.y, v.im.y);
+}
+
+// Axis-0 (AXIS 0: lines (i1, i2), blockIdx.y = i1) or axis-1 (blockIdx.y = live plane) pass over
+// 16 columns i2. INV: reads only the live planes / the plane's live rows (others are
+// zero), writes every element. Forward: reads every element (times `mul` when given),
+// writes only the live ones. `dst` may be `src`.
+template <int L, bool INV, int AXIS>
+__global__ void __launch_bounds__(Pk<L>::NT) k_sphp_cols(const float2* src, float2* dst, const float* __restrict__ mul,
+                                                         const SphereTables st, const float2* __restrict__ tw_g) {
+  constexpr int M = Pk<L>::M, NT = Pk<L>::NT, LS = Pk<L>::LS;
+  constexpr long S = AXIS == 0 ? (long)L * L : L;
+  __shared__ pk2 tw[L];
+  __shared__ pk2 ex[CPB * LS];
+  __shared__ unsigned char live[L];
+  const int tid = threadIdx.x, cp = tid % CPB, u = tid / CPB;
+  const int line = AXIS == 0 ? (int)blockIdx.y : st.planes[blockIdx.y];
+  const unsigned char* lv = AXIS == 0 ? st.planelive : st.rowlive + line * L;
+  for (int t = tid; t < L; t += NT) live[t] = lv[t];
+  load_tw<L>(tw, tw_g, tid);
+  const long off = (AXIS == 0 ? (long)line * L : (long)line * L * L) + blockIdx.x * (2 * CPB) + 2 * cp;
+  const long vol = (long)blockIdx.z * L * L * L;
+  const float2* s = src + vol + off;
+  float2* d = dst + vol + off;
+  if (INV) {
+    __syncthreads();   // live flags and twiddles
+    if (u < 8) {
+      pk2 v[M];
+#pragma unroll
+      for (int k1 = 0; k1 < M; ++k1)
+        v[k1] = live[u + 8 * k1] ? pk_load(s + (u + 8 * k1) * S) : pk2{f2(0.f), f2(0.f)};
+      pk_dft<M, true>(v);
+      ex[cp * LS + u * M] = v[0];
+#pragma unroll
+      for (int m = 1; m < M; ++m) ex[cp * LS + u * M + m] = ptwiddle<true>(v[m], tw[u * M + m]);
+    }
+    __syncthreads();
+    if (u < M) {
+      pk2 v[8];
+#pragma unroll
+      for (int k2 = 0; k2 < 8; ++k2) v[k2] = ex[cp * LS + k2 * M + u];
+      pk_dft<8, true>(v);
+#pragma unroll
+      for (int n2 = 0; n2 < 8; ++n2) pk_store(d + (u + M * n2) * S, v[n2]);
+    }
+  } else {
+    pk2 v[8];
+    if (u < M) {
+#pragma unroll
+      for (int n2 = 0; n2 < 8; ++n2) v[n2] = pk_load(s + (u + M * n2) * S);
+      if (mul != nullptr) {
+#pragma unroll
+        for (int n2 = 0; n2 < 8; ++n2) {
+          const float2 f = __ldg(reinterpret_cast<const float2*>(mul + off + (u + M * n2) * S));
+          v[n2] = {vmul(v[n2].re, f), vmul(v[n2].im, f)};
+        }
+      }
+      pk_dft<8, false>(v);
+    }
+    __syncthreads();
+    if (u < M) {
+      ex[cp * LS + u] = v[0];
+#pragma unroll
+      for (int k2 = 1; k2 < 8; ++k2) ex[cp * LS + k2 * M + u] = ptwiddle<false>(v[k2], tw[k2 * M + u]);
+    }
+    __syncthreads();
+    if (u < 8) {
+      pk2 w[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) w[m] = ex[cp * LS + u * M + m];
+      pk_dft<M, false>(w);
+#pragma unroll
+      for (int k1 = 0; k1 < M; ++k1)
+        if (live[u + 8 * k1]) pk_store(d + (u + 8 * k1) * S, w[k1]);
+    }
+  }
+}
+
+// Inverse along axis 2 of 16 live rows, the rows' basis coefficients scattered in.
+template <int L>
+__global__ void __launch_bounds__(Pk<L>::NT) k_sphp_rows_inv(const double2* __restrict__ coef, long ldc,
+                                                             float2* __restrict__ vol, const SphereTables st,
+                                                             const int* __restrict__ basis, double scale,
+                                                             const float2* __restrict__ tw_g) {
+  constexpr int M = Pk<L>::M, NT = Pk<L>::NT, LS = Pk<L>::LS;
+  __shared__ pk2 tw[L];
+  __shared__ pk2 buf[RPB * LS];
+  const int tid = threadIdx.x, rp = tid % RPB, u = tid / RPB;
+  const int r0 = blockIdx.x * (2 * RPB), nr = min(2 * RPB, st.nrows - r0);
+  load_tw<L>(tw, tw_g, tid);
+  for (int e = tid; e < RPB * LS; e += NT) buf[e] = pk2{f2(0.f), f2(0.f)};
+  __syncthreads();
+  const int kb = st.row_kbeg[r0], ke = st.row_kbeg[r0 + nr];
+  const double2* cv = coef + blockIdx.y * ldc;
+  for (int k = kb + tid; k < ke; k += NT) {
+    const int r = st.krow[k] - r0;
+    float* p = reinterpret_cast<float*>(buf + (r >> 1) * LS + basis[k] % L) + (r & 1);
+    const double2 c = cv[k];
+    p[0] = (float)(c.x * scale);
+    p[2] = (float)(c.y * scale);
+  }
+  __syncthreads();
+  pk2* mine = buf + rp * LS;
+  if (u < 8) {   // element u + 8 k1 -> m of k2 = u, in place
+    pk2 v[M];
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) v[k1] = mine[u + 8 * k1];
+    pk_dft<M, true>(v);
+    mine[u] = v[0];
+#pragma unroll
+    for (int m = 1; m < M; ++m) mine[u + 8 * m] = ptwiddle<true>(v[m], tw[u * M + m]);
+  }
+  __syncthreads();
+  if (u < M) {
+    pk2 v[8];
+#pragma unroll
+    for (int k2 = 0; k2 < 8; ++k2) v[k2] = mine[8 * u + k2];
+    pk_dft<8, true>(v);
+    float2* vv = vol + (long)blockIdx.y * L * L * L + u;
+    if (2 * rp < nr) {
+      float2* d = vv + (long)st.row_idx[r0 + 2 * rp] * L;
+#pragma unroll
+      for (int n2 = 0; n2 < 8; ++n2) d[M * n2] = make_float2(v[n2].re.x, v[n2].im.x);
+    }
+    if (2 * rp + 1 < nr) {
+      float2* d = vv + (long)st.row_idx[r0 + 2 * rp + 1] * L;
+#pragma unroll
+      for (int n2 = 0; n2 < 8; ++n2) d[M * n2] = make_float2(v[n2].re.y, v[n2].im.y);
+    }
+  }
+}
+
+// Forward along axis 2 of 16 live rows, then out[k] = scale * F[k] (+ kin[k] x[k]) (+ out[k])
+// for the rows' basis vectors.
+template <int L>
+__global__ void __launch_bounds__(Pk<L>::NT) k_sphp_rows_fwd(const float2* __restrict__ vol, const SphereTables st,
+                                                             const int* __restrict__ basis, double scale,
+                                                             const double* __restrict__ kin,
+                                                             const double2* __restrict__ x, long ldx,
+                                                             double2* __restrict__ out, long ldo, int accumulate,
+                                                             const float2* __restrict__ tw_g) {
+  constexpr int M = Pk<L>::M, NT = Pk<L>::NT, LS = Pk<L>::LS;
+  __shared__ pk2 tw[L];
+  __shared__ pk2 buf[RPB * LS];
+  const int tid = threadIdx.x, rp = tid % RPB, u = tid / RPB;
+  const int r0 = blockIdx.x * (2 * RPB), nr = min(2 * RPB, st.nrows - r0);
+  load_tw<L>(tw, tw_g, tid);
+  __syncthreads();
+  pk2* mine = buf + rp * LS;
+  if (u < M) {
+    const float2* vv = vol + (long)blockIdx.y * L * L * L + u;
+    const float2* p = vv + (long)st.row_idx[r0 + min(2 * rp, nr - 1)] * L;
+    const float2* q = vv + (long)st.row_idx[r0 + min(2 * rp + 1, nr - 1)] * L;   // past the last row: any live one
+    pk2 v[8];
+#pragma unroll
+    for (int n2 = 0; n2 < 8; ++n2) {
+      const float2 a = p[M * n2], b = q[M * n2];
+      v[n2] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+    }
+    pk_dft<8, false>(v);
+    mine[8 * u] = v[0];
+#pragma unroll
+    for (int k2 = 1; k2 < 8; ++k2) mine[8 * u + k2] = ptwiddle<false>(v[k2], tw[k2 * M + u]);
+  }
+  __syncthreads();
+  if (u < 8) {
+    pk2 v[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) v[m] = mine[u + 8 * m];
+    pk_dft<M, false>(v);
+#pragma unroll
+    for (int k1 = 0; k1 < M; ++k1) mine[u + 8 * k1] = v[k1];
+  }
+  __syncthreads();
+  const int kb = st.row_kbeg[r0], ke = st.row_kbeg[r0 + nr];
+  double2* ov = out + blockIdx.y * ldo;
+  const double2* xv = x != nullptr ? x + blockIdx.y * ldx : nullptr;
+  for (int k = kb + tid; k < ke; k += NT) {
+    const int r = st.krow[k] - r0;
+    const float* f = reinterpret_cast<const float*>(buf + (r >> 1) * LS + basis[k] % L) + (r & 1);
+    double2 t = make_double2((double)f[0] * scale, (double)f[2] * scale);
+    if (kin != nullptr) {
+      const double2 c = xv[k];
+      t.x += kin[k] * c.x;
+      t.y += kin[k] * c.y;
+    }
+    if (accumulate) {
+      const double2 o = ov[k];
+      t.x += o.x;
+      t.y += o.y;
+    }
+    ov[k] = t;
+  }
+}
+
+template <int L>
+cudaError_t to_real_t(const double2* coef, long ldc, float2* vol, long nvol, const SphereTables& st, const int* basis,
+                      double scale, const float2* tw, cudaStream_t s) {
+  if (st.nrows == 0) return cudaMemsetAsync(vol, 0, sizeof(float2) * (size_t)L * L * L * nvol, s);
+  constexpr int NT = Pk<L>::NT;
+  k_sphp_rows_inv<L><<<dim3((unsigned)((st.nrows + 2 * RPB - 1) / (2 * RPB)), (unsigned)nvol), NT, 0, s>>>(
+      coef, ldc, vol, st, basis, scale, tw);
+  k_sphp_cols<L, true, 1><<<dim3(L / (2 * CPB), (unsigned)st.nplanes, (unsigned)nvol), NT, 0, s>>>(vol, vol, nullptr, st, tw);
+  k_sphp_cols<L, true, 0><<<dim3(L / (2 * CPB), L, (unsigned)nvol), NT, 0, s>>>(vol, vol, nullptr, st, tw);
+  launched(3);
+  return cudaGetLastError();
+}
+
+template <int L>
+cudaError_t to_sphere_t(const float2* vol, const float* mul, float2* work, long nvol, const SphereTables& st,
+                        const int* basis, double scale, const double* kin, const double2* x, long ldx, double2* out,
+                        long ldo, int accumulate, const float2* tw, cudaStream_t s) {
+  if (st.nrows == 0) return cudaSuccess;
+  constexpr int NT = Pk<L>::NT;
+  k_sphp_cols<L, false, 0><<<dim3(L / (2 * CPB), L, (unsigned)nvol), NT, 0, s>>>(vol, work, mul, st, tw);
+  k_sphp_cols<L, false, 1><<<dim3(L / (2 * CPB), (unsigned)st.nplanes, (unsigned)nvol), NT, 0, s>>>(work, work, nullptr, st, tw);
+  k_sphp_rows_fwd<L><<<dim3((unsigned)((st.nrows + 2 * RPB - 1) / (2 * RPB)), (unsigned)nvol), NT, 0, s>>>(
+      work, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw);
+  launched(3);
+  return cudaGetLastError();
+}
+
+// ---- FP64 ---------------------------------------------------------------------------
+template <int L, typename C>
 cudaError_t to_real_t(const double2* coef, long ldc, C* vol, long nvol, const SphereTables& st, const int* basis,
                       double scale, const C* tw, cudaStream_t s) {
   if (st.nrows == 0) return cudaMemsetAsync(vol, 0, sizeof(C) * (size_t)L * L * L * nvol, s);
@@ -192,7 +443,7 @@ cudaError_t to_real_t(const double2* coef, long ldc, C* vol, long nvol, const Sp
   return cudaGetLastError();
 }
 
-template <typename C, int L>
+template <int L, typename C>
 cudaError_t to_sphere_t(const C* vol, const typename real_of<C>::type* mul, C* work, long nvol,
                         const SphereTables& st, const int* basis, double scale, const double* kin, const double2* x,
                         long ldx, double2* out, long ldo, int accumulate, const C* tw, cudaStream_t s) {
@@ -220,10 +471,10 @@ static cudaError_t to_real_any(const double2* coef, long ldc, C* vol, long nvol,
   if (nvol <= 0) return cudaSuccess;
   if (nvol > 65535) return cudaErrorInvalidValue;
   switch (g.n0) {
-    case 32: return to_real_t<C, 32>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
-    case 48: return to_real_t<C, 48>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
-    case 64: return to_real_t<C, 64>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
-    case 96: return to_real_t<C, 96>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
+    case 32: return to_real_t<32>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
+    case 48: return to_real_t<48>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
+    case 64: return to_real_t<64>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
+    case 96: return to_real_t<96>(coef, ldc, vol, nvol, st, basis, scale, tw_L, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -236,10 +487,10 @@ static cudaError_t from_real_any(const C* vol, const typename real_of<C>::type* 
   if (nvol <= 0) return cudaSuccess;
   if (nvol > 65535) return cudaErrorInvalidValue;
   switch (g.n0) {
-    case 32: return to_sphere_t<C, 32>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
-    case 48: return to_sphere_t<C, 48>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
-    case 64: return to_sphere_t<C, 64>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
-    case 96: return to_sphere_t<C, 96>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
+    case 32: return to_sphere_t<32>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
+    case 48: return to_sphere_t<48>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
+    case 64: return to_sphere_t<64>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
+    case 96: return to_sphere_t<96>(vol, mul, work, nvol, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw_L, s);
     default: return cudaErrorInvalidValue;
   }
 }
