@@ -282,18 +282,28 @@ __global__ void k_anderson_dots(const H* __restrict__ dR, long slot_stride, Slot
 // Gathers the sums into gram[b][slot_q][new] (and its conjugate at [new][slot_q]) and the
 // right-hand side <dR_q, r> (slots in order, oldest first), then solves
 // (G + 1e-14 tr(G) I) gamma = rhs per band by Cholesky; gamma = 0 when the trace is zero
-// or a pivot is not positive. One warp per band, the matrix in shared memory: the k^3 / 6
-// multiply-adds of a column's update are spread over the lanes.
-__global__ void __launch_bounds__(32) k_anderson_solve(const double4_16a* __restrict__ part, SlotList sl, int newslot,
-                                                       int mdim, double2* __restrict__ gram,
-                                                       double2* __restrict__ gamma) {
-  __shared__ double2 L[kSlotMax][kSlotMax + 1];
-  const int b = blockIdx.x, lane = threadIdx.x, k = sl.k;
+// or a pivot is not positive. One block per band, the matrix in shared memory with the
+// right-hand side as its last row (so the forward substitution is part of the
+// factorisation). Latency bounds it: k dependent pivots, each a reciprocal square root,
+// a scaled column and an update that the block's threads share.
+constexpr int kSolveThreads = 128;
+
+__global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_16a* __restrict__ part, SlotList sl,
+                                                                  int newslot, int mdim, double2* __restrict__ gram,
+                                                                  double2* __restrict__ gamma) {
+  __shared__ double2 L[kSlotMax + 1][kSlotMax + 1];
+  __shared__ double inv[kSlotMax];   // 1 / L[j][j]
+  const int b = blockIdx.x, tid = threadIdx.x, k = sl.k;
   double2* G = gram + (long)b * mdim * mdim;
-  double2 y = make_double2(0.0, 0.0);   // right-hand side, then the solution, of row `lane`
-  const int mine = lane < k ? sl.s[lane] : 0;
-  if (lane < k) {
-    const double4_16a* p = part + ((long)b * k + lane) * kDotChunks;
+  // L L^H = A with A[i][j] = G[s_i][s_j]  (G[s][t] = <dR_s, dR_t>); older entries
+#pragma unroll 4
+  for (int t = tid; t < k * k; t += kSolveThreads) {
+    const int i = t / k, j = t % k;
+    if (j <= i && sl.s[i] != newslot && sl.s[j] != newslot) L[i][j] = G[(long)sl.s[i] * mdim + sl.s[j]];
+  }
+  if (tid < k) {
+    const int q = tid, mine = sl.s[q];
+    const double4_16a* p = part + ((long)b * k + q) * kDotChunks;
     double4_16a t = p[0];
 #pragma unroll
     for (int c = 1; c < kDotChunks; ++c) {
@@ -302,66 +312,60 @@ __global__ void __launch_bounds__(32) k_anderson_solve(const double4_16a* __rest
       t.z += p[c].z;
       t.w += p[c].w;
     }
-    if (mine == newslot) {
-      G[(long)mine * mdim + mine] = make_double2(t.x, 0.0);
-    } else {
-      G[(long)mine * mdim + newslot] = make_double2(t.x, t.y);
-      G[(long)newslot * mdim + mine] = make_double2(t.x, -t.y);
-    }
-    y = make_double2(t.z, t.w);
+    int at = 0;   // the new slot's place in the list
+    while (sl.s[at] != newslot) ++at;
+    const double2 fwd = make_double2(t.x, q == at ? 0.0 : t.y), rev = make_double2(t.x, q == at ? 0.0 : -t.y);
+    G[(long)mine * mdim + newslot] = fwd;
+    G[(long)newslot * mdim + mine] = rev;
+    if (q >= at) L[q][at] = fwd;
+    if (q <= at) L[at][q] = rev;
+    L[k][q] = make_double2(t.z, -t.w);   // conj(rhs): row k becomes y^H, L y = rhs
   }
-  __syncwarp();
-  // L L^H = A with A[i][j] = G[s_i][s_j]  (G[s][t] = <dR_s, dR_t>)
-  for (int t = lane; t < k * k; t += 32) {
-    const int i = t / k, j = t % k;
-    if (j <= i) L[i][j] = G[(long)sl.s[i] * mdim + sl.s[j]];
-  }
-  __syncwarp();
+  __syncthreads();
   double tr = 0.0;
   for (int q = 0; q < k; ++q) tr += L[q][q].x;
   bool ok = tr > 0.0;
   const double shift = 1e-14 * tr;
-  double inv = 0.0;   // 1 / L[lane][lane]
   for (int j = 0; j < k && ok; ++j) {
     const double d = L[j][j].x + shift;
     if (!(d > 0.0)) { ok = false; break; }
     const double r = rsqrt(d);
-    if (lane == j) inv = r;
-    if (lane > j && lane < k) L[lane][j] = make_double2(L[lane][j].x * r, L[lane][j].y * r);
-    __syncwarp();
-    const int m = k - 1 - j;
-    for (int t = lane; t < m * m; t += 32) {
+    if (tid == 0) inv[j] = r;
+    // rows i > j of column j scaled, and A[i][p] -= L[i][j] conj(L[p][j]) for j < p <= i
+    const int m = k - j;   // rows j + 1 .. k
+    const double r2 = r * r;
+    for (int t = tid; t < m * m; t += kSolveThreads) {
       const int i = j + 1 + t % m, p = j + 1 + t / m;
-      if (p > i) continue;
+      if (p > i || p == k) continue;
       const double2 u = L[i][j], w = L[p][j];
-      L[i][p].x -= u.x * w.x + u.y * w.y;
-      L[i][p].y -= u.y * w.x - u.x * w.y;
+      L[i][p].x -= r2 * (u.x * w.x + u.y * w.y);
+      L[i][p].y -= r2 * (u.y * w.x - u.x * w.y);
     }
-    __syncwarp();
+    __syncthreads();
+    if (tid < m) {
+      double2& v = L[j + 1 + tid][j];
+      v = make_double2(v.x * r, v.y * r);
+    }
+    // the next round reads column j + 1, which only the update above wrote
   }
+  __syncthreads();
+  if (tid >= 32) return;
   if (!ok) {
-    if (lane < k) gamma[(long)b * mdim + lane] = make_double2(0.0, 0.0);
+    if (tid < k) gamma[(long)b * mdim + tid] = make_double2(0.0, 0.0);
     return;
   }
-  for (int i = 0; i < k; ++i) {   // L y = rhs
-    if (lane == i) { y.x *= inv; y.y *= inv; }
-    const double yx = __shfl_sync(0xffffffffu, y.x, i), yy = __shfl_sync(0xffffffffu, y.y, i);
-    if (lane > i && lane < k) {
-      const double2 l = L[lane][i];
-      y.x -= l.x * yx - l.y * yy;
-      y.y -= l.x * yy + l.y * yx;
-    }
-  }
+  double2 y = tid < k ? make_double2(L[k][tid].x, -L[k][tid].y) : make_double2(0.0, 0.0);
+  const double di = tid < k ? inv[tid] : 0.0;
   for (int i = k - 1; i >= 0; --i) {   // L^H g = y
-    if (lane == i) { y.x *= inv; y.y *= inv; }
+    if (tid == i) { y.x *= di; y.y *= di; }
     const double yx = __shfl_sync(0xffffffffu, y.x, i), yy = __shfl_sync(0xffffffffu, y.y, i);
-    if (lane < i) {
-      const double2 l = L[i][lane];
+    if (tid < i) {
+      const double2 l = L[i][tid];
       y.x -= l.x * yx + l.y * yy;
       y.y -= l.x * yy - l.y * yx;
     }
   }
-  if (lane < k) gamma[(long)b * mdim + lane] = y;
+  if (tid < k) gamma[(long)b * mdim + tid] = y;
 }
 
 cudaError_t anderson_gamma(const void* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r,
@@ -376,7 +380,7 @@ cudaError_t anderson_gamma(const void* dR, long slot_stride, const SlotList& sl,
   else
     k_anderson_dots<double2><<<grid, 32 * sl.k, 0, s>>>((const double2*)dR, slot_stride, sl, newslot, r, npw,
                                                         (double4_16a*)part);
-  k_anderson_solve<<<ne, 32, 0, s>>>((const double4_16a*)part, sl, newslot, mdim, gram, gamma);
+  k_anderson_solve<<<ne, kSolveThreads, 0, s>>>((const double4_16a*)part, sl, newslot, mdim, gram, gamma);
   launched(2);
   return cudaGetLastError();
 }

@@ -55,7 +55,21 @@ __global__ void __launch_bounds__(64) k_gemm(int opA, int opB, int M, int N, int
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int b = 0; b < 2; ++b) acc[a][b] = C{};
-  C ra[P], rb[P];   // next slice
+  // FP32 sums run over kRun terms, then go into FP64 ones: their rounding does not grow with K
+  constexpr int kRun = 512;
+  double2 sum[2][2] = {};
+  auto flush = [&]() {
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const double2 v = to_d(acc[a][b]);
+        sum[a][b].x += v.x;
+        sum[a][b].y += v.y;
+        acc[a][b] = C{};
+      }
+  };
+  TI ra[P], rb[P];   // next slice, converted when it is stored: the loads stay in flight together
   auto fetch = [&](int k0) {
 #pragma unroll
     for (int q = 0; q < P; ++q) {
@@ -71,16 +85,16 @@ __global__ void __launch_bounds__(64) k_gemm(int opA, int opB, int M, int N, int
         if (opB == OP_N) vb = ld_op(B + (k0 + kb) + (long)(n0 + jb) * ldb);
         else { vb = ld_op(B + (n0 + jb) + (long)(k0 + kb) * ldb); vb.y = -vb.y; }
       }
-      ra[q] = mk_as<C>(va);
-      rb[q] = mk_as<C>(vb);
+      ra[q] = va;
+      rb[q] = vb;
     }
   };
   auto stash = [&](int buf) {
 #pragma unroll
     for (int q = 0; q < P; ++q) {
       const int u = tid & 15, w = (tid >> 4) + 4 * q;
-      if (opA == OP_N) As[buf][w][u] = ra[q]; else As[buf][u][w] = ra[q];
-      if (opB == OP_N) Bs[buf][u][w] = rb[q]; else Bs[buf][w][u] = rb[q];
+      if (opA == OP_N) As[buf][w][u] = mk_as<C>(ra[q]); else As[buf][u][w] = mk_as<C>(ra[q]);
+      if (opB == OP_N) Bs[buf][u][w] = mk_as<C>(rb[q]); else Bs[buf][w][u] = mk_as<C>(rb[q]);
     }
   };
   int buf = 0;
@@ -117,14 +131,16 @@ __global__ void __launch_bounds__(64) k_gemm(int opA, int opB, int M, int N, int
     if (more) stash(buf ^ 1);
     __syncthreads();
     buf ^= 1;
+    if (sizeof(C) == sizeof(float2) && (k0 - kbeg) % kRun == kRun - GK) flush();
   }
+  if (sizeof(C) == sizeof(float2)) flush();
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int i = m0 + tx + 8 * a, j = n0 + ty + 8 * b;
       if (i >= M || j >= N || (structure == GEMM_HERM && i < j)) continue;   // i < j: mirrored from (j, i)
-      const double2 v = to_d(acc[a][b]);
+      const double2 v = sizeof(C) == sizeof(float2) ? sum[a][b] : to_d(acc[a][b]);
       if (ksplit > 1) {
         part[((long)kz * N + j) * (long)M + i] = v;
         continue;
@@ -279,7 +295,7 @@ cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const double2
 // and inverts its factor, the rows below are multiplied by that inverse, and the trailing
 // matrix takes the rank-CB update: 3 launches per CB columns. Bound by FP64 (two
 // multiply-adds a clock and SM) in the single diagonal block, so only one thread takes
-// each pivot's reciprocal square root.
+// each pivot's square root and reciprocal.
 constexpr int CB = 32;
 
 // Factor of the nb x nb block at (j0, j0), zeros above its diagonal, and the factor's
@@ -306,9 +322,9 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* __restrict__ A, doub
       if (!(d > 0.0)) {
         bad = 1;
       } else {
-        const double r = rsqrt(d);
-        a[j][j] = make_double2(d * r, 0.0);
-        rinv[j] = r;
+        const double s = sqrt(d);
+        a[j][j] = make_double2(s, 0.0);
+        rinv[j] = 1.0 / s;
       }
     }
     __syncthreads();
