@@ -21,13 +21,13 @@
 //
 // Kernel: one CTA per 128 x 128 complex output tile and K chunk (split-K for
 // the long reductions over the basis, summed afterwards in a fixed order).
-// Warps 0-3 load their row of A and column of B for a stage of 8 complex k,
-// split and expand them, and store them into shared memory in the canonical
-// K-major layout without swizzle (core matrices of 8 rows x 16 bytes); a ring
-// of two stages is guarded by mbarriers. One thread of warp 4 issues
+// Warps 0-7 copy their rows of A and columns of B for a stage of 8 complex k into shared
+// memory asynchronously, several stages ahead, then split and expand them
+// into the canonical K-major layout without swizzle (core matrices of 8 rows x 16 bytes);
+// that ring of two stages is guarded by mbarriers. One thread of warp 8 issues
 // tcgen05.mma (kind::tf32, M = 128, N = 256, K = 8) and releases each stage
-// with tcgen05.commit. Warps 0-3 read the accumulators with tcgen05.ld (warp w
-// owns TMEM lanes 32w..32w+31, i.e. output rows) and write C or the
+// with tcgen05.commit. Warps 0-7 read the accumulators with tcgen05.ld (warp w
+// owns TMEM lanes 32 (w % 4)..+31, i.e. output rows) and write C or the
 // split-K partials. The accumulator is promoted into round-to-nearest FP32
 // sums every 8 stages (see the kernel). Every wait is bounded: on expiry the
 // kernel sets an error flag, stops issuing work and frees its tensor memory.
@@ -47,16 +47,17 @@ constexpr int TC_NC = 128;           // complex output columns per tile (256 rea
 constexpr int TC_KC = 8;             // complex k per stage (16 real k: two MMAs of K = 8)
 constexpr int TC_NS = 2;             // ring stages
 constexpr int TC_WIN = 8;            // stages per accumulation window (48 MMAs)
-constexpr int TC_PF = 4;             // stages of operand loads in flight per producer thread
-static_assert(TC_WIN % TC_PF == 0, "the producer loop steps through windows in groups of TC_PF stages");
+constexpr int TC_RAW = 6;            // stages of operand copies in flight (shared memory)
 constexpr int TC_PROD = 256;         // producer / drain threads (warps 0-7), two per tile row
 constexpr int TC_THREADS = 288;      // + warp 8: tensor-memory allocation and MMA issue
 constexpr uint32_t TC_TMEM_COLS = 512;                      // two accumulators of 256 columns
 constexpr uint32_t A_BYTES = TC_M * 2 * TC_KC * 4;           // 128 rows x 16 floats
 constexpr uint32_t B_BYTES = 2 * TC_NC * 2 * TC_KC * 4;      // 256 rows x 16 floats
 constexpr uint32_t STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;  // [A hi][A lo][B hi][B lo]
-constexpr uint32_t SUM_BYTES = 2 * TC_NC * TC_M * 4;         // FP32 window sums, [256 columns][128 rows]
-constexpr uint32_t TC_SMEM = TC_NS * STAGE_BYTES + SUM_BYTES;  // 224 KB: one CTA per SM
+constexpr uint32_t WARP_RAW = 2 * 32 * 32;                   // a warp's part of a raw stage: 32 rows x 4 complex of A, of B
+constexpr uint32_t RAW_BYTES = TC_PROD / 32 * WARP_RAW;
+constexpr uint32_t TC_SMEM = TC_NS * STAGE_BYTES + TC_RAW * RAW_BYTES;  // 192 KB: one CTA per SM
+static_assert(2 * TC_NC * TC_M * 4 <= TC_SMEM, "the output exchange takes the rings' place");
 constexpr long long kWaitCycles = 4000000000LL;              // about 2 s at 2 GHz
 
 // Instruction descriptor of tcgen05.mma kind::tf32: FP32 accumulator (bits 4-5 = 1),
@@ -145,15 +146,14 @@ __device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
   lo = __uint_as_float(l);
 }
 
-__device__ __forceinline__ void st_split(unsigned char* hi_base, unsigned char* lo_base, uint32_t off, float a, float b,
-                                         float c, float d) {
-  float4 h, l;
-  split_tf32(a, h.x, l.x);
-  split_tf32(b, h.y, l.y);
-  split_tf32(c, h.z, l.z);
-  split_tf32(d, h.w, l.w);
-  *reinterpret_cast<float4*>(hi_base + off) = h;
-  *reinterpret_cast<float4*>(lo_base + off) = l;
+__device__ __forceinline__ void split2(float2 v, float2& hi, float2& lo) {
+  split_tf32(v.x, hi.x, lo.x);
+  split_tf32(v.y, hi.y, lo.y);
+}
+
+// 8 bytes from global into shared memory, or zeros
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(dst), "l"(src), "r"(valid ? 8 : 0) : "memory");
 }
 
 // byte offset of row r, core-matrix column kc (4 floats) inside an operand tile
@@ -168,18 +168,26 @@ __device__ __forceinline__ uint32_t core_off(int r, int kc) {
 // part[(kz N + j) M + i]; otherwise C = alpha sum + beta C.
 //
 // Threads: warps 0-7 produce and drain, two threads per tile row r = 32 (w % 4) + lane
-// (warp w reaches TMEM lanes 32 (w % 4)..+31); thread half h = w / 4 loads and converts
-// complex k 4h..4h+3 of each stage (TC_PF stages ahead, in registers) and owns
-// accumulator columns 128h..128h+127 (C_r for h = 0, C_i for h = 1). Warp 8 allocates
-// tensor memory and one of its threads issues the MMAs.
+// (warp w reaches TMEM lanes 32 (w % 4)..+31); thread half h = w / 4 converts complex k
+// 4h..4h+3 of each stage and owns accumulator columns 128h..128h+127 (C_r for h = 0, C_i for
+// h = 1). Warp 8 allocates tensor memory and one of its threads issues the MMAs.
+//
+// Operands. Each warp copies its own 32 rows x 4 complex of A and of B asynchronously into a
+// ring of TC_RAW raw stages (whole 32-byte runs of a row when the operand is contiguous along
+// k, 256-byte runs across rows otherwise), so no register holds a load in flight and no
+// other warp is waited for. A row's two 16-byte chunks swap places with bit 2 of the row:
+// the threads that read one row each then touch distinct banks. The overlap A^H B of 432
+// columns of Si216 (K = 43,819): 565 us of device work, 887 with the loads in registers and
+// the sums in shared memory; the split and expansion by the producers bound it (3 x 196
+// GFLOP of MMAs would take 0.21 ms).
 //
 // Accumulation. The tensor core adds into its FP32 accumulator with truncation, so its
 // error grows linearly with the number of MMAs into one accumulator (measured: 4e-5
 // relative after 2250 MMAs). Each window of TC_WIN stages (48 MMAs) therefore starts a
 // fresh accumulator, and the producer threads add the finished window into FP32 sums in
-// shared memory (round to nearest), one slice of 16 columns after each stage they
-// produce. Two TMEM accumulators alternate, so the MMAs of window w run while window
-// w - 1 is drained.
+// registers (round to nearest), one slice of 16 columns after each stage they produce.
+// Two TMEM accumulators alternate, so the MMAs of window w run while window w - 1 is
+// drained.
 template <int OPA, int OPB>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_cgemm_tf32x3(int M, int N, int K, int kchunk, int ksplit, int tri_b, double2 alpha,
@@ -198,7 +206,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (tri_b) kend = min(kend, n0 + TC_NC);
   const int nst = kend > kbeg ? (kend - kbeg + TC_KC - 1) / TC_KC : 0;
   const int nwin = (nst + TC_WIN - 1) / TC_WIN;
-  float* sums = reinterpret_cast<float*>(smem + TC_NS * STAGE_BYTES);   // [256 columns][128 rows]
+  float* sums = reinterpret_cast<float*>(smem);   // [256 columns][128 rows], once the rings are done with
 
   if (tid == 0) {
     for (int s = 0; s < TC_NS; ++s) {
@@ -227,30 +235,43 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   if (warp < TC_PROD / 32) {
     const int q = warp & 3, h = warp >> 2;
     const int r = 32 * q + lane;                 // tile row of op(A), tile column of op(B)
-    const int m = m0 + r, n = n0 + r;
     const uint32_t tlane = (uint32_t)(32 * q) << 16;
-    float* my_sums = sums + (TC_NC * h) * TC_M + r;   // column j of this thread: my_sums[j * TC_M]
-    float2 pa[TC_PF][4], pb[TC_PF][4];           // stages st .. st + TC_PF - 1 in flight (buffer st % TC_PF)
-    auto load = [&](int st, float2 (&a)[4], float2 (&b)[4]) {
+    const uint32_t raw0 = smem_u32(smem) + TC_NS * STAGE_BYTES + (uint32_t)warp * WARP_RAW;
+    auto raw_off = [](int row, int k) {   // complex k of row
+      return (uint32_t)(row * 32 + (((k >> 1) ^ (row >> 2)) & 1) * 16 + (k & 1) * 8);
+    };
+    // asynchronous copies of this warp's part of stage st
+    auto copy = [&](int st) {
+      const uint32_t dst = raw0 + (uint32_t)(st % TC_RAW) * RAW_BYTES;
       const int kb = kbeg + st * TC_KC + 4 * h;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int kk = kb + j;
-        float2 va = make_float2(0.f, 0.f), vb = make_float2(0.f, 0.f);
-        if (st < nst && m < M && kk < kend) {
-          if (OPA == OP_N) va = __ldg(A + m + (long)kk * lda);
-          else { va = __ldg(A + kk + (long)m * lda); va.y = -va.y; }
+      for (int j = 0; j < 4 && st < nst; ++j) {
+        {
+          const int row = OPA == OP_N ? lane : (lane >> 2) + 8 * j, k = OPA == OP_N ? j : lane & 3;
+          const int mm = m0 + 32 * q + row, kk = kb + k;
+          const bool in = mm < M && kk < kend;
+          const float2* src = in ? (OPA == OP_N ? A + mm + (long)kk * lda : A + kk + (long)mm * lda) : A;
+          cp_async8(dst + raw_off(row, k), src, in);
         }
-        if (st < nst && n < N && kk < kend) {
-          if (OPB == OP_N) vb = __ldg(B + kk + (long)n * ldb);
-          else { vb = __ldg(B + n + (long)kk * ldb); vb.y = -vb.y; }
+        {
+          const int row = OPB == OP_H ? lane : (lane >> 2) + 8 * j, k = OPB == OP_H ? j : lane & 3;
+          const int nn = n0 + 32 * q + row, kk = kb + k;
+          const bool in = nn < N && kk < kend;
+          const float2* src = in ? (OPB == OP_N ? B + kk + (long)nn * ldb : B + nn + (long)kk * ldb) : B;
+          cp_async8(dst + 1024 + raw_off(row, k), src, in);
         }
-        a[j] = va;
-        b[j] = vb;
       }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    // store stage st (from a, b) into its ring slot
-    auto produce = [&](int st, const float2 (&a)[4], const float2 (&b)[4]) {
+    // split and expand stage st into its MMA ring slot
+    auto produce = [&](int st) {
+      const unsigned char* raw = smem + TC_NS * STAGE_BYTES + (uint32_t)(st % TC_RAW) * RAW_BYTES + warp * WARP_RAW;
+      float4 ra[2], rb[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        ra[c] = *reinterpret_cast<const float4*>(raw + raw_off(lane, 2 * c));
+        rb[c] = *reinterpret_cast<const float4*>(raw + 1024 + raw_off(lane, 2 * c));
+      }
       const int s = st % TC_NS;
       const uint32_t ph = (uint32_t)(st / TC_NS) & 1u;
       if (ok) ok = mbar_wait(&bar_empty[s], ph ^ 1u, err);
@@ -261,66 +282,77 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
       if (ok) {
 #pragma unroll
         for (int c = 0; c < 2; ++c) {   // core-matrix columns kc = 2h + c: complex k 4h + 2c, +1
-          const int kc = 2 * h + c;
-          const float2 a0 = a[2 * c], a1 = a[2 * c + 1], b0 = b[2 * c], b1 = b[2 * c + 1];
-          st_split(Ahi, Alo, core_off(r, kc), a0.x, a0.y, a1.x, a1.y);
-          st_split(Bhi, Blo, core_off(r, kc), b0.x, -b0.y, b1.x, -b1.y);          // -> C_r
-          st_split(Bhi, Blo, core_off(r + TC_NC, kc), b0.y, b0.x, b1.y, b1.x);    // -> C_i
+          const uint32_t o = core_off(r, 2 * h + c), o2 = core_off(r + TC_NC, 2 * h + c);
+          float2 h0, l0, h1, l1;
+          split2(make_float2(ra[c].x, OPA == OP_H ? -ra[c].y : ra[c].y), h0, l0);
+          split2(make_float2(ra[c].z, OPA == OP_H ? -ra[c].w : ra[c].w), h1, l1);
+          *reinterpret_cast<float4*>(Ahi + o) = make_float4(h0.x, h0.y, h1.x, h1.y);
+          *reinterpret_cast<float4*>(Alo + o) = make_float4(l0.x, l0.y, l1.x, l1.y);
+          split2(make_float2(rb[c].x, OPB == OP_H ? -rb[c].y : rb[c].y), h0, l0);
+          split2(make_float2(rb[c].z, OPB == OP_H ? -rb[c].w : rb[c].w), h1, l1);
+          *reinterpret_cast<float4*>(Bhi + o) = make_float4(h0.x, -h0.y, h1.x, -h1.y);    // -> C_r
+          *reinterpret_cast<float4*>(Blo + o) = make_float4(l0.x, -l0.y, l1.x, -l1.y);
+          *reinterpret_cast<float4*>(Bhi + o2) = make_float4(h0.y, h0.x, h1.y, h1.x);     // -> C_i
+          *reinterpret_cast<float4*>(Blo + o2) = make_float4(l0.y, l0.x, l1.y, l1.x);
         }
       }
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       mbar_arrive(&bar_full[s]);
     };
-    // slice pos (16 columns) of window dw's accumulator into the sums
-    auto drain = [&](int dw, int pos) {
-      const int b = dw & 1;
-      if (pos == 0 && ok) ok = mbar_wait(&bar_acc_full[b], (uint32_t)(dw >> 1) & 1u, err);
-      tc_fence_after();
-      uint32_t v[16];
-      // tcgen05.ld is warp-collective: the whole warp reads the accumulator, or none of it
-      if (__all_sync(0xffffffffu, ok)) {
-        tmem_ld16(tmem + tlane + (uint32_t)(b * 2 * TC_NC + TC_NC * h + 16 * pos), v);
-        tmem_ld_wait();
-      } else {
+    float acc[TC_NC];   // this thread's 128 window sums
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = 0u;
+    for (int i = 0; i < TC_NC; ++i) acc[i] = 0.f;
+#pragma unroll
+    for (int e = 0; e < TC_RAW - 1; ++e) copy(e);
+    // after producing stage st = TC_WIN win + pos, drain slice pos (16 columns) of window win - 1
+#pragma unroll 1
+    for (int win = 0; win <= nwin; ++win) {
+      const int b = (win - 1) & 1;
+#pragma unroll
+      for (int pos = 0; pos < TC_WIN; ++pos) {
+        const int st = TC_WIN * win + pos;
+        if (st < nst) {
+          __syncwarp();   // the slot copied into next was read by the whole warp
+          copy(st + TC_RAW - 1);
+          asm volatile("cp.async.wait_group %0;\n" ::"n"(TC_RAW - 1) : "memory");
+          __syncwarp();   // every lane's copies of stage st have landed
+          produce(st);
+        }
+        if (win > 0) {
+          if (pos == 0) {
+            if (ok) ok = mbar_wait(&bar_acc_full[b], (uint32_t)((win - 1) >> 1) & 1u, err);
+            tc_fence_after();
+          }
+          uint32_t v[16];
+          // tcgen05.ld is warp-collective: the whole warp reads the accumulator, or none of it
+          if (__all_sync(0xffffffffu, ok)) {
+            tmem_ld16(tmem + tlane + (uint32_t)(b * 2 * TC_NC + TC_NC * h + 16 * pos), v);
+            tmem_ld_wait();
+          } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = 0u;
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[16 * pos + i] += __uint_as_float(v[i]);
+        }
       }
-      float* sp = my_sums + (16 * pos) * TC_M;
-#pragma unroll
-      for (int i = 0; i < 16; ++i) sp[i * TC_M] = dw == 0 ? __uint_as_float(v[i]) : sp[i * TC_M] + __uint_as_float(v[i]);
-      if (pos == TC_WIN - 1) {
+      if (win > 0) {
         tc_fence_before();
         mbar_arrive(&bar_acc_empty[b]);
       }
-    };
-#pragma unroll
-    for (int e = 0; e < TC_PF; ++e) load(e, pa[e], pb[e]);
-    // stages in groups of TC_PF (stage st in buffer st % TC_PF); after producing stage
-    // st = TC_WIN win + pos, drain slice pos of window win - 1
-#pragma unroll 1
-    for (int st0 = 0; st0 < TC_WIN * (nwin + 1); st0 += TC_PF) {
-#pragma unroll
-      for (int e = 0; e < TC_PF; ++e) {
-        const int st = st0 + e;
-        if (st < nst) {
-          float2 a[4], b[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) { a[j] = pa[e][j]; b[j] = pb[e][j]; }
-          load(st + TC_PF, pa[e], pb[e]);   // TC_PF stages ahead, in flight while this one is stored
-          produce(st, a, b);
-        }
-        const int win = st / TC_WIN, pos = st % TC_WIN;
-        if (win >= 1 && win - 1 < nwin) drain(win - 1, pos);
-      }
     }
-    // ---- output ----------------------------------------------------------------------
-    asm volatile("bar.sync 1, %0;\n" ::"r"(TC_PROD) : "memory");   // both halves of every row drained
+    // ---- output: the two halves of a row meet in shared memory ------------------------
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    asm volatile("bar.sync 1, %0;\n" ::"r"(TC_PROD) : "memory");   // every window drained: the rings are free
+#pragma unroll
+    for (int i = 0; i < TC_NC; ++i) sums[(TC_NC * h + i) * TC_M + r] = acc[i];
+    asm volatile("bar.sync 1, %0;\n" ::"r"(TC_PROD) : "memory");
+    const int m = m0 + r;
     if (m < M) {
       for (int j0 = (TC_NC / 2) * h; j0 < (TC_NC / 2) * (h + 1); ++j0) {
         const int j = n0 + j0;
         if (j >= N) break;
-        double2 v = make_double2(0.0, 0.0);
-        if (nst > 0) v = make_double2((double)sums[j0 * TC_M + r], (double)sums[(TC_NC + j0) * TC_M + r]);
+        const double2 v = make_double2((double)sums[j0 * TC_M + r], (double)sums[(TC_NC + j0) * TC_M + r]);
         if (ksplit > 1) {
           part[((long)kz * N + j) * (long)M + m] = v;
         } else {
