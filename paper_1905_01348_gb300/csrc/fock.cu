@@ -20,13 +20,22 @@
 //       output orbital sums its pair contributions in a fixed order and
 //       updates its W row once.
 // X traffic is four passes of the pair volume (write, read+write, read).
+//
+// These kernels serve every grid in FP64 and the non-cubic ones in FP32. FP64 arithmetic
+// bounds them (an SM does two FP64 multiply-adds a clock), so they save operations: a
+// line takes at most two steps of large codelets (fft_pk.cuh) with the fewest twiddles,
+// and the slabs (axis 2) and columns (axis 1) of frequencies that products of the basis
+// cannot reach are neither transformed nor stored. 27 orbitals on 24 x 48 x 32 points, an
+// exchange in FP64: 3.63 ms with lines of three small codelets, 3.46 pruned with the large
+// ones, 3.29 with coprime factors; the FP64 pipe is then busy 3/4 of the time.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <cstring>
 #include <vector>
 
 #include "common.cuh"
-#include "fft.cuh"
+#include "fft_pk.cuh"
 #include "internal.h"
 
 namespace pt {
@@ -37,91 +46,231 @@ static const cplx<T>* twp(const DevTwiddles& tw, int L) {
 }
 
 // ---------------------------------------------------------------------------
+// Lines in shared memory, L = R M, take two in-place steps: A, R-point DFTs, and B, M-point
+// DFTs. For 24 = 8 x 3 and 48 = 16 x 3 (coprime factors) element 3 q + R m (mod L) has index q
+// in step A and m in step B, without twiddles; otherwise element m + M q has, and step A
+// applies W_L^(m q). place_of(k) is where frequency k ends: (R + 3) k mod L, or
+// M (k mod R) + k / R. The inverse starts from there.
+template <typename T> struct value_of;
+template <> struct value_of<float> { using type = cf; };
+template <> struct value_of<double> { using type = cd; };
+
+__host__ __device__ constexpr bool coprime(int L) { return L == 24 || L == 48; }
+__host__ __device__ constexpr int first_radix(int L) { return L == 12 ? 12 : L == 16 || L == 48 ? 16 : 8; }
+__device__ __forceinline__ int place_of(int k, int L) {
+  const int R = first_radix(L), M = L / R;
+  return coprime(L) ? (R + 3) * k % L : M * (k % R) + k / R;
+}
+__device__ __forceinline__ int freq_at(int place, int L) {
+  const int R = first_radix(L), M = L / R;
+  return coprime(L) ? (L == 24 ? 11 : 43) * place % L : place / M + R * (place % M);
+}
+
+// Transforms `nlines` lines: element e of line i at buf[lines(i) + e es].
+template <int L, bool INV, typename V, class Lines>
+__device__ __forceinline__ void line_pass(V* buf, int nlines, int es, const V* tw, int tid, int nthr, Lines lines) {
+  constexpr int R = first_radix(L), M = L / R;
+  constexpr bool twiddled = M > 1 && !coprime(L);
+  // element q of the DFT number m of step A (b = false), element m of DFT q of step B
+  auto at = [](int q, int m) {
+    if (!coprime(L)) return m + M * q;
+    const int e = 3 * q + R * m;
+    return e >= L ? e - L : e;
+  };
+  auto step_a = [&]() {
+    for (int b = tid; b < nlines * M; b += nthr) {
+      const int m = b / nlines;
+      V* p = buf + lines(b - m * nlines);
+      V v[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) v[q] = p[at(q, m) * es];
+      if (INV && twiddled) {
+#pragma unroll
+        for (int q = 1; q < R; ++q) v[q] = ptwiddle<true>(v[q], tw[q * m]);
+      }
+      pk_dft<R, INV>(v);
+      if (!INV && twiddled) {
+#pragma unroll
+        for (int q = 1; q < R; ++q) v[q] = ptwiddle<false>(v[q], tw[q * m]);
+      }
+#pragma unroll
+      for (int q = 0; q < R; ++q) p[at(q, m) * es] = v[q];
+    }
+    __syncthreads();
+  };
+  auto step_b = [&]() {
+    for (int b = tid; b < nlines * R; b += nthr) {
+      const int q = b / nlines;
+      V* p = buf + lines(b - q * nlines);
+      V v[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) v[m] = p[at(q, m) * es];
+      pk_dft<M, INV>(v);
+#pragma unroll
+      for (int m = 0; m < M; ++m) p[at(q, m) * es] = v[m];
+    }
+    __syncthreads();
+  };
+  if constexpr (M == 1) {
+    step_a();
+  } else if constexpr (!INV) {
+    step_a();
+    step_b();
+  } else {
+    step_b();
+    step_a();
+  }
+}
+
+template <bool INV, typename V, class Lines>
+__device__ __forceinline__ void line_pass_any(V* buf, int L, int nlines, int es, const V* tw, int tid, int nthr,
+                                              Lines lines) {
+  switch (L) {
+    case 8: line_pass<8, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 12: line_pass<12, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 16: line_pass<16, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 24: line_pass<24, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 32: line_pass<32, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 48: line_pass<48, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 64: line_pass<64, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 96: line_pass<96, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    default: break;
+  }
+}
+
+// twiddles c - i s as (c, s)
+template <typename V, typename C> __device__ __forceinline__ void load_tw(V* tw, const C* tw_g, int L, int tid, int nthr) {
+  for (int t = tid; t < L; t += nthr) tw[t] = V{tw_g[t].x, -tw_g[t].y};
+}
+
+// Largest frequency along axis 1 of the pair products in the axis-2 slab of frequency +-g2,
+// and the axis-2 reach (n1, n2 or more: every one is reached).
+struct PairReach {
+  int g2;
+  unsigned char g1[kMaxLength / 2 + 1];
+};
+
+__device__ __forceinline__ bool live(int k, int n, int reach) { return k <= reach || k >= n - reach; }
+
 template <typename T>
-__global__ void k_fock_f1(const PairTile* __restrict__ tiles, int tile0, cplx<T>* __restrict__ X, int n0, int n1,
-                          int n2, int rr, const cplx<T>* __restrict__ tw_g) {
-  using C = cplx<T>;
+__global__ void __launch_bounds__(256, 2) k_fock_f1(const PairTile* __restrict__ tiles, int tile0,
+                                                    cplx<T>* __restrict__ Xc, int n0, int n1, int n2, int rr,
+                                                    int reach2, const cplx<T>* __restrict__ tw_g) {
+  using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PairTile tl;
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int rowlen = rr * n2;
-  C* tw = reinterpret_cast<C*>(smem_raw);
-  C* orb = tw + n2;
-  C* work = orb + 2 * kTileMax * rowlen;
-  if (tid == 0) tl = tiles[tile0 + blockIdx.y];
-  for (int t = tid; t < n2; t += nthr) tw[t] = tw_g[t];
+  const int rowlen = rr * n2, ls = n2 + 1;
+  V* X = reinterpret_cast<V*>(Xc);
+  V* tw = reinterpret_cast<V*>(smem_raw);
+  V* orb = tw + n2;
+  V* work = orb + 2 * kTileMax * rowlen;
+  for (int t = tid; t < (int)(sizeof(PairTile) / 4); t += nthr)
+    reinterpret_cast<unsigned*>(&tl)[t] = reinterpret_cast<const unsigned*>(tiles + tile0 + blockIdx.y)[t];
+  load_tw(tw, tw_g, n2, tid, nthr);
   __syncthreads();
   const int nb1 = n1 / rr;
   const int i0 = blockIdx.x / nb1;
   const int i1s = (blockIdx.x - i0 * nb1) * rr;
   const long roff = ((long)i0 * n1 + i1s) * n2;
   for (int o = 0; o < tl.n_orb; ++o) {
-    const C* src = (const C*)tl.in[o] + roff;
+    const V* src = (const V*)tl.in[o] + roff;
     for (int e = tid; e < rowlen; e += nthr) orb[o * rowlen + e] = src[e];
   }
   __syncthreads();
   const int np = tl.n_pairs;
   for (int idx = tid; idx < np * rowlen; idx += nthr) {
-    const int p = idx / rowlen, e = idx - p * rowlen;
-    work[idx] = cmulc(orb[tl.pi[p] * rowlen + e], orb[tl.pj[p] * rowlen + e]);
+    const int l = idx / n2, p = l / rr, e = idx - p * rowlen;
+    const V a = orb[tl.pi[p] * rowlen + e], b = orb[tl.pj[p] * rowlen + e];
+    work[l * ls + idx - l * n2] = V{vfma(a.re, b.re, vmul(a.im, b.im)), vdet(a.re, b.im, a.im, b.re)};   // conj(a) b
   }
   __syncthreads();
-  fft_lines<T, false, true>(work, n2, np * rr, n2, 1, tw, tid, nthr);
+  line_pass_any<false>(work, n2, np * rr, 1, tw, tid, nthr, [ls](int l) { return l * ls; });
   // store X[slot][i2][i0][i1s + r]; consecutive threads take consecutive r
   const long slot0 = (long)blockIdx.y * kTileMax * kTileMax;
   for (int idx = tid; idx < np * rowlen; idx += nthr) {
-    const int r = idx % rr;
-    const int rest = idx / rr;
-    const int i2 = rest % n2;
-    const int p = rest / n2;
-    X[(((slot0 + p) * n2 + i2) * n0 + i0) * n1 + i1s + r] = work[(p * rr + r) * n2 + i2];
+    const int r = idx % rr, rest = idx / rr;
+    const int i2 = rest % n2, p = rest / n2;
+    if (live(i2, n2, reach2))
+      X[(((slot0 + p) * n2 + i2) * n0 + i0) * n1 + i1s + r] = work[(p * rr + r) * ls + place_of(i2, n2)];
   }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(768, 1) k_fock_f2(cplx<T>* __restrict__ X, const PairTile* __restrict__ tiles, int tile0, int n0, int n1,
-                          int n2, const T* __restrict__ khat_t, const cplx<T>* __restrict__ tw0_g,
-                          const cplx<T>* __restrict__ tw1_g) {
-  using C = cplx<T>;
+__global__ void __launch_bounds__(256, 2) k_fock_f2(cplx<T>* __restrict__ Xc, const PairTile* __restrict__ tiles,
+                                                    int tile0, int n0, int n1, int n2, PairReach reach,
+                                                    const T* __restrict__ khat_t, const cplx<T>* __restrict__ tw0_g,
+                                                    const cplx<T>* __restrict__ tw1_g) {
+  using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int n_cols;
+  __shared__ unsigned char cols[kMaxLength], dead[kMaxLength];
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int slot = blockIdx.y;
   const int p = slot % (kTileMax * kTileMax);
   if (p >= tiles[tile0 + slot / (kTileMax * kTileMax)].n_pairs) return;
-  const int i2 = blockIdx.x;
-  C* tw0 = reinterpret_cast<C*>(smem_raw);
-  C* tw1 = tw0 + n0;
-  C* buf = tw1 + n1;
-  for (int t = tid; t < n0; t += nthr) tw0[t] = tw0_g[t];
-  for (int t = tid; t < n1; t += nthr) tw1[t] = tw1_g[t];
-  const int cnt = n0 * n1;
-  C* slab = X + ((long)slot * n2 + i2) * cnt;
-  for (int e = tid; e < cnt; e += nthr) buf[e] = slab[e];
+  // live slabs only: blockIdx.x in [0, n_live) maps to frequencies 0..R, then -R..-1
+  const int i2 = (int)blockIdx.x <= reach.g2 ? (int)blockIdx.x : (int)blockIdx.x + (n2 - (int)gridDim.x);
+  const int reach1 = reach.g1[min(i2, n2 - i2)];
+  const int ls = n1 + 1, cnt = n0 * n1;
+  V* tw0 = reinterpret_cast<V*>(smem_raw);
+  V* tw1 = tw0 + n0;
+  V* buf = tw1 + n1;
+  load_tw(tw0, tw0_g, n0, tid, nthr);
+  load_tw(tw1, tw1_g, n1, tid, nthr);
+  if (tid < 32) {   // places of the live axis-1 frequencies, then of the dead ones
+    int nl = 0, nd = 0;
+    for (int c0 = 0; c0 < n1; c0 += 32) {
+      const int c = c0 + tid;
+      const bool in = c < n1, lv = in && live(freq_at(c, n1), n1, reach1);
+      const unsigned ml = __ballot_sync(0xffffffffu, lv), md = __ballot_sync(0xffffffffu, in && !lv);
+      const unsigned below = (1u << tid) - 1u;
+      if (lv) cols[nl + __popc(ml & below)] = (unsigned char)c;
+      else if (in) dead[nd + __popc(md & below)] = (unsigned char)c;
+      nl += __popc(ml);
+      nd += __popc(md);
+    }
+    if (tid == 0) n_cols = nl;
+  }
+  V* slab = reinterpret_cast<V*>(Xc) + ((long)slot * n2 + i2) * cnt;
+#pragma unroll 4
+  for (int e = tid; e < cnt; e += nthr) buf[e / n1 * ls + e % n1] = slab[e];
   __syncthreads();
-  fft_lines<T, false, true>(buf, n1, n0, n1, 1, tw1, tid, nthr);    // axis 1
-  fft_lines<T, false, false>(buf, n0, n1, 1, n1, tw0, tid, nthr);   // axis 0
+  const int nc = n_cols;
+  auto rows = [ls](int l) { return l * ls; };
+  auto live_cols = [](int l) { return (int)cols[l]; };
+  line_pass_any<false>(buf, n1, n0, 1, tw1, tid, nthr, rows);           // axis 1
+  line_pass_any<false>(buf, n0, nc, ls, tw0, tid, nthr, live_cols);     // axis 0, live columns
   const T* kt = khat_t + (long)i2 * cnt;
-  for (int e = tid; e < cnt; e += nthr) buf[e] = cscale(buf[e], kt[e]);
+  for (int e = tid; e < nc * n0; e += nthr) {
+    const int r = e / nc, c = cols[e - r * nc];
+    V& v = buf[r * ls + c];
+    const T k = kt[freq_at(r, n0) * n1 + freq_at(c, n1)];
+    v = V{v.re * k, v.im * k};
+  }
+  for (int e = tid; e < (n1 - nc) * n0; e += nthr) buf[e / (n1 - nc) * ls + dead[e % (n1 - nc)]] = V{(T)0, (T)0};
   __syncthreads();
-  fft_lines<T, true, false>(buf, n0, n1, 1, n1, tw0, tid, nthr);
-  fft_lines<T, true, true>(buf, n1, n0, n1, 1, tw1, tid, nthr);
-  for (int e = tid; e < cnt; e += nthr) slab[e] = buf[e];
+  line_pass_any<true>(buf, n0, nc, ls, tw0, tid, nthr, live_cols);
+  line_pass_any<true>(buf, n1, n0, 1, tw1, tid, nthr, rows);
+  for (int e = tid; e < cnt; e += nthr) slab[e] = buf[e / n1 * ls + e % n1];
 }
 
 template <typename T>
-__global__ void k_fock_f3(const PairTile* __restrict__ tiles, int tile0, const cplx<T>* __restrict__ X, int n0, int n1,
-                          int n2, int rr, int sym,
-                          const cplx<T>* __restrict__ tw_g) {
-  using C = cplx<T>;
+__global__ void __launch_bounds__(256, 2) k_fock_f3(const PairTile* __restrict__ tiles, int tile0,
+                                                    const cplx<T>* __restrict__ Xc, int n0, int n1, int n2, int rr,
+                                                    int reach2, const cplx<T>* __restrict__ tw_g) {
+  using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PairTile tl;
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int rowlen = rr * n2;
-  C* tw = reinterpret_cast<C*>(smem_raw);
-  C* orb = tw + n2;
-  C* work = orb + 2 * kTileMax * rowlen;
-  if (tid == 0) tl = tiles[tile0 + blockIdx.y];
-  for (int t = tid; t < n2; t += nthr) tw[t] = tw_g[t];
+  const int rowlen = rr * n2, ls = n2 + 1;
+  const V* X = reinterpret_cast<const V*>(Xc);
+  V* tw = reinterpret_cast<V*>(smem_raw);
+  V* orb = tw + n2;
+  V* work = orb + 2 * kTileMax * rowlen;
+  for (int t = tid; t < (int)(sizeof(PairTile) / 4); t += nthr)
+    reinterpret_cast<unsigned*>(&tl)[t] = reinterpret_cast<const unsigned*>(tiles + tile0 + blockIdx.y)[t];
+  load_tw(tw, tw_g, n2, tid, nthr);
   __syncthreads();
   const int nb1 = n1 / rr;
   const int i0 = blockIdx.x / nb1;
@@ -129,31 +278,32 @@ __global__ void k_fock_f3(const PairTile* __restrict__ tiles, int tile0, const c
   const long roff = ((long)i0 * n1 + i1s) * n2;
   const int np = tl.n_pairs;
   const long slot0 = (long)blockIdx.y * kTileMax * kTileMax;
+#pragma unroll 4
   for (int idx = tid; idx < np * rowlen; idx += nthr) {
-    const int r = idx % rr;
-    const int rest = idx / rr;
-    const int i2 = rest % n2;
-    const int p = rest / n2;
-    work[(p * rr + r) * n2 + i2] = X[(((slot0 + p) * n2 + i2) * n0 + i0) * n1 + i1s + r];
+    const int r = idx % rr, rest = idx / rr;
+    const int i2 = rest % n2, p = rest / n2;
+    work[(p * rr + r) * ls + place_of(i2, n2)] =
+        live(i2, n2, reach2) ? X[(((slot0 + p) * n2 + i2) * n0 + i0) * n1 + i1s + r] : V{(T)0, (T)0};
   }
   for (int o = 0; o < tl.n_orb; ++o) {
-    const C* src = (const C*)tl.in[o] + roff;
+    const V* src = (const V*)tl.in[o] + roff;
     for (int e = tid; e < rowlen; e += nthr) orb[o * rowlen + e] = src[e];
   }
   __syncthreads();
-  fft_lines<T, true, true>(work, n2, np * rr, n2, 1, tw, tid, nthr);
+  line_pass_any<true>(work, n2, np * rr, 1, tw, tid, nthr, [ls](int l) { return l * ls; });
   // each output orbital: fixed-order sum over the tile's pairs, one RMW of its row
   for (int o = 0; o < tl.n_orb; ++o) {
     if (!tl.is_out[o]) continue;
-    C* dst = (C*)tl.out[o] + roff;
+    V* dst = (V*)tl.out[o] + roff;
     for (int e = tid; e < rowlen; e += nthr) {
-      C acc = mk((T)0, (T)0);
-      for (int p = 0; p < np; ++p) {
-        const C v = work[p * rowlen + e];
-        if (tl.pj[p] == o) acc = cadd(acc, cmul(orb[tl.pi[p] * rowlen + e], v));
-        if (sym && tl.pi[p] == o && tl.pi[p] != tl.pj[p]) acc = cadd(acc, cmul_conj(orb[tl.pj[p] * rowlen + e], v));
+      const int r = e / n2;
+      V acc = {(T)0, (T)0};
+      for (int c = 0; c < tl.out_n[o]; ++c) {
+        const V v = work[(tl.out_pair[o][c] * rr + r) * ls + e - r * n2], a = orb[tl.out_other[o][c] * rowlen + e];
+        if (tl.out_conj[o][c]) acc = padd(acc, V{vfma(a.re, v.re, vmul(a.im, v.im)), vdet(a.im, v.re, a.re, v.im)});
+        else acc = padd(acc, V{vdet(a.re, v.re, a.im, v.im), vfma(a.re, v.im, vmul(a.im, v.re))});
       }
-      dst[e] = cadd(dst[e], acc);
+      dst[e] = padd(dst[e], acc);
     }
   }
 }
@@ -166,27 +316,18 @@ static int rows_per_block(int n1, bool fp64) {
   return 1;
 }
 
-static int round_threads(int t) {
-  t = ((t + 31) / 32) * 32;
-  return std::max(64, std::min(1024, t));
-}
-
 template <typename T>
 cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, void* scratch, const DevTwiddles& tw,
                        cudaStream_t s) {
   using C = cplx<T>;
+  (void)sym;   // the tiles' contribution lists know which pairs feed both orbitals
   if constexpr (sizeof(T) == 4) {
     if (fock_fast_supported(g)) return fock_pairs_fast(plan, g, khat_t, scratch, twp<float>(tw, g.n0), s);
   }
   const bool fp64 = sizeof(T) == 8;
   const int rr = rows_per_block(g.n1, fp64);
-  const int rowlen = rr * g.n2;
-  const int lines13 = kTileMax * kTileMax * rr;
-  const int thr13 = round_threads(std::max(fft_threads_needed(g.n2, lines13, fp64), 128));
-  const size_t smem13 = (size_t)(g.n2 + 2 * kTileMax * rowlen + kTileMax * kTileMax * rowlen) * sizeof(C);
-  const int thr2 = round_threads(std::max(fft_threads_needed(g.n1, g.n0, fp64), fft_threads_needed(g.n0, g.n1, fp64)));
-  const size_t smem2 = (size_t)(g.n0 + g.n1 + g.n0 * g.n1) * sizeof(C);
-  if (thr13 > 1024 || thr2 > 768) return cudaErrorInvalidConfiguration;
+  const size_t smem13 = (size_t)(g.n2 + 2 * kTileMax * rr * g.n2 + kTileMax * kTileMax * rr * (g.n2 + 1)) * sizeof(C);
+  const size_t smem2 = (size_t)(g.n0 + g.n1 + g.n0 * (g.n1 + 1)) * sizeof(C);
   cudaError_t e;
   static std::atomic<unsigned long long> attr_done{0};
   if (const unsigned long long bit = device_bit_todo(attr_done)) {
@@ -199,17 +340,26 @@ cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, 
     attr_done.fetch_or(bit, std::memory_order_release);
   }
   if (smem13 > 200 * 1024 || smem2 > 200 * 1024) return cudaErrorInvalidConfiguration;
+  // four blocks per SM keep the FP64 pipe busy across barriers; large tiles take wider blocks
+  const int thr13 = smem13 > 50 * 1024 ? 256 : 128, thr2 = smem2 > 50 * 1024 ? 256 : 128;
   const C* tw0 = twp<T>(tw, g.n0);
   const C* tw1 = twp<T>(tw, g.n1);
   const C* tw2 = twp<T>(tw, g.n2);
   C* X = (C*)scratch;
+  // frequencies of pair products; with aliasing along axis 1 or 2 any may hold one
+  PairReach reach;
+  const bool free2 = 2 * plan.g2_reach + 1 <= g.n2, free1 = 2 * plan.g1_reach[0] + 1 <= g.n1;
+  reach.g2 = free2 ? plan.g2_reach : g.n2;
+  for (int k = 0; k <= kMaxLength / 2; ++k)
+    reach.g1[k] = (unsigned char)(free1 && free2 && k <= plan.g2_reach ? plan.g1_reach[k] : g.n1);
+  const unsigned n_live = free2 ? 2 * plan.g2_reach + 1 : g.n2;
   for (int l = 0; l < plan.n_launch; ++l) {
     const int t0 = plan.launch_first[l], nt = plan.launch_count[l];
     dim3 g13((unsigned)(g.n0 * (g.n1 / rr)), (unsigned)nt);
-    k_fock_f1<T><<<g13, thr13, smem13, s>>>(plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, tw2); launched();
-    dim3 g2((unsigned)g.n2, (unsigned)(nt * kTileMax * kTileMax));
-    k_fock_f2<T><<<g2, thr2, smem2, s>>>(X, plan.d_tiles, t0, g.n0, g.n1, g.n2, khat_t, tw0, tw1); launched();
-    k_fock_f3<T><<<g13, thr13, smem13, s>>>(plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, sym, tw2); launched();
+    k_fock_f1<T><<<g13, thr13, smem13, s>>>(plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
+    dim3 g2(n_live, (unsigned)(nt * kTileMax * kTileMax));
+    k_fock_f2<T><<<g2, thr2, smem2, s>>>(X, plan.d_tiles, t0, g.n0, g.n1, g.n2, reach, khat_t, tw0, tw1); launched();
+    k_fock_f3<T><<<g13, thr13, smem13, s>>>(plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
   }
   return cudaGetLastError();
 }

@@ -13,6 +13,7 @@ namespace pt {
 // Supported FFT lengths and the offset of each length's twiddle table.
 constexpr int kNumLengths = 8;
 constexpr int kLengths[kNumLengths] = {8, 12, 16, 24, 32, 48, 64, 96};
+constexpr int kMaxLength = 96;
 constexpr int kTwiddleTotal = 8 + 12 + 16 + 24 + 32 + 48 + 64 + 96;
 int twiddle_offset(int L);   // -1 if unsupported
 void twiddle_host(double2* out);   // all tables, exp(-2 pi i t / L)
@@ -162,6 +163,9 @@ struct FockPlan {
   // exactly beyond it on an alias-free grid, so the fast path skips those
   // axis-2 slabs. A value >= n2 / 2 disables the skip.
   int g2_reach;
+  // Largest |G1| a pair product can reach at |G2| = k (k <= g2_reach and kMaxLength / 2): the
+  // products lie in the ball of twice the basis cutoff's radius.
+  unsigned char g1_reach[kMaxLength / 2 + 1];
 };
 
 // The pair kernels of `plan` (tiles bound to their orbitals and accumulators).
