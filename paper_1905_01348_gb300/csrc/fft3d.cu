@@ -174,45 +174,69 @@ cudaError_t fft_cols(void* data, long nvol, Grid3 g, int axis, int inverse, int 
 }
 
 // ---------------------------------------------------------------------------
-// Convolution of a real field with a reciprocal-space factor (the Hartree solve, the Kerker
-// mixing) on cubic grids of 32, 48 or 64 points: a block transforms a whole plane (axes 1 and
-// 2) in shared memory, so the solve takes three launches instead of seven, with the field's
-// load, the factor and the potential's assembly inside them. One volume is too little work
-// to fill the chip: launches and latency bound it (32^3: 100 us in seven launches).
+// Convolution of a real field with an even real reciprocal-space factor (the Hartree solve,
+// the Kerker mixing) on cubic grids of 32 to 96 points: a block transforms a whole plane
+// (axes 1 and 2) in shared memory, so the solve takes three launches instead of seven, with
+// the field's load, the factor and the potential's assembly inside them. FP64 arithmetic and
+// latency bound it (one volume is little work), so the transforms use that the field is
+// real: two rows share one complex line, and only the frequencies 0..L/2 of axis 2 are kept.
+// The three launches at 32^3: 40 us, 48 with complex fields (64^3 with complex fields: 140).
 namespace {
 
 template <int L> struct ConvCfg {
-  static constexpr int NT = L == 32 ? 128 : L == 48 ? 192 : 256;   // plane kernels
+  static constexpr int H = L / 2 + 1;                              // columns of the half spectrum
+  static constexpr int HS = H | 1;                                 // odd row stride
+  static constexpr int NT = L == 32 ? 128 : L == 48 ? 192 : L == 64 ? 256 : 384;   // plane kernels
   static constexpr int NC = 8;                                     // columns of an axis-0 block
-  static constexpr int NT0 = L == 48 ? 96 : 64;
-  static constexpr size_t smem_plane = sizeof(double2) * (L + L * (L + 1));
+  static constexpr int NT0 = L >= 48 && L != 64 ? 96 : 64;
+  static constexpr size_t smem_plane = sizeof(double2) * (L + L / 2 * (L + 1) + L * HS);
   static constexpr size_t smem_axis0 = sizeof(double2) * (L + L * (NC + 1));
 };
 
-// plane i0 of a (minus b, when given), transformed along axes 2 and 1
+// plane i0 of a (minus b, when given), transformed along axes 2 and 1, frequencies 0..L/2 of
+// axis 2; the blocks beyond the planes write the part of the local potential that does not
+// wait for the result, on SMs the planes leave idle
 template <int L>
 __global__ void __launch_bounds__(ConvCfg<L>::NT) k_conv_plane_fwd(const double* __restrict__ a,
                                                                    const double* __restrict__ b,
-                                                                   double2* __restrict__ out,
+                                                                   double2* __restrict__ out, ConvSink sink,
                                                                    const double2* __restrict__ tw_g) {
-  constexpr int NT = ConvCfg<L>::NT;
+  constexpr int NT = ConvCfg<L>::NT, H = ConvCfg<L>::H, HS = ConvCfg<L>::HS, W = L + 1;
+  if (blockIdx.x >= L) {
+#pragma unroll 2
+    for (int p = (blockIdx.x - L) * NT + threadIdx.x; p < L * L * L; p += (gridDim.x - L) * NT)
+      sink.vloc[p] = static_potential(sink, p);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* tw = reinterpret_cast<double2*>(smem_raw);
-  double2* buf = tw + L;
+  double2* buf = tw + L;             // [row pair][i2]
+  double2* half = buf + L / 2 * W;   // [i1][frequency]
   const int tid = threadIdx.x;
   const long off = (long)blockIdx.x * L * L;
   for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
 #pragma unroll 4
-  for (int e = tid; e < L * L; e += NT) {
-    double v = a[off + e];
-    if (b != nullptr) v -= b[off + e];
-    buf[(e / L) * (L + 1) + e % L] = make_double2(v, 0.0);
+  for (int e = tid; e < L / 2 * L; e += NT) {
+    const int r = e / L, i2 = e % L;
+    const long p = off + 2 * r * L + i2;
+    double2 v = make_double2(a[p], a[p + L]);
+    if (b != nullptr) v = make_double2(v.x - b[p], v.y - b[p + L]);
+    buf[r * W + i2] = v;
   }
   __syncthreads();
-  ct_forward<double2, L, L, NT, L + 1, 1>(buf, L, tw, tid);
-  ct_forward<double2, L, L, NT, 1, L + 1>(buf, L, tw, tid);
+  ct_forward<double2, L, L / 2, NT, W, 1>(buf, L / 2, tw, tid);
+  // the two rows of a line: (Z_k + conj Z_-k) / 2 and (Z_k - conj Z_-k) / 2i
+  for (int e = tid; e < L / 2 * H; e += NT) {
+    const int r = e / H, k = e % H;
+    const double2 z = buf[r * W + k], c = buf[r * W + (k ? L - k : 0)];
+    half[2 * r * HS + k] = make_double2(0.5 * (z.x + c.x), 0.5 * (z.y - c.y));
+    half[(2 * r + 1) * HS + k] = make_double2(0.5 * (z.y + c.y), 0.5 * (c.x - z.x));
+  }
+  __syncthreads();
+  ct_forward<double2, L, H, NT, 1, HS>(half, H, tw, tid);
+  double2* o = out + (long)blockIdx.x * L * H;
 #pragma unroll 4
-  for (int e = tid; e < L * L; e += NT) out[off + e] = buf[(e / L) * (L + 1) + e % L];
+  for (int e = tid; e < L * H; e += NT) o[e] = half[(e / H) * HS + e % H];
 }
 
 // axis 0 of NC columns: forward, times f, inverse, in place
@@ -220,48 +244,63 @@ template <int L>
 __global__ void __launch_bounds__(ConvCfg<L>::NT0) k_conv_axis0(double2* __restrict__ data,
                                                                 const double* __restrict__ f,
                                                                 const double2* __restrict__ tw_g) {
-  constexpr int NT = ConvCfg<L>::NT0, NC = ConvCfg<L>::NC;
+  constexpr int NT = ConvCfg<L>::NT0, NC = ConvCfg<L>::NC, H = ConvCfg<L>::H;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* tw = reinterpret_cast<double2*>(smem_raw);
   double2* buf = tw + L;
   const int tid = threadIdx.x;
-  const long off = (long)blockIdx.x * NC;
+  const int c0 = blockIdx.x * NC, nc = min(NC, L * H - c0);
   for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
 #pragma unroll 4
-  for (int e = tid; e < L * NC; e += NT) buf[(e / NC) * (NC + 1) + e % NC] = data[(long)(e / NC) * L * L + off + e % NC];
+  for (int e = tid; e < L * NC; e += NT)
+    if (e % NC < nc) buf[(e / NC) * (NC + 1) + e % NC] = data[(long)(e / NC) * L * H + c0 + e % NC];
   __syncthreads();
-  ct_forward<double2, L, NC, NT, 1, NC + 1>(buf, NC, tw, tid);
+  ct_forward<double2, L, NC, NT, 1, NC + 1>(buf, nc, tw, tid);
   for (int e = tid; e < L * NC; e += NT) {
+    if (e % NC >= nc) continue;
+    const int col = c0 + e % NC;
     double2& v = buf[(e / NC) * (NC + 1) + e % NC];
-    v = cscale(v, f[(long)(e / NC) * L * L + off + e % NC]);
+    v = cscale(v, f[((long)(e / NC) * L + col / H) * L + col % H]);
   }
   __syncthreads();
-  ct_inverse<double2, L, NC, NT, 1, NC + 1>(buf, NC, tw, tid);
+  ct_inverse<double2, L, NC, NT, 1, NC + 1>(buf, nc, tw, tid);
 #pragma unroll 4
-  for (int e = tid; e < L * NC; e += NT) data[(long)(e / NC) * L * L + off + e % NC] = buf[(e / NC) * (NC + 1) + e % NC];
+  for (int e = tid; e < L * NC; e += NT)
+    if (e % NC < nc) data[(long)(e / NC) * L * H + c0 + e % NC] = buf[(e / NC) * (NC + 1) + e % NC];
 }
 
-// plane i0 back along axes 1 and 2; the real part goes to the sink
+// plane i0 back along axes 1 and 2 (row pairs as one complex line), the result to the sink
 template <int L>
 __global__ void __launch_bounds__(ConvCfg<L>::NT) k_conv_plane_inv(const double2* __restrict__ in, ConvSink sink,
                                                                    const double2* __restrict__ tw_g) {
-  constexpr int NT = ConvCfg<L>::NT;
+  constexpr int NT = ConvCfg<L>::NT, H = ConvCfg<L>::H, HS = ConvCfg<L>::HS, W = L + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* tw = reinterpret_cast<double2*>(smem_raw);
   double2* buf = tw + L;
+  double2* half = buf + L / 2 * W;
   const int tid = threadIdx.x;
   const long off = (long)blockIdx.x * L * L;
   for (int t = tid; t < L; t += NT) tw[t] = tw_g[t];
+  const double2* src = in + (long)blockIdx.x * L * H;
 #pragma unroll 4
-  for (int e = tid; e < L * L; e += NT) buf[(e / L) * (L + 1) + e % L] = in[off + e];
+  for (int e = tid; e < L * H; e += NT) half[(e / H) * HS + e % H] = src[e];
   __syncthreads();
-  ct_inverse<double2, L, L, NT, 1, L + 1>(buf, L, tw, tid);
-  ct_inverse<double2, L, L, NT, L + 1, 1>(buf, L, tw, tid);
-#pragma unroll 2
-  for (int e = tid; e < L * L; e += NT) {
-    const double h = buf[(e / L) * (L + 1) + e % L].x;
-    if (sink.acc != nullptr) sink.acc[off + e] += h;
-    else sink_potential(sink, off + e, h);
+  ct_inverse<double2, L, H, NT, 1, HS>(half, H, tw, tid);
+  for (int e = tid; e < L / 2 * L; e += NT) {   // Z_k = A_k + i B_k, A_-k = conj A_k
+    const int r = e / L, k = e % L;
+    const bool up = k < H;
+    const double2 x = half[2 * r * HS + (up ? k : L - k)], y = half[(2 * r + 1) * HS + (up ? k : L - k)];
+    buf[r * W + k] = up ? make_double2(x.x - y.y, x.y + y.x) : make_double2(x.x + y.y, y.x - x.y);
+  }
+  __syncthreads();
+  ct_inverse<double2, L, L / 2, NT, W, 1>(buf, L / 2, tw, tid);
+#pragma unroll 4
+  for (int e = tid; e < L / 2 * L; e += NT) {
+    const int r = e / L, i2 = e % L;
+    const long p = off + 2 * r * L + i2;
+    const double2 h = buf[r * W + i2];
+    sink_result(sink, p, h.x);
+    sink_result(sink, p + L, h.y);
   }
 }
 
@@ -278,8 +317,9 @@ cudaError_t convolve_t(const double* a, const double* b, const double* f, double
     if (e != cudaSuccess) return e;
     attr_done.fetch_or(bit, std::memory_order_release);
   }
-  k_conv_plane_fwd<L><<<L, G::NT, G::smem_plane, s>>>(a, b, work, tw);
-  k_conv_axis0<L><<<L * L / G::NC, G::NT0, G::smem_axis0, s>>>(work, f, tw);
+  const int extra = sink.acc == nullptr ? std::max(32, sm_count() - L) : 0;
+  k_conv_plane_fwd<L><<<L + extra, G::NT, G::smem_plane, s>>>(a, b, work, sink, tw);
+  k_conv_axis0<L><<<(L * G::H + G::NC - 1) / G::NC, G::NT0, G::smem_axis0, s>>>(work, f, tw);
   k_conv_plane_inv<L><<<L, G::NT, G::smem_plane, s>>>(work, sink, tw);
   launched(3);
   return cudaGetLastError();
@@ -288,7 +328,7 @@ cudaError_t convolve_t(const double* a, const double* b, const double* f, double
 }  // namespace
 
 bool convolve_supported(Grid3 g) {
-  return g.n0 == g.n1 && g.n1 == g.n2 && (g.n0 == 32 || g.n0 == 48 || g.n0 == 64);
+  return g.n0 == g.n1 && g.n1 == g.n2 && (g.n0 == 32 || g.n0 == 48 || g.n0 == 64 || g.n0 == 96);
 }
 
 cudaError_t convolve(const double* a, const double* b, const double* f, double2* work, const ConvSink& sink, Grid3 g,
@@ -298,6 +338,7 @@ cudaError_t convolve(const double* a, const double* b, const double* f, double2*
     case 32: return convolve_t<32>(a, b, f, work, sink, t, s);
     case 48: return convolve_t<48>(a, b, f, work, sink, t, s);
     case 64: return convolve_t<64>(a, b, f, work, sink, t, s);
+    case 96: return convolve_t<96>(a, b, f, work, sink, t, s);
     default: return cudaErrorInvalidValue;
   }
 }

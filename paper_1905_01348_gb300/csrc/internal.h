@@ -75,19 +75,24 @@ __device__ __forceinline__ double cbrt_pos(double x) {
   y = fma(fma(-y * y, y, x), c, y);
   return fma(fma(-y * y, y, x), c, y);
 }
-// vh, vloc (and vloc32) of grid point r with Hartree potential h (vh null: no Hartree)
-__device__ __forceinline__ void sink_potential(const ConvSink& k, long r, double h) {
-  double v = k.vion[r];
-  if (k.vh != nullptr) {
-    k.vh[r] = h;
-    v += h;
+// the local potential of grid point r without Hartree
+__device__ __forceinline__ double static_potential(const ConvSink& k, long r) {
+  return k.w_lda != 0.0 ? fma(-k.w_lda, cbrt_pos(3.0 / M_PI * k.rho[r]), k.vion[r]) : k.vion[r];
+}
+// adds the convolution's result h at r to acc, or as the Hartree potential to vloc, which
+// holds static_potential
+__device__ __forceinline__ void sink_result(const ConvSink& k, long r, double h) {
+  if (k.acc != nullptr) {
+    k.acc[r] += h;
+    return;
   }
-  if (k.w_lda != 0.0) v += k.w_lda * -cbrt_pos(3.0 / M_PI * k.rho[r]);
+  k.vh[r] = h;
+  const double v = k.vloc[r] + h;
   k.vloc[r] = v;
   if (k.vloc32 != nullptr) k.vloc32[r] = (float)v;
 }
 #endif
-// h = F^-1[f F[a - b]] (b may be null; f carries the 1 / N) on the supported cubic grids;
+// h = F^-1[f F[a - b]] (b may be null; f real, even, with the 1 / N) on the supported cubic grids;
 // work: one complex128 volume.
 bool convolve_supported(Grid3 g);
 cudaError_t convolve(const double* a, const double* b, const double* f, double2* work, const ConvSink& sink, Grid3 g,

@@ -101,8 +101,16 @@ __global__ void k_rho_to_complex(const double* __restrict__ rho, double2* __rest
 }
 
 __global__ void k_vloc(const double2* __restrict__ vh_c, ConvSink sink, long N) {
-  for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x)
-    sink_potential(sink, r, vh_c != nullptr ? vh_c[r].x : 0.0);
+  for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x) {
+    double v = static_potential(sink, r);
+    if (vh_c != nullptr) {
+      const double h = vh_c[r].x;
+      sink.vh[r] = h;
+      v += h;
+    }
+    sink.vloc[r] = v;
+    if (sink.vloc32 != nullptr) sink.vloc32[r] = (float)v;
+  }
 }
 
 cudaError_t rho_to_complex(const double* rho, double2* buf, long N, cudaStream_t s) {
