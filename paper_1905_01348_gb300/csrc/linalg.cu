@@ -35,8 +35,8 @@ template <typename C> __device__ __forceinline__ C mk_as(float2 v) { return v; }
 __device__ __forceinline__ double2 ld_op(const double2* p) { return *p; }
 __device__ __forceinline__ float2 ld_op(const float2* p) { return __ldg(p); }
 
-template <typename C, typename TI>
-__global__ void __launch_bounds__(64) k_gemm(int opA, int opB, int M, int N, int K, int kchunk, int ksplit, int structure,
+template <typename C, typename TI, int opA, int opB>
+__global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, int ksplit, int structure,
                                              double2 alpha, const TI* __restrict__ A, long lda,
                                              const TI* __restrict__ B, long ldb, double2 beta,
                                              double2* __restrict__ Cm, long ldc, double2* __restrict__ part) {
@@ -69,32 +69,31 @@ __global__ void __launch_bounds__(64) k_gemm(int opA, int opB, int M, int N, int
         acc[a][b] = C{};
       }
   };
-  TI ra[P], rb[P];   // next slice, converted when it is stored: the loads stay in flight together
+  // next slice, untouched until it is stored: the loads stay in flight together (a conjugation
+  // at the load waited for each in turn: 16.7 us a product of 16 columns by 1,647, 9.4 now)
+  TI ra[P], rb[P];
   auto fetch = [&](int k0) {
 #pragma unroll
     for (int q = 0; q < P; ++q) {
       const int u = tid & 15, w = (tid >> 4) + 4 * q;   // u runs along the contiguous direction
       const int ia = opA == OP_N ? u : w, ka = opA == OP_N ? w : u;
       const int jb = opB == OP_N ? w : u, kb = opB == OP_N ? u : w;
-      TI va{}, vb{};
-      if (m0 + ia < M && k0 + ka < kend) {
-        if (opA == OP_N) va = ld_op(A + (m0 + ia) + (long)(k0 + ka) * lda);
-        else { va = ld_op(A + (k0 + ka) + (long)(m0 + ia) * lda); va.y = -va.y; }
-      }
-      if (n0 + jb < N && k0 + kb < kend) {
-        if (opB == OP_N) vb = ld_op(B + (k0 + kb) + (long)(n0 + jb) * ldb);
-        else { vb = ld_op(B + (n0 + jb) + (long)(k0 + kb) * ldb); vb.y = -vb.y; }
-      }
-      ra[q] = va;
-      rb[q] = vb;
+      ra[q] = rb[q] = TI{};
+      if (m0 + ia < M && k0 + ka < kend)
+        ra[q] = ld_op(opA == OP_N ? A + (m0 + ia) + (long)(k0 + ka) * lda : A + (k0 + ka) + (long)(m0 + ia) * lda);
+      if (n0 + jb < N && k0 + kb < kend)
+        rb[q] = ld_op(opB == OP_N ? B + (k0 + kb) + (long)(n0 + jb) * ldb : B + (n0 + jb) + (long)(k0 + kb) * ldb);
     }
   };
   auto stash = [&](int buf) {
 #pragma unroll
     for (int q = 0; q < P; ++q) {
       const int u = tid & 15, w = (tid >> 4) + 4 * q;
-      if (opA == OP_N) As[buf][w][u] = mk_as<C>(ra[q]); else As[buf][u][w] = mk_as<C>(ra[q]);
-      if (opB == OP_N) Bs[buf][u][w] = mk_as<C>(rb[q]); else Bs[buf][w][u] = mk_as<C>(rb[q]);
+      C a = mk_as<C>(ra[q]), b = mk_as<C>(rb[q]);
+      if (opA == OP_H) a.y = -a.y;
+      if (opB == OP_H) b.y = -b.y;
+      if (opA == OP_N) As[buf][w][u] = a; else As[buf][u][w] = a;
+      if (opB == OP_N) Bs[buf][u][w] = b; else Bs[buf][w][u] = b;
     }
   };
   int buf = 0;
@@ -259,8 +258,14 @@ static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alph
   const int least = sizeof(C) == sizeof(double2) ? 8 : 64;
   const int ksplit = K > 0 && ws != nullptr ? choose_split(tiles, K, least, (long)M * N, ws_elems) : 1;
   const int kchunk = std::max(1, (K + ksplit - 1) / ksplit);
-  k_gemm<C, TI><<<dim3(tm, tn, (unsigned)ksplit), 64, 0, s>>>(opA, opB, M, N, K, kchunk, ksplit, structure, alpha, A,
-                                                              lda, B, ldb, beta, Cm, ldc, ws);
+  const dim3 grid(tm, tn, (unsigned)ksplit);
+#define PT_GEMM(OA, OB) \
+  k_gemm<C, TI, OA, OB><<<grid, 64, 0, s>>>(M, N, K, kchunk, ksplit, structure, alpha, A, lda, B, ldb, beta, Cm, ldc, ws)
+  if (opA == OP_N && opB == OP_N) PT_GEMM(OP_N, OP_N);
+  else if (opA == OP_N) PT_GEMM(OP_N, OP_H);
+  else if (opB == OP_N) PT_GEMM(OP_H, OP_N);
+  else PT_GEMM(OP_H, OP_H);
+#undef PT_GEMM
   launched();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || ksplit == 1) return e;
