@@ -301,6 +301,9 @@ __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_
                                                                   double2* __restrict__ gamma) {
   __shared__ double2 L[kSlotMax + 1][kSlotMax + 1];
   __shared__ double inv[kSlotMax];   // 1 / L[j][j]
+  // entries (i, p), p <= i <= k, p < k, by falling p: those a column j still changes (p > j)
+  // come first
+  __shared__ unsigned char ent[kSlotMax * (kSlotMax + 3) / 2][2];
   const int b = blockIdx.x, tid = threadIdx.x, k = sl.k;
   double2* G = gram + (long)b * mdim * mdim;
   // L L^H = A with A[i][j] = G[s_i][s_j]  (G[s][t] = <dR_s, dR_t>); older entries
@@ -308,6 +311,14 @@ __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_
   for (int t = tid; t < k * k; t += kSolveThreads) {
     const int i = t / k, j = t % k;
     if (j <= i && sl.s[i] != newslot && sl.s[j] != newslot) L[i][j] = G[(long)sl.s[i] * mdim + sl.s[j]];
+  }
+  if (tid < k) {
+    const int p = k - 1 - tid;   // rows p .. k after the sum of 2, 3, .. (tid + 1) earlier entries
+    int at = tid * (tid + 3) / 2;
+    for (int i = p; i <= k; ++i, ++at) {
+      ent[at][0] = (unsigned char)i;
+      ent[at][1] = (unsigned char)p;
+    }
   }
   if (tid < k) {
     const int q = tid, mine = sl.s[q];
@@ -342,9 +353,8 @@ __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_
     // rows i > j of column j scaled, and A[i][p] -= L[i][j] conj(L[p][j]) for j < p <= i
     const int m = k - j;   // rows j + 1 .. k
     const double r2 = r * r;
-    for (int t = tid; t < m * m; t += kSolveThreads) {
-      const int i = j + 1 + t % m, p = j + 1 + t / m;
-      if (p > i || p == k) continue;
+    for (int t = tid; t < (m - 1) * (m + 2) / 2; t += kSolveThreads) {
+      const int i = ent[t][0], p = ent[t][1];
       const double2 u = L[i][j], w = L[p][j];
       L[i][p].x -= r2 * (u.x * w.x + u.y * w.y);
       L[i][p].y -= r2 * (u.y * w.x - u.x * w.y);
