@@ -56,6 +56,7 @@ static int round_threads(int t) {
 template <typename T, bool INV>
 __global__ void k_rows(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out, long nrows, int L, int rpc,
                        const cplx<T>* __restrict__ tw_g, T scale, const T* __restrict__ mul, long rows_per_vol) {
+  grid_entry();
   using C = cplx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
@@ -83,6 +84,7 @@ __global__ void k_rows(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out
 template <typename T, bool INV, int MODE>
 __global__ void k_cols(cplx<T>* __restrict__ data, int n0, int n1, int n2, int axis, int chunk,
                        const cplx<T>* __restrict__ tw_g, T scale, const T* __restrict__ mul) {
+  grid_entry();
   using C = cplx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int L = axis == 0 ? n0 : n1;
@@ -136,10 +138,10 @@ cudaError_t fft_rows(const void* in, void* out, long nvol, Grid3 g, int inverse,
   const T sc = (T)scale;
   const long rpv = (long)g.n0 * g.n1;
   if (inverse)
-    k_rows<T, true><<<(unsigned)nblk, nthr, smem, s>>>((const C*)in, (C*)out, nrows, L, rpc, tw_for<T>(tw, L), sc,
+    launch((unsigned)nblk, nthr, smem, s)(k_rows<T, true>, (const C*)in, (C*)out, nrows, L, rpc, tw_for<T>(tw, L), sc,
                                                       mul_real, rpv);
   else
-    k_rows<T, false><<<(unsigned)nblk, nthr, smem, s>>>((const C*)in, (C*)out, nrows, L, rpc, tw_for<T>(tw, L), sc,
+    launch((unsigned)nblk, nthr, smem, s)(k_rows<T, false>, (const C*)in, (C*)out, nrows, L, rpc, tw_for<T>(tw, L), sc,
                                                        mul_real, rpv);
   launched();
   return cudaGetLastError();
@@ -160,7 +162,7 @@ cudaError_t fft_cols(void* data, long nvol, Grid3 g, int axis, int inverse, int 
   dim3 grid((g.n2 + chunk - 1) / chunk, axis == 0 ? g.n1 : g.n0, (unsigned)nvol);
   const T sc = (T)scale;
   const C* twp = tw_for<T>(tw, L);
-#define PT_COLS(INV, MODE) k_cols<T, INV, MODE><<<grid, nthr, smem, s>>>((C*)data, g.n0, g.n1, g.n2, axis, chunk, twp, sc, mul_real)
+#define PT_COLS(INV, MODE) launch(grid, nthr, smem, s)(k_cols<T, INV, MODE>, (C*)data, g.n0, g.n1, g.n2, axis, chunk, twp, sc, mul_real)
   if (mode == 0) {
     if (inverse) PT_COLS(true, 0); else PT_COLS(false, 0);
   } else if (mode == 1) {
@@ -201,6 +203,7 @@ __global__ void __launch_bounds__(ConvCfg<L>::NT) k_conv_plane_fwd(const double*
                                                                    const double* __restrict__ b,
                                                                    double2* __restrict__ out, ConvSink sink,
                                                                    const double2* __restrict__ tw_g) {
+  grid_entry();
   constexpr int NT = ConvCfg<L>::NT, H = ConvCfg<L>::H, HS = ConvCfg<L>::HS, W = L + 1;
   if (blockIdx.x >= L) {
 #pragma unroll 2
@@ -244,6 +247,7 @@ template <int L>
 __global__ void __launch_bounds__(ConvCfg<L>::NT0) k_conv_axis0(double2* __restrict__ data,
                                                                 const double* __restrict__ f,
                                                                 const double2* __restrict__ tw_g) {
+  grid_entry();
   constexpr int NT = ConvCfg<L>::NT0, NC = ConvCfg<L>::NC, H = ConvCfg<L>::H;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* tw = reinterpret_cast<double2*>(smem_raw);
@@ -273,6 +277,7 @@ __global__ void __launch_bounds__(ConvCfg<L>::NT0) k_conv_axis0(double2* __restr
 template <int L>
 __global__ void __launch_bounds__(ConvCfg<L>::NT) k_conv_plane_inv(const double2* __restrict__ in, ConvSink sink,
                                                                    const double2* __restrict__ tw_g) {
+  grid_entry();
   constexpr int NT = ConvCfg<L>::NT, H = ConvCfg<L>::H, HS = ConvCfg<L>::HS, W = L + 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* tw = reinterpret_cast<double2*>(smem_raw);
@@ -318,9 +323,9 @@ cudaError_t convolve_t(const double* a, const double* b, const double* f, double
     attr_done.fetch_or(bit, std::memory_order_release);
   }
   const int extra = sink.acc == nullptr ? std::max(32, sm_count() - L) : 0;
-  k_conv_plane_fwd<L><<<L + extra, G::NT, G::smem_plane, s>>>(a, b, work, sink, tw);
-  k_conv_axis0<L><<<(L * G::H + G::NC - 1) / G::NC, G::NT0, G::smem_axis0, s>>>(work, f, tw);
-  k_conv_plane_inv<L><<<L, G::NT, G::smem_plane, s>>>(work, sink, tw);
+  launch(L + extra, G::NT, G::smem_plane, s)(k_conv_plane_fwd<L>, a, b, work, sink, tw);
+  launch((L * G::H + G::NC - 1) / G::NC, G::NT0, G::smem_axis0, s)(k_conv_axis0<L>, work, f, tw);
+  launch(L, G::NT, G::smem_plane, s)(k_conv_plane_inv<L>, work, sink, tw);
   launched(3);
   return cudaGetLastError();
 }
@@ -347,6 +352,7 @@ cudaError_t convolve(const double* a, const double* b, const double* f, double2*
 template <typename T>
 __global__ void k_scatter(const double2* __restrict__ in, long in_ld, cplx<T>* __restrict__ out, long N,
                           const int* __restrict__ basis, int npw, double scale) {
+  grid_entry();
   const long v = blockIdx.y;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npw; k += gridDim.x * blockDim.x) {
     const double2 c = in[v * in_ld + k];
@@ -358,6 +364,7 @@ template <typename T>
 __global__ void k_gather(const cplx<T>* __restrict__ in, double2* __restrict__ out, long out_ld, long N,
                          const int* __restrict__ basis, int npw, double scale, const double* __restrict__ kin,
                          const double2* __restrict__ x, long x_ld, int accumulate) {
+  grid_entry();
   const long v = blockIdx.y;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npw; k += gridDim.x * blockDim.x) {
     const double2 f = to_d(in[v * N + basis[k]]);
@@ -380,7 +387,7 @@ cudaError_t scatter_basis(const double2* in, long in_ld, void* out, long nvol, G
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(C) * g.N() * nvol, s);
   if (e != cudaSuccess) return e;
   dim3 grid((npw + 255) / 256, (unsigned)nvol);
-  k_scatter<T><<<grid, 256, 0, s>>>(in, in_ld, (C*)out, g.N(), basis, npw, scale); launched();
+  launch(grid, 256, 0, s)(k_scatter<T>, in, in_ld, (C*)out, g.N(), basis, npw, scale); launched();
   return cudaGetLastError();
 }
 
@@ -389,18 +396,19 @@ cudaError_t gather_basis(const void* in, double2* out, long out_ld, long nvol, G
                          double scale, const double* kin, const double2* x, long x_ld, int accumulate, cudaStream_t s) {
   using C = cplx<T>;
   dim3 grid((npw + 255) / 256, (unsigned)nvol);
-  k_gather<T><<<grid, 256, 0, s>>>((const C*)in, out, out_ld, g.N(), basis, npw, scale, kin, x, x_ld, accumulate); launched();
+  launch(grid, 256, 0, s)(k_gather<T>, (const C*)in, out, out_ld, g.N(), basis, npw, scale, kin, x, x_ld, accumulate); launched();
   return cudaGetLastError();
 }
 
 __global__ void k_c128_to_c64(const double2* __restrict__ in, float2* __restrict__ out, long n) {
+  grid_entry();
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
     out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 
 cudaError_t convert_c128_to_c64(const double2* in, float2* out, long n, cudaStream_t s) {
   long blocks = std::min<long>((n + 255) / 256, 152L * 32);
-  k_c128_to_c64<<<(unsigned)std::max<long>(blocks, 1), 256, 0, s>>>(in, out, n); launched();
+  launch((unsigned)std::max<long>(blocks, 1), 256, 0, s)(k_c128_to_c64, in, out, n); launched();
   return cudaGetLastError();
 }
 

@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(SNT) k_sph_rows_inv(const double2* __restrict_
                                                       C* __restrict__ vol, const SphereTables st,
                                                       const int* __restrict__ basis, double scale,
                                                       const C* __restrict__ tw_g) {
+  grid_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* buf = tw + L;
@@ -76,6 +77,7 @@ __global__ void __launch_bounds__(SNT) k_sph_rows_inv(const double2* __restrict_
 template <typename C, int L, bool INV>
 __global__ void __launch_bounds__(SNT) k_sph_axis1(C* __restrict__ vol, const SphereTables st,
                                                    const C* __restrict__ tw_g) {
+  grid_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* buf = tw + L;
@@ -106,6 +108,7 @@ __global__ void __launch_bounds__(SNT) k_sph_axis1(C* __restrict__ vol, const Sp
 template <typename C, int L, bool INV>
 __global__ void __launch_bounds__(SNT) k_sph_axis0(const C* src, C* dst, const typename real_of<C>::type* __restrict__ mul,
                                                    const SphereTables st, const C* __restrict__ tw_g) {
+  grid_entry();
   using R = typename real_of<C>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
@@ -144,6 +147,7 @@ __global__ void __launch_bounds__(SNT) k_sph_rows_fwd(const C* __restrict__ vol,
                                                       const double* __restrict__ kin, const double2* __restrict__ x,
                                                       long ldx, double2* __restrict__ out, long ldo, int accumulate,
                                                       const C* __restrict__ tw_g) {
+  grid_entry();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* buf = tw + L;
@@ -216,6 +220,7 @@ __device__ __forceinline__ void pk_store(float2* p, pk2 v) {
 template <int L, bool INV, int AXIS>
 __global__ void __launch_bounds__(Pk<L>::NT) k_sphp_cols(const float2* src, float2* dst, const float* __restrict__ mul,
                                                          const SphereTables st, const float2* __restrict__ tw_g) {
+  grid_entry();
   constexpr int M = Pk<L>::M, NT = Pk<L>::NT, LS = Pk<L>::LS;
   constexpr long S = AXIS == 0 ? (long)L * L : L;
   __shared__ pk2 tw[L];
@@ -290,6 +295,7 @@ __global__ void __launch_bounds__(Pk<L>::NT) k_sphp_rows_inv(const double2* __re
                                                              float2* __restrict__ vol, const SphereTables st,
                                                              const int* __restrict__ basis, double scale,
                                                              const float2* __restrict__ tw_g) {
+  grid_entry();
   constexpr int M = Pk<L>::M, NT = Pk<L>::NT, LS = Pk<L>::LS;
   __shared__ pk2 tw[L];
   __shared__ pk2 buf[RPB * LS];
@@ -347,6 +353,7 @@ __global__ void __launch_bounds__(Pk<L>::NT) k_sphp_rows_fwd(const float2* __res
                                                              const double2* __restrict__ x, long ldx,
                                                              double2* __restrict__ out, long ldo, int accumulate,
                                                              const float2* __restrict__ tw_g) {
+  grid_entry();
   constexpr int M = Pk<L>::M, NT = Pk<L>::NT, LS = Pk<L>::LS;
   __shared__ pk2 tw[L];
   __shared__ pk2 buf[RPB * LS];
@@ -406,10 +413,9 @@ cudaError_t to_real_t(const double2* coef, long ldc, float2* vol, long nvol, con
                       double scale, const float2* tw, cudaStream_t s) {
   if (st.nrows == 0) return cudaMemsetAsync(vol, 0, sizeof(float2) * (size_t)L * L * L * nvol, s);
   constexpr int NT = Pk<L>::NT;
-  k_sphp_rows_inv<L><<<dim3((unsigned)((st.nrows + 2 * RPB - 1) / (2 * RPB)), (unsigned)nvol), NT, 0, s>>>(
-      coef, ldc, vol, st, basis, scale, tw);
-  k_sphp_cols<L, true, 1><<<dim3(L / (2 * CPB), (unsigned)st.nplanes, (unsigned)nvol), NT, 0, s>>>(vol, vol, nullptr, st, tw);
-  k_sphp_cols<L, true, 0><<<dim3(L / (2 * CPB), L, (unsigned)nvol), NT, 0, s>>>(vol, vol, nullptr, st, tw);
+  launch(dim3((unsigned)((st.nrows + 2 * RPB - 1) / (2 * RPB)), (unsigned)nvol), NT, 0, s)(k_sphp_rows_inv<L>, coef, ldc, vol, st, basis, scale, tw);
+  launch(dim3(L / (2 * CPB), (unsigned)st.nplanes, (unsigned)nvol), NT, 0, s)(k_sphp_cols<L, true, 1>, vol, vol, nullptr, st, tw);
+  launch(dim3(L / (2 * CPB), L, (unsigned)nvol), NT, 0, s)(k_sphp_cols<L, true, 0>, vol, vol, nullptr, st, tw);
   launched(3);
   return cudaGetLastError();
 }
@@ -420,10 +426,9 @@ cudaError_t to_sphere_t(const float2* vol, const float* mul, float2* work, long 
                         long ldo, int accumulate, const float2* tw, cudaStream_t s) {
   if (st.nrows == 0) return cudaSuccess;
   constexpr int NT = Pk<L>::NT;
-  k_sphp_cols<L, false, 0><<<dim3(L / (2 * CPB), L, (unsigned)nvol), NT, 0, s>>>(vol, work, mul, st, tw);
-  k_sphp_cols<L, false, 1><<<dim3(L / (2 * CPB), (unsigned)st.nplanes, (unsigned)nvol), NT, 0, s>>>(work, work, nullptr, st, tw);
-  k_sphp_rows_fwd<L><<<dim3((unsigned)((st.nrows + 2 * RPB - 1) / (2 * RPB)), (unsigned)nvol), NT, 0, s>>>(
-      work, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw);
+  launch(dim3(L / (2 * CPB), L, (unsigned)nvol), NT, 0, s)(k_sphp_cols<L, false, 0>, vol, work, mul, st, tw);
+  launch(dim3(L / (2 * CPB), (unsigned)st.nplanes, (unsigned)nvol), NT, 0, s)(k_sphp_cols<L, false, 1>, work, work, nullptr, st, tw);
+  launch(dim3((unsigned)((st.nrows + 2 * RPB - 1) / (2 * RPB)), (unsigned)nvol), NT, 0, s)(k_sphp_rows_fwd<L>, work, st, basis, scale, kin, x, ldx, out, ldo, accumulate, tw);
   launched(3);
   return cudaGetLastError();
 }
@@ -434,11 +439,11 @@ cudaError_t to_real_t(const double2* coef, long ldc, C* vol, long nvol, const Sp
                       double scale, const C* tw, cudaStream_t s) {
   if (st.nrows == 0) return cudaMemsetAsync(vol, 0, sizeof(C) * (size_t)L * L * L * nvol, s);
   const dim3 gr((unsigned)((st.nrows + SC - 1) / SC), (unsigned)nvol);
-  k_sph_rows_inv<C, L><<<gr, SNT, smem_rows<C, L>(), s>>>(coef, ldc, vol, st, basis, scale, tw);
+  launch(gr, SNT, smem_rows<C, L>(), s)(k_sph_rows_inv<C, L>, coef, ldc, vol, st, basis, scale, tw);
   const dim3 g1((unsigned)(L / SC), (unsigned)st.nplanes, (unsigned)nvol);
-  k_sph_axis1<C, L, true><<<g1, SNT, smem_cols<C, L>(), s>>>(vol, st, tw);
+  launch(g1, SNT, smem_cols<C, L>(), s)(k_sph_axis1<C, L, true>, vol, st, tw);
   const dim3 g0((unsigned)(L / SC), (unsigned)L, (unsigned)nvol);
-  k_sph_axis0<C, L, true><<<g0, SNT, smem_cols<C, L>(), s>>>(vol, vol, nullptr, st, tw);
+  launch(g0, SNT, smem_cols<C, L>(), s)(k_sph_axis0<C, L, true>, vol, vol, nullptr, st, tw);
   launched(3);
   return cudaGetLastError();
 }
@@ -449,11 +454,11 @@ cudaError_t to_sphere_t(const C* vol, const typename real_of<C>::type* mul, C* w
                         long ldx, double2* out, long ldo, int accumulate, const C* tw, cudaStream_t s) {
   if (st.nrows == 0) return cudaSuccess;
   const dim3 g0((unsigned)(L / SC), (unsigned)L, (unsigned)nvol);
-  k_sph_axis0<C, L, false><<<g0, SNT, smem_cols<C, L>(), s>>>(vol, work, mul, st, tw);
+  launch(g0, SNT, smem_cols<C, L>(), s)(k_sph_axis0<C, L, false>, vol, work, mul, st, tw);
   const dim3 g1((unsigned)(L / SC), (unsigned)st.nplanes, (unsigned)nvol);
-  k_sph_axis1<C, L, false><<<g1, SNT, smem_cols<C, L>(), s>>>(work, st, tw);
+  launch(g1, SNT, smem_cols<C, L>(), s)(k_sph_axis1<C, L, false>, work, st, tw);
   const dim3 gr((unsigned)((st.nrows + SC - 1) / SC), (unsigned)nvol);
-  k_sph_rows_fwd<C, L><<<gr, SNT, smem_rows<C, L>(), s>>>(work, st, basis, scale, kin, x, ldx, out, ldo, accumulate,
+  launch(gr, SNT, smem_rows<C, L>(), s)(k_sph_rows_fwd<C, L>, work, st, basis, scale, kin, x, ldx, out, ldo, accumulate,
                                                           tw);
   launched(3);
   return cudaGetLastError();

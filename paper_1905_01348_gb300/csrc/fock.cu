@@ -156,6 +156,7 @@ template <typename T>
 __global__ void __launch_bounds__(256, 2) k_fock_f1(const PairTile* __restrict__ tiles, int tile0,
                                                     cplx<T>* __restrict__ Xc, int n0, int n1, int n2, int rr,
                                                     int reach2, const cplx<T>* __restrict__ tw_g) {
+  grid_entry();
   using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PairTile tl;
@@ -201,6 +202,7 @@ __global__ void __launch_bounds__(256, 2) k_fock_f2(cplx<T>* __restrict__ Xc, co
                                                     int tile0, int n0, int n1, int n2, PairReach reach,
                                                     const T* __restrict__ khat_t, const cplx<T>* __restrict__ tw0_g,
                                                     const cplx<T>* __restrict__ tw1_g) {
+  grid_entry();
   using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int n_cols;
@@ -259,6 +261,7 @@ template <typename T>
 __global__ void __launch_bounds__(256, 2) k_fock_f3(const PairTile* __restrict__ tiles, int tile0,
                                                     const cplx<T>* __restrict__ Xc, int n0, int n1, int n2, int rr,
                                                     int reach2, const cplx<T>* __restrict__ tw_g) {
+  grid_entry();
   using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PairTile tl;
@@ -356,10 +359,10 @@ cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, 
   for (int l = 0; l < plan.n_launch; ++l) {
     const int t0 = plan.launch_first[l], nt = plan.launch_count[l];
     dim3 g13((unsigned)(g.n0 * (g.n1 / rr)), (unsigned)nt);
-    k_fock_f1<T><<<g13, thr13, smem13, s>>>(plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
+    launch(g13, thr13, smem13, s)(k_fock_f1<T>, plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
     dim3 g2(n_live, (unsigned)(nt * kTileMax * kTileMax));
-    k_fock_f2<T><<<g2, thr2, smem2, s>>>(X, plan.d_tiles, t0, g.n0, g.n1, g.n2, reach, khat_t, tw0, tw1); launched();
-    k_fock_f3<T><<<g13, thr13, smem13, s>>>(plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
+    launch(g2, thr2, smem2, s)(k_fock_f2<T>, X, plan.d_tiles, t0, g.n0, g.n1, g.n2, reach, khat_t, tw0, tw1); launched();
+    launch(g13, thr13, smem13, s)(k_fock_f3<T>, plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
   }
   return cudaGetLastError();
 }

@@ -161,6 +161,7 @@ template <int L>
 __global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES1) k_fast_f1(const PairTile* __restrict__ tiles, int n_items,
                                                           pk2* __restrict__ X, const float2* __restrict__ tw_g,
                                                           int reach) {
+  grid_entry();
   using S = Sizes<L>;
   constexpr int M = S::M, MP = S::MP, QS = S::QS, RG = S::RG;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -266,6 +267,7 @@ template <int L>
 __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     k_fast_f2(pk2* __restrict__ X, const PairTile* __restrict__ tiles, const float2* __restrict__ kt2,
               const float2* __restrict__ tw_g, int reach) {
+  grid_entry();
   using S = Sizes<L>;
   constexpr int Q = S::Q, CP = S::CP, CPQ = S::CPQ, SC = S::SC, ROT = S::ROT, NT = S::NT2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -412,6 +414,7 @@ template <int L>
 __global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES3) k_fast_f3(const PairTile* __restrict__ tiles, int n_items,
                                                           const pk2* __restrict__ X,
                                                           const float2* __restrict__ tw_g, int reach) {
+  grid_entry();
   using S = Sizes<L>;
   constexpr int M = S::M, MP = S::MP, QS = S::QS, RG = S::RG;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -585,10 +588,10 @@ static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* 
     const PairTile* tiles = plan.d_tiles + plan.launch_first[l];
     const int nt = plan.launch_count[l], items = nt * S::RG;
     const unsigned g1 = (unsigned)std::min(items, S::RES1 * sms), g3 = (unsigned)std::min(items, S::RES3 * sms);
-    k_fast_f1<L><<<g1, S::NT, S::smem13, s>>>(tiles, items, X, tw, reach);
+    launch(g1, S::NT, S::smem13, s)(k_fast_f1<L>, tiles, items, X, tw, reach);
     dim3 g2((unsigned)n_live, (unsigned)(nt * NPAIR));
-    k_fast_f2<L><<<g2, S::NT2, S::smem2, s>>>(X, tiles, kt2, tw, reach);
-    k_fast_f3<L><<<g3, S::NT, S::smem13, s>>>(tiles, items, X, tw, reach);
+    launch(g2, S::NT2, S::smem2, s)(k_fast_f2<L>, X, tiles, kt2, tw, reach);
+    launch(g3, S::NT, S::smem13, s)(k_fast_f3<L>, tiles, items, X, tw, reach);
     launched(3);
   }
   return cudaGetLastError();

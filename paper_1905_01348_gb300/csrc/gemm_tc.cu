@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     k_cgemm_tf32x3(int M, int N, int K, int kchunk, int ksplit, int tri_b, double2 alpha,
                    const float2* __restrict__ A, long lda, const float2* __restrict__ B, long ldb, double2 beta,
                    double2* __restrict__ Cm, long ldc, double2* __restrict__ part, int* __restrict__ err) {
+  grid_entry();
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar_full[TC_NS];
   __shared__ __align__(8) uint64_t bar_empty[TC_NS];
@@ -413,7 +414,7 @@ static cudaError_t launch_tc(int M, int N, int K, int kchunk, int ksplit, int tr
     attr_done.fetch_or(bit, std::memory_order_release);
   }
   dim3 grid((unsigned)((M + TC_M - 1) / TC_M), (unsigned)((N + TC_NC - 1) / TC_NC), (unsigned)ksplit);
-  k_cgemm_tf32x3<OPA, OPB><<<grid, TC_THREADS, TC_SMEM, s>>>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb,
+  launch(grid, TC_THREADS, TC_SMEM, s)(k_cgemm_tf32x3<OPA, OPB>, M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb,
                                                              beta, C, ldc, ws, err);
   launched();
   return cudaGetLastError();

@@ -7,6 +7,7 @@
 #include <cstddef>
 #include <string>
 #include <atomic>
+#include <utility>
 
 namespace pt {
 
@@ -239,6 +240,38 @@ inline unsigned long long device_bit_todo(const std::atomic<unsigned long long>&
   const unsigned long long bit = 1ull << (dev & 63);
   return (mask.load(std::memory_order_acquire) & bit) ? 0ull : bit;
 }
+
+// Kernel launches that overlap the end of their predecessor. launch(grid, block, shared bytes,
+// stream)(kernel, arguments...) lets the kernel's blocks take their places, and its launch
+// latency pass, while the last blocks of the kernel before it on the stream finish; every
+// kernel begins with grid_entry(), which holds it until that kernel has ended and its writes
+// are visible (and so, as each kernel waits in turn, all before it). A PT-CN step of Si8 is some
+// 500 launches of a few microseconds each: 4.23 ms with plain launches, 3.10 with these. No kernel
+// lets the next one in before its blocks end: blocks that came in early crowded onto the SMs
+// that had room (the FP64 step of Si8 took 7.40 ms instead of 5.66, that of Si64 42.4 instead of
+// 39.7). Errors are left to cudaGetLastError.
+struct launch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  launch(dim3 grid, dim3 block, size_t smem, cudaStream_t s) {
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.numAttrs = 1;
+  }
+#ifdef __CUDACC__
+  template <typename... P, typename... A> void operator()(void (*kernel)(P...), A&&... args) {
+    cfg.attrs = &attr;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  }
+#endif
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_entry() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+#endif
 
 // Count of kernels this library has launched (all systems, this process).
 void launched(int n = 1);

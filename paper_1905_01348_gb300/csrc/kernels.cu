@@ -39,6 +39,7 @@ __device__ __forceinline__ void block_sums(double (&v)[NS], double* part) {
 // out[q] = sum of part[b ns + q] over the nblocks partials, in an order that depends on
 // nblocks alone: one warp per sum, lane l adding partials l, l + 32, ... first.
 __global__ void k_finalize(const double* __restrict__ part, int nblocks, int ns, double* __restrict__ out) {
+  grid_entry();
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (q >= ns) return;
   double t = 0.0;
@@ -49,11 +50,12 @@ __global__ void k_finalize(const double* __restrict__ part, int nblocks, int ns,
 }
 
 static void finalize(const double* part, int nblocks, int ns, double* out, cudaStream_t s) {
-  k_finalize<<<1, 32 * ns, 0, s>>>(part, nblocks, ns, out); launched();
+  launch(1, 32 * ns, 0, s)(k_finalize, part, nblocks, ns, out); launched();
 }
 
 // ---- density ------------------------------------------------------------------
 __global__ void k_density(const double2* __restrict__ psi_r, long N, int ne, double* __restrict__ rho) {
+  grid_entry();
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int k = 0; k < ne; ++k) {
@@ -65,13 +67,14 @@ __global__ void k_density(const double2* __restrict__ psi_r, long N, int ne, dou
 }
 
 cudaError_t density(const double2* psi_r, long N, int ne, double* rho, cudaStream_t s) {
-  k_density<<<nblk(N, 256, 152L * 64), 256, 0, s>>>(psi_r, N, ne, rho); launched();
+  launch(nblk(N, 256, 152L * 64), 256, 0, s)(k_density, psi_r, N, ne, rho); launched();
   return cudaGetLastError();
 }
 
 // FP32 squares summed in FP32 over groups of 16 bands (eight loads in flight
 // per thread), the group sums accumulated in FP64: FP64 work drops 16-fold.
 __global__ void k_density32(const float2* __restrict__ psi_r, long N, int ne, double* __restrict__ rho) {
+  grid_entry();
   constexpr int G = 16;
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x) {
     double s = 0.0;
@@ -90,17 +93,19 @@ __global__ void k_density32(const float2* __restrict__ psi_r, long N, int ne, do
 }
 
 cudaError_t density32(const float2* psi_r, long N, int ne, double* rho, cudaStream_t s) {
-  k_density32<<<nblk(N, 256, 152L * 64), 256, 0, s>>>(psi_r, N, ne, rho); launched();
+  launch(nblk(N, 256, 152L * 64), 256, 0, s)(k_density32, psi_r, N, ne, rho); launched();
   return cudaGetLastError();
 }
 
 // ---- local potential -----------------------------------------------------------
 __global__ void k_rho_to_complex(const double* __restrict__ rho, double2* __restrict__ buf, long N) {
+  grid_entry();
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x)
     buf[r] = make_double2(rho[r], 0.0);
 }
 
 __global__ void k_vloc(const double2* __restrict__ vh_c, ConvSink sink, long N) {
+  grid_entry();
   for (long r = blockIdx.x * (long)blockDim.x + threadIdx.x; r < N; r += (long)gridDim.x * blockDim.x) {
     double v = static_potential(sink, r);
     if (vh_c != nullptr) {
@@ -114,18 +119,19 @@ __global__ void k_vloc(const double2* __restrict__ vh_c, ConvSink sink, long N) 
 }
 
 cudaError_t rho_to_complex(const double* rho, double2* buf, long N, cudaStream_t s) {
-  k_rho_to_complex<<<nblk(N, 256), 256, 0, s>>>(rho, buf, N); launched();
+  launch(nblk(N, 256), 256, 0, s)(k_rho_to_complex, rho, buf, N); launched();
   return cudaGetLastError();
 }
 
 cudaError_t assemble_vloc(const double2* vh_c, const ConvSink& sink, long N, cudaStream_t s) {
-  k_vloc<<<nblk(N, 256), 256, 0, s>>>(vh_c, sink, N); launched();
+  launch(nblk(N, 256), 256, 0, s)(k_vloc, vh_c, sink, N); launched();
   return cudaGetLastError();
 }
 
 // Gaussian wells summed over atoms and periodic images in real space.
 __global__ void k_vion(double* __restrict__ v, int n0, int n1, int n2, double a0, double a1, double a2,
                        const double* __restrict__ atoms, int na, double depth, double sigma, double rcut) {
+  grid_entry();
   const long N = (long)n0 * n1 * n2;
   const double inv2s2 = 1.0 / (2.0 * sigma * sigma);
   const int m0 = (int)ceil(rcut / a0), m1 = (int)ceil(rcut / a1), m2 = (int)ceil(rcut / a2);
@@ -159,7 +165,7 @@ cudaError_t ion_potential(double* v, Grid3 g, const double* cell, const double* 
                           double sigma, cudaStream_t s) {
   // exp(-d^2 / (2 sigma^2)) < 1e-20 beyond rcut
   const double rcut = sigma * std::sqrt(2.0 * 46.0);
-  k_vion<<<nblk(g.N(), 128, 152L * 64), 128, 0, s>>>(v, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2], d_atoms, na,
+  launch(nblk(g.N(), 128, 152L * 64), 128, 0, s)(k_vion, v, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2], d_atoms, na,
                                                      depth, sigma, rcut); launched();
   return cudaGetLastError();
 }
@@ -168,6 +174,7 @@ cudaError_t ion_potential(double* v, Grid3 g, const double* cell, const double* 
 // psi_half = psi - i dt/2 R
 __global__ void k_half_step(const double2* __restrict__ psi, const double2* __restrict__ R, double hdt,
                             double2* __restrict__ out, long n) {
+  grid_entry();
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
     const double2 p = psi[t], r = R[t];
     // -i hdt (rx + i ry) = hdt ry - i hdt rx
@@ -176,13 +183,14 @@ __global__ void k_half_step(const double2* __restrict__ psi, const double2* __re
 }
 
 cudaError_t half_step(const double2* psi, const double2* R, double hdt, double2* out, long n, cudaStream_t s) {
-  k_half_step<<<nblk(n, 256), 256, 0, s>>>(psi, R, hdt, out, n); launched();
+  launch(nblk(n, 256), 256, 0, s)(k_half_step, psi, R, hdt, out, n); launched();
   return cudaGetLastError();
 }
 
 // y = x - tau * P * R, P = 1 / (1 + kin) per basis vector (start-state relaxation)
 __global__ void k_precond_step(double2* __restrict__ x, const double2* __restrict__ R, const double* __restrict__ kin,
                                int npw, long n, double tau) {
+  grid_entry();
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
     const double p = tau / (1.0 + kin[t % npw]);
     const double2 r = R[t];
@@ -194,7 +202,7 @@ __global__ void k_precond_step(double2* __restrict__ x, const double2* __restric
 }
 
 cudaError_t precond_step(double2* x, const double2* R, const double* kin, int npw, long n, double tau, cudaStream_t s) {
-  k_precond_step<<<nblk(n, 256), 256, 0, s>>>(x, R, kin, npw, n, tau); launched();
+  launch(nblk(n, 256), 256, 0, s)(k_precond_step, x, R, kin, npw, n, tau); launched();
   return cudaGetLastError();
 }
 
@@ -211,6 +219,7 @@ __global__ void __launch_bounds__(256) k_resid_push(const double2* __restrict__ 
                                                     const double2* __restrict__ xp, double2* __restrict__ r,
                                                     H* __restrict__ dx, H* __restrict__ dr, long n, int have_prev,
                                                     double* __restrict__ part) {
+  grid_entry();
   using A = decltype(H::x);
   double acc[1] = {0.0};
 #pragma unroll 2
@@ -236,9 +245,9 @@ cudaError_t residual_push(const double2* x, const double2* T, const double2* ph,
                           cudaStream_t s) {
   const unsigned b = resid_blocks(n);
   if (f32)
-    k_resid_push<float2><<<b, 256, 0, s>>>(x, T, ph, hdt, xp, r, (float2*)dx, (float2*)dr, n, have_prev, part);
+    launch(b, 256, 0, s)(k_resid_push<float2>, x, T, ph, hdt, xp, r, (float2*)dx, (float2*)dr, n, have_prev, part);
   else
-    k_resid_push<double2><<<b, 256, 0, s>>>(x, T, ph, hdt, xp, r, (double2*)dx, (double2*)dr, n, have_prev, part);
+    launch(b, 256, 0, s)(k_resid_push<double2>, x, T, ph, hdt, xp, r, (double2*)dx, (double2*)dr, n, have_prev, part);
   launched();
   return cudaGetLastError();
 }
@@ -261,6 +270,7 @@ constexpr int kDotChunks = 8;
 template <typename H>
 __global__ void k_anderson_dots(const H* __restrict__ dR, long slot_stride, SlotList sl, int newslot,
                                 const double2* __restrict__ r, int npw, double4_16a* __restrict__ part) {
+  grid_entry();
   using A = decltype(H::x);
   const int b = blockIdx.y, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int len = (npw + kDotChunks - 1) / kDotChunks;
@@ -299,6 +309,7 @@ constexpr int kSolveThreads = 128;
 __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_16a* __restrict__ part, SlotList sl,
                                                                   int newslot, int mdim, double2* __restrict__ gram,
                                                                   double2* __restrict__ gamma) {
+  grid_entry();
   __shared__ double2 L[kSlotMax + 1][kSlotMax + 1];
   __shared__ double inv[kSlotMax];   // 1 / L[j][j]
   // entries (i, p), p <= i <= k, p < k, by falling p: those a column j still changes (p > j)
@@ -393,12 +404,12 @@ cudaError_t anderson_gamma(const void* dR, long slot_stride, const SlotList& sl,
   if (ne > 65535) return cudaErrorInvalidValue;
   const dim3 grid(kDotChunks, (unsigned)ne);
   if (f32)
-    k_anderson_dots<float2><<<grid, 32 * sl.k, 0, s>>>((const float2*)dR, slot_stride, sl, newslot, r, npw,
+    launch(grid, 32 * sl.k, 0, s)(k_anderson_dots<float2>, (const float2*)dR, slot_stride, sl, newslot, r, npw,
                                                        (double4_16a*)part);
   else
-    k_anderson_dots<double2><<<grid, 32 * sl.k, 0, s>>>((const double2*)dR, slot_stride, sl, newslot, r, npw,
+    launch(grid, 32 * sl.k, 0, s)(k_anderson_dots<double2>, (const double2*)dR, slot_stride, sl, newslot, r, npw,
                                                         (double4_16a*)part);
-  k_anderson_solve<<<ne, kSolveThreads, 0, s>>>((const double4_16a*)part, sl, newslot, mdim, gram, gamma);
+  launch(ne, kSolveThreads, 0, s)(k_anderson_solve, (const double4_16a*)part, sl, newslot, mdim, gram, gamma);
   launched(2);
   return cudaGetLastError();
 }
@@ -412,6 +423,7 @@ __global__ void __launch_bounds__(256) k_anderson_update(const double2* __restri
                                                          long slot_stride, SlotList sl,
                                                          const double2* __restrict__ gamma, int mdim, int npw,
                                                          double beta, double2* __restrict__ out) {
+  grid_entry();
   using A = decltype(H::x);
   const int k = sl.k;
   const int b = blockIdx.y;
@@ -449,10 +461,10 @@ cudaError_t anderson_update(const double2* x, const double2* r, const void* dX, 
   if (ne == 0) return cudaSuccess;
   const dim3 grid((unsigned)std::min(32, (npw + 255) / 256), (unsigned)ne);
   if (f32)
-    k_anderson_update<float2><<<grid, 256, 0, s>>>(x, r, (const float2*)dX, (const float2*)dR, slot_stride, sl, gamma,
+    launch(grid, 256, 0, s)(k_anderson_update<float2>, x, r, (const float2*)dX, (const float2*)dR, slot_stride, sl, gamma,
                                                    mdim, npw, beta, out);
   else
-    k_anderson_update<double2><<<grid, 256, 0, s>>>(x, r, (const double2*)dX, (const double2*)dR, slot_stride, sl,
+    launch(grid, 256, 0, s)(k_anderson_update<double2>, x, r, (const double2*)dX, (const double2*)dR, slot_stride, sl,
                                                     gamma, mdim, npw, beta, out);
   launched();
   return cudaGetLastError();
@@ -461,6 +473,7 @@ cudaError_t anderson_update(const double2* x, const double2* r, const void* dX, 
 // kin[k] = |gk[k] + a|^2 / 2 with gk the basis vectors G + kick (three arrays of npw)
 __global__ void k_kinetic_shifted(const double* __restrict__ gk3, int npw, double ax, double ay, double az,
                                   double* __restrict__ kin) {
+  grid_entry();
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < npw; k += gridDim.x * blockDim.x) {
     const double x = gk3[k] + ax, y = gk3[npw + k] + ay, z = gk3[2 * (long)npw + k] + az;
     kin[k] = 0.5 * (x * x + y * y + z * z);
@@ -468,12 +481,13 @@ __global__ void k_kinetic_shifted(const double* __restrict__ gk3, int npw, doubl
 }
 
 cudaError_t kinetic_shifted(const double* gk3, int npw, double ax, double ay, double az, double* kin, cudaStream_t s) {
-  k_kinetic_shifted<<<nblk(npw, 256), 256, 0, s>>>(gk3, npw, ax, ay, az, kin); launched();
+  launch(nblk(npw, 256), 256, 0, s)(k_kinetic_shifted, gk3, npw, ax, ay, az, kin); launched();
   return cudaGetLastError();
 }
 
 // ---- density change, energy, dipole ---------------------------------------------------
 __global__ void k_drho(const double* __restrict__ a, const double* __restrict__ b, long N, double* __restrict__ part) {
+  grid_entry();
   double acc[1] = {0.0};
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < N; t += (long)gridDim.x * blockDim.x)
     acc[0] += fabs(a[t] - b[t]);
@@ -482,7 +496,7 @@ __global__ void k_drho(const double* __restrict__ a, const double* __restrict__ 
 
 cudaError_t rho_change(const double* a, const double* b, long N, double* part, double* out, cudaStream_t s) {
   const unsigned nb = nblk(N, 256, 1024);
-  k_drho<<<nb, 256, 0, s>>>(a, b, N, part); launched();
+  launch(nb, 256, 0, s)(k_drho, a, b, N, part); launched();
   finalize(part, nb, 1, out, s);
   return cudaGetLastError();
 }
@@ -491,6 +505,7 @@ cudaError_t rho_change(const double* a, const double* b, long N, double* part, d
 __global__ void k_grid_sums(const double* __restrict__ rho, const double* __restrict__ vion,
                             const double* __restrict__ vh, int use_h, int n0, int n1, int n2, double a0, double a1,
                             double a2, double* __restrict__ part) {
+  grid_entry();
   const long N = (long)n0 * n1 * n2;
   double acc[6] = {0, 0, 0, 0, 0, 0};
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < N; t += (long)gridDim.x * blockDim.x) {
@@ -511,6 +526,7 @@ __global__ void k_grid_sums(const double* __restrict__ rho, const double* __rest
 // [0] sum kin |c|^2
 __global__ void k_kin_sum(const double2* __restrict__ c, const double* __restrict__ kin, int npw, long n,
                           double* __restrict__ part) {
+  grid_entry();
   double acc[1] = {0.0};
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
     const double2 v = c[t];
@@ -520,6 +536,7 @@ __global__ void k_kin_sum(const double2* __restrict__ c, const double* __restric
 }
 
 __global__ void k_trace_real(const double2* __restrict__ M, int n, double* __restrict__ out) {
+  grid_entry();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     double t = 0.0;
     for (int i = 0; i < n; ++i) t += M[i + (long)i * n].x;
@@ -531,17 +548,18 @@ cudaError_t energy_sums(const double* rho, const double* vion, const double* vh,
                         const double2* c, const double* kin, int npw, int ne, const double2* negM, double* part,
                         double* out8, cudaStream_t s) {
   const unsigned nb = nblk(g.N(), 256, 1024);
-  k_grid_sums<<<nb, 256, 0, s>>>(rho, vion, vh, use_h, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2], part); launched();
+  launch(nb, 256, 0, s)(k_grid_sums, rho, vion, vh, use_h, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2], part); launched();
   finalize(part, nb, 6, out8, s);
   const long n = (long)npw * ne;
   const unsigned nb2 = nblk(n, 256, 1024);
-  k_kin_sum<<<nb2, 256, 0, s>>>(c, kin, npw, n, part + 6 * 1024); launched();
+  launch(nb2, 256, 0, s)(k_kin_sum, c, kin, npw, n, part + 6 * 1024); launched();
   finalize(part + 6 * 1024, nb2, 1, out8 + 6, s);
-  if (negM != nullptr) { k_trace_real<<<1, 32, 0, s>>>(negM, ne, out8 + 7); launched(); }
+  if (negM != nullptr) { launch(1, 32, 0, s)(k_trace_real, negM, ne, out8 + 7); launched(); }
   return cudaGetLastError();
 }
 
 __global__ void k_hartree_factor(double* __restrict__ f, int n0, int n1, int n2, double a0, double a1, double a2) {
+  grid_entry();
   const long N = (long)n0 * n1 * n2;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < N; t += (long)gridDim.x * blockDim.x) {
     const int i2 = (int)(t % n2);
@@ -557,7 +575,7 @@ __global__ void k_hartree_factor(double* __restrict__ f, int n0, int n1, int n2,
 }
 
 cudaError_t hartree_factor(double* f, Grid3 g, const double* cell, cudaStream_t s) {
-  k_hartree_factor<<<nblk(g.N(), 256), 256, 0, s>>>(f, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2]); launched();
+  launch(nblk(g.N(), 256), 256, 0, s)(k_hartree_factor, f, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2]); launched();
   return cudaGetLastError();
 }
 
@@ -566,6 +584,7 @@ cudaError_t hartree_factor(double* f, Grid3 g, const double* cell, cudaStream_t 
 namespace pt {
 
 __global__ void k_axpy(double2 a, const double2* __restrict__ x, double2* __restrict__ y, long n) {
+  grid_entry();
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
     const double2 v = x[t];
     double2 w = y[t];
@@ -576,7 +595,7 @@ __global__ void k_axpy(double2 a, const double2* __restrict__ x, double2* __rest
 }
 
 cudaError_t axpy(double2 a, const double2* x, double2* y, long n, cudaStream_t s) {
-  k_axpy<<<nblk(n, 256), 256, 0, s>>>(a, x, y, n); launched();
+  launch(nblk(n, 256), 256, 0, s)(k_axpy, a, x, y, n); launched();
   return cudaGetLastError();
 }
 
@@ -586,28 +605,31 @@ namespace pt {
 
 __global__ void k_diff_to_complex(const double* __restrict__ a, const double* __restrict__ b, double2* __restrict__ buf,
                                   long N) {
+  grid_entry();
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < N; t += (long)gridDim.x * blockDim.x)
     buf[t] = make_double2(a[t] - b[t], 0.0);
 }
 
 __global__ void k_add_real(const double2* __restrict__ buf, double* __restrict__ a, long N) {
+  grid_entry();
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < N; t += (long)gridDim.x * blockDim.x)
     a[t] += buf[t].x;
 }
 
 cudaError_t diff_to_complex(const double* a, const double* b, double2* buf, long N, cudaStream_t s) {
-  k_diff_to_complex<<<nblk(N, 256), 256, 0, s>>>(a, b, buf, N); launched();
+  launch(nblk(N, 256), 256, 0, s)(k_diff_to_complex, a, b, buf, N); launched();
   return cudaGetLastError();
 }
 
 cudaError_t add_real(const double2* buf, double* a, long N, cudaStream_t s) {
-  k_add_real<<<nblk(N, 256), 256, 0, s>>>(buf, a, N); launched();
+  launch(nblk(N, 256), 256, 0, s)(k_add_real, buf, a, N); launched();
   return cudaGetLastError();
 }
 
 // b |G|^2 / (|G|^2 + q0^2) / N  (Kerker weight with the inverse-FFT normalisation)
 __global__ void k_kerker_factor(double* __restrict__ f, int n0, int n1, int n2, double a0, double a1, double a2,
                                 double b, double q2) {
+  grid_entry();
   const long N = (long)n0 * n1 * n2;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < N; t += (long)gridDim.x * blockDim.x) {
     const int i2 = (int)(t % n2);
@@ -623,7 +645,7 @@ __global__ void k_kerker_factor(double* __restrict__ f, int n0, int n1, int n2, 
 }
 
 cudaError_t kerker_factor(double* f, Grid3 g, const double* cell, double b, double q0, cudaStream_t s) {
-  k_kerker_factor<<<nblk(g.N(), 256), 256, 0, s>>>(f, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2], b, q0 * q0);
+  launch(nblk(g.N(), 256), 256, 0, s)(k_kerker_factor, f, g.n0, g.n1, g.n2, cell[0], cell[1], cell[2], b, q0 * q0);
   launched();
   return cudaGetLastError();
 }

@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, in
                                              double2 alpha, const TI* __restrict__ A, long lda,
                                              const TI* __restrict__ B, long ldb, double2 beta,
                                              double2* __restrict__ Cm, long ldc, double2* __restrict__ part) {
+  grid_entry();
   constexpr int P = GT * GK / 64;   // operand elements per thread per slice
   __shared__ C As[2][GK][GT + 1];
   __shared__ C Bs[2][GK][GT + 1];
@@ -164,6 +165,7 @@ __global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, in
 template <int G>
 __global__ void k_splitk_reduce(int M, int N, int ksplit, int structure, double2 alpha, const double2* __restrict__ part,
                                 double2 beta, double2* __restrict__ Cm, long ldc) {
+  grid_entry();
   constexpr int E = 32 / G;   // entries per warp
   const long total = (long)M * N;
   const int lane = threadIdx.x & 31, g = lane / E;
@@ -211,8 +213,8 @@ static cudaError_t reduce_partials(int M, int N, int ksplit, int structure, doub
   // eight threads per entry while one per entry would leave the chip mostly idle
   const int G = ksplit >= 8 && total < 65536 ? 8 : 1;
   const int blocks = (int)std::min<long>((total * G + 255) / 256, 152L * 16);
-  if (G == 8) k_splitk_reduce<8><<<blocks, 256, 0, s>>>(M, N, ksplit, structure, alpha, part, beta, C, ldc);
-  else k_splitk_reduce<1><<<blocks, 256, 0, s>>>(M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  if (G == 8) launch(blocks, 256, 0, s)(k_splitk_reduce<8>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  else launch(blocks, 256, 0, s)(k_splitk_reduce<1>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
   launched();
   return cudaGetLastError();
 }
@@ -260,7 +262,7 @@ static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alph
   const int kchunk = std::max(1, (K + ksplit - 1) / ksplit);
   const dim3 grid(tm, tn, (unsigned)ksplit);
 #define PT_GEMM(OA, OB) \
-  k_gemm<C, TI, OA, OB><<<grid, 64, 0, s>>>(M, N, K, kchunk, ksplit, structure, alpha, A, lda, B, ldb, beta, Cm, ldc, ws)
+  launch(grid, 64, 0, s)(k_gemm<C, TI, OA, OB>, M, N, K, kchunk, ksplit, structure, alpha, A, lda, B, ldb, beta, Cm, ldc, ws)
   if (opA == OP_N && opB == OP_N) PT_GEMM(OP_N, OP_N);
   else if (opA == OP_N) PT_GEMM(OP_N, OP_H);
   else if (opB == OP_N) PT_GEMM(OP_H, OP_N);
@@ -307,6 +309,7 @@ constexpr int CB = 32;
 // inverse into the same block of Linv.
 __global__ void __launch_bounds__(256) k_chol_diag(double2* __restrict__ A, double2* __restrict__ Linv, int n, int j0,
                                                    int* __restrict__ status) {
+  grid_entry();
   __shared__ double2 a[CB][CB + 1], x[CB][CB + 1];
   __shared__ double rinv[CB];
   __shared__ int bad;
@@ -378,6 +381,7 @@ __global__ void __launch_bounds__(256) k_chol_diag(double2* __restrict__ A, doub
 // of the columns j0.. above the diagonal (rows of A12) is zeroed.
 __global__ void __launch_bounds__(256) k_chol_panel(double2* __restrict__ A, const double2* __restrict__ Linv, int n,
                                                     int j0, const int* __restrict__ status) {
+  grid_entry();
   __shared__ double2 a[8][CB + 1], x[CB][CB + 1];
   if (*status != 0) return;
   const int tid = threadIdx.x, i0 = j0 + CB + 8 * blockIdx.x;
@@ -401,6 +405,7 @@ __global__ void __launch_bounds__(256) k_chol_panel(double2* __restrict__ A, con
 // A22 -= L21 L21^H on and below the diagonal, one 16 x 16 tile per block
 __global__ void __launch_bounds__(256) k_chol_trail(double2* __restrict__ A, int n, int j0,
                                                     const int* __restrict__ status) {
+  grid_entry();
   __shared__ double2 u[CB][17], w[CB][17];
   if (blockIdx.x < blockIdx.y || *status != 0) return;
   const int tid = threadIdx.x, base = j0 + CB;
@@ -430,19 +435,20 @@ cudaError_t cholesky_inverse(double2* A, double2* Linv, int n, int* d_status, cu
   cudaError_t e = cudaMemsetAsync(d_status, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   for (int j0 = 0; j0 < n; j0 += CB) {
-    k_chol_diag<<<1, 256, 0, s>>>(A, Linv, n, j0, d_status); launched();
+    launch(1, 256, 0, s)(k_chol_diag, A, Linv, n, j0, d_status); launched();
     const int rest = n - j0 - CB;
     if (rest <= 0) continue;
-    k_chol_panel<<<(rest + 7) / 8, 256, 0, s>>>(A, Linv, n, j0, d_status); launched();
+    launch((rest + 7) / 8, 256, 0, s)(k_chol_panel, A, Linv, n, j0, d_status); launched();
     const unsigned t = (unsigned)((rest + 15) / 16);
-    k_chol_trail<<<dim3(t, t), 256, 0, s>>>(A, n, j0, d_status); launched();
+    launch(dim3(t, t), 256, 0, s)(k_chol_trail, A, n, j0, d_status); launched();
   }
-  if (n > CB) { k_tri_inverse<<<n, 128, sizeof(double2) * n, s>>>(A, Linv, n); launched(); }
+  if (n > CB) { launch(n, 128, sizeof(double2) * n, s)(k_tri_inverse, A, Linv, n); launched(); }
   return cudaGetLastError();
 }
 
 // Column c of L^{-1}: solve L x = e_c by forward substitution (one block per column).
 __global__ void k_tri_inverse(const double2* __restrict__ L, double2* __restrict__ Li, int n) {
+  grid_entry();
   extern __shared__ double2 b[];
   const int c = blockIdx.x;
   for (int i = threadIdx.x; i < n; i += blockDim.x) b[i] = make_double2(i == c ? 1.0 : 0.0, 0.0);
