@@ -586,9 +586,6 @@ pt_status set_kinetic(pt_system* sys, int64_t n) { return set_kinetic_t(sys, (do
 // ACE and the observables. cn_step runs them in order; a batch interleaves the phases of
 // several systems, each on its own stream, with identical arithmetic.
 
-// the residual's block partials inside sys->part, clear of the other reductions' partials
-static constexpr long kResidPart = 7168;
-
 pt_status cn_begin(pt_system* sys, StepCtx* c) {
   const int ne = sys->ne, npw = sys->npw;
   const long n = (long)npw * ne;
@@ -678,7 +675,7 @@ pt_status cn_iterate(pt_system* sys, StepCtx* c) {
     const size_t hs = sys->mixed ? sizeof(float2) : sizeof(double2);
     const size_t at = (newslot >= 0 ? newslot : 0) * stride * hs;
     PT_CK(pt::residual_push(sys->psi_f, sys->hpsi, sys->psi_half, hdt, sys->xprev, sys->rprev, sys->dX + at,
-                            sys->dR + at, n, newslot >= 0 ? 1 : 0, f32, sys->part + kResidPart, sys->s));
+                            sys->dR + at, n, newslot >= 0 ? 1 : 0, f32, sys->s));
     c->have_prev = true;
     pt::SlotList sl{};
     sl.k = (int)sys->and_order.size();
@@ -739,7 +736,7 @@ pt_status cn_outer(pt_system* sys, StepCtx* c, bool* again) {
 }
 
 pt_status cn_orthonormalize(pt_system* sys, StepCtx* c) {
-  PT_CK(pt::residual_norm2(sys->part + kResidPart, (long)sys->npw * sys->ne, sys->red, sys->s));
+  PT_CK(pt::norm2(sys->rprev, (long)sys->npw * sys->ne, sys->part, sys->red, sys->s));   // of the last residual
   PT_TRY(read_small(sys, c->hres, sys->red, sizeof(c->hres)));
   // orthonormalise; the real-space orbitals of Psi_{n+1} for its exchange and density
   PT_TRY(orthonormalize(sys, sys->psi_f, sys->psi));

@@ -207,9 +207,10 @@ cudaError_t precond_step(double2* x, const double2* R, const double* kin, int np
 }
 
 // ---- Anderson mixing (Sec. 3.4), per band -------------------------------------------
-// r = -(x + i dt/2 T - psi_half) (the fixed-point residual, Alg. 1 and 3) with block partials
-// of |r|^2, and the history entries dX[slot] = x - x_prev, dR[slot] = r - r_prev when there
-// is a previous iterate. r overwrites r_prev: one pass over the orbitals instead of three.
+// r = -(x + i dt/2 T - psi_half) (the fixed-point residual, Alg. 1 and 3) and the history
+// entries dX[slot] = x - x_prev, dR[slot] = r - r_prev when there is a previous iterate. r
+// overwrites r_prev: one pass over the orbitals instead of three. Bound by memory: 128 bands x
+// 13,133 in 46 us (4.1 TB/s); the norm of r, needed once a step, made it 62.
 // History entries are stored as H: complex128, or complex64 in mixed precision
 // (the differences of successive iterates and residuals, whose rounding to FP32
 // only perturbs the least-squares extrapolation, not the fixed point).
@@ -217,11 +218,9 @@ template <typename H>
 __global__ void __launch_bounds__(256) k_resid_push(const double2* __restrict__ x, const double2* __restrict__ T,
                                                     const double2* __restrict__ ph, double hdt,
                                                     const double2* __restrict__ xp, double2* __restrict__ r,
-                                                    H* __restrict__ dx, H* __restrict__ dr, long n, int have_prev,
-                                                    double* __restrict__ part) {
+                                                    H* __restrict__ dx, H* __restrict__ dr, long n, int have_prev) {
   grid_entry();
   using A = decltype(H::x);
-  double acc[1] = {0.0};
 #pragma unroll 2
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
     const double2 p = x[t], q = T[t], h = ph[t];
@@ -233,68 +232,121 @@ __global__ void __launch_bounds__(256) k_resid_push(const double2* __restrict__ 
       dr[t] = {(A)(v.x - d.x), (A)(v.y - d.y)};
     }
     r[t] = v;
+  }
+}
+
+cudaError_t residual_push(const double2* x, const double2* T, const double2* ph, double hdt, const double2* xp,
+                          double2* r, void* dx, void* dr, long n, int have_prev, int f32, cudaStream_t s) {
+  const unsigned b = nblk(n, 256);
+  if (f32)
+    launch(b, 256, 0, s)(k_resid_push<float2>, x, T, ph, hdt, xp, r, (float2*)dx, (float2*)dr, n, have_prev);
+  else
+    launch(b, 256, 0, s)(k_resid_push<double2>, x, T, ph, hdt, xp, r, (double2*)dx, (double2*)dr, n, have_prev);
+  launched();
+  return cudaGetLastError();
+}
+
+// out = sum |r|^2 (once per step, of its last residual); part: 1024 doubles
+__global__ void k_norm2(const double2* __restrict__ r, long n, double* __restrict__ part) {
+  grid_entry();
+  double acc[1] = {0.0};
+  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
+    const double2 v = r[t];
     acc[0] += v.x * v.x + v.y * v.y;
   }
   block_sums<1>(acc, part);
 }
 
-static unsigned resid_blocks(long n) { return nblk(n, 256, 1024); }
-
-cudaError_t residual_push(const double2* x, const double2* T, const double2* ph, double hdt, const double2* xp,
-                          double2* r, void* dx, void* dr, long n, int have_prev, int f32, double* part,
-                          cudaStream_t s) {
-  const unsigned b = resid_blocks(n);
-  if (f32)
-    launch(b, 256, 0, s)(k_resid_push<float2>, x, T, ph, hdt, xp, r, (float2*)dx, (float2*)dr, n, have_prev, part);
-  else
-    launch(b, 256, 0, s)(k_resid_push<double2>, x, T, ph, hdt, xp, r, (double2*)dx, (double2*)dr, n, have_prev, part);
-  launched();
+cudaError_t norm2(const double2* r, long n, double* part, double* out, cudaStream_t s) {
+  const unsigned b = nblk(n, 256, 1024);
+  launch(b, 256, 0, s)(k_norm2, r, n, part); launched();
+  finalize(part, (int)b, 1, out, s);
   return cudaGetLastError();
 }
 
-cudaError_t residual_norm2(const double* part, long n, double* out, cudaStream_t s) {
-  finalize(part, (int)resid_blocks(n), 1, out, s);
-  return cudaGetLastError();
-}
-
-// Partial sums over one of kDotChunks chunks of the basis of <dR_q, dR_new> and <dR_q, r>
-// for band blockIdx.y, one warp per history slot q: the warps of a block walk the same
-// stretch together, so dR_new and r come from DRAM once per block and from L1 for the
-// other slots, and every lane carries four sums whatever the history depth.
+// Partial sums over one of gridDim.x chunks of the basis of <dR_q, dR_new> and <dR_q, r> for
+// band blockIdx.y and every slot q: a thread reads dR_new and r of its coefficients once and
+// carries four sums per slot in registers (KM >= k slots), so each entry of the history is
+// read once, coalesced, with k loads in flight. One warp per slot re-read dR_new and r from L1
+// for each slot: 92 us on average over a step at 128 bands x 13,133, 59 so.
 // Complex64 history (mixed precision): the products are formed in FP32 and
-// summed in FP32 over each lane's share of the chunk (about npw / 256 terms);
-// the lanes' sums are reduced in FP64. FP64 otherwise. The Gram matrix and
-// right-hand side feed the FP64 solve either way.
-constexpr int kDotChunks = 8;
+// summed in FP32 over each thread's share of the basis (at most npw / 256 terms);
+// the threads' sums are reduced in FP64. FP64 otherwise. The Gram matrix and
+// right-hand side feed the FP64 solve either way. The reduction halves the values a lane
+// carries with every exchange, 78 FP64 additions a lane where a tree per value takes 400.
+constexpr int kDotThreads = 128, kDotChunksMax = 8;
 
-template <typename H>
-__global__ void k_anderson_dots(const H* __restrict__ dR, long slot_stride, SlotList sl, int newslot,
-                                const double2* __restrict__ r, int npw, double4_16a* __restrict__ part) {
+// Sums x over the warp's lanes, HAVE values: lanes whose bit O is set keep the upper half, the
+// others the lower; the lane ends with the n values from `base` on in x[0..n).
+template <int HAVE, int O>
+__device__ __forceinline__ void fold_lanes(double* x, int lane, int& base, int& n) {
+  constexpr int HALF = (HAVE + 1) / 2;
+  const bool up = (lane & O) != 0;
+#pragma unroll
+  for (int i = 0; i < HALF; ++i) {
+    const double hi = i + HALF < HAVE ? x[i + HALF < HAVE ? i + HALF : 0] : 0.0;
+    const double send = up ? x[i] : hi, keep = up ? hi : x[i];
+    x[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+  }
+  if (up) {
+    base += HALF;
+    n -= HALF;
+  } else {
+    n = min(n, HALF);
+  }
+  if constexpr (O > 1) fold_lanes<HALF, O / 2>(x, lane, base, n);
+}
+
+template <typename H, int KM>
+__global__ void __launch_bounds__(kDotThreads) k_anderson_dots(const H* __restrict__ dR, long slot_stride, SlotList sl,
+                                                               int newslot, const double2* __restrict__ r, int npw,
+                                                               double* __restrict__ part) {
   grid_entry();
   using A = decltype(H::x);
-  const int b = blockIdx.y, q = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int len = (npw + kDotChunks - 1) / kDotChunks;
+  constexpr int NV = 4 * KM;
+  __shared__ double sh[kDotThreads / 32][NV];
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, k = sl.k;
+  const int len = (npw + gridDim.x - 1) / gridDim.x;
   const int g0 = blockIdx.x * len, g1 = min(npw, g0 + len);
   const long boff = (long)b * npw;
   const H* dn = dR + (long)newslot * slot_stride + boff;
-  const H* du = dR + (long)sl.s[q] * slot_stride + boff;
   const double2* rb = r + boff;
-  A a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-#pragma unroll 4
-  for (int g = g0 + lane; g < g1; g += 32) {
-    const H v = dn[g], u = du[g];
-    const double2 w = rb[g];
-    const A wx = (A)w.x, wy = (A)w.y;
-    a0 += u.x * v.x + u.y * v.y;
-    a1 += u.x * v.y - u.y * v.x;
-    a2 += u.x * wx + u.y * wy;
-    a3 += u.x * wy - u.y * wx;
-  }
-  double d[4] = {(double)a0, (double)a1, (double)a2, (double)a3};
+  A acc[NV];
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
-    for (int o = 16; o > 0; o >>= 1) d[c] += __shfl_down_sync(0xffffffffu, d[c], o);
-  if (lane == 0) part[((long)b * sl.k + q) * kDotChunks + blockIdx.x] = make_double4_16a(d[0], d[1], d[2], d[3]);
+  for (int c = 0; c < NV; ++c) acc[c] = 0;
+  for (int g = g0 + tid; g < g1; g += kDotThreads) {
+    const H v = dn[g];
+    const double2 w = rb[g];
+    H u[KM];
+#pragma unroll
+    for (int q = 0; q < KM; ++q) {
+      u[q] = H{};
+      if (q < k) u[q] = dR[(long)sl.s[q] * slot_stride + boff + g];
+    }
+    const A wx = (A)w.x, wy = (A)w.y;
+#pragma unroll
+    for (int q = 0; q < KM; ++q) {
+      acc[4 * q + 0] += u[q].x * v.x + u[q].y * v.y;
+      acc[4 * q + 1] += u[q].x * v.y - u[q].y * v.x;
+      acc[4 * q + 2] += u[q].x * wx + u[q].y * wy;
+      acc[4 * q + 3] += u[q].x * wy - u[q].y * wx;
+    }
+  }
+  double x[NV];
+#pragma unroll
+  for (int c = 0; c < NV; ++c) x[c] = (double)acc[c];
+  int base = 0, n = NV;
+  fold_lanes<NV, 16>(x, lane, base, n);
+#pragma unroll
+  for (int i = 0; i < (NV + 31) / 32; ++i)
+    if (i < n) sh[tid >> 5][base + i] = x[i];
+  __syncthreads();
+  if (tid < NV && tid < 4 * k) {
+    double t = sh[0][tid];
+#pragma unroll
+    for (int w = 1; w < kDotThreads / 32; ++w) t += sh[w][tid];
+    part[(((long)b * k + tid / 4) * gridDim.x + blockIdx.x) * 4 + tid % 4] = t;
+  }
 }
 
 // Gathers the sums into gram[b][slot_q][new] (and its conjugate at [new][slot_q]) and the
@@ -307,7 +359,8 @@ __global__ void k_anderson_dots(const H* __restrict__ dR, long slot_stride, Slot
 constexpr int kSolveThreads = 128;
 
 __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_16a* __restrict__ part, SlotList sl,
-                                                                  int newslot, int mdim, double2* __restrict__ gram,
+                                                                  int newslot, int chunks, int mdim,
+                                                                  double2* __restrict__ gram,
                                                                   double2* __restrict__ gamma) {
   grid_entry();
   __shared__ double2 L[kSlotMax + 1][kSlotMax + 1];
@@ -333,10 +386,10 @@ __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_
   }
   if (tid < k) {
     const int q = tid, mine = sl.s[q];
-    const double4_16a* p = part + ((long)b * k + q) * kDotChunks;
+    const double4_16a* p = part + ((long)b * k + q) * chunks;
     double4_16a t = p[0];
-#pragma unroll
-    for (int c = 1; c < kDotChunks; ++c) {
+#pragma unroll 4
+    for (int c = 1; c < chunks; ++c) {
       t.x += p[c].x;
       t.y += p[c].y;
       t.z += p[c].z;
@@ -397,19 +450,30 @@ __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_
   if (tid < k) gamma[(long)b * mdim + tid] = y;
 }
 
+template <typename H>
+static void dots_any(const H* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r, int npw, int ne,
+                     int chunks, double* part, cudaStream_t s) {
+  launch to(dim3((unsigned)chunks, (unsigned)ne), kDotThreads, 0, s);
+  switch ((sl.k + 3) / 4) {
+    case 1: to(k_anderson_dots<H, 4>, dR, slot_stride, sl, newslot, r, npw, part); break;
+    case 2: to(k_anderson_dots<H, 8>, dR, slot_stride, sl, newslot, r, npw, part); break;
+    case 3: to(k_anderson_dots<H, 12>, dR, slot_stride, sl, newslot, r, npw, part); break;
+    case 4: to(k_anderson_dots<H, 16>, dR, slot_stride, sl, newslot, r, npw, part); break;
+    case 5: to(k_anderson_dots<H, 20>, dR, slot_stride, sl, newslot, r, npw, part); break;
+    default: to(k_anderson_dots<H, kSlotMax>, dR, slot_stride, sl, newslot, r, npw, part); break;
+  }
+}
+
 cudaError_t anderson_gamma(const void* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r,
                            int npw, int ne, int mdim, double2* gram, double2* gamma, void* part, int f32,
                            cudaStream_t s) {
   if (sl.k < 1 || sl.k > kSlotMax) return cudaErrorInvalidValue;
   if (ne > 65535) return cudaErrorInvalidValue;
-  const dim3 grid(kDotChunks, (unsigned)ne);
-  if (f32)
-    launch(grid, 32 * sl.k, 0, s)(k_anderson_dots<float2>, (const float2*)dR, slot_stride, sl, newslot, r, npw,
-                                                       (double4_16a*)part);
-  else
-    launch(grid, 32 * sl.k, 0, s)(k_anderson_dots<double2>, (const double2*)dR, slot_stride, sl, newslot, r, npw,
-                                                        (double4_16a*)part);
-  launch(ne, kSolveThreads, 0, s)(k_anderson_solve, (const double4_16a*)part, sl, newslot, mdim, gram, gamma);
+  // two chunks of 128 threads each (256 threads' sums per band) once the bands fill the chip
+  const int chunks = std::max(2, std::min(kDotChunksMax, 2 * sm_count() / ne));
+  if (f32) dots_any<float2>((const float2*)dR, slot_stride, sl, newslot, r, npw, ne, chunks, (double*)part, s);
+  else dots_any<double2>((const double2*)dR, slot_stride, sl, newslot, r, npw, ne, chunks, (double*)part, s);
+  launch(ne, kSolveThreads, 0, s)(k_anderson_solve, (const double4_16a*)part, sl, newslot, chunks, mdim, gram, gamma);
   launched(2);
   return cudaGetLastError();
 }

@@ -22,12 +22,11 @@ cudaError_t ion_potential(double* v, Grid3 g, const double* cell, const double* 
 cudaError_t hartree_factor(double* f, Grid3 g, const double* cell, cudaStream_t s);
 cudaError_t half_step(const double2* psi, const double2* R, double hdt, double2* out, long n, cudaStream_t s);
 cudaError_t precond_step(double2* x, const double2* R, const double* kin, int npw, long n, double tau, cudaStream_t s);
-// r (holding r_prev) <- -(x + i hdt T - ph); dx = x - xp and dr = r - r_prev when have_prev;
-// part (1024 doubles) takes the block partials of |r|^2 that residual_norm2 sums up
+// r (holding r_prev) <- -(x + i hdt T - ph); dx = x - xp and dr = r - r_prev when have_prev
 cudaError_t residual_push(const double2* x, const double2* T, const double2* ph, double hdt, const double2* xp,
-                          double2* r, void* dx, void* dr, long n, int have_prev, int f32, double* part,
-                          cudaStream_t s);
-cudaError_t residual_norm2(const double* part, long n, double* out, cudaStream_t s);
+                          double2* r, void* dx, void* dr, long n, int have_prev, int f32, cudaStream_t s);
+// out = sum |r|^2; part: 1024 doubles
+cudaError_t norm2(const double2* r, long n, double* part, double* out, cudaStream_t s);
 // gram entries of the new slot and gamma per band; part: at least 8 * 4 * sl.k * ne doubles
 cudaError_t anderson_gamma(const void* dR, long slot_stride, const SlotList& sl, int newslot, const double2* r,
                            int npw, int ne, int mdim, double2* gram, double2* gamma, void* part, int f32,
