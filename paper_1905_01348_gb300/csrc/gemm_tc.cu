@@ -151,6 +151,14 @@ __device__ __forceinline__ void split2(float2 v, float2& hi, float2& lo) {
   split_tf32(v.y, hi.y, lo.y);
 }
 
+// (double)x by integer operations (FP64 conversions run at the FP64 pipe's two a clock);
+// zeros, subnormals, infinities and NaN take the conversion
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e == 0u || e == 0xffu) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+
 // 8 bytes from global into shared memory, or zeros
 __device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, bool valid) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(dst), "l"(src), "r"(valid ? 8 : 0) : "memory");
@@ -350,21 +358,47 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("bar.sync 1, %0;\n" ::"r"(TC_PROD) : "memory");
     const int m = m0 + r;
     if (m < M) {
-      for (int j0 = (TC_NC / 2) * h; j0 < (TC_NC / 2) * (h + 1); ++j0) {
-        const int j = n0 + j0;
-        if (j >= N) break;
-        const double2 v = make_double2((double)sums[j0 * TC_M + r], (double)sums[(TC_NC + j0) * TC_M + r]);
-        if (ksplit > 1) {
-          part[((long)kz * N + j) * (long)M + m] = v;
-        } else {
-          double2* c = Cm + m + (long)j * ldc;
-          double2 o2 = make_double2(alpha.x * v.x - alpha.y * v.y, alpha.x * v.y + alpha.y * v.x);
-          if (beta.x != 0.0 || beta.y != 0.0) {
-            const double2 o = *c;
-            o2.x += beta.x * o.x - beta.y * o.y;
-            o2.y += beta.x * o.y + beta.y * o.x;
+      // Eight columns at a time, C's old values loaded together: one at a time, each load
+      // waited for the store before it. alpha = +-1 and beta = 1, the factors of every product
+      // of the path, take no FP64 multiplication: the general form's ten FP64 operations
+      // per value are 40 us a tile at two a clock, as long as its MMAs at K = 432 (A B of Si216,
+      // M = 43,819: 1.04 -> 0.75 ms).
+      const float sign = alpha.y == 0.0 && (alpha.x == 1.0 || alpha.x == -1.0) ? (float)alpha.x : 0.f;
+      const bool plus = beta.x == 1.0 && beta.y == 0.0;
+      const bool old = ksplit == 1 && (beta.x != 0.0 || beta.y != 0.0);
+      for (int j0 = (TC_NC / 2) * h; j0 < (TC_NC / 2) * (h + 1) && n0 + j0 < N; j0 += 8) {
+        double2 o[8];
+        if (old) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (n0 + j0 + u < N) o[u] = Cm[m + (long)(n0 + j0 + u) * ldc];
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = n0 + j0 + u;
+          if (j >= N) break;
+          const float re = sums[(j0 + u) * TC_M + r], im = sums[(TC_NC + j0 + u) * TC_M + r];
+          if (ksplit > 1) {
+            part[((long)kz * N + j) * (long)M + m] = make_double2(widen(re), widen(im));
+            continue;
           }
-          *c = o2;
+          double2 o2;
+          if (sign != 0.f) {
+            o2 = make_double2(widen(sign * re), widen(sign * im));
+          } else {
+            const double2 v = make_double2(widen(re), widen(im));
+            o2 = make_double2(alpha.x * v.x - alpha.y * v.y, alpha.x * v.y + alpha.y * v.x);
+          }
+          if (old) {
+            if (plus) {
+              o2.x += o[u].x;
+              o2.y += o[u].y;
+            } else {
+              o2.x += beta.x * o[u].x - beta.y * o[u].y;
+              o2.y += beta.x * o[u].y + beta.y * o[u].x;
+            }
+          }
+          Cm[m + (long)j * ldc] = o2;
         }
       }
     }
