@@ -83,7 +83,9 @@ pt_status merge_schedule(const std::vector<pt_system*>& sys, int tile, int tpl, 
   for (size_t i = 0; i < sys.size(); ++i) {
     pt::PairTile* t = nullptr;
     int *lf = nullptr, *lc = nullptr, nl = 0;
-    const int nt = pt::fock_build_tiles(sys[i]->ne, 0, tile, 1, INT_MAX, &t, &lf, &lc, &nl);
+    // the order of each system's own schedule, so that its sums are the same to the bit
+    const int order = pt::fock_tile_order(sys[i]->gf, sys[i]->mixed, sys[i]->ne, tile, 1, false);
+    const int nt = pt::fock_build_tiles(sys[i]->ne, 0, tile, 1, order, INT_MAX, &t, &lf, &lc, &nl);
     if (nt < 0) { *why = "tile schedule"; return PT_ERR_INVALID; }
     pt::fock_bind_tiles(t, nt, fock_orbitals_addr(sys[i]), nullptr, sys[i]->w_r, nullptr, sys[i]->Nf,
                         exchange_cs(sys[i]));

@@ -251,7 +251,7 @@ static pt_status ensure_plan_x(pt_system* sys, int ncols) {
   pt::PairTile* tiles = nullptr;
   int *lf = nullptr, *lc = nullptr, nl = 0;
   const int tile = choose_tile(&sys->p);
-  const int nt = pt::fock_build_tiles(sys->ne, ncols, tile, 0, tiles_per_launch(&sys->p, sys->Nf, sys->mixed), &tiles,
+  const int nt = pt::fock_build_tiles(sys->ne, ncols, tile, 0, pt::TILE_ROUNDS, tiles_per_launch(&sys->p, sys->Nf, sys->mixed), &tiles,
                                       &lf, &lc, &nl);
   if (nt < 0 || (size_t)nt > sys->max_tiles_x) {
     std::free(tiles); std::free(lf); std::free(lc);
@@ -271,6 +271,7 @@ static pt_status ensure_plan_x(pt_system* sys, int ncols) {
   sys->plan_x.launch_count = lc;
   sys->plan_x.d_tiles = sys->d_tiles_x;
   sys->plan_x.n_tiles = nt;
+  sys->plan_x.group = 1;
   set_pair_reach(&sys->plan_x, &sys->p);
   sys->plan_x_ncols = ncols;
   return PT_OK;

@@ -393,9 +393,16 @@ void fock_bind_tiles(PairTile* tiles, int n, const void* psi_r, const void* x_r,
 // round (off-diagonal tiles: all |A| x |B| pairs), then one round of the
 // diagonal tiles (pairs a <= b inside a block). Non-symmetric (V_X applied to
 // other vectors): round r pairs X-block b with occupied block (b + r) mod nbo.
-int fock_build_tiles(int n_occ, int n_x, int tile, int sym, int tiles_per_launch, PairTile** tiles_out,
+// Paired order: blocks go two by two, (A, A') and (B, B'), through the tournament, and each
+// meeting is the tiles A B, A' B', then A B', A' B; the diagonal ones are A A, A' A', then A A'.
+long fock_max_tiles(int n_occ, int tile) {
+  const long nb = (n_occ + tile - 1) / tile, np = (nb + 1) / 2;
+  return 2 * np * (np + 1);
+}
+
+int fock_build_tiles(int n_occ, int n_x, int tile, int sym, int order, int tiles_per_launch, PairTile** tiles_out,
                      int** launch_first, int** launch_count, int* n_launch) {
-  if (tile < 1 || tile > kTileMax || n_occ < 1 || tiles_per_launch < 1) return -1;
+  if (tile < 1 || tile > kTileMax || n_occ < 1 || tiles_per_launch < (order == TILE_GROUPED ? 4 : 1)) return -1;
   std::vector<PairTile> tiles;
   std::vector<std::vector<int>> rounds;   // tile indices per round
   auto block_range = [&](int b, int n, int* lo) { *lo = b * tile; return std::min(n, (b + 1) * tile) - b * tile; };
@@ -427,7 +434,45 @@ int fock_build_tiles(int n_occ, int n_x, int tile, int sym, int tiles_per_launch
     tiles.push_back(t);
     return (int)tiles.size() - 1;
   };
-  if (sym) {
+  if (sym && order != TILE_ROUNDS) {
+    const int nb = (n_occ + tile - 1) / tile, np = (nb + 1) / 2, npp = np + (np & 1);
+    auto pair_tile = [&](int a, int b) {
+      int alo, blo;
+      const int an = block_range(a, n_occ, &alo), bn = block_range(b, n_occ, &blo);
+      return make_tile(alo, an, 0, blo, bn, 0, a == b, 1, 1);
+    };
+    // a meeting's tiles, the first `apart` of them without a common block; the rest likewise
+    auto add = [&](std::vector<int>* first, std::vector<int>* second, const std::vector<int>& t, size_t apart) {
+      for (size_t k = 0; k < t.size(); ++k) (order == TILE_GROUPED || k < apart ? first : second)->push_back(t[k]);
+      if (order == TILE_GROUPED) first->resize((first->size() + 3) / 4 * 4, -1);
+    };
+    auto end_round = [&](std::vector<int>* rd) {
+      if (!rd->empty()) rounds.push_back(*rd);
+      rd->clear();
+    };
+    std::vector<int> one, two;
+    for (int r = 0; r < npp - 1; ++r) {
+      for (int i = 0; i < npp / 2; ++i) {
+        int a = i == 0 ? r : (r + i) % (npp - 1), b = i == 0 ? npp - 1 : (r - i + npp - 1) % (npp - 1);
+        if (a >= np || b >= np) continue;
+        if (a > b) std::swap(a, b);
+        if (2 * b + 1 < nb)
+          add(&one, &two, {pair_tile(2 * a, 2 * b), pair_tile(2 * a + 1, 2 * b + 1), pair_tile(2 * a, 2 * b + 1),
+                           pair_tile(2 * a + 1, 2 * b)}, 2);
+        else
+          add(&one, &two, {pair_tile(2 * a, 2 * b), pair_tile(2 * a + 1, 2 * b)}, 1);
+      }
+      end_round(&one);
+      end_round(&two);
+    }
+    for (int a = 0; a < np; ++a) {
+      if (2 * a + 1 < nb) add(&one, &two, {pair_tile(2 * a, 2 * a), pair_tile(2 * a + 1, 2 * a + 1), pair_tile(2 * a, 2 * a + 1)}, 2);
+      else add(&one, &two, {pair_tile(2 * a, 2 * a)}, 1);
+    }
+    end_round(&one);
+    end_round(&two);
+    if (order == TILE_GROUPED) tiles_per_launch -= tiles_per_launch % 4;
+  } else if (sym) {
     const int nb = (n_occ + tile - 1) / tile;
     const int nbp = nb + (nb & 1);
     for (int r = 0; r < nbp - 1; ++r) {
@@ -472,7 +517,7 @@ int fock_build_tiles(int n_occ, int n_x, int tile, int sym, int tiles_per_launch
       const int cnt = (int)std::min<size_t>(tiles_per_launch, rd.size() - k);
       lf.push_back((int)ordered.size());
       lc.push_back(cnt);
-      for (int q = 0; q < cnt; ++q) ordered.push_back(tiles[rd[k + q]]);
+      for (int q = 0; q < cnt; ++q) ordered.push_back(rd[k + q] < 0 ? PairTile{} : tiles[rd[k + q]]);
     }
   }
   *tiles_out = (PairTile*)std::malloc(sizeof(PairTile) * ordered.size());

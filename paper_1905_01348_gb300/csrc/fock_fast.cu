@@ -75,6 +75,19 @@ template <int L> __device__ __forceinline__ unsigned live_mask(int k2, int reach
 // pair 4a + b = (a, 4 + b).
 __device__ __forceinline__ bool full_tile(const PairTile& tl) { return tl.n_orb == 2 * TT && tl.n_pairs == NPAIR; }
 
+// The walk of an F1 or F3 block: an item is a row group of a group of 1 << glog tiles,
+// which the block takes one after another, so that the orbital rows (and W rows) they share
+// come from L2 the second time. Unit u is tile u % (1 << glog) of the block's item u >> glog.
+template <int L> struct Walk {
+  int first, stride, glog, units;
+  __device__ __forceinline__ Walk(int n_items, int glog_)
+      : first(blockIdx.x), stride(gridDim.x), glog(glog_),
+        units(((n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1) << glog_) {}
+  __device__ __forceinline__ int item(int u) const { return first + (u >> glog) * stride; }
+  __device__ __forceinline__ int tile(int u) const { return ((item(u) / Sizes<L>::RG) << glog) + (u & ((1 << glog) - 1)); }
+  __device__ __forceinline__ int rows(int u) const { return item(u) % Sizes<L>::RG; }   // row group
+};
+
 // the tile record into shared memory, asynchronously
 __device__ __forceinline__ void copy_tile(PairTile* dst, const PairTile* src, int tid) {
   static_assert(sizeof(PairTile) % 16 == 0, "copied by 16 bytes");
@@ -158,31 +171,32 @@ __device__ __forceinline__ pk2 pk_shfl_xor(pk2 a, int m) {
 // index of the first step, so one read of a left orbital serves four pairs; a full tile
 // keeps the right orbitals' values in registers for all of its left ones.
 template <int L>
-__global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES1) k_fast_f1(const PairTile* __restrict__ tiles, int n_items,
+__global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES1) k_fast_f1(const PairTile* __restrict__ tiles, int n_items, int glog,
                                                           pk2* __restrict__ X, const float2* __restrict__ tw_g,
                                                           int reach) {
   grid_entry();
   using S = Sizes<L>;
-  constexpr int M = S::M, MP = S::MP, QS = S::QS, RG = S::RG;
+  constexpr int M = S::M, MP = S::MP, QS = S::QS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) PairTile ring[3];   // the tiles of this item, the next and the one after
   pk2* tw = reinterpret_cast<pk2*>(smem_raw);
   float2* orb = reinterpret_cast<float2*>(smem_raw + S::tw_bytes);
   pk2* ex = reinterpret_cast<pk2*>(smem_raw + S::tw_bytes + S::orb_bytes);
-  const int tid = threadIdx.x, stride = gridDim.x;
-  copy_tile(&ring[0], tiles + blockIdx.x / RG, tid);
-  if (blockIdx.x + stride < n_items) copy_tile(&ring[1], tiles + (blockIdx.x + stride) / RG, tid);
+  const int tid = threadIdx.x;
+  const Walk<L> walk(n_items, glog);
+  copy_tile(&ring[0], tiles + walk.tile(0), tid);
+  if (walk.units > 1) copy_tile(&ring[1], tiles + walk.tile(1), tid);
   load_twiddles<L>(tw, tw_g, tid, S::NT);
   cp_async_wait_all();
   __syncthreads();
-  load_orbitals<L>(orb, ring[0], 0, 2 * TT, (long)(blockIdx.x % RG) * (RR * L), tid);
+  load_orbitals<L>(orb, ring[0], 0, 2 * TT, (long)walk.rows(0) * (RR * L), tid);
   const int qa = tid % QB, n1 = (tid / QB) % M, rpa = tid / (QB * M);
   const int rpb = tid % RP, k2b = (tid / RP) % 8, qb = tid / (8 * RP);
   const bool first = rpa < RP;   // M < 8: the last threads only take part in the second step
   const unsigned live = live_mask<L>(k2b, reach);
   int cur = 0;
   bool was_full = false;
-  for (int item = blockIdx.x; item < n_items; item += stride) {
+  for (int u = 0; u < walk.units; ++u) {
     // After a full item four groups are in flight, orbitals (0, right), 1, 2, 3; a full item
     // waits for each as it comes to it.
     const bool piped = was_full && full_tile(ring[cur]);
@@ -190,12 +204,13 @@ __global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES1) k_fast_f1(const 
     __syncthreads();
     const int nxt = cur == 2 ? 0 : cur + 1, far = cur == 0 ? 2 : cur - 1;
     const PairTile& tl = ring[cur];
-    const bool more = item + stride < n_items;
-    const long noff = (long)((item + stride) % RG) * (RR * L);
-    if (item + 2 * stride < n_items) copy_tile(&ring[far], tiles + (item + 2 * stride) / RG, tid);
+    const bool more = u + 1 < walk.units;
+    const long noff = (long)walk.rows(u + 1) * (RR * L);
+    if (u + 2 < walk.units) copy_tile(&ring[far], tiles + walk.tile(u + 2), tid);
     const int np = tl.n_pairs;
     const bool full = full_tile(tl);
-    pk2* xb = X + (((long)(item / RG) * NPAIR + qb) * L + k2b) * (L * S::CP) + (item % RG) * RP + rpb;
+    pk2* xb = X + (((long)walk.tile(u) * NPAIR + qb) * L + k2b) * (L * S::CP) + walk.rows(u) * RP + rpb;
+    if (np == 0 && more) load_orbitals<L>(orb, ring[nxt], 0, 2 * TT, noff, tid);   // an empty tile
     pk2 b[8];
     if (full && first) {
 #pragma unroll
@@ -411,55 +426,60 @@ __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
 // as in F1: X values are loaded into registers one group of pairs (or item) ahead,
 // orbital rows refill their places asynchronously, and the additions to W do not wait.
 template <int L>
-__global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES3) k_fast_f3(const PairTile* __restrict__ tiles, int n_items,
+__global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES3) k_fast_f3(const PairTile* __restrict__ tiles, int n_items, int glog,
                                                           const pk2* __restrict__ X,
                                                           const float2* __restrict__ tw_g, int reach) {
   grid_entry();
   using S = Sizes<L>;
-  constexpr int M = S::M, MP = S::MP, QS = S::QS, RG = S::RG;
+  constexpr int M = S::M, MP = S::MP, QS = S::QS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(16) PairTile ring[3];
   pk2* tw = reinterpret_cast<pk2*>(smem_raw);
   float2* orb = reinterpret_cast<float2*>(smem_raw + S::tw_bytes);
   pk2* ex = reinterpret_cast<pk2*>(smem_raw + S::tw_bytes + S::orb_bytes);
-  const int tid = threadIdx.x, stride = gridDim.x;
-  copy_tile(&ring[0], tiles + blockIdx.x / RG, tid);
-  if (blockIdx.x + stride < n_items) copy_tile(&ring[1], tiles + (blockIdx.x + stride) / RG, tid);
+  const int tid = threadIdx.x;
+  const Walk<L> walk(n_items, glog);
+  copy_tile(&ring[0], tiles + walk.tile(0), tid);
+  if (walk.units > 1) copy_tile(&ring[1], tiles + walk.tile(1), tid);
   load_twiddles<L>(tw, tw_g, tid, S::NT);
   cp_async_wait_all();
   __syncthreads();
-  load_orbitals<L>(orb, ring[0], 0, 2 * TT, (long)(blockIdx.x % RG) * (RR * L), tid);
+  load_orbitals<L>(orb, ring[0], 0, 2 * TT, (long)walk.rows(0) * (RR * L), tid);
   const int qa = tid % QB, n1 = (tid / QB) % M, rpa = tid / (QB * M);
   const int rpb = tid % RP, k2b = (tid / RP) % 8, qb = tid / (8 * RP);
   const bool second = rpa < RP;   // M < 8: the last threads only take part in the first step
   const unsigned live = live_mask<L>(k2b, reach);
   const pk2 zero = {f2(0.f), f2(0.f)};
   pk2 x[M];
-  // X values of pairs p0.. of an item into registers
-  auto load_x = [&](int item, int p0, int np) {
+  // X values of pairs p0.. of a unit into registers
+  auto load_x = [&](int u, int p0, int np) {
     if (qb < QB && p0 + qb < np) {
-      const pk2* src = X + (((long)(item / RG) * NPAIR + p0 + qb) * L + k2b) * (L * S::CP) + (item % RG) * RP + rpb;
+      const pk2* src = X + (((long)walk.tile(u) * NPAIR + p0 + qb) * L + k2b) * (L * S::CP) + walk.rows(u) * RP + rpb;
 #pragma unroll
       for (int k1 = 0; k1 < M; ++k1)
         x[k1] = live & (1u << k1) ? load_now(src + (long)k1 * 8 * L * S::CP) : zero;
     }
   };
-  load_x(blockIdx.x, 0, ring[0].n_pairs);
+  load_x(0, 0, ring[0].n_pairs);
   int cur = 0;
   bool was_full = false;
-  for (int item = blockIdx.x; item < n_items; item += stride) {
+  for (int u = 0; u < walk.units; ++u) {
     // After a full item five groups are in flight: the right orbitals, 0, 1, 2, 3.
     const bool piped = was_full && full_tile(ring[cur]);
     if (piped) cp_async_wait<4>(); else cp_async_wait_all();
     __syncthreads();
     const int nxt = cur == 2 ? 0 : cur + 1, far = cur == 0 ? 2 : cur - 1;
     const PairTile& tl = ring[cur];
-    const bool more = item + stride < n_items;
-    const long noff = (long)((item + stride) % RG) * (RR * L);
-    if (item + 2 * stride < n_items) copy_tile(&ring[far], tiles + (item + 2 * stride) / RG, tid);
+    const bool more = u + 1 < walk.units;
+    const long noff = (long)walk.rows(u + 1) * (RR * L);
+    if (u + 2 < walk.units) copy_tile(&ring[far], tiles + walk.tile(u + 2), tid);
     const int np = tl.n_pairs;
     const bool full = full_tile(tl);
-    const long roff = (long)(item % RG) * (RR * L), aoff = roff + (long)2 * rpa * L + n1;
+    const long roff = (long)walk.rows(u) * (RR * L), aoff = roff + (long)2 * rpa * L + n1;
+    if (np == 0 && more) {   // an empty tile
+      load_x(u + 1, 0, ring[nxt].n_pairs);
+      load_orbitals<L>(orb, ring[nxt], 0, 2 * TT, noff, tid);
+    }
     pk2 b[8], wb[8];
     if (full && second) {
 #pragma unroll
@@ -476,8 +496,8 @@ __global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES3) k_fast_f3(const 
 #pragma unroll
         for (int m = 1; m < M; ++m) dst[m] = ptwiddle<true>(x[m], tw[k2b * M + m]);
       }
-      if (p0 + QB < np) load_x(item, p0 + QB, np);
-      else if (more) load_x(item + stride, 0, ring[nxt].n_pairs);
+      if (p0 + QB < np) load_x(u, p0 + QB, np);
+      else if (more) load_x(u + 1, 0, ring[nxt].n_pairs);
       if (piped) {
         if (p0 == 0) cp_async_wait<3>(); else cp_async_wait<4>();
       }
@@ -584,14 +604,15 @@ static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* 
   const int reach = 2 * plan.g2_reach + 1 < L ? plan.g2_reach : L;
   const int n_live = reach >= L ? L : 2 * reach + 1;
   const int sms = sm_count();   // F1 and F3 run the blocks the chip holds at once
+  const int glog = plan.group == 4 ? 2 : 0;
   for (int l = 0; l < plan.n_launch; ++l) {
     const PairTile* tiles = plan.d_tiles + plan.launch_first[l];
-    const int nt = plan.launch_count[l], items = nt * S::RG;
+    const int nt = plan.launch_count[l], items = (nt >> glog) * S::RG;
     const unsigned g1 = (unsigned)std::min(items, S::RES1 * sms), g3 = (unsigned)std::min(items, S::RES3 * sms);
-    launch(g1, S::NT, S::smem13, s)(k_fast_f1<L>, tiles, items, X, tw, reach);
+    launch(g1, S::NT, S::smem13, s)(k_fast_f1<L>, tiles, items, glog, X, tw, reach);
     dim3 g2((unsigned)n_live, (unsigned)(nt * NPAIR));
     launch(g2, S::NT2, S::smem2, s)(k_fast_f2<L>, X, tiles, kt2, tw, reach);
-    launch(g3, S::NT, S::smem13, s)(k_fast_f3<L>, tiles, items, X, tw, reach);
+    launch(g3, S::NT, S::smem13, s)(k_fast_f3<L>, tiles, items, glog, X, tw, reach);
     launched(3);
   }
   return cudaGetLastError();
@@ -599,6 +620,19 @@ static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* 
 
 bool fock_fast_supported(Grid3 g) {
   return g.n0 == g.n1 && g.n1 == g.n2 && (g.n0 == 32 || g.n0 == 48 || g.n0 == 64 || g.n0 == 96);
+}
+
+// Paired tiles on the fast path once the orbitals and their sums (16 bytes a point) leave L2:
+// four tiles of two pairs of blocks then read 16 orbitals' rows from memory instead of 32.
+// The order depends on the system alone, so its sums are the same in a batch, for any
+// tiles_per_launch and in the static entry. Grouped from six rounds of resident blocks on, where
+// the last, partly filled one matters little (128 orbitals at 64^3: 18.98 -> 18.44 ms, 288
+// at 96^3: 333.2 -> 331.1).
+int fock_tile_order(Grid3 g, bool mixed, int n_occ, int tile, int tiles_per_launch, bool may_group) {
+  if (!mixed || !fock_fast_supported(g) || 16.0 * g.N() * n_occ < 64e6) return TILE_ROUNDS;
+  const long nb = (n_occ + tile - 1) / tile, meetings = std::min<long>((nb + 1) / 4, tiles_per_launch / 4);
+  const int L = g.n0, res = L == 96 ? Sizes<96>::RES1 : Sizes<32>::RES1;
+  return may_group && meetings * (L * (L / RR)) >= 6L * res * sm_count() ? TILE_GROUPED : TILE_PAIRED;
 }
 
 size_t fast_khat_index(int L, int i0, int i1, int i2) {

@@ -164,6 +164,7 @@ struct FockPlan {
   int* launch_count;
   PairTile* d_tiles;      // device
   int n_tiles;
+  int group;              // consecutive tiles of a launch that share orbitals (TILE_GROUPED: 4; else 1)
   // Largest |G2| (frequency index along axis 2) a pair product can reach: twice
   // the largest |g2| of the basis. Products of band-limited orbitals vanish
   // exactly beyond it on an alias-free grid, so the fast path skips those
@@ -190,8 +191,17 @@ cudaError_t fock_pairs_fast(const FockPlan& plan, Grid3 g, const float* khat_t, 
 void fock_bind_tiles(PairTile* tiles, int n, const void* psi_r, const void* x_r, void* w_occ, void* w_x, long N,
                      size_t cs);
 // Host tile schedules. sym: pairs i <= j of n_occ orbitals; otherwise n_occ x n_x pairs.
-int fock_build_tiles(int n_occ, int n_x, int tile, int sym, int tiles_per_launch, PairTile** tiles_out,
+// order (sym only): TILE_ROUNDS; TILE_PAIRED, where two blocks meet two others, tile after
+// tile; TILE_GROUPED, the same sums in the same order, but with the four tiles of such a
+// meeting side by side in one launch (unused places are empty tiles). The tiles of a
+// launch share no output, those of a group excepted.
+enum { TILE_ROUNDS = 0, TILE_PAIRED = 1, TILE_GROUPED = 2 };
+int fock_build_tiles(int n_occ, int n_x, int tile, int sym, int order, int tiles_per_launch, PairTile** tiles_out,
                      int** launch_first, int** launch_count, int* n_launch);
+// tiles that any symmetric schedule of n_occ orbitals holds at most
+long fock_max_tiles(int n_occ, int tile);
+// the order of the symmetric tiles on grid g; may_group: for a launch of one system
+int fock_tile_order(Grid3 g, bool mixed, int n_occ, int tile, int tiles_per_launch, bool may_group);
 
 // ---- dense linear algebra (linalg.cu) -------------------------------------
 // C(M x N) = alpha * op(A) op(B) + beta * C, complex128, column-major, on the CUDA cores.

@@ -291,7 +291,7 @@ size_t carve(pt_system* sys, const pt_params* p, uintptr_t base) {
   t->part = c.take<double>(8192);
   t->red = c.take<double>(64);
   t->status = c.take<int>(16);
-  t->d_tiles_sym = c.take<pt::PairTile>((size_t)(nb * (nb - 1) / 2 + nb));
+  t->d_tiles_sym = c.take<pt::PairTile>((size_t)pt::fock_max_tiles(p->n_orb, choose_tile(p)));
   t->max_tiles_x = (size_t)nb * nb;
   t->d_tiles_x = c.take<pt::PairTile>(t->max_tiles_x);
   return c.off + 256;
@@ -398,7 +398,8 @@ pt_status init_body(pt_system* sys, const double* psi0_host) {
     int *lf = nullptr, *lc = nullptr, nl = 0;
     const int tile = choose_tile(p);
     const int tpl = tiles_per_launch(p, sys->Nf, sys->mixed);
-    const int nt = pt::fock_build_tiles(sys->ne, 0, tile, 1, tpl, &tiles, &lf, &lc, &nl);
+    const int order = pt::fock_tile_order(sys->gf, sys->mixed, sys->ne, tile, tpl, true);
+    const int nt = pt::fock_build_tiles(sys->ne, 0, tile, 1, order, tpl, &tiles, &lf, &lc, &nl);
     if (nt < 0) { sys->err = "tile schedule"; return PT_ERR_INVALID; }
     pt::fock_bind_tiles(tiles, nt, fock_orbitals_addr(sys), nullptr, sys->w_r, nullptr, sys->Nf, exchange_cs(sys));
     PT_CK(cudaMemcpyAsync(sys->d_tiles_sym, tiles, sizeof(pt::PairTile) * nt, cudaMemcpyHostToDevice, s));
@@ -411,6 +412,7 @@ pt_status init_body(pt_system* sys, const double* psi0_host) {
     sys->plan_sym.launch_count = lc;
     sys->plan_sym.d_tiles = sys->d_tiles_sym;
     sys->plan_sym.n_tiles = nt;
+    sys->plan_sym.group = order == pt::TILE_GROUPED ? 4 : 1;
     set_pair_reach(&sys->plan_sym, p);
   }
   PT_CK(cudaMemsetAsync(sys->status, 0, sizeof(int) * 16, s));
@@ -507,13 +509,16 @@ pt_status exchange_static_body(pt_system* t, const pt_params* p, const std::vect
   PT_CK(upload_fft_tables(p, t->g, t->mixed, t->tw64, t->tw32, t->khat64, t->khat32, s));
   pt::PairTile* tiles = nullptr;
   int *lf = nullptr, *lc = nullptr, nl = 0;
-  const int nt = pt::fock_build_tiles(t->ne, 0, t->plan_sym.tile, 1, t->plan_sym.tiles_per_launch, &tiles, &lf, &lc, &nl);
+  const int order = pt::fock_tile_order(t->g, t->mixed, t->ne, t->plan_sym.tile, t->plan_sym.tiles_per_launch, false);
+  const int nt = pt::fock_build_tiles(t->ne, 0, t->plan_sym.tile, 1, order, t->plan_sym.tiles_per_launch, &tiles, &lf, &lc,
+                                      &nl);
   if (nt < 0) { t->err = "pt_exchange_static: tile schedule"; return PT_ERR_INVALID; }
   pt::fock_bind_tiles(tiles, nt, fock_orbitals_addr(t), nullptr, t->w_r, nullptr, t->N, exchange_cs(t));
   t->plan_sym.n_launch = nl;
   t->plan_sym.launch_first = lf;
   t->plan_sym.launch_count = lc;
   t->plan_sym.n_tiles = nt;
+  t->plan_sym.group = 1;
   t->plan_sym.d_tiles = t->d_tiles_sym;
   set_pair_reach(&t->plan_sym, p);
   PT_CK(cudaMemsetAsync(t->status, 0, sizeof(int) * 16, s));
