@@ -276,6 +276,7 @@ pt_status pt_batch_create(pt_system* const* systems, int nsys, int pair_tile, in
   b->plan.d_tiles = d_tiles;
   b->plan.n_tiles = (int)m.tiles.size();
   b->plan.g2_reach = sys[0]->plan_sym.g2_reach;   // the systems share cell and cutoff
+  std::memcpy(b->plan.g0_reach, sys[0]->plan_sym.g0_reach, sizeof(b->plan.g0_reach));
   std::memcpy(b->plan.g1_reach, sys[0]->plan_sym.g1_reach, sizeof(b->plan.g1_reach));
   b->ev_sys.assign(sys.size(), nullptr);
   for (size_t i = 0; e == cudaSuccess && i < sys.size(); ++i) e = cudaEventCreateWithFlags(&b->ev_sys[i], cudaEventDisableTiming);

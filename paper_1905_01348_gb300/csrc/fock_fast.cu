@@ -159,6 +159,11 @@ __device__ __forceinline__ pk2 pk_shfl_xor(pk2 a, int m) {
           make_float2(__shfl_xor_sync(0xffffffffu, a.im.x, m), __shfl_xor_sync(0xffffffffu, a.im.y, m))};
 }
 
+// the largest |k0| that pair products hold at axis-2 frequency |k2| (L: all)
+struct RowReach {
+  unsigned char at[kMaxLength / 2 + 1];
+};
+
 }  // namespace
 
 // F1: pair products of RR grid rows for every pair of the tile, forward FFT along axis 2,
@@ -278,10 +283,13 @@ __global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES1) k_fast_f1(const 
 // outputs overwrite its own inputs): place (c', u, k2) = c' SC + u Q + k2 with c' = c / 2 and
 // u = (n1, p) before and (k1, c & 1, q / 2) after B; at odd u, k2 is rotated by ROT. Threads
 // of neighbouring c' (A) and of neighbouring k2 (B, C) touch distinct banks.
+// Rows k0 outside the ball that holds the pair products (a quarter of a live slab's) are not
+// stored by B and not taken by C, whose threads share the rest (288 orbitals at 96^3: 335.6 ->
+// 331.1 ms an exchange).
 template <int L>
 __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     k_fast_f2(pk2* __restrict__ X, const PairTile* __restrict__ tiles, const float2* __restrict__ kt2,
-              const float2* __restrict__ tw_g, int reach) {
+              const float2* __restrict__ tw_g, int reach, const __grid_constant__ RowReach rows) {
   grid_entry();
   using S = Sizes<L>;
   constexpr int Q = S::Q, CP = S::CP, CPQ = S::CPQ, SC = S::SC, ROT = S::ROT, NT = S::NT2;
@@ -304,6 +312,8 @@ __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     twb[t] = {make_float2(w.x, z.x), make_float2(-w.y, -z.y)};
   }
   pk2* slab = X + ((long)slot * L + i2) * (L * CP);
+  const int r0 = rows.at[min(i2, L - i2)];   // rows (frequencies k0) that hold pair products
+  auto live0 = [&](int k0) { return k0 <= r0 || k0 >= L - r0; };
   __syncthreads();
 #pragma unroll 1
   for (int t = tid; t < 8 * Q; t += NT) {
@@ -341,18 +351,22 @@ __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     }
 #pragma unroll
     for (int h = 0; h < 4; ++h)
+      if (live0(t % Q + Q * h)) {
 #pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        const pk2 a = v[h][2 * g], b = v[h][2 * g + 1];
-        (g ? r : p)[(4 * h + g) * Q] = {make_float2(a.re.x, b.re.x), make_float2(a.im.x, b.im.x)};
-        (g ? r : p)[(4 * h + 2 + g) * Q] = {make_float2(a.re.y, b.re.y), make_float2(a.im.y, b.im.y)};
+        for (int g = 0; g < 2; ++g) {
+          const pk2 a = v[h][2 * g], b = v[h][2 * g + 1];
+          (g ? r : p)[(4 * h + g) * Q] = {make_float2(a.re.x, b.re.x), make_float2(a.im.x, b.im.x)};
+          (g ? r : p)[(4 * h + 2 + g) * Q] = {make_float2(a.re.y, b.re.y), make_float2(a.im.y, b.im.y)};
+        }
       }
   }
   __syncthreads();
   const float2* kt = kt2 + (long)i2 * (L * CP);
+  const int n0 = min(L, 2 * r0 + 1);
 #pragma unroll 1
-  for (int t = tid; t < 8 * Q; t += NT) {
-    const int k2 = t % Q, k1 = (t / Q) % 4, g = t / (4 * Q);
+  for (int t = tid; t < 2 * n0; t += NT) {
+    const int g = t >= n0, j = t - g * n0, k0 = j <= r0 ? j : j + L - n0;
+    const int k2 = k0 % Q, k1 = k0 / Q;
     pk2* p = buf + (4 * k1 + g) * Q + (k2 + g * ROT) % Q;
     pk2 v[Q];
 #pragma unroll
@@ -360,7 +374,7 @@ __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     pk_dft<Q, false>(v);
 #pragma unroll
     for (int m = 0; m < Q; ++m) {
-      const float2 kk = __ldg(kt + m * 8 * Q + t);   // [m][g][k1][k2]: t itself
+      const float2 kk = __ldg(kt + (2 * m + g) * L + k0);
       v[m] = {vmul(v[m].re, kk), vmul(v[m].im, kk)};
     }
     pk_dft<Q, true>(v);
@@ -378,7 +392,11 @@ __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     for (int h = 0; h < 4; ++h)
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
-        const pk2 a = (g ? r : p)[(4 * h + g) * Q], b = (g ? r : p)[(4 * h + 2 + g) * Q];
+        pk2 a = {f2(0.f), f2(0.f)}, b = a;
+        if (live0(t % Q + Q * h)) {
+          a = (g ? r : p)[(4 * h + g) * Q];
+          b = (g ? r : p)[(4 * h + 2 + g) * Q];
+        }
         v[h][2 * g] = {make_float2(a.re.x, b.re.x), make_float2(a.im.x, b.im.x)};
         v[h][2 * g + 1] = {make_float2(a.re.y, b.re.y), make_float2(a.im.y, b.im.y)};
       }
@@ -603,6 +621,10 @@ static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* 
   const float2* kt2 = reinterpret_cast<const float2*>(khat_t);
   const int reach = 2 * plan.g2_reach + 1 < L ? plan.g2_reach : L;
   const int n_live = reach >= L ? L : 2 * reach + 1;
+  RowReach rows;
+  const bool free0 = reach < L && 2 * plan.g0_reach[0] + 1 <= L;
+  for (int k = 0; k <= kMaxLength / 2; ++k)
+    rows.at[k] = (unsigned char)(free0 && k <= plan.g2_reach ? plan.g0_reach[k] : L);
   const int sms = sm_count();   // F1 and F3 run the blocks the chip holds at once
   const int glog = plan.group == 4 ? 2 : 0;
   for (int l = 0; l < plan.n_launch; ++l) {
@@ -611,7 +633,7 @@ static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* 
     const unsigned g1 = (unsigned)std::min(items, S::RES1 * sms), g3 = (unsigned)std::min(items, S::RES3 * sms);
     launch(g1, S::NT, S::smem13, s)(k_fast_f1<L>, tiles, items, glog, X, tw, reach);
     dim3 g2((unsigned)n_live, (unsigned)(nt * NPAIR));
-    launch(g2, S::NT2, S::smem2, s)(k_fast_f2<L>, X, tiles, kt2, tw, reach);
+    launch(g2, S::NT2, S::smem2, s)(k_fast_f2<L>, X, tiles, kt2, tw, reach, rows);
     launch(g3, S::NT, S::smem13, s)(k_fast_f3<L>, tiles, items, glog, X, tw, reach);
     launched(3);
   }

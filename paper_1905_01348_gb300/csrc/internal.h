@@ -173,6 +173,7 @@ struct FockPlan {
   // Largest |G1| a pair product can reach at |G2| = k (k <= g2_reach and kMaxLength / 2): the
   // products lie in the ball of twice the basis cutoff's radius.
   unsigned char g1_reach[kMaxLength / 2 + 1];
+  unsigned char g0_reach[kMaxLength / 2 + 1];   // the same along axis 0
 };
 
 // The pair kernels of `plan` (tiles bound to their orbitals and accumulators).

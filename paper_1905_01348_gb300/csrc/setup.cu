@@ -107,23 +107,25 @@ void seeded_coefficients(const pt_params* p, double* out) {
     }
 }
 
-// The reach of pair products along axes 2 and 1 (Eq. 3: products of two basis-limited
+// The reach of pair products along axes 2, 1 and 0 (Eq. 3: products of two basis-limited
 // orbitals): at most twice the largest |g| index of the basis, and inside the ball of twice
 // the cutoff sphere's radius, |G|^2 <= 4 * 2 ecut (widened by rounding).
 void set_pair_reach(pt::FockPlan* plan, const pt_params* p) {
   std::vector<int> idx;
   basis_list(p, &idx, nullptr);
-  int m1 = 0, m2 = 0;
+  int m0 = 0, m1 = 0, m2 = 0;
   for (int v : idx) {
     m2 = std::max(m2, std::abs(freq(v % p->n[2], p->n[2])));
     m1 = std::max(m1, std::abs(freq((v / p->n[2]) % p->n[1], p->n[1])));
+    m0 = std::max(m0, std::abs(freq(v / p->n[2] / p->n[1], p->n[0])));
   }
   plan->g2_reach = 2 * m2;
   for (int k = 0; k <= pt::kMaxLength / 2; ++k) {
     const double gz = 2.0 * M_PI * k / p->cell[2];
     const double left = 8.0 * p->ecut * (1.0 + 1e-9) - gz * gz;
-    const int ball = left > 0.0 ? (int)std::floor(std::sqrt(left) * p->cell[1] / (2.0 * M_PI)) : 0;
-    plan->g1_reach[k] = (unsigned char)std::min(2 * m1, ball);
+    const double index = left > 0.0 ? std::sqrt(left) / (2.0 * M_PI) : 0.0;
+    plan->g0_reach[k] = (unsigned char)std::min(2 * m0, (int)std::floor(index * p->cell[0]));
+    plan->g1_reach[k] = (unsigned char)std::min(2 * m1, (int)std::floor(index * p->cell[1]));
   }
 }
 
