@@ -46,6 +46,10 @@ template <int L> struct Sizes {
   // 5%, and by 12% three of 192, whose 96 registers spill
   static constexpr int NT2 = L == 96 ? 192 : L == 64 ? 128 : L == 48 ? 96 : 64;
   static constexpr int MINB2 = L == 96 ? 2 : L == 64 ? 4 : 6;
+  // F2 brings the slab of the block that will take its place into L2: with two blocks an SM
+  // their loads are not hidden (96: 334.3 -> 331.1 ms, 288 orbitals); with four and more they are
+  // (64: 18.2 ms without, 18.4 with)
+  static constexpr bool AHEAD2 = L == 96;
   static constexpr int RG = L * (L / RR);               // row groups of a tile
   static constexpr int RES1 = L == 96 ? 2 : 4;          // resident F1 and F3 blocks per SM
   static constexpr int RES3 = L == 96 ? 2 : 3;
@@ -163,6 +167,10 @@ __device__ __forceinline__ pk2 pk_shfl_xor(pk2 a, int m) {
 struct RowReach {
   unsigned char at[kMaxLength / 2 + 1];
 };
+
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
+}
 
 }  // namespace
 
@@ -289,7 +297,7 @@ __global__ void __launch_bounds__(Sizes<L>::NT, Sizes<L>::RES1) k_fast_f1(const 
 template <int L>
 __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     k_fast_f2(pk2* __restrict__ X, const PairTile* __restrict__ tiles, const float2* __restrict__ kt2,
-              const float2* __restrict__ tw_g, int reach, const __grid_constant__ RowReach rows) {
+              const float2* __restrict__ tw_g, int reach, const __grid_constant__ RowReach rows, int ahead) {
   grid_entry();
   using S = Sizes<L>;
   constexpr int Q = S::Q, CP = S::CP, CPQ = S::CPQ, SC = S::SC, ROT = S::ROT, NT = S::NT2;
@@ -312,6 +320,14 @@ __global__ void __launch_bounds__(Sizes<L>::NT2, Sizes<L>::MINB2)
     twb[t] = {make_float2(w.x, z.x), make_float2(-w.y, -z.y)};
   }
   pk2* slab = X + ((long)slot * L + i2) * (L * CP);
+  // the slab of the block that takes this one's place, into L2
+  if (tid == 0 && ahead > 0) {
+    const unsigned next = blockIdx.y * gridDim.x + blockIdx.x + ahead, y = next / gridDim.x, x = next % gridDim.x;
+    if (y < gridDim.y && y % NPAIR < (unsigned)tiles[y / NPAIR].n_pairs) {
+      const int j2 = (int)x <= reach ? (int)x : (int)x + (L - (int)gridDim.x);
+      prefetch_l2(X + ((long)y * L + j2) * (L * CP), L * CP * sizeof(pk2));
+    }
+  }
   const int r0 = rows.at[min(i2, L - i2)];   // rows (frequencies k0) that hold pair products
   auto live0 = [&](int k0) { return k0 <= r0 || k0 >= L - r0; };
   __syncthreads();
@@ -633,7 +649,7 @@ static cudaError_t launch_fast(const FockPlan& plan, const float* khat_t, void* 
     const unsigned g1 = (unsigned)std::min(items, S::RES1 * sms), g3 = (unsigned)std::min(items, S::RES3 * sms);
     launch(g1, S::NT, S::smem13, s)(k_fast_f1<L>, tiles, items, glog, X, tw, reach);
     dim3 g2((unsigned)n_live, (unsigned)(nt * NPAIR));
-    launch(g2, S::NT2, S::smem2, s)(k_fast_f2<L>, X, tiles, kt2, tw, reach, rows);
+    launch(g2, S::NT2, S::smem2, s)(k_fast_f2<L>, X, tiles, kt2, tw, reach, rows, S::AHEAD2 ? S::MINB2 * sms : 0);
     launch(g3, S::NT, S::smem13, s)(k_fast_f3<L>, tiles, items, glog, X, tw, reach);
     launched(3);
   }
