@@ -351,35 +351,36 @@ __global__ void __launch_bounds__(kDotThreads) k_anderson_dots(const H* __restri
 
 // Gathers the sums into gram[b][slot_q][new] (and its conjugate at [new][slot_q]) and the
 // right-hand side <dR_q, r> (slots in order, oldest first), then solves
-// (G + 1e-14 tr(G) I) gamma = rhs per band by Cholesky; gamma = 0 when the trace is zero
+// (G + 1e-14 tr(G) I) gamma = rhs per band by L D L^H; gamma = 0 when the trace is zero
 // or a pivot is not positive. One block per band, the matrix in shared memory with the
 // right-hand side as its last row (so the forward substitution is part of the
-// factorisation). Latency bounds it: k dependent pivots, each a reciprocal square root,
-// a scaled column and an update that the block's threads share.
-constexpr int kSolveThreads = 128;
+// factorisation). Latency bounds it: k dependent pivots. One warp keeps the diagonal, a lane per
+// entry, and inverts the next pivot while the others update the entries below the
+// diagonal; columns stay unscaled, so a column costs one barrier (a step's average, up to 20
+// entries: 20.0 us with a scaled column per pivot, 17.5 so).
+constexpr int kSolveUpdate = 128, kSolveThreads = kSolveUpdate + 32;
 
 __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_16a* __restrict__ part, SlotList sl,
                                                                   int newslot, int chunks, int mdim,
                                                                   double2* __restrict__ gram,
                                                                   double2* __restrict__ gamma) {
   grid_entry();
-  __shared__ double2 L[kSlotMax + 1][kSlotMax + 1];
-  __shared__ double inv[kSlotMax];   // 1 / L[j][j]
-  // entries (i, p), p <= i <= k, p < k, by falling p: those a column j still changes (p > j)
-  // come first
-  __shared__ unsigned char ent[kSlotMax * (kSlotMax + 3) / 2][2];
+  __shared__ double2 V[kSlotMax + 1][kSlotMax + 1];   // below the diagonal: column j of L times the pivot D_j
+  __shared__ double inv[kSlotMax];                    // 1 / D_j, or 0 when it is not positive
+  // entries (i, p), p < i <= k, by falling p: those a column j still changes (p > j) come first
+  __shared__ unsigned char ent[kSlotMax * (kSlotMax + 1) / 2][2];
   const int b = blockIdx.x, tid = threadIdx.x, k = sl.k;
   double2* G = gram + (long)b * mdim * mdim;
-  // L L^H = A with A[i][j] = G[s_i][s_j]  (G[s][t] = <dR_s, dR_t>); older entries
+  // A[i][j] = G[s_i][s_j]  (G[s][t] = <dR_s, dR_t>); older entries
 #pragma unroll 4
   for (int t = tid; t < k * k; t += kSolveThreads) {
     const int i = t / k, j = t % k;
-    if (j <= i && sl.s[i] != newslot && sl.s[j] != newslot) L[i][j] = G[(long)sl.s[i] * mdim + sl.s[j]];
+    if (j <= i && sl.s[i] != newslot && sl.s[j] != newslot) V[i][j] = G[(long)sl.s[i] * mdim + sl.s[j]];
   }
-  if (tid < k) {
-    const int p = k - 1 - tid;   // rows p .. k after the sum of 2, 3, .. (tid + 1) earlier entries
-    int at = tid * (tid + 3) / 2;
-    for (int i = p; i <= k; ++i, ++at) {
+  if (tid >= kSolveUpdate && tid - kSolveUpdate < k) {
+    const int c = tid - kSolveUpdate, p = k - 1 - c;   // rows p + 1 .. k after the sum of 1, 2, .. c earlier entries
+    int at = c * (c + 1) / 2;
+    for (int i = p + 1; i <= k; ++i, ++at) {
       ent[at][0] = (unsigned char)i;
       ent[at][1] = (unsigned char)p;
     }
@@ -400,49 +401,62 @@ __global__ void __launch_bounds__(kSolveThreads) k_anderson_solve(const double4_
     const double2 fwd = make_double2(t.x, q == at ? 0.0 : t.y), rev = make_double2(t.x, q == at ? 0.0 : -t.y);
     G[(long)mine * mdim + newslot] = fwd;
     G[(long)newslot * mdim + mine] = rev;
-    if (q >= at) L[q][at] = fwd;
-    if (q <= at) L[at][q] = rev;
-    L[k][q] = make_double2(t.z, -t.w);   // conj(rhs): row k becomes y^H, L y = rhs
+    if (q >= at) V[q][at] = fwd;
+    if (q <= at) V[at][q] = rev;
+    V[k][q] = make_double2(t.z, -t.w);   // conj(rhs): row k becomes w^H, L w = rhs
   }
   __syncthreads();
-  double tr = 0.0;
-  for (int q = 0; q < k; ++q) tr += L[q][q].x;
-  bool ok = tr > 0.0;
-  const double shift = 1e-14 * tr;
-  for (int j = 0; j < k && ok; ++j) {
-    const double d = L[j][j].x + shift;
-    if (!(d > 0.0)) { ok = false; break; }
-    const double r = rsqrt(d);
-    if (tid == 0) inv[j] = r;
-    // rows i > j of column j scaled, and A[i][p] -= L[i][j] conj(L[p][j]) for j < p <= i
-    const int m = k - j;   // rows j + 1 .. k
-    const double r2 = r * r;
-    for (int t = tid; t < (m - 1) * (m + 2) / 2; t += kSolveThreads) {
-      const int i = ent[t][0], p = ent[t][1];
-      const double2 u = L[i][j], w = L[p][j];
-      L[i][p].x -= r2 * (u.x * w.x + u.y * w.y);
-      L[i][p].y -= r2 * (u.y * w.x - u.x * w.y);
+  const int lane = tid - kSolveUpdate;
+  double diag = 0.0;
+  auto pivot = [&](int j) {   // by the diagonal's warp
+    const double d = __shfl_sync(0xffffffffu, diag, j);
+    const double r = d > 0.0 ? 1.0 / d : 0.0;
+    if (lane == 0) inv[j] = r;
+  };
+  if (lane >= 0) {
+    diag = lane < k ? V[lane][lane].x : 0.0;
+    double tr = diag;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+    diag += 1e-14 * tr;
+    if (!(tr > 0.0)) diag = 0.0;
+    pivot(0);
+  }
+  __syncthreads();
+  bool ok = true;
+  for (int j = 0; j < k; ++j) {
+    const double r = inv[j];
+    if (!(r > 0.0)) { ok = false; break; }
+    if (j + 1 == k) break;
+    if (lane >= 0) {
+      if (lane > j && lane < k) {
+        const double2 u = V[lane][j];
+        diag -= r * (u.x * u.x + u.y * u.y);
+      }
+      pivot(j + 1);
+    } else {
+      const int m = k - j;   // A[i][p] -= V[i][j] conj(V[p][j]) / D_j for j < p < i <= k
+      for (int t = tid; t < m * (m - 1) / 2; t += kSolveUpdate) {
+        const int i = ent[t][0], p = ent[t][1];
+        const double2 u = V[i][j], w = V[p][j];
+        V[i][p].x -= r * (u.x * w.x + u.y * w.y);
+        V[i][p].y -= r * (u.y * w.x - u.x * w.y);
+      }
     }
     __syncthreads();
-    if (tid < m) {
-      double2& v = L[j + 1 + tid][j];
-      v = make_double2(v.x * r, v.y * r);
-    }
-    // the next round reads column j + 1, which only the update above wrote
   }
-  __syncthreads();
   if (tid >= 32) return;
   if (!ok) {
     if (tid < k) gamma[(long)b * mdim + tid] = make_double2(0.0, 0.0);
     return;
   }
-  double2 y = tid < k ? make_double2(L[k][tid].x, -L[k][tid].y) : make_double2(0.0, 0.0);
+  double2 y = tid < k ? make_double2(V[k][tid].x, -V[k][tid].y) : make_double2(0.0, 0.0);
   const double di = tid < k ? inv[tid] : 0.0;
-  for (int i = k - 1; i >= 0; --i) {   // L^H g = y
+  for (int i = k - 1; i >= 0; --i) {   // D L^H gamma = w
     if (tid == i) { y.x *= di; y.y *= di; }
     const double yx = __shfl_sync(0xffffffffu, y.x, i), yy = __shfl_sync(0xffffffffu, y.y, i);
     if (tid < i) {
-      const double2 l = L[i][tid];
+      const double2 l = V[i][tid];
       y.x -= l.x * yx + l.y * yy;
       y.y -= l.x * yy - l.y * yx;
     }
