@@ -43,6 +43,16 @@ __device__ __forceinline__ void lower_tile(int t, int& i, int& j) {
   j = t - i * (i + 1) / 2;
 }
 
+// *c = r + beta *c
+__device__ __forceinline__ void put_output(double2* c, double2 beta, double2 r) {
+  if (beta.x != 0.0 || beta.y != 0.0) {
+    const double2 o = *c;
+    r.x += beta.x * o.x - beta.y * o.y;
+    r.y += beta.x * o.y + beta.y * o.x;
+  }
+  *c = r;
+}
+
 template <typename C, typename TI, int opA, int opB>
 __global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, int ksplit, int structure,
                                              double2 alpha, const TI* __restrict__ A, long lda,
@@ -154,76 +164,66 @@ __global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, in
         part[((long)kz * N + j) * (long)M + i] = v;
         continue;
       }
-      auto put = [&](double2* c, double2 r) {
-        if (beta.x != 0.0 || beta.y != 0.0) {
-          const double2 o = *c;
-          r.x += beta.x * o.x - beta.y * o.y;
-          r.y += beta.x * o.y + beta.y * o.x;
-        }
-        *c = r;
-      };
-      put(Cm + i + (long)j * ldc, make_double2(alpha.x * v.x - alpha.y * v.y, alpha.x * v.y + alpha.y * v.x));
+      put_output(Cm + i + (long)j * ldc, beta, make_double2(alpha.x * v.x - alpha.y * v.y, alpha.x * v.y + alpha.y * v.x));
       if (structure == GEMM_HERM && i != j)   // alpha conj(v)
-        put(Cm + j + (long)i * ldc, make_double2(alpha.x * v.x + alpha.y * v.y, alpha.y * v.x - alpha.x * v.y));
+        put_output(Cm + j + (long)i * ldc, beta, make_double2(alpha.x * v.x + alpha.y * v.y, alpha.y * v.x - alpha.x * v.y));
     }
 }
 
-// Sums the split-K partials in a fixed order: G threads per entry (lanes 32 / G apart) sum
-// consecutive runs of partials, then add up pairwise. For GEMM_HERM the partials exist
-// on and below the diagonal; an entry above it is the conjugate of its mirror.
-template <int G>
-__global__ void k_splitk_reduce(int M, int N, int ksplit, int structure, double2 alpha, const double2* __restrict__ part,
-                                double2 beta, double2* __restrict__ Cm, long ldc) {
+// Sums the split-K partials in a fixed order: G groups of a block's threads (32 entries each)
+// sum consecutive runs of partials, then add up in shared memory. For GEMM_HERM the partials
+// exist on and below the diagonal; an entry above it is the conjugate of its mirror. Bound by
+// the partials' read and by FP64 additions; 32 entries side by side read whole 128-byte lines
+// (four a warp read 32 bytes of FP32 partials at a time, and took 32 us for 152 partials of
+// 128 x 128).
+template <int G, typename P>
+__global__ void __launch_bounds__(256) k_splitk_reduce(int M, int N, int ksplit, int structure, double2 alpha,
+                                                       const P* __restrict__ part, double2 beta,
+                                                       double2* __restrict__ Cm, long ldc) {
   grid_entry();
-  constexpr int E = 32 / G;   // entries per warp
+  constexpr int E = 256 / G;   // entries of a block
+  __shared__ double2 sums[G > 1 ? G - 1 : 1][E];
   const long total = (long)M * N;
-  const int lane = threadIdx.x & 31, g = lane / E;
+  const int g = threadIdx.x / E, at = threadIdx.x % E;
   const int run = (ksplit + G - 1) / G;
   const int z0 = g * run, z1 = min(ksplit, z0 + run);
-  const long warps = (long)gridDim.x * (blockDim.x >> 5);
-  for (long w = blockIdx.x * (long)(blockDim.x >> 5) + (threadIdx.x >> 5); w * E < total; w += warps) {
-    const long t = w * E + lane % E;
-    double2 s = make_double2(0.0, 0.0);
-    int i = 0, j = 0;
-    bool mirror = false;
-    if (t < total) {
-      i = (int)(t % M);
-      j = (int)(t / M);
-      mirror = structure == GEMM_HERM && i < j;
-      const double2* p = part + (mirror ? (long)i * M + j : (long)j * M + i);
-#pragma unroll 4
-      for (int kz = z0; kz < z1; ++kz) {
-        const double2 v = p[(long)kz * total];
-        s.x += v.x;
-        s.y += v.y;
-      }
+  const long t = (long)blockIdx.x * E + at;
+  const int i = (int)(t % M), j = (int)(t / M);
+  const bool in = t < total, mirror = structure == GEMM_HERM && i < j;
+  double2 s = make_double2(0.0, 0.0);
+  if (in) {
+    const P* p = part + (mirror ? (long)i * M + j : t);
+#pragma unroll 8
+    for (int kz = z0; kz < z1; ++kz) {
+      const P v = p[(long)kz * total];
+      s.x += widen(v.x);
+      s.y += widen(v.y);
     }
-#pragma unroll
-    for (int o = E; o < 32; o <<= 1) {
-      s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-      s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-    }
-    if (t >= total || g != 0) continue;
-    if (mirror) s.y = -s.y;
-    double2* c = Cm + i + (long)j * ldc;
-    double2 r = make_double2(alpha.x * s.x - alpha.y * s.y, alpha.x * s.y + alpha.y * s.x);
-    if (beta.x != 0.0 || beta.y != 0.0) {
-      const double2 o = *c;
-      r.x += beta.x * o.x - beta.y * o.y;
-      r.y += beta.x * o.y + beta.y * o.x;
-    }
-    *c = r;
   }
+  if (G > 1) {
+    if (g > 0) sums[g - 1][at] = s;
+    __syncthreads();
+    if (g > 0) return;
+#pragma unroll
+    for (int q = 0; q < G - 1; ++q) {
+      s.x += sums[q][at].x;
+      s.y += sums[q][at].y;
+    }
+  }
+  if (!in) return;
+  if (mirror) s.y = -s.y;
+  put_output(Cm + i + (long)j * ldc, beta, make_double2(alpha.x * s.x - alpha.y * s.y, alpha.x * s.y + alpha.y * s.x));
 }
 
-static cudaError_t reduce_partials(int M, int N, int ksplit, int structure, double2 alpha, const double2* part,
+template <typename P>
+static cudaError_t reduce_partials(int M, int N, int ksplit, int structure, double2 alpha, const P* part,
                                    double2 beta, double2* C, long ldc, cudaStream_t s) {
   const long total = (long)M * N;
-  // eight threads per entry while one per entry would leave the chip mostly idle
+  // eight groups while one per entry would leave the chip mostly idle
   const int G = ksplit >= 8 && total < 65536 ? 8 : 1;
-  const int blocks = (int)std::min<long>((total * G + 255) / 256, 152L * 16);
-  if (G == 8) launch(blocks, 256, 0, s)(k_splitk_reduce<8>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
-  else launch(blocks, 256, 0, s)(k_splitk_reduce<1>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  const unsigned blocks = (unsigned)((total * G + 255) / 256);
+  if (G == 8) launch(blocks, 256, 0, s)(k_splitk_reduce<8, P>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  else launch(blocks, 256, 0, s)(k_splitk_reduce<1, P>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
   launched();
   return cudaGetLastError();
 }
@@ -303,7 +303,7 @@ cudaError_t gemm32_small(int opA, int opB, int M, int N, int K, double2 alpha, c
   return gemm_impl<float2>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_elems, s, structure);
 }
 
-cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const double2* part, double2 beta, double2* C,
+cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const float2* part, double2 beta, double2* C,
                           long ldc, cudaStream_t s) {
   return reduce_partials(M, N, ksplit, GEMM_GENERAL, alpha, part, beta, C, ldc, s);
 }
