@@ -189,8 +189,9 @@ template <int L> struct ConvCfg {
   static constexpr int H = L / 2 + 1;                              // columns of the half spectrum
   static constexpr int HS = H | 1;                                 // odd row stride
   static constexpr int NT = L == 32 ? 128 : L == 48 ? 192 : L == 64 ? 256 : 384;   // plane kernels
-  static constexpr int NC = 8;                                     // columns of an axis-0 block
-  static constexpr int NT0 = L >= 48 && L != 64 ? 96 : 64;
+  // columns of an axis-0 block: at 32, 136 blocks of four instead of 68 of eight
+  static constexpr int NC = L == 32 ? 4 : 8;
+  static constexpr int NT0 = L == 32 ? 32 : L == 64 ? 64 : 96;
   static constexpr size_t smem_plane = sizeof(double2) * (L + L / 2 * (L + 1) + L * HS);
   static constexpr size_t smem_axis0 = sizeof(double2) * (L + L * (NC + 1));
 };
