@@ -24,16 +24,7 @@ template <typename C> __device__ __forceinline__ C csub(C a, C b) { return mk(a.
 template <typename C> __device__ __forceinline__ C cmul(C a, C b) {
   return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-// conj(a) * b
-template <typename C> __device__ __forceinline__ C cmulc(C a, C b) {
-  return mk(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
-// a * conj(b)
-template <typename C> __device__ __forceinline__ C cmul_conj(C a, C b) {
-  return mk(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
-}
 template <typename C, typename R> __device__ __forceinline__ C cscale(C a, R s) { return mk(a.x * s, a.y * s); }
-template <typename C> __device__ __forceinline__ C cconj(C a) { return mk(a.x, -a.y); }
 // multiply by -i (forward) or +i (inverse)
 template <bool INV, typename C> __device__ __forceinline__ C mul_mi(C a) {
   return INV ? mk(-a.y, a.x) : mk(a.y, -a.x);

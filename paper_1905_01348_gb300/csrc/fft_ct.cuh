@@ -1,13 +1,9 @@
-// Compile-time-sized line FFTs for the pair pipeline (lengths 32, 48, 64, 96).
+// Compile-time-sized line FFTs (lengths 32, 48, 64, 96) for the FP64 sphere transforms and
+// the convolution.
 //
 // Each length L = R1 * R2 is transformed by two Stockham stages (radix R1,
 // then radix R2 with sub-transform length R1), so one line costs two
-// shared-memory round trips. The inverse uses the reversed plan (R2, R1):
-// the forward stage 2 butterfly j reads and writes elements j + r R1, which
-// are exactly the inputs of inverse stage 1 butterfly j, so "forward stage 2,
-// multiply by the kernel, inverse stage 1" runs in registers (ct_fused).
-// Shared-memory line buffers use a padded index i + i / 8, which spreads the
-// radix-8 stride of stage-1 writes over all banks.
+// shared-memory round trips. The inverse uses the reversed plan (R2, R1).
 #pragma once
 
 #include "common.cuh"
@@ -63,19 +59,11 @@ template <> struct Plan2<96> { static constexpr int R1 = 8, R2 = 12; };
 // on 16 distinct bank pairs for row- and column-wise stages alike, and the
 // twiddle index is uniform across the warp (a shared-memory broadcast).
 
-// Shared-memory layouts: Strided<LS, ES> puts element e of line l at
-// l * LS + e * ES; kernels may define their own (a struct with a static at(l, e)).
-template <int LS, int ES> struct Strided {
-  __device__ __forceinline__ static int at(int l, int e) { return l * LS + e * ES; }
-};
-
-// One Stockham stage over lines [line0, line0 + nl) of length L, reading
-// through layout SA from `src` and writing through layout DA to `dst`
-// (src == dst: in place; every read of the stage finishes before the first
-// write). Lines at or beyond nl are skipped (NL is the per-call capacity).
-template <typename C, bool INV, int L, int R, int NS, int NL, int NT, class SA, class DA>
-__device__ __forceinline__ void ct_stage_lay(const C* src, C* dst, int nl, const C* __restrict__ tw, int tid,
-                                             int line0 = 0) {
+// One Stockham stage in place over lines [line0, line0 + nl) of length L, element e of
+// line l at l * LS + e * ES (every read of the stage finishes before the first write).
+// Lines at or beyond nl are skipped (NL is the per-call capacity).
+template <typename C, bool INV, int L, int R, int NS, int NL, int NT, int LS, int ES>
+__device__ __forceinline__ void ct_stage(C* buf, int nl, const C* __restrict__ tw, int tid, int line0 = 0) {
   constexpr int NBL = L / R;
   constexpr int MB = (NL * NBL + NT - 1) / NT;
   constexpr int TWS = L / (NS * R);
@@ -87,7 +75,7 @@ __device__ __forceinline__ void ct_stage_lay(const C* src, C* dst, int nl, const
     if (j < NBL && ll < nl) {
       const int line = line0 + ll;
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[q][r] = src[SA::at(line, j + r * NBL)];
+      for (int r = 0; r < R; ++r) v[q][r] = buf[line * LS + (j + r * NBL) * ES];
       if (NS > 1) {
         const int k = j % NS;
 #pragma unroll
@@ -110,71 +98,7 @@ __device__ __forceinline__ void ct_stage_lay(const C* src, C* dst, int nl, const
       const int k = j % NS;
       const int o = (j - k) * R + k;
 #pragma unroll
-      for (int r = 0; r < R; ++r) dst[DA::at(line, o + r * NS)] = v[q][r];
-    }
-  }
-  __syncthreads();
-}
-
-template <typename C, bool INV, int L, int R, int NS, int NL, int NT, int SLS, int SES, int DLS, int DES>
-__device__ __forceinline__ void ct_stage_io(const C* src, C* dst, int nl, const C* __restrict__ tw, int tid,
-                                            int line0 = 0) {
-  ct_stage_lay<C, INV, L, R, NS, NL, NT, Strided<SLS, SES>, Strided<DLS, DES>>(src, dst, nl, tw, tid, line0);
-}
-
-template <typename C, int L, int NL, int NT, class A>
-__device__ __forceinline__ void ct_forward_lay(C* buf, int nl, const C* tw, int tid) {
-  constexpr int R1 = Plan2<L>::R1, R2 = Plan2<L>::R2;
-  ct_stage_lay<C, false, L, R1, 1, NL, NT, A, A>(buf, buf, nl, tw, tid);
-  ct_stage_lay<C, false, L, R2, R1, NL, NT, A, A>(buf, buf, nl, tw, tid);
-}
-
-template <typename C, int L, int NL, int NT, class A>
-__device__ __forceinline__ void ct_inverse_lay(C* buf, int nl, const C* tw, int tid) {
-  constexpr int R1 = Plan2<L>::R1, R2 = Plan2<L>::R2;
-  ct_stage_lay<C, true, L, R2, 1, NL, NT, A, A>(buf, buf, nl, tw, tid);
-  ct_stage_lay<C, true, L, R1, R2, NL, NT, A, A>(buf, buf, nl, tw, tid);
-}
-
-template <typename C, bool INV, int L, int R, int NS, int NL, int NT, int LS, int ES>
-__device__ __forceinline__ void ct_stage(C* buf, int nl, const C* __restrict__ tw, int tid, int line0 = 0) {
-  ct_stage_io<C, INV, L, R, NS, NL, NT, LS, ES, LS, ES>(buf, buf, nl, tw, tid, line0);
-}
-
-// Forward stage 2 of plan (R1, R2), multiply each element by mul(line, e),
-// inverse stage 1 of plan (R2, R1); all in registers between one read and one write.
-template <typename C, int L, int NL, int NT, int LS, int ES, class Mul>
-__device__ __forceinline__ void ct_fused(C* buf, int nl, const C* __restrict__ tw, int tid, Mul mul, int line0 = 0) {
-  constexpr int R1 = Plan2<L>::R1, R2 = Plan2<L>::R2;
-  constexpr int NBL = R1;   // = L / R2
-  constexpr int MB = (NL * NBL + NT - 1) / NT;
-  C v[MB][R2];
-#pragma unroll
-  for (int q = 0; q < MB; ++q) {
-    const int b = tid + q * NT;
-    const int ll = b % NL, j = b / NL;
-    if (j < NBL && ll < nl) {
-      const int line = line0 + ll;
-      const int base = line * LS;
-#pragma unroll
-      for (int r = 0; r < R2; ++r) v[q][r] = buf[base + (j + r * R1) * ES];
-#pragma unroll
-      for (int r = 1; r < R2; ++r) v[q][r] = cmul(v[q][r], tw[r * j]);
-      dftc<R2, false>(v[q]);
-#pragma unroll
-      for (int r = 0; r < R2; ++r) v[q][r] = cscale(v[q][r], mul(line, j + r * R1));
-      dftc<R2, true>(v[q]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < MB; ++q) {
-    const int b = tid + q * NT;
-    const int ll = b % NL, j = b / NL;
-    if (j < NBL && ll < nl) {
-      const int base = (line0 + ll) * LS;
-#pragma unroll
-      for (int r = 0; r < R2; ++r) buf[base + (j * R2 + r) * ES] = v[q][r];
+      for (int r = 0; r < R; ++r) buf[line * LS + (o + r * NS) * ES] = v[q][r];
     }
   }
   __syncthreads();
