@@ -249,8 +249,10 @@ pt_status pt_launch_count(uint64_t* count);
  * element (i, k) of op(A) is A[i + k lda] for op_a = 0 and conj(A[k + i lda]) for
  * op_a = 1; likewise op(B) with ldb. op(A) is M x K, op(B) K x N, C M x N (ldc).
  * upper_b = 1 promises that op(B) is upper triangular (op(B)(k, j) = 0 for k > j),
- * which lets each output tile stop its reduction at its last column. Arithmetic: 3xTF32 (each operand split into two TF32 parts,
- * three products) with FP32 accumulation. d_ws: device scratch of ws_bytes >= 256
+ * which lets each output tile stop its reduction at its last column. Arithmetic: 3xTF32
+ * (each operand split into two TF32 parts, three products) with FP32 accumulation; an
+ * output that would leave most of its 128 x 128 tiles empty takes FP32 multiply-adds on the
+ * CUDA cores instead, with FP64 sums over the split. d_ws: device scratch of ws_bytes >= 256
  * (256-byte aligned): its first 256 bytes hold a status word, the rest takes the
  * split-K partials of long reductions (M N complex128 per split; with no room the
  * reduction is not split). Enqueued on `stream`, which is synchronised before the
