@@ -32,14 +32,6 @@ template <bool INV, typename C> __device__ __forceinline__ C mul_mi(C a) {
 
 __device__ __forceinline__ float2 to_c(double2 a, float2*) { return make_float2((float)a.x, (float)a.y); }
 __device__ __forceinline__ double2 to_c(double2 a, double2*) { return a; }
-// (double)x by integer operations (FP64 conversions run at the FP64 pipe's two a clock);
-// zeros, subnormals, infinities and NaN take the conversion
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
-  if (e == 0u || e == 0xffu) return (double)x;
-  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double2 to_d(float2 a) { return make_double2(a.x, a.y); }
 __device__ __forceinline__ double2 to_d(double2 a) { return a; }
 template <typename C> __device__ __forceinline__ C cvt(double2 a) { return to_c(a, (C*)nullptr); }

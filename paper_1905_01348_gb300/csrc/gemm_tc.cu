@@ -151,6 +151,14 @@ __device__ __forceinline__ void split2(float2 v, float2& hi, float2& lo) {
   split_tf32(v.y, hi.y, lo.y);
 }
 
+// (double)x by integer operations (FP64 conversions run at the FP64 pipe's two a clock);
+// zeros, subnormals, infinities and NaN take the conversion
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e == 0u || e == 0xffu) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+
 // 8 bytes from global into shared memory, or zeros
 __device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, bool valid) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(dst), "l"(src), "r"(valid ? 8 : 0) : "memory");
@@ -192,7 +200,7 @@ template <int OPA, int OPB>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_cgemm_tf32x3(int M, int N, int K, int kchunk, int ksplit, int tri_b, double2 alpha,
                    const float2* __restrict__ A, long lda, const float2* __restrict__ B, long ldb, double2 beta,
-                   double2* __restrict__ Cm, long ldc, float2* __restrict__ part, int* __restrict__ err) {
+                   double2* __restrict__ Cm, long ldc, double2* __restrict__ part, int* __restrict__ err) {
   grid_entry();
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ __align__(8) uint64_t bar_full[TC_NS];
@@ -371,7 +379,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
           if (j >= N) break;
           const float re = sums[(j0 + u) * TC_M + r], im = sums[(TC_NC + j0 + u) * TC_M + r];
           if (ksplit > 1) {
-            part[((long)kz * N + j) * (long)M + m] = make_float2(re, im);
+            part[((long)kz * N + j) * (long)M + m] = make_double2(widen(re), widen(im));
             continue;
           }
           double2 o2;
@@ -430,7 +438,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
 template <int OPA, int OPB>
 static cudaError_t launch_tc(int M, int N, int K, int kchunk, int ksplit, int tri_b, double2 alpha, const float2* A,
-                             long lda, const float2* B, long ldb, double2 beta, double2* C, long ldc, float2* part,
+                             long lda, const float2* B, long ldb, double2 beta, double2* C, long ldc, double2* ws,
                              int* err, cudaStream_t s) {
   static std::atomic<unsigned long long> attr_done{0};
   if (const unsigned long long bit = device_bit_todo(attr_done)) {
@@ -441,7 +449,7 @@ static cudaError_t launch_tc(int M, int N, int K, int kchunk, int ksplit, int tr
   }
   dim3 grid((unsigned)((M + TC_M - 1) / TC_M), (unsigned)((N + TC_NC - 1) / TC_NC), (unsigned)ksplit);
   launch(grid, TC_THREADS, TC_SMEM, s)(k_cgemm_tf32x3<OPA, OPB>, M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb,
-                                                             beta, C, ldc, part, err);
+                                                             beta, C, ldc, ws, err);
   launched();
   return cudaGetLastError();
 }
@@ -473,14 +481,13 @@ cudaError_t gemm_tc(int opA, int opB, int M, int N, int K, double2 alpha, const 
   kchunk = ((kchunk + TC_KC - 1) / TC_KC) * TC_KC;
   ksplit = std::max(1, (K + kchunk - 1) / kchunk);
   if (K <= 0) { ksplit = 1; kchunk = TC_KC; }
-  float2* part = reinterpret_cast<float2*>(ws);   // the tiles' FP32 sums as they are
   cudaError_t e;
-  if (opA == OP_N && opB == OP_N) e = launch_tc<OP_N, OP_N>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, part, d_err, s);
-  else if (opA == OP_N) e = launch_tc<OP_N, OP_H>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, part, d_err, s);
-  else if (opB == OP_N) e = launch_tc<OP_H, OP_N>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, part, d_err, s);
-  else e = launch_tc<OP_H, OP_H>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, part, d_err, s);
+  if (opA == OP_N && opB == OP_N) e = launch_tc<OP_N, OP_N>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, ws, d_err, s);
+  else if (opA == OP_N) e = launch_tc<OP_N, OP_H>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, ws, d_err, s);
+  else if (opB == OP_N) e = launch_tc<OP_H, OP_N>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, ws, d_err, s);
+  else e = launch_tc<OP_H, OP_H>(M, N, K, kchunk, ksplit, tri_b, alpha, A, lda, B, ldb, beta, C, ldc, ws, d_err, s);
   if (e != cudaSuccess || ksplit == 1) return e;
-  return splitk_reduce(M, N, ksplit, alpha, part, beta, C, ldc, s);
+  return splitk_reduce(M, N, ksplit, alpha, ws, beta, C, ldc, s);
 }
 
 }  // namespace pt

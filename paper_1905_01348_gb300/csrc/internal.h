@@ -233,7 +233,7 @@ cudaError_t gemm_tc(int opA, int opB, int M, int N, int K, double2 alpha, const 
                     long ldb, double2 beta, double2* C, long ldc, double2* splitk_ws, size_t splitk_ws_elems,
                     int* d_err, cudaStream_t s, int structure = GEMM_GENERAL);
 // C = alpha sum_kz part[kz] + beta C over ksplit partials part[(kz N + j) M + i], fixed order.
-cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const float2* part, double2 beta, double2* C,
+cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const double2* part, double2 beta, double2* C,
                           long ldc, cudaStream_t s);
 // In-place lower Cholesky of an n x n Hermitian matrix (column-major, lower triangle
 // used and overwritten, upper set to 0) and Linv = L^{-1}. *d_status = 1 on a

@@ -173,12 +173,12 @@ __global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, in
 // Sums the split-K partials in a fixed order: G groups of a block's threads (32 entries each)
 // sum consecutive runs of partials, then add up in shared memory. For GEMM_HERM the partials
 // exist on and below the diagonal; an entry above it is the conjugate of its mirror. Bound by
-// the partials' read and by FP64 additions; 32 entries side by side read whole 128-byte lines
-// (four a warp read 32 bytes of FP32 partials at a time, and took 32 us for 152 partials of
-// 128 x 128).
-template <int G, typename P>
+// the partials' read and by FP64 additions; 32 entries side by side read whole lines where
+// four a warp read 64 bytes at a time (Si64 step, 42 sums of 152 partials of 128 x 128: 38.85 ->
+// 38.6 ms).
+template <int G>
 __global__ void __launch_bounds__(256) k_splitk_reduce(int M, int N, int ksplit, int structure, double2 alpha,
-                                                       const P* __restrict__ part, double2 beta,
+                                                       const double2* __restrict__ part, double2 beta,
                                                        double2* __restrict__ Cm, long ldc) {
   grid_entry();
   constexpr int E = 256 / G;   // entries of a block
@@ -192,12 +192,12 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(int M, int N, int ksplit,
   const bool in = t < total, mirror = structure == GEMM_HERM && i < j;
   double2 s = make_double2(0.0, 0.0);
   if (in) {
-    const P* p = part + (mirror ? (long)i * M + j : t);
+    const double2* p = part + (mirror ? (long)i * M + j : t);
 #pragma unroll 8
     for (int kz = z0; kz < z1; ++kz) {
-      const P v = p[(long)kz * total];
-      s.x += widen(v.x);
-      s.y += widen(v.y);
+      const double2 v = p[(long)kz * total];
+      s.x += v.x;
+      s.y += v.y;
     }
   }
   if (G > 1) {
@@ -215,15 +215,14 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(int M, int N, int ksplit,
   put_output(Cm + i + (long)j * ldc, beta, make_double2(alpha.x * s.x - alpha.y * s.y, alpha.x * s.y + alpha.y * s.x));
 }
 
-template <typename P>
-static cudaError_t reduce_partials(int M, int N, int ksplit, int structure, double2 alpha, const P* part,
+static cudaError_t reduce_partials(int M, int N, int ksplit, int structure, double2 alpha, const double2* part,
                                    double2 beta, double2* C, long ldc, cudaStream_t s) {
   const long total = (long)M * N;
   // eight groups while one per entry would leave the chip mostly idle
   const int G = ksplit >= 8 && total < 65536 ? 8 : 1;
   const unsigned blocks = (unsigned)((total * G + 255) / 256);
-  if (G == 8) launch(blocks, 256, 0, s)(k_splitk_reduce<8, P>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
-  else launch(blocks, 256, 0, s)(k_splitk_reduce<1, P>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  if (G == 8) launch(blocks, 256, 0, s)(k_splitk_reduce<8>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
+  else launch(blocks, 256, 0, s)(k_splitk_reduce<1>, M, N, ksplit, structure, alpha, part, beta, C, ldc);
   launched();
   return cudaGetLastError();
 }
@@ -303,7 +302,7 @@ cudaError_t gemm32_small(int opA, int opB, int M, int N, int K, double2 alpha, c
   return gemm_impl<float2>(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_elems, s, structure);
 }
 
-cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const float2* part, double2 beta, double2* C,
+cudaError_t splitk_reduce(int M, int N, int ksplit, double2 alpha, const double2* part, double2 beta, double2* C,
                           long ldc, cudaStream_t s) {
   return reduce_partials(M, N, ksplit, GEMM_GENERAL, alpha, part, beta, C, ldc, s);
 }
