@@ -263,9 +263,10 @@ static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alph
   const int tm = (M + GT - 1) / GT, tn = (N + GT - 1) / GT;
   if (tn > 65535) return cudaErrorInvalidValue;
   const long tiles = structure == GEMM_HERM ? (long)tm * (tm + 1) / 2 : (long)tm * tn;
-  // FP64 chunks down to one slice pay (its multiply-adds are the time); FP32 ones cost a
-  // partial to sum, so they keep four slices
-  const int least = sizeof(C) == sizeof(double2) ? 8 : 64;
+  // FP64 chunks down to half a slice pay (its multiply-adds are the time: FP64 step of Si8 5.64
+  // ms, 5.74 with whole slices); FP32 ones down to a slice (16 columns by 1,647, the
+  // products' share of a Si8 step: 2.71 ms a step, 2.74 with two slices, 2.80 with four)
+  const int least = sizeof(C) == sizeof(double2) ? 8 : 16;
   const int ksplit = K > 0 && ws != nullptr ? choose_split(tiles, K, least, (long)M * N, ws_elems) : 1;
   const int kchunk = std::max(1, (K + ksplit - 1) / ksplit);
   // GEMM_HERM: only the lower triangle's tiles, as blocks that return at once would leave some
