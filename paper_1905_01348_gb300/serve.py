@@ -286,9 +286,10 @@ class BatchedServer:
     from the budget when the group starts and returned when it ends. Systems are opened
     on their own threads (start-state relaxation can take seconds) and join their
     group's running batch at the next tick. A group with nothing running holds its first
-    tick for up to gather_s while more of its requests are being opened or are due: a batch
-    of small systems steps in little more time than one of them, and without the wait
-    requests that arrive closer together than one runs would each run alone.
+    tick while more of its requests are being opened, or are due and could be admitted with
+    the slots and memory now free: a batch of small systems steps in little more time than
+    one of them. It holds for gather_s at most, and for no longer than its last tick took
+    once it has had one: started at once, a tick keeps a later request waiting no longer.
     """
 
     def __init__(self, footprint, open_system, make_batch, budget_bytes: int, max_active: int = 8,
@@ -352,9 +353,33 @@ class BatchedServer:
                 ready[self.group_of(req)].append((req, o, system))
                 cv.notify_all()
 
+        def joins_by(key, soon):
+            # with cv held: a request of the group arrives by `soon` and could be admitted, in
+            # arrival order, with the slots and bytes that are free now
+            room, slots, starting = self.budget - used[0], len(free_slots), set()
+            for r in pending:
+                if r.arrival_s > soon or slots == 0:
+                    return False
+                k = self.group_of(r)
+                held = k in groups or k in starting
+                need = out[r.rid].footprint + (0 if held else int(self.group_reserve(k)))
+                if need > self.budget:    # will be turned away
+                    continue
+                if need > room:
+                    return False
+                if r.steps < 1:           # finishes as it is admitted
+                    continue
+                if k == key:
+                    return True
+                room -= need
+                slots -= 1
+                starting.add(k)
+            return False
+
         def worker(key):
             running = []      # [req, outcome, system, steps done]
             batch, members = None, ()
+            hold_s = self.gather_s
             while True:
                 with cv:
                     while not ready[key] and not running:
@@ -368,13 +393,11 @@ class BatchedServer:
                             cv.notify_all()
                             return
                         cv.wait(timeout=0.05)
-                    until = self.clock() + self.gather_s
+                    until = self.clock() + hold_s
                     while not running and free_slots and self.clock() < until:
-                        soon = self.clock() - t0 + self.gather_s
-                        due = any(self.group_of(r) == key and r.arrival_s <= soon for r in pending)
                         mine = sum(self.group_of(r) == key and out[r.rid].admitted_s is not None and
                                    out[r.rid].finished_s is None for r in reqs)
-                        if not due and mine == len(ready[key]):   # none is due, none is being opened
+                        if mine == len(ready[key]) and not joins_by(key, until - t0):   # nor is one being opened
                             break
                         cv.wait(timeout=0.002)
                     for req, o, system in ready[key]:
@@ -390,6 +413,7 @@ class BatchedServer:
                     t = self.clock()
                     _, infos = batch.step()
                     dt_ms = (self.clock() - t) * 1e3
+                    hold_s = min(self.gather_s, 1e-3 * dt_ms)
                 except Exception as e:   # the whole group fails this tick; every member is reported
                     msg = f"{type(e).__name__}: {e}"
                     with cv:
