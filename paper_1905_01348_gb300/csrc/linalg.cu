@@ -8,6 +8,7 @@
 // factor stop the reduction at the diagonal.
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 
 #include "common.cuh"
@@ -54,7 +55,7 @@ __device__ __forceinline__ void put_output(double2* c, double2 beta, double2 r) 
 }
 
 template <typename C, typename TI, int opA, int opB>
-__global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, int ksplit, int structure,
+__global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, int ksplit, int structure, int swapped,
                                              double2 alpha, const TI* __restrict__ A, long lda,
                                              const TI* __restrict__ B, long ldb, double2 beta,
                                              double2* __restrict__ Cm, long ldc, double2* __restrict__ part) {
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(64) k_gemm(int M, int N, int K, int kchunk, in
   __shared__ C Bs[2][GK][GT + 1];
   const int tid = threadIdx.x;
   const int tx = tid & 7, ty = tid >> 3;
-  int bi = blockIdx.x, bj = blockIdx.y;
+  int bi = swapped ? blockIdx.y : blockIdx.x, bj = swapped ? blockIdx.x : blockIdx.y;
   if (structure == GEMM_HERM) lower_tile(blockIdx.x, bi, bj);
   const int m0 = bi * GT, n0 = bj * GT, kz = blockIdx.z;
   const int kbeg = kz * kchunk;
@@ -260,9 +261,11 @@ static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alph
                              cudaStream_t s, int structure) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (structure == GEMM_HERM && M != N) return cudaErrorInvalidValue;
-  const int tm = (M + GT - 1) / GT, tn = (N + GT - 1) / GT;
-  if (tn > 65535) return cudaErrorInvalidValue;
-  const long tiles = structure == GEMM_HERM ? (long)tm * (tm + 1) / 2 : (long)tm * tn;
+  const long tm = ((long)M + GT - 1) / GT, tn = ((long)N + GT - 1) / GT;
+  const long tiles = structure == GEMM_HERM ? tm * (tm + 1) / 2 : tm * tn;
+  // grid axis y takes 65,535 tiles, x any number: a longer row of tiles goes along x
+  const int swapped = tn > 65535;
+  if (std::min(tm, tn) > 65535 || (structure == GEMM_HERM && tiles > INT_MAX)) return cudaErrorInvalidValue;
   // FP64 chunks down to half a slice pay (its multiply-adds are the time: FP64 step of Si8 5.64
   // ms, 5.74 with whole slices); FP32 ones down to a slice (16 columns by 1,647, the
   // products' share of a Si8 step: 2.71 ms a step, 2.74 with two slices, 2.80 with four)
@@ -271,9 +274,11 @@ static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alph
   const int kchunk = std::max(1, (K + ksplit - 1) / ksplit);
   // GEMM_HERM: only the lower triangle's tiles, as blocks that return at once would leave some
   // SMs with seven of the others and some with four (Psi^H Psi of Si216: 41.5 ms, 30.6 so)
-  const dim3 grid = structure == GEMM_HERM ? dim3((unsigned)tiles, 1, (unsigned)ksplit) : dim3(tm, tn, (unsigned)ksplit);
+  const dim3 grid = structure == GEMM_HERM ? dim3((unsigned)tiles, 1, (unsigned)ksplit)
+                    : swapped              ? dim3((unsigned)tn, (unsigned)tm, (unsigned)ksplit)
+                                           : dim3((unsigned)tm, (unsigned)tn, (unsigned)ksplit);
 #define PT_GEMM(OA, OB) \
-  launch(grid, 64, 0, s)(k_gemm<C, TI, OA, OB>, M, N, K, kchunk, ksplit, structure, alpha, A, lda, B, ldb, beta, Cm, ldc, ws)
+  launch(grid, 64, 0, s)(k_gemm<C, TI, OA, OB>, M, N, K, kchunk, ksplit, structure, swapped, alpha, A, lda, B, ldb, beta, Cm, ldc, ws)
   if (opA == OP_N && opB == OP_N) PT_GEMM(OP_N, OP_N);
   else if (opA == OP_N) PT_GEMM(OP_N, OP_H);
   else if (opB == OP_N) PT_GEMM(OP_H, OP_N);

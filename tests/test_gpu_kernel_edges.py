@@ -159,3 +159,19 @@ def test_product_small_outputs(pkg, op_a, op_b, M, N, K, scratch):
     pkg.pt_complex_product(op_a, op_b, M, N, K, 0.5 - 1j, dA.data_ptr(), a_shape[1], dB.data_ptr(), b_shape[1], 2j,
                            dC.data_ptr(), M, False, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
     assert rel(dC.cpu().numpy().T, exact) < 1e-5
+
+
+@pytest.mark.parametrize("op_a,op_b,M,N,K", [(0, 0, 1, 1048561, 3), (1, 0, 17, 1048577, 16), (0, 1, 3, 1100001, 5),
+                                             (0, 0, 1048577, 2, 9)])
+def test_product_long_outputs(pkg, op_a, op_b, M, N, K):
+    """Outputs of a few rows or columns whose other edge takes more than 65,535 tiles of 16."""
+    import torch
+    a_shape, b_shape = ((K, M) if op_a == 0 else (M, K)), ((N, K) if op_b == 0 else (K, N))
+    A, B = (syn.gaussian_vectors(sh, q).astype(np.complex64) for q, sh in enumerate((a_shape, b_shape)))
+    exact = (A.T if op_a == 0 else A.conj()).astype(complex) @ (B.T if op_b == 0 else B.conj())
+    dA, dB = (torch.from_numpy(np.ascontiguousarray(t)).to("cuda:0") for t in (A, B))
+    dC = torch.full((N, M), float("nan"), dtype=torch.complex128, device="cuda:0")
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda:0")
+    pkg.pt_complex_product(op_a, op_b, M, N, K, 1.0, dA.data_ptr(), a_shape[1], dB.data_ptr(), b_shape[1], 0.0,
+                           dC.data_ptr(), M, False, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
+    assert rel(dC.cpu().numpy().T, exact) < 1e-5
