@@ -241,17 +241,49 @@ int sm_count() {
   return sms;
 }
 
-// Chunks of the reduction: the blocks of an SM share its multiply pipe, so the time goes as
-// the blocks of the fullest SM times the chunk length. Take the fewest chunks within 3%
-// of the least such time that the workspace allows, none shorter than `least_chunk`.
-static int choose_split(long tiles, int K, int least_chunk, long out_elems, size_t ws_elems) {
+// Chunks of the reduction: of those that the workspace allows, the fewest within 3% (FP32: 1%)
+// of the least time. FP64: the blocks of an SM share its multiply pipe, so the time goes as the
+// blocks of the fullest SM times the chunk length, and chunks of half a slice pay (FP64 step
+// of Si8 5.64 ms, 5.74 with whole slices). FP32 (microseconds, small32_us): a block alone on
+// its SM waits for its slices, and hides the waits of a few others.
+static int choose_split64(long tiles, int K, long out_elems, size_t ws_elems) {
   const long sms = sm_count();
-  const long most = std::max<long>(1, std::min<long>({(long)(K / least_chunk), (long)(ws_elems / out_elems), 4 * sms}));
+  const long most = std::max<long>(1, std::min<long>({(long)(K / 8), (long)(ws_elems / out_elems), 4 * sms}));
   auto cost = [&](long ks) { return (double)((tiles * ks + sms - 1) / sms) * (double)((K + ks - 1) / ks); };
   double least = cost(1);
   for (long ks = 2; ks <= most; ++ks) least = std::min(least, cost(ks));
   for (long ks = 1; ks <= most; ++ks)
     if (cost(ks) <= 1.03 * least) return (int)ks;
+  return 1;
+}
+
+// Microseconds that summing ks partials of an output takes.
+static double reduce_us(long ks, long out_elems) {
+  return ks > 1 ? 2.0 + 1.5e-5 * (double)out_elems + (double)ks * (double)out_elems * 32 / 8e6 : 0.0;
+}
+
+// The FP32 kernel on `tiles` tiles of 16 x 16 in ks chunks: a step along the reduction takes a
+// block alone on its SM 54 ns, b blocks 16 + 10.3 b (fitted to 33 products, 16 x 16 to 4096 x
+// 32 by 300 to 60,000, each in 1 to 1024 chunks; 32 x 300 by 60,000 took 830 us in the four
+// chunks that give every SM one block, 191 in 128).
+static double small32_us(long tiles, long K, long ks, long out_elems) {
+  const long sms = sm_count(), blocks = (tiles * ks + sms - 1) / sms;
+  const long steps = ((K + ks - 1) / ks + GK - 1) / GK * GK;
+  return 1e-3 * (double)steps * std::max(54.0, 16.0 + 10.3 * (double)blocks) + reduce_us(ks, out_elems);
+}
+
+static int choose_split32(long tiles, int K, long out_elems, size_t ws_elems) {
+  const long slices = ((long)K + GK - 1) / GK;
+  const long most = std::max<long>(1, std::min<long>({slices, (long)(ws_elems / out_elems), 256}));
+  // the fewest chunks of each length: q slices, then q - 1 or the next that leaves fewer chunks
+  auto next = [&](long ks) {
+    const long q = (slices + ks - 1) / ks;
+    return q > 1 ? (slices + q - 2) / (q - 1) : most + 1;
+  };
+  double least = small32_us(tiles, K, 1, out_elems);
+  for (long ks = next(1); ks <= most; ks = next(ks)) least = std::min(least, small32_us(tiles, K, ks, out_elems));
+  for (long ks = 1; ks <= most; ks = next(ks))
+    if (small32_us(tiles, K, ks, out_elems) <= 1.01 * least) return (int)ks;
   return 1;
 }
 
@@ -266,11 +298,10 @@ static cudaError_t gemm_impl(int opA, int opB, int M, int N, int K, double2 alph
   // grid axis y takes 65,535 tiles, x any number: a longer row of tiles goes along x
   const int swapped = tn > 65535;
   if (std::min(tm, tn) > 65535 || (structure == GEMM_HERM && tiles > INT_MAX)) return cudaErrorInvalidValue;
-  // FP64 chunks down to half a slice pay (its multiply-adds are the time: FP64 step of Si8 5.64
-  // ms, 5.74 with whole slices); FP32 ones down to a slice (16 columns by 1,647, the
-  // products' share of a Si8 step: 2.71 ms a step, 2.74 with two slices, 2.80 with four)
-  const int least = sizeof(C) == sizeof(double2) ? 8 : 16;
-  const int ksplit = K > 0 && ws != nullptr ? choose_split(tiles, K, least, (long)M * N, ws_elems) : 1;
+  int ksplit = 1;
+  if (K > 0 && ws != nullptr)
+    ksplit = sizeof(C) == sizeof(double2) ? choose_split64(tiles, K, (long)M * N, ws_elems)
+                                          : choose_split32(tiles, K, (long)M * N, ws_elems);
   const int kchunk = std::max(1, (K + ksplit - 1) / ksplit);
   // GEMM_HERM: only the lower triangle's tiles, as blocks that return at once would leave some
   // SMs with seven of the others and some with four (Psi^H Psi of Si216: 41.5 ms, 30.6 so)

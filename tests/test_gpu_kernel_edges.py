@@ -175,3 +175,20 @@ def test_product_long_outputs(pkg, op_a, op_b, M, N, K):
     pkg.pt_complex_product(op_a, op_b, M, N, K, 1.0, dA.data_ptr(), a_shape[1], dB.data_ptr(), b_shape[1], 0.0,
                            dC.data_ptr(), M, False, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
     assert rel(dC.cpu().numpy().T, exact) < 1e-5
+
+
+@pytest.mark.parametrize("op_a,op_b,M,N,K,scratch", [(1, 0, 32, 300, 20000, True), (0, 1, 2000, 32, 6000, True),
+                                                     (1, 0, 16, 16, 70001, True), (1, 1, 40, 40, 33, True),
+                                                     (0, 0, 300, 17, 9999, False), (1, 0, 1, 1, 4097, True)])
+def test_product_long_reductions(pkg, op_a, op_b, M, N, K, scratch):
+    """Small outputs whose reduction takes few to the most chunks, ragged last ones included."""
+    import torch
+    a_shape, b_shape = ((K, M) if op_a == 0 else (M, K)), ((N, K) if op_b == 0 else (K, N))
+    A, B = (syn.gaussian_vectors(sh, q).astype(np.complex64) for q, sh in enumerate((a_shape, b_shape)))
+    exact = (A.T if op_a == 0 else A.conj()).astype(complex) @ (B.T if op_b == 0 else B.conj())
+    dA, dB = (torch.from_numpy(np.ascontiguousarray(t)).to("cuda:0") for t in (A, B))
+    dC = torch.full((N, M), float("nan"), dtype=torch.complex128, device="cuda:0")
+    ws = torch.empty((64 << 20) if scratch else 256, dtype=torch.uint8, device="cuda:0")
+    pkg.pt_complex_product(op_a, op_b, M, N, K, 1.0, dA.data_ptr(), a_shape[1], dB.data_ptr(), b_shape[1], 0.0,
+                           dC.data_ptr(), M, False, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
+    assert rel(dC.cpu().numpy().T, exact) < 1e-5
