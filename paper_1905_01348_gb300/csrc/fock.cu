@@ -47,33 +47,41 @@ static const cplx<T>* twp(const DevTwiddles& tw, int L) {
 
 // ---------------------------------------------------------------------------
 // Lines in shared memory, L = R M, take two in-place steps: A, R-point DFTs, and B, M-point
-// DFTs. For 24 = 8 x 3 and 48 = 16 x 3 (coprime factors) element 3 q + R m (mod L) has index q
-// in step A and m in step B, without twiddles; otherwise element m + M q has, and step A
-// applies W_L^(m q). place_of(k) is where frequency k ends: (R + 3) k mod L, or
+// DFTs. For M = 3 (24 = 8 x 3, 48 = 16 x 3, 12 = 4 x 3: coprime factors) element 3 q + R m (mod
+// L) has index q in step A and m in step B, without twiddles; otherwise element m + M q has,
+// and step A applies W_L^(m q). place_of(k) is where frequency k ends: (R + 3) k mod L, or
 // M (k mod R) + k / R. The inverse starts from there.
+//
+// Few lines (FEW, FP64): a codelet per line of 8 to 16 points leaves most of a warp idle when
+// there are fewer than 32 lines, and the FP64 pipe, which bounds the kernels, is as long busy with
+// a part of a warp as with all of it. Such lines take R = 4 (F2 of slabs of two short axes, a
+// launch of 32 pairs on 16 x 16 x 64 points: 133 us with 16-point codelets, 55 so).
 template <typename T> struct value_of;
 template <> struct value_of<float> { using type = cf; };
 template <> struct value_of<double> { using type = cd; };
 
-__host__ __device__ constexpr bool coprime(int L) { return L == 24 || L == 48; }
-__host__ __device__ constexpr int first_radix(int L) { return L == 12 ? 12 : L == 16 || L == 48 ? 16 : 8; }
-__device__ __forceinline__ int place_of(int k, int L) {
-  const int R = first_radix(L), M = L / R;
-  return coprime(L) ? (R + 3) * k % L : M * (k % R) + k / R;
+template <bool FEW> __host__ __device__ constexpr int first_radix(int L) {
+  return FEW ? 4 : L == 12 ? 12 : L == 16 || L == 48 ? 16 : 8;
 }
-__device__ __forceinline__ int freq_at(int place, int L) {
-  const int R = first_radix(L), M = L / R;
-  return coprime(L) ? (L == 24 ? 11 : 43) * place % L : place / M + R * (place % M);
+template <bool FEW> __host__ __device__ constexpr bool coprime(int L) { return L == 3 * first_radix<FEW>(L); }
+template <bool FEW = false> __device__ __forceinline__ int place_of(int k, int L) {
+  const int R = first_radix<FEW>(L), M = L / R;
+  return coprime<FEW>(L) ? (R + 3) * k % L : M * (k % R) + k / R;
+}
+// (the inverses of 7 mod 12, 11 mod 24 and 19 mod 48)
+template <bool FEW = false> __device__ __forceinline__ int freq_at(int place, int L) {
+  const int R = first_radix<FEW>(L), M = L / R;
+  return coprime<FEW>(L) ? (L == 12 ? 7 : L == 24 ? 11 : 43) * place % L : place / M + R * (place % M);
 }
 
 // Transforms `nlines` lines: element e of line i at buf[lines(i) + e es].
-template <int L, bool INV, typename V, class Lines>
+template <int L, bool INV, bool FEW, typename V, class Lines>
 __device__ __forceinline__ void line_pass(V* buf, int nlines, int es, const V* tw, int tid, int nthr, Lines lines) {
-  constexpr int R = first_radix(L), M = L / R;
-  constexpr bool twiddled = M > 1 && !coprime(L);
+  constexpr int R = first_radix<FEW>(L), M = L / R;
+  constexpr bool twiddled = M > 1 && !coprime<FEW>(L);
   // element q of the DFT number m of step A (b = false), element m of DFT q of step B
   auto at = [](int q, int m) {
-    if (!coprime(L)) return m + M * q;
+    if (!coprime<FEW>(L)) return m + M * q;
     const int e = 3 * q + R * m;
     return e >= L ? e - L : e;
   };
@@ -122,18 +130,53 @@ __device__ __forceinline__ void line_pass(V* buf, int nlines, int es, const V* t
   }
 }
 
-template <bool INV, typename V, class Lines>
+template <bool INV, bool FEW = false, typename V, class Lines>
 __device__ __forceinline__ void line_pass_any(V* buf, int L, int nlines, int es, const V* tw, int tid, int nthr,
                                               Lines lines) {
   switch (L) {
-    case 8: line_pass<8, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
-    case 12: line_pass<12, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
-    case 16: line_pass<16, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
-    case 24: line_pass<24, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
-    case 32: line_pass<32, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
-    case 48: line_pass<48, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
-    case 64: line_pass<64, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
-    case 96: line_pass<96, INV>(buf, nlines, es, tw, tid, nthr, lines); break;
+    case 8: line_pass<8, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); return;
+    case 12: line_pass<12, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); return;
+    case 16: line_pass<16, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); return;
+    default: break;
+  }
+  if constexpr (!FEW) {
+    switch (L) {
+      case 24: line_pass<24, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); break;
+      case 32: line_pass<32, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); break;
+      case 48: line_pass<48, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); break;
+      case 64: line_pass<64, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); break;
+      case 96: line_pass<96, INV, FEW>(buf, nlines, es, tw, tid, nthr, lines); break;
+      default: break;
+    }
+  }
+}
+
+// whether F1 and F3 take the transforms of few lines for a tile's lines
+template <typename T> __device__ __forceinline__ bool few_lines(int L, int nlines) {
+  return sizeof(T) == 8 && L <= 16 && nlines < 32;
+}
+
+// where the frequencies of a line are, by the transforms of many and (FP64) of few lines: a
+// table, as the divisions for a length known at run time took F1 and F3 a tenth of their time
+// (FP32, 33 orbitals on 32 x 32 x 64 points: 1640 us an exchange without, 1495 so)
+template <typename T, int L>
+__device__ __forceinline__ void load_places_of(unsigned char (&places)[2][kMaxLength], int tid, int nthr) {
+  for (int t = tid; t < L; t += nthr) {
+    places[0][t] = (unsigned char)place_of(t, L);
+    if (sizeof(T) == 8 && L <= 16) places[1][t] = (unsigned char)place_of<true>(t, L);
+  }
+}
+template <typename T>
+__device__ __forceinline__ void load_places(unsigned char (&places)[2][kMaxLength], int L, int tid, int nthr) {
+  switch (L) {
+    case 8: load_places_of<T, 8>(places, tid, nthr); break;
+    case 12: load_places_of<T, 12>(places, tid, nthr); break;
+    case 16: load_places_of<T, 16>(places, tid, nthr); break;
+    case 24: load_places_of<T, 24>(places, tid, nthr); break;
+    case 32: load_places_of<T, 32>(places, tid, nthr); break;
+    case 48: load_places_of<T, 48>(places, tid, nthr); break;
+    case 64: load_places_of<T, 64>(places, tid, nthr); break;
+    case 96: load_places_of<T, 96>(places, tid, nthr); break;
     default: break;
   }
 }
@@ -152,14 +195,20 @@ struct PairReach {
 
 __device__ __forceinline__ bool live(int k, int n, int reach) { return k <= reach || k >= n - reach; }
 
+// Blocks of 256 threads that share an SM's registers. FP64 needs those of two. FP32 is bound by
+// latency and memory, and four of 64 registers fit without a spill (16 orbitals on 96 x 64 x 64
+// points: 2026 us an exchange with the 72 to 80 registers the compiler would take, 1878 so).
+template <typename T> struct PairBlocks { static constexpr int value = sizeof(T) == 8 ? 2 : 4; };
+
 template <typename T>
-__global__ void __launch_bounds__(256, 2) k_fock_f1(const PairTile* __restrict__ tiles, int tile0,
+__global__ void __launch_bounds__(256, PairBlocks<T>::value) k_fock_f1(const PairTile* __restrict__ tiles, int tile0,
                                                     cplx<T>* __restrict__ Xc, int n0, int n1, int n2, int rr,
                                                     int reach2, const cplx<T>* __restrict__ tw_g) {
   grid_entry();
   using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PairTile tl;
+  __shared__ unsigned char places[2][kMaxLength];
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int rowlen = rr * n2, ls = n2 + 1;
   V* X = reinterpret_cast<V*>(Xc);
@@ -169,11 +218,13 @@ __global__ void __launch_bounds__(256, 2) k_fock_f1(const PairTile* __restrict__
   for (int t = tid; t < (int)(sizeof(PairTile) / 4); t += nthr)
     reinterpret_cast<unsigned*>(&tl)[t] = reinterpret_cast<const unsigned*>(tiles + tile0 + blockIdx.y)[t];
   load_tw(tw, tw_g, n2, tid, nthr);
+  load_places<T>(places, n2, tid, nthr);
   __syncthreads();
   const int nb1 = n1 / rr;
   const int i0 = blockIdx.x / nb1;
   const int i1s = (blockIdx.x - i0 * nb1) * rr;
   const long roff = ((long)i0 * n1 + i1s) * n2;
+  const bool few = few_lines<T>(n2, tl.n_pairs * rr);
   for (int o = 0; o < tl.n_orb; ++o) {
     const V* src = (const V*)tl.in[o] + roff;
     for (int e = tid; e < rowlen; e += nthr) orb[o * rowlen + e] = src[e];
@@ -186,22 +237,24 @@ __global__ void __launch_bounds__(256, 2) k_fock_f1(const PairTile* __restrict__
     work[l * ls + idx - l * n2] = V{vfma(a.re, b.re, vmul(a.im, b.im)), vdet(a.re, b.im, a.im, b.re)};   // conj(a) b
   }
   __syncthreads();
-  line_pass_any<false>(work, n2, np * rr, 1, tw, tid, nthr, [ls](int l) { return l * ls; });
+  auto rows = [ls](int l) { return l * ls; };
+  if (few) line_pass_any<false, true>(work, n2, np * rr, 1, tw, tid, nthr, rows);
+  else line_pass_any<false>(work, n2, np * rr, 1, tw, tid, nthr, rows);
   // store X[slot][i2][i0][i1s + r]; consecutive threads take consecutive r
   const long slot0 = (long)blockIdx.y * kTileMax * kTileMax;
   for (int idx = tid; idx < np * rowlen; idx += nthr) {
     const int r = idx % rr, rest = idx / rr;
     const int i2 = rest % n2, p = rest / n2;
     if (live(i2, n2, reach2))
-      X[(((slot0 + p) * n2 + i2) * n0 + i0) * n1 + i1s + r] = work[(p * rr + r) * ls + place_of(i2, n2)];
+      X[(((slot0 + p) * n2 + i2) * n0 + i0) * n1 + i1s + r] = work[(p * rr + r) * ls + places[few][i2]];
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256, 2) k_fock_f2(cplx<T>* __restrict__ Xc, const PairTile* __restrict__ tiles,
-                                                    int tile0, int n0, int n1, int n2, PairReach reach,
-                                                    const T* __restrict__ khat_t, const cplx<T>* __restrict__ tw0_g,
-                                                    const cplx<T>* __restrict__ tw1_g) {
+template <typename T, bool FEW>
+__global__ void __launch_bounds__(sizeof(T) == 8 && !FEW ? 512 : 256, FEW ? 4 : sizeof(T) == 8 ? 1 : PairBlocks<T>::value)
+    k_fock_f2(cplx<T>* __restrict__ Xc, const PairTile* __restrict__ tiles, int tile0, int n0, int n1, int n2,
+              const __grid_constant__ PairReach reach, const T* __restrict__ khat_t, const cplx<T>* __restrict__ tw0_g,
+              const cplx<T>* __restrict__ tw1_g) {
   grid_entry();
   using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -224,7 +277,7 @@ __global__ void __launch_bounds__(256, 2) k_fock_f2(cplx<T>* __restrict__ Xc, co
     int nl = 0, nd = 0;
     for (int c0 = 0; c0 < n1; c0 += 32) {
       const int c = c0 + tid;
-      const bool in = c < n1, lv = in && live(freq_at(c, n1), n1, reach1);
+      const bool in = c < n1, lv = in && live(freq_at<FEW>(c, n1), n1, reach1);
       const unsigned ml = __ballot_sync(0xffffffffu, lv), md = __ballot_sync(0xffffffffu, in && !lv);
       const unsigned below = (1u << tid) - 1u;
       if (lv) cols[nl + __popc(ml & below)] = (unsigned char)c;
@@ -234,37 +287,38 @@ __global__ void __launch_bounds__(256, 2) k_fock_f2(cplx<T>* __restrict__ Xc, co
     }
     if (tid == 0) n_cols = nl;
   }
-  V* slab = reinterpret_cast<V*>(Xc) + ((long)slot * n2 + i2) * cnt;
+  V* X = reinterpret_cast<V*>(Xc) + (long)slot * n2 * cnt;
 #pragma unroll 4
-  for (int e = tid; e < cnt; e += nthr) buf[e / n1 * ls + e % n1] = slab[e];
+  for (int e = tid; e < cnt; e += nthr) buf[e / n1 * ls + e % n1] = X[(long)i2 * cnt + e];
   __syncthreads();
   const int nc = n_cols;
   auto rows = [ls](int l) { return l * ls; };
   auto live_cols = [](int l) { return (int)cols[l]; };
-  line_pass_any<false>(buf, n1, n0, 1, tw1, tid, nthr, rows);           // axis 1
-  line_pass_any<false>(buf, n0, nc, ls, tw0, tid, nthr, live_cols);     // axis 0, live columns
+  line_pass_any<false, FEW>(buf, n1, n0, 1, tw1, tid, nthr, rows);           // axis 1
+  line_pass_any<false, FEW>(buf, n0, nc, ls, tw0, tid, nthr, live_cols);     // axis 0, live columns
   const T* kt = khat_t + (long)i2 * cnt;
   for (int e = tid; e < nc * n0; e += nthr) {
     const int r = e / nc, c = cols[e - r * nc];
     V& v = buf[r * ls + c];
-    const T k = kt[freq_at(r, n0) * n1 + freq_at(c, n1)];
+    const T k = kt[freq_at<FEW>(r, n0) * n1 + freq_at<FEW>(c, n1)];
     v = V{v.re * k, v.im * k};
   }
   for (int e = tid; e < (n1 - nc) * n0; e += nthr) buf[e / (n1 - nc) * ls + dead[e % (n1 - nc)]] = V{(T)0, (T)0};
   __syncthreads();
-  line_pass_any<true>(buf, n0, nc, ls, tw0, tid, nthr, live_cols);
-  line_pass_any<true>(buf, n1, n0, 1, tw1, tid, nthr, rows);
-  for (int e = tid; e < cnt; e += nthr) slab[e] = buf[e / n1 * ls + e % n1];
+  line_pass_any<true, FEW>(buf, n0, nc, ls, tw0, tid, nthr, live_cols);
+  line_pass_any<true, FEW>(buf, n1, n0, 1, tw1, tid, nthr, rows);
+  for (int e = tid; e < cnt; e += nthr) X[(long)i2 * cnt + e] = buf[e / n1 * ls + e % n1];
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256, 2) k_fock_f3(const PairTile* __restrict__ tiles, int tile0,
+__global__ void __launch_bounds__(256, PairBlocks<T>::value) k_fock_f3(const PairTile* __restrict__ tiles, int tile0,
                                                     const cplx<T>* __restrict__ Xc, int n0, int n1, int n2, int rr,
                                                     int reach2, const cplx<T>* __restrict__ tw_g) {
   grid_entry();
   using V = typename value_of<T>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ PairTile tl;
+  __shared__ unsigned char places[2][kMaxLength];
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int rowlen = rr * n2, ls = n2 + 1;
   const V* X = reinterpret_cast<const V*>(Xc);
@@ -274,6 +328,7 @@ __global__ void __launch_bounds__(256, 2) k_fock_f3(const PairTile* __restrict__
   for (int t = tid; t < (int)(sizeof(PairTile) / 4); t += nthr)
     reinterpret_cast<unsigned*>(&tl)[t] = reinterpret_cast<const unsigned*>(tiles + tile0 + blockIdx.y)[t];
   load_tw(tw, tw_g, n2, tid, nthr);
+  load_places<T>(places, n2, tid, nthr);
   __syncthreads();
   const int nb1 = n1 / rr;
   const int i0 = blockIdx.x / nb1;
@@ -281,11 +336,12 @@ __global__ void __launch_bounds__(256, 2) k_fock_f3(const PairTile* __restrict__
   const long roff = ((long)i0 * n1 + i1s) * n2;
   const int np = tl.n_pairs;
   const long slot0 = (long)blockIdx.y * kTileMax * kTileMax;
+  const bool few = few_lines<T>(n2, np * rr);
 #pragma unroll 4
   for (int idx = tid; idx < np * rowlen; idx += nthr) {
     const int r = idx % rr, rest = idx / rr;
     const int i2 = rest % n2, p = rest / n2;
-    work[(p * rr + r) * ls + place_of(i2, n2)] =
+    work[(p * rr + r) * ls + places[few][i2]] =
         live(i2, n2, reach2) ? X[(((slot0 + p) * n2 + i2) * n0 + i0) * n1 + i1s + r] : V{(T)0, (T)0};
   }
   for (int o = 0; o < tl.n_orb; ++o) {
@@ -293,7 +349,9 @@ __global__ void __launch_bounds__(256, 2) k_fock_f3(const PairTile* __restrict__
     for (int e = tid; e < rowlen; e += nthr) orb[o * rowlen + e] = src[e];
   }
   __syncthreads();
-  line_pass_any<true>(work, n2, np * rr, 1, tw, tid, nthr, [ls](int l) { return l * ls; });
+  auto rows = [ls](int l) { return l * ls; };
+  if (few) line_pass_any<true, true>(work, n2, np * rr, 1, tw, tid, nthr, rows);
+  else line_pass_any<true>(work, n2, np * rr, 1, tw, tid, nthr, rows);
   // each output orbital: fixed-order sum over the tile's pairs, one RMW of its row
   for (int o = 0; o < tl.n_orb; ++o) {
     if (!tl.is_out[o]) continue;
@@ -336,19 +394,27 @@ cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, 
   if (const unsigned long long bit = device_bit_todo(attr_done)) {
     e = cudaFuncSetAttribute(k_fock_f1<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_fock_f2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    e = cudaFuncSetAttribute(k_fock_f2<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_fock_f3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     attr_done.fetch_or(bit, std::memory_order_release);
   }
   if (smem13 > 200 * 1024 || smem2 > 200 * 1024) return cudaErrorInvalidConfiguration;
-  // four blocks per SM keep the FP64 pipe busy across barriers; large tiles take wider blocks
-  const int thr13 = smem13 > 50 * 1024 ? 256 : 128, thr2 = smem2 > 50 * 1024 ? 256 : 128;
+  // Threads. FP64: four blocks per SM keep its pipe busy across barriers, large tiles take wider
+  // blocks. Lines of up to 16 points (one codelet each) fill 64 threads, which pays once there
+  // are more blocks than four per SM (16 orbitals on 64 x 48 x 16 points: 1605 us an exchange
+  // with 128, 1346 so; on 24 x 8 x 16: 249 and 263). FP32: lines of 48 and more points fill 256
+  // (16 orbitals on 64 x 48 x 64: 1105 us with 128, 947 so; on 64 x 48 x 32: 514 and 592).
+  const bool few = fp64 && g.n0 <= 16 && g.n1 <= 16;
+  const int thr13 = g.n2 >= (fp64 ? 96 : 48) ? 256 : 128;
+  const int thr2 = few ? 64 : smem2 > 50 * 1024 ? 256 : 128;
   const C* tw0 = twp<T>(tw, g.n0);
   const C* tw1 = twp<T>(tw, g.n1);
   const C* tw2 = twp<T>(tw, g.n2);
   C* X = (C*)scratch;
+  auto f2 = k_fock_f2<T, false>;
+  if constexpr (sizeof(T) == 8) f2 = few ? k_fock_f2<T, true> : f2;
   // frequencies of pair products; with aliasing along axis 1 or 2 any may hold one
   PairReach reach;
   const bool free2 = 2 * plan.g2_reach + 1 <= g.n2, free1 = 2 * plan.g1_reach[0] + 1 <= g.n1;
@@ -359,10 +425,16 @@ cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, 
   for (int l = 0; l < plan.n_launch; ++l) {
     const int t0 = plan.launch_first[l], nt = plan.launch_count[l];
     dim3 g13((unsigned)(g.n0 * (g.n1 / rr)), (unsigned)nt);
-    launch(g13, thr13, smem13, s)(k_fock_f1<T>, plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
+    const int t13 = fp64 && g.n2 <= 16 && (long)g13.x * nt > 4L * sm_count() ? 64 : thr13;
+    launch(g13, t13, smem13, s)(k_fock_f1<T>, plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
     dim3 g2(n_live, (unsigned)(nt * kTileMax * kTileMax));
-    launch(g2, thr2, smem2, s)(k_fock_f2<T>, X, plan.d_tiles, t0, g.n0, g.n1, g.n2, reach, khat_t, tw0, tw1); launched();
-    launch(g13, thr13, smem13, s)(k_fock_f3<T>, plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
+    // FP64, large slabs: 512 threads (the registers of an SM) where no second block shares the
+    // SM, for its shared memory or because there are no more slabs (5 orbitals on 64 x 96 x 12
+    // points: 641 us an exchange with 256, 526 so)
+    const bool alone = fp64 && smem2 > 50 * 1024 &&
+                       (2 * smem2 > 220 * 1024 || (long)n_live * nt * kTileMax * kTileMax <= 2L * sm_count());
+    launch(g2, alone ? 512 : thr2, smem2, s)(f2, X, plan.d_tiles, t0, g.n0, g.n1, g.n2, reach, khat_t, tw0, tw1); launched();
+    launch(g13, t13, smem13, s)(k_fock_f3<T>, plan.d_tiles, t0, X, g.n0, g.n1, g.n2, rr, reach.g2, tw2); launched();
   }
   return cudaGetLastError();
 }

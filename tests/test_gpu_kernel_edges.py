@@ -192,3 +192,17 @@ def test_product_long_reductions(pkg, op_a, op_b, M, N, K, scratch):
     pkg.pt_complex_product(op_a, op_b, M, N, K, 1.0, dA.data_ptr(), a_shape[1], dB.data_ptr(), b_shape[1], 0.0,
                            dC.data_ptr(), M, False, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
     assert rel(dC.cpu().numpy().T, exact) < 1e-5
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("mixed", 2e-5)])
+@pytest.mark.parametrize("n,n_orb", [((8, 8, 16), 5), ((8, 12, 12), 3), ((12, 12, 8), 9), ((16, 12, 16), 6),
+                                     ((16, 16, 96), 2), ((12, 8, 48), 8), ((16, 24, 16), 5), ((64, 96, 12), 5),
+                                     ((96, 96, 8), 3)])
+def test_exchange_short_lines_and_large_slabs(pkg, n, n_orb, precision, tol):
+    """Slabs of two short axes, tiles of few short lines, and slabs that have an SM to themselves."""
+    w = workload(n, n_orb, precision=precision)
+    model, C0 = make(w, seed=4)
+    st = model.init_state(C0)
+    s = pkg.System(w, C0)
+    assert rel(s.exchange().cpu().numpy().T, st.W) < tol
+    s.close()
