@@ -8,8 +8,8 @@
 // Pair intermediate X: [pair slot][i2][i0][i1 / 2] of pk2, a pk2 holding i1 and i1 + 1
 // (the byte count and position of two complex64 values); only the axis-2 slabs that
 // pair products can reach are written or read.
-// Kernel table (fast_khat_index): [i2][i1 / 4][(i1 / 2) % 2][i0] pairs of K(i1), K(i1 + 1),
-// i1 even: the two frequencies one pk2 of F2's inner step holds, in the order its threads read.
+// Kernel table (fast_khat_index): [i2][i1 / 2][i0] pairs of K(i1), K(i1 + 1), i1 even: the two
+// frequencies one pk2 of F2's inner step holds, in the order its threads read.
 #include <algorithm>
 
 #include "common.cuh"
@@ -679,11 +679,6 @@ int fock_tile_order(Grid3 g, bool mixed, int n_occ, int tile, int tiles_per_laun
   const long nb = (n_occ + tile - 1) / tile, meetings = std::min<long>((nb + 1) / 4, tiles_per_launch / 4);
   const int L = g.n0, res = L == 96 ? Sizes<96>::RES1 : Sizes<32>::RES1;
   return may_group && meetings * (L * (L / RR)) >= 6L * res * sm_count() ? TILE_GROUPED : TILE_PAIRED;
-}
-
-size_t fast_khat_index(int L, int i0, int i1, int i2) {
-  const int Q = L / 4, m = i1 / 4, g = (i1 / 2) % 2;
-  return ((((size_t)i2 * Q + m) * 2 + g) * 4 + i0 / Q) * Q * 2 + (size_t)(i0 % Q) * 2 + i1 % 2;
 }
 
 cudaError_t fock_pairs_fast(const FockPlan& plan, Grid3 g, const float* khat_t, void* scratch, const float2* tw_L,

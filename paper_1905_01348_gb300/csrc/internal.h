@@ -183,7 +183,9 @@ cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, 
 // FP32 cubic fast path (fock_fast.cu): n0 == n1 == n2 in {32, 48, 64, 96}.
 bool fock_fast_supported(Grid3 g);
 // place of K(i0, i1, i2) in the kernel table of the fast path (grid of edge L)
-size_t fast_khat_index(int L, int i0, int i1, int i2);
+inline size_t fast_khat_index(int L, int i0, int i1, int i2) {
+  return (((size_t)i2 * (L / 2) + i1 / 2) * L + i0) * 2 + i1 % 2;
+}
 cudaError_t fock_pairs_fast(const FockPlan& plan, Grid3 g, const float* khat_t, void* scratch, const float2* tw_L,
                             cudaStream_t s);
 // Sets in[] / out[] of host tiles from their orbital slots: slot o reads
