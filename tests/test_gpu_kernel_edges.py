@@ -206,3 +206,23 @@ def test_exchange_short_lines_and_large_slabs(pkg, n, n_orb, precision, tol):
     s = pkg.System(w, C0)
     assert rel(s.exchange().cpu().numpy().T, st.W) < tol
     s.close()
+
+
+@pytest.mark.parametrize("edge,n_orb,groups", [(96, 49, 10), (96, 41, 13), (64, 130, 20)])
+def test_grouped_tiles_of_odd_block_counts(pkg, edge, n_orb, groups):
+    """Tiles side by side where a block has no partner (meetings of two tiles and empty places, a
+    diagonal group of one) and, with 41, rounds that take two launch groups: the sums of one tile
+    at a time, to the bit, and those of the FP64 kernels."""
+    C0 = np.random.default_rng(2).standard_normal((n_orb, make_basis(workload((edge,) * 3, 1)), 2))
+    C0 = C0.view(np.complex128)[..., 0]
+    out, launches = [], []
+    for more in (dict(precision="mixed"), dict(precision="mixed", pair_tiles_per_launch=1), dict(precision="fp64")):
+        s = pkg.System(workload((edge,) * 3, n_orb, **more), C0)
+        pkg.pt_set_timing(s.handle, True)
+        pkg.pt_get_timing(s.handle, reset=True)
+        out.append(s.exchange().clone())
+        launches.append(pkg.pt_get_timing(s.handle)[2])
+        s.close()
+    assert launches[0] == groups   # one tile after the other it would be 16, 12 and 36
+    assert out[0].equal(out[1])
+    assert float((out[0] - out[2]).abs().max() / out[2].abs().max()) < 2e-5
