@@ -473,7 +473,6 @@ static void dots_any(const H* dR, long slot_stride, const SlotList& sl, int news
     case 2: to(k_anderson_dots<H, 8>, dR, slot_stride, sl, newslot, r, npw, part); break;
     case 3: to(k_anderson_dots<H, 12>, dR, slot_stride, sl, newslot, r, npw, part); break;
     case 4: to(k_anderson_dots<H, 16>, dR, slot_stride, sl, newslot, r, npw, part); break;
-    case 5: to(k_anderson_dots<H, 20>, dR, slot_stride, sl, newslot, r, npw, part); break;
     default: to(k_anderson_dots<H, kSlotMax>, dR, slot_stride, sl, newslot, r, npw, part); break;
   }
 }

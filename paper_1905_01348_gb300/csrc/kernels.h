@@ -6,7 +6,7 @@
 
 namespace pt {
 
-constexpr int kSlotMax = 24;   // Anderson history slots a kernel accepts
+constexpr int kSlotMax = 20;   // deepest Anderson history (a multiple of four)
 struct SlotList {
   int k;                       // valid entries
   int s[kSlotMax];             // history slots, oldest first

@@ -226,3 +226,19 @@ def test_grouped_tiles_of_odd_block_counts(pkg, edge, n_orb, groups):
     assert launches[0] == groups   # one tile after the other it would be 16, 12 and 36
     assert out[0].equal(out[1])
     assert float((out[0] - out[2]).abs().max() / out[2].abs().max()) < 2e-5
+
+
+@pytest.mark.parametrize("depth", [7, 11, 16, 20])
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-10), ("mixed", 1e-4)])
+def test_anderson_deep_histories(pkg, depth, precision, tol):
+    """Every size of the history kernels, filled and wrapped around, in both history precisions."""
+    w = workload((12, 16, 24), 5, precision=precision, fock_mode="ace", scf_fixed_iters=depth + 3, anderson_dim=depth,
+                 dt=0.5)
+    w["relax_iters"] = 3
+    model, C0 = make(w, seed=2)
+    st, info_o = model.step(model.init_state(C0))
+    s = pkg.System(w, C0)
+    _, info_g = s.step()
+    assert rel(s.orbitals().T, st.Psi) < tol
+    assert abs(info_g["energy"] - info_o.energy) < tol * abs(info_o.energy)
+    s.close()
