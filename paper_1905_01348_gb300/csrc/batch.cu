@@ -152,9 +152,9 @@ size_t batch_layout(const Merged& m, int tpl, const pt_system* s0, uintptr_t bas
 
 pt_status pair_launches(pt_batch* b) {
   if (b->mixed)
-    return pt::fock_pairs<float>(b->plan, 1, b->gf, (const float*)b->khat, b->X, b->tw, b->s) == cudaSuccess
+    return pt::fock_pairs<float>(b->plan, b->gf, (const float*)b->khat, b->X, b->tw, b->s) == cudaSuccess
                ? PT_OK : PT_ERR_CUDA;
-  return pt::fock_pairs<double>(b->plan, 1, b->gf, (const double*)b->khat, b->X, b->tw, b->s) == cudaSuccess
+  return pt::fock_pairs<double>(b->plan, b->gf, (const double*)b->khat, b->X, b->tw, b->s) == cudaSuccess
              ? PT_OK : PT_ERR_CUDA;
 }
 

@@ -224,7 +224,7 @@ static pt_status exchange_sym_t(pt_system* sys, const double2* coef, double2* ou
   PT_TRY(exchange_prepare_t<T>(sys, coef));
   const T* kt = sys->mixed ? (const T*)(const void*)sys->khat32 : (const T*)(const void*)sys->khat64;
   if (sys->timing) PT_CK(cudaEventRecord(sys->ev0, sys->s));
-  PT_CK(pt::fock_pairs<T>(sys->plan_sym, 1, fock_grid(sys).g, kt, sys->scratch, sys->tw, sys->s));
+  PT_CK(pt::fock_pairs<T>(sys->plan_sym, fock_grid(sys).g, kt, sys->scratch, sys->tw, sys->s));
   if (sys->timing) {
     PT_CK(cudaEventRecord(sys->ev1, sys->s));
     PT_CK(cudaEventSynchronize(sys->ev1));
@@ -288,7 +288,7 @@ static pt_status exchange_x_t(pt_system* sys, const double2* X, int ncols, doubl
   PT_TRY(fock_orbitals<T>(sys, sys->psi, &pr));
   const T* kt = sys->mixed ? (const T*)(const void*)sys->khat32 : (const T*)(const void*)sys->khat64;
   (void)pr;   // the tiles of plan_x are bound to these orbitals, x_r and w_r
-  PT_CK(pt::fock_pairs<T>(sys->plan_x, 0, fv.g, kt, sys->scratch, sys->tw, sys->s));
+  PT_CK(pt::fock_pairs<T>(sys->plan_x, fv.g, kt, sys->scratch, sys->tw, sys->s));
   return to_basis<T>(sys, fv, sys->w_r, ncols, out, 1, nullptr, nullptr);
 }
 

@@ -59,11 +59,11 @@ template <> struct Plan2<96> { static constexpr int R1 = 8, R2 = 12; };
 // on 16 distinct bank pairs for row- and column-wise stages alike, and the
 // twiddle index is uniform across the warp (a shared-memory broadcast).
 
-// One Stockham stage in place over lines [line0, line0 + nl) of length L, element e of
+// One Stockham stage in place over nl lines of length L, element e of
 // line l at l * LS + e * ES (every read of the stage finishes before the first write).
 // Lines at or beyond nl are skipped (NL is the per-call capacity).
 template <typename C, bool INV, int L, int R, int NS, int NL, int NT, int LS, int ES>
-__device__ __forceinline__ void ct_stage(C* buf, int nl, const C* __restrict__ tw, int tid, int line0 = 0) {
+__device__ __forceinline__ void ct_stage(C* buf, int nl, const C* __restrict__ tw, int tid) {
   constexpr int NBL = L / R;
   constexpr int MB = (NL * NBL + NT - 1) / NT;
   constexpr int TWS = L / (NS * R);
@@ -73,9 +73,8 @@ __device__ __forceinline__ void ct_stage(C* buf, int nl, const C* __restrict__ t
     const int b = tid + q * NT;
     const int ll = b % NL, j = b / NL;
     if (j < NBL && ll < nl) {
-      const int line = line0 + ll;
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[q][r] = buf[line * LS + (j + r * NBL) * ES];
+      for (int r = 0; r < R; ++r) v[q][r] = buf[ll * LS + (j + r * NBL) * ES];
       if (NS > 1) {
         const int k = j % NS;
 #pragma unroll
@@ -94,11 +93,10 @@ __device__ __forceinline__ void ct_stage(C* buf, int nl, const C* __restrict__ t
     const int b = tid + q * NT;
     const int ll = b % NL, j = b / NL;
     if (j < NBL && ll < nl) {
-      const int line = line0 + ll;
       const int k = j % NS;
       const int o = (j - k) * R + k;
 #pragma unroll
-      for (int r = 0; r < R; ++r) buf[line * LS + (o + r * NS) * ES] = v[q][r];
+      for (int r = 0; r < R; ++r) buf[ll * LS + (o + r * NS) * ES] = v[q][r];
     }
   }
   __syncthreads();
@@ -106,17 +104,17 @@ __device__ __forceinline__ void ct_stage(C* buf, int nl, const C* __restrict__ t
 
 // Full forward (plan R1, R2) and inverse (plan R2, R1) line transforms in place.
 template <typename C, int L, int NL, int NT, int LS, int ES>
-__device__ __forceinline__ void ct_forward(C* buf, int nl, const C* tw, int tid, int line0 = 0) {
+__device__ __forceinline__ void ct_forward(C* buf, int nl, const C* tw, int tid) {
   constexpr int R1 = Plan2<L>::R1, R2 = Plan2<L>::R2;
-  ct_stage<C, false, L, R1, 1, NL, NT, LS, ES>(buf, nl, tw, tid, line0);
-  ct_stage<C, false, L, R2, R1, NL, NT, LS, ES>(buf, nl, tw, tid, line0);
+  ct_stage<C, false, L, R1, 1, NL, NT, LS, ES>(buf, nl, tw, tid);
+  ct_stage<C, false, L, R2, R1, NL, NT, LS, ES>(buf, nl, tw, tid);
 }
 
 template <typename C, int L, int NL, int NT, int LS, int ES>
-__device__ __forceinline__ void ct_inverse(C* buf, int nl, const C* tw, int tid, int line0 = 0) {
+__device__ __forceinline__ void ct_inverse(C* buf, int nl, const C* tw, int tid) {
   constexpr int R1 = Plan2<L>::R1, R2 = Plan2<L>::R2;
-  ct_stage<C, true, L, R2, 1, NL, NT, LS, ES>(buf, nl, tw, tid, line0);
-  ct_stage<C, true, L, R1, R2, NL, NT, LS, ES>(buf, nl, tw, tid, line0);
+  ct_stage<C, true, L, R2, 1, NL, NT, LS, ES>(buf, nl, tw, tid);
+  ct_stage<C, true, L, R1, R2, NL, NT, LS, ES>(buf, nl, tw, tid);
 }
 
 }  // namespace pt

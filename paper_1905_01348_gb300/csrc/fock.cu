@@ -378,10 +378,9 @@ static int rows_per_block(int n1, bool fp64) {
 }
 
 template <typename T>
-cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, void* scratch, const DevTwiddles& tw,
+cudaError_t fock_pairs(const FockPlan& plan, Grid3 g, const T* khat_t, void* scratch, const DevTwiddles& tw,
                        cudaStream_t s) {
   using C = cplx<T>;
-  (void)sym;   // the tiles' contribution lists know which pairs feed both orbitals
   if constexpr (sizeof(T) == 4) {
     if (fock_fast_supported(g)) return fock_pairs_fast(plan, g, khat_t, scratch, twp<float>(tw, g.n0), s);
   }
@@ -439,9 +438,9 @@ cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, 
   return cudaGetLastError();
 }
 
-template cudaError_t fock_pairs<float>(const FockPlan&, int, Grid3, const float*, void*, const DevTwiddles&,
+template cudaError_t fock_pairs<float>(const FockPlan&, Grid3, const float*, void*, const DevTwiddles&,
                                        cudaStream_t);
-template cudaError_t fock_pairs<double>(const FockPlan&, int, Grid3, const double*, void*, const DevTwiddles&,
+template cudaError_t fock_pairs<double>(const FockPlan&, Grid3, const double*, void*, const DevTwiddles&,
                                         cudaStream_t);
 
 void fock_bind_tiles(PairTile* tiles, int n, const void* psi_r, const void* x_r, void* w_occ, void* w_x, long N,

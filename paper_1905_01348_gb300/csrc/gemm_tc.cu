@@ -186,8 +186,8 @@ __device__ __forceinline__ uint32_t core_off(int r, int kc) {
 // other warp is waited for. A row's two 16-byte chunks swap places with bit 2 of the row:
 // the threads that read one row each then touch distinct banks. The overlap A^H B of 432
 // columns of Si216 (K = 43,819): 565 us of device work, 887 with the loads in registers and
-// the sums in shared memory; the split and expansion by the producers bound it (3 x 196
-// GFLOP of MMAs would take 0.21 ms).
+// the sums in shared memory; the split and expansion by the producers bound it (3 x 65
+// GFLOP take 0.21 ms at 952 TFLOP/s, 0.29 ms with the padding to 512 columns).
 //
 // Accumulation. The tensor core adds into its FP32 accumulator with truncation, so its
 // error grows linearly with the number of MMAs into one accumulator (measured: 4e-5

@@ -178,7 +178,7 @@ struct FockPlan {
 
 // The pair kernels of `plan` (tiles bound to their orbitals and accumulators).
 template <typename T>
-cudaError_t fock_pairs(const FockPlan& plan, int sym, Grid3 g, const T* khat_t, void* scratch, const DevTwiddles& tw,
+cudaError_t fock_pairs(const FockPlan& plan, Grid3 g, const T* khat_t, void* scratch, const DevTwiddles& tw,
                        cudaStream_t s);
 // FP32 cubic fast path (fock_fast.cu): n0 == n1 == n2 in {32, 48, 64, 96}.
 bool fock_fast_supported(Grid3 g);

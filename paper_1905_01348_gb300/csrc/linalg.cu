@@ -497,30 +497,6 @@ __global__ void __launch_bounds__(256) k_chol_trail(double2* __restrict__ A, int
   A[i + (long)k * n] = s;
 }
 
-__global__ void k_tri_inverse(const double2* __restrict__ L, double2* __restrict__ Li, int n);
-
-cudaError_t cholesky_inverse(double2* A, double2* Linv, int n, int* d_status, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(d_status, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
-  for (int j0 = 0; j0 < n; j0 += CB) {
-    launch(1, kCholUpdate + 32, 0, s)(k_chol_diag, A, Linv, n, j0, d_status); launched();
-    const int rest = n - j0 - CB;
-    if (rest <= 0) continue;
-    launch((rest + 7) / 8, 256, 0, s)(k_chol_panel, A, Linv, n, j0, d_status); launched();
-    const unsigned t = (unsigned)((rest + 15) / 16);
-    launch(dim3(t, t), 256, 0, s)(k_chol_trail, A, n, j0, d_status); launched();
-  }
-  if (n > CB) {
-    const size_t smem = (sizeof(double2) + sizeof(double)) * n;
-    if (smem > 48 * 1024) {
-      e = cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    launch(n, 128, smem, s)(k_tri_inverse, A, Linv, n); launched();
-  }
-  return cudaGetLastError();
-}
-
 // Column c of L^{-1}: solve L x = e_c by forward substitution (one block per column), with the
 // pivots' reciprocals taken at the start and the next column of L on its way during a step
 // (n = 128: 185 us with a division by every thread in every step, and the column then loaded).
@@ -569,6 +545,28 @@ __global__ void __launch_bounds__(128) k_tri_inverse(const double2* __restrict__
   }
   for (int i = tid; i < n; i += 128)
     Li[i + (long)c * n] = i < c ? make_double2(0.0, 0.0) : make_double2(b[i].x * rinv[i], b[i].y * rinv[i]);
+}
+
+cudaError_t cholesky_inverse(double2* A, double2* Linv, int n, int* d_status, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(d_status, 0, sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  for (int j0 = 0; j0 < n; j0 += CB) {
+    launch(1, kCholUpdate + 32, 0, s)(k_chol_diag, A, Linv, n, j0, d_status); launched();
+    const int rest = n - j0 - CB;
+    if (rest <= 0) continue;
+    launch((rest + 7) / 8, 256, 0, s)(k_chol_panel, A, Linv, n, j0, d_status); launched();
+    const unsigned t = (unsigned)((rest + 15) / 16);
+    launch(dim3(t, t), 256, 0, s)(k_chol_trail, A, n, j0, d_status); launched();
+  }
+  if (n > CB) {
+    const size_t smem = (sizeof(double2) + sizeof(double)) * n;
+    if (smem > 48 * 1024) {
+      e = cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    launch(n, 128, smem, s)(k_tri_inverse, A, Linv, n); launched();
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace pt
