@@ -257,33 +257,41 @@ static int choose_split64(long tiles, int K, long out_elems, size_t ws_elems) {
   return 1;
 }
 
-// Microseconds that summing ks partials of an output takes.
+// Microseconds that summing ks partials of an output takes: a launch, the wait for the first
+// partials of a thread, one after the other, and their bytes.
 static double reduce_us(long ks, long out_elems) {
-  return ks > 1 ? 2.0 + 1.5e-5 * (double)out_elems + (double)ks * (double)out_elems * 32 / 8e6 : 0.0;
+  if (ks <= 1) return 0.0;
+  return 2.0 + 0.06 * (double)std::min(ks, 32L) + 1.5e-5 * (double)out_elems + (double)ks * (double)out_elems * 32 / 8e6;
 }
 
 // The FP32 kernel on `tiles` tiles of 16 x 16 in ks chunks: a step along the reduction takes a
 // block alone on its SM 54 ns, b blocks 16 + 10.3 b (fitted to 33 products, 16 x 16 to 4096 x
 // 32 by 300 to 60,000, each in 1 to 1024 chunks; 32 x 300 by 60,000 took 830 us in the four
 // chunks that give every SM one block, 191 in 128).
-static double small32_us(long tiles, long K, long ks, long out_elems) {
-  const long sms = sm_count(), blocks = (tiles * ks + sms - 1) / sms;
+static double small32_us(long tiles, long K, long ks, long out_elems, long sms) {
+  const long blocks = (tiles * ks + sms - 1) / sms;
   const long steps = ((K + ks - 1) / ks + GK - 1) / GK * GK;
   return 1e-3 * (double)steps * std::max(54.0, 16.0 + 10.3 * (double)blocks) + reduce_us(ks, out_elems);
 }
 
 static int choose_split32(long tiles, int K, long out_elems, size_t ws_elems) {
-  const long slices = ((long)K + GK - 1) / GK;
-  const long most = std::max<long>(1, std::min<long>({slices, (long)(ws_elems / out_elems), 256}));
+  constexpr long kMost = 256;
+  const long sms = sm_count(), slices = ((long)K + GK - 1) / GK;
+  const long most = std::max<long>(1, std::min<long>({slices, (long)(ws_elems / out_elems), kMost}));
   // the fewest chunks of each length: q slices, then q - 1 or the next that leaves fewer chunks
-  auto next = [&](long ks) {
+  int chunks[kMost], n = 0;
+  double us[kMost], least = 0.0;
+  for (long ks = 1; ks <= most;) {
+    chunks[n] = (int)ks;
+    us[n] = small32_us(tiles, K, ks, out_elems, sms);
+    least = n == 0 ? us[0] : std::min(least, us[n]);
+    ++n;
     const long q = (slices + ks - 1) / ks;
-    return q > 1 ? (slices + q - 2) / (q - 1) : most + 1;
-  };
-  double least = small32_us(tiles, K, 1, out_elems);
-  for (long ks = next(1); ks <= most; ks = next(ks)) least = std::min(least, small32_us(tiles, K, ks, out_elems));
-  for (long ks = 1; ks <= most; ks = next(ks))
-    if (small32_us(tiles, K, ks, out_elems) <= 1.01 * least) return (int)ks;
+    if (q <= 1) break;
+    ks = (slices + q - 2) / (q - 1);
+  }
+  for (int i = 0; i < n; ++i)
+    if (us[i] <= 1.01 * least) return chunks[i];
   return 1;
 }
 
