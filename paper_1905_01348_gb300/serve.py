@@ -12,7 +12,7 @@ first step to the last, and its memory returns to the budget when it ends.
 Requests that arrive while others run are admitted the moment a slot and
 memory free up (continuous admission, not a queue drained one at a time).
 
-The library's kernels are deterministic (no atomics; fixed reduction orders)
+The library's kernels are deterministic (every sum has one order)
 and distinct systems share no device state, so a request's results are the
 same alone and in any mix; `--check-alone` re-runs every request by itself and
 reports the largest difference.
